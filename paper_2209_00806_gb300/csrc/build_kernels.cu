@@ -712,6 +712,7 @@ int build_diag2(BuildOutput &b, cudaStream_t st, std::string &msg)
     CK(cudaMalloc(&d2, (size_t)std::max<int64_t>(b.n_rows, 1) * sizeof(double)));
     k_twice<<<blocks_for(b.n_rows, 256), 256, 0, st>>>(b.n_rows, b.diag64, d2);
     cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);     // read ahead of dep_wait()
     if (e != cudaSuccess) {
         cudaFree(d2);
         msg = std::string("2 d: ") + cudaGetErrorString(e);

@@ -83,20 +83,9 @@ __device__ __forceinline__ W32F pack(const Cv<float, 4> &o)
 }
 
 // 16-byte lanes load as one vector access, 32-byte lanes as two.
-template <typename T> __device__ __forceinline__ T lane_ldg(const T *p) { return __ldg(p); }
 template <typename T> __device__ __forceinline__ T lane_ldcs(const T *p) { return __ldcs(p); }
 template <typename T> __device__ __forceinline__ T lane_ld(const T *p) { return *p; }
 template <typename T> __device__ __forceinline__ void lane_st(T *p, const T &v) { *p = v; }
-template <> __device__ __forceinline__ W32F lane_ldg(const W32F *p)
-{
-    const float4 *q = reinterpret_cast<const float4 *>(p);
-    W32F v; v.a = __ldg(q); v.b = __ldg(q + 1); return v;
-}
-template <> __device__ __forceinline__ W32D lane_ldg(const W32D *p)
-{
-    const double2 *q = reinterpret_cast<const double2 *>(p);
-    W32D v; v.a = __ldg(q); v.b = __ldg(q + 1); return v;
-}
 template <> __device__ __forceinline__ W32F lane_ldcs(const W32F *p)
 {
     const float4 *q = reinterpret_cast<const float4 *>(p);
@@ -128,13 +117,15 @@ template <> __device__ __forceinline__ void lane_st(W32D *p, const W32D &v)
     q[0] = v.a; q[1] = v.b;
 }
 
-// Load the lane data of row `r` through the read-only path.
+// Load the lane data of row `r` of a vector that this kernel does not write.
+// A plain load: the kernels are dependent launches (launch_dependent), and a
+// read-only load of a vector could be moved above dep_wait().
 template <typename V, int L, int SPL>
 __device__ __forceinline__ Cv<V, SPL> ld_ro(const void *base, int64_t r, int l)
 {
     typedef typename LaneT<V, SPL>::type Lane;
     Cv<V, SPL> o;
-    unpack(lane_ldg(reinterpret_cast<const Lane *>(base) + r * L + l), o);
+    unpack(lane_ld(reinterpret_cast<const Lane *>(base) + r * L + l), o);
     return o;
 }
 template <typename V, int L, int SPL>
@@ -331,15 +322,14 @@ __device__ __forceinline__ Cv<double, SPL> term_row_sum(const TermArgs &a, int64
     return combine_sum<SPL>(a, gd, xo, s, p, zz);
 }
 
-// CX: complex matrix values (re, im) per stored entry (Peierls phases);
-// otherwise real values.  RS > 1 splits each row's entries over RS adjacent
-// threads (part = 0 .. RS-1 takes entries part, part + RS, ...; shuffles add
-// the parts): long rows get RS times the gathers in flight.
-template <typename V, int L, int SPL, bool CX, int RS = 1>
+// Row split (real values): each row's entries over RS adjacent threads
+// (part = 0 .. RS-1 takes entries part, part + RS, ...; shuffles add the
+// parts): long rows get RS times the gathers in flight.
+template <typename V, int L, int SPL, int RS>
 __device__ __forceinline__ Cv<V, SPL> term_row(const TermArgs &a, int64_t r, int l,
-                                               const V *sc, int part = 0)
+                                               const V *sc, int part)
 {
-    if constexpr (sizeof(V) == 8 && !CX) {
+    if constexpr (sizeof(V) == 8) {
         if (a.uniform) return term_row_sum<L, SPL, RS>(a, r, l, sc, part);
     }
     Cv<V, SPL> p, zz;
@@ -374,26 +364,16 @@ __device__ __forceinline__ Cv<V, SPL> term_row(const TermArgs &a, int64_t r, int
     Cv<V, SPL> y = ld_ro<V, L, SPL>(a.x, r, l);
 #pragma unroll
     for (int j = 0; j < SPL; ++j) { y.re[j] *= d; y.im[j] *= d; }
-    typedef typename Val2<V>::type V2;
-    const V2 *valp2 = reinterpret_cast<const V2 *>(a.H.val) + base + lr;
     for (int k = part; k < w; k += 4 * RS) {
         int32_t c[4];
-        V h[4], hm[4];
+        V h[4];
         bool ok[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int ku = k + u * RS;
             ok[u] = ku < w;
             c[u] = ok[u] ? __ldg(colp + (int64_t)ku * kSliceRows) : (int32_t)r;
-            hm[u] = (V)0;
-            if (CX) {
-                V2 v2;
-                v2.x = (V)0;
-                v2.y = (V)0;
-                if (ok[u]) v2 = __ldg(valp2 + (int64_t)ku * kSliceRows);
-                h[u] = v2.x;
-                hm[u] = v2.y;
-            } else if (a.uniform) {
+            if (a.uniform) {
                 // one value for all entries; padded slots (col == own row) add nothing
                 ok[u] = ok[u] && c[u] != (int32_t)r;
                 h[u] = Coef<V>::hu(a);
@@ -411,10 +391,6 @@ __device__ __forceinline__ Cv<V, SPL> term_row(const TermArgs &a, int64_t r, int
                 for (int j = 0; j < SPL; ++j) {
                     y.re[j] = fma(h[u], xv[u].re[j], y.re[j]);
                     y.im[j] = fma(h[u], xv[u].im[j], y.im[j]);
-                    if (CX) {       // (h + i hm)(x_re + i x_im)
-                        y.re[j] = fma(-hm[u], xv[u].im[j], y.re[j]);
-                        y.im[j] = fma(hm[u], xv[u].re[j], y.im[j]);
-                    }
                 }
             }
         }
@@ -454,6 +430,246 @@ __device__ __forceinline__ Cv<V, SPL> term_row(const TermArgs &a, int64_t r, int
     return o;
 }
 
+// Matrix values a kernel is compiled for: one real value for all entries
+// (TermArgs::uniform), a real value per entry, a complex one per entry.
+enum Vals { kOne, kReal, kComplex };
+
+// One row's matrix part, read ahead of the vectors: no kernel of the time
+// step writes it, so a dependent launch loads it before dep_wait(), and the
+// register-pipelined kernel loads the next row's before this row's gathers.
+// AHEAD: the values and the diagonal too, else the columns only (the caller's
+// registers then hold the values for a shorter time).
+template <typename V, Vals M, bool AHEAD>
+struct RowAhead {
+    int w;              // entries of the row's slice
+    int32_t c[4];
+    V h[AHEAD && M == kReal ? 4 : 1];
+    V d;
+};
+
+template <typename V, Vals M>
+__device__ __forceinline__ V row_diag(const TermArgs &a, uint32_t r)
+{
+    if constexpr (sizeof(V) == 8 && M == kOne) return a.zero_diag ? 0.0 : gdiag_at(a, r);   // gamma d
+    else return __ldg(reinterpret_cast<const V *>(a.H.diag) + r);
+}
+
+// Offset of row r's first entry and its slice's entries per row.
+__device__ __forceinline__ int64_t row_base(const TermArgs &a, uint32_t r, int &w)
+{
+    const uint32_t q = r / kSliceRows, lr = r % kSliceRows;
+    if (a.fixed_width) {        // no slice-pointer load: one dependent round trip less
+        w = a.fixed_width;
+        return (int64_t)q * (kSliceRows * w) + lr;
+    }
+    const int64_t base = __ldg(a.H.slice_ptr + q);
+    w = (int)((__ldg(a.H.slice_ptr + q + 1) - base) / kSliceRows);
+    return base + lr;
+}
+
+template <typename V, Vals M, bool AHEAD>
+__device__ __forceinline__ void row_ahead(const TermArgs &a, uint32_t r, RowAhead<V, M, AHEAD> &n)
+{
+    const int64_t base = row_base(a, r, n.w);
+    const int32_t *colp = a.H.col + base;
+    const V *valp = reinterpret_cast<const V *>(a.H.val) + base;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const bool ok = u < n.w;
+        n.c[u] = ok ? __ldg(colp + u * kSliceRows) : (int32_t)r;
+        if constexpr (AHEAD && M == kReal) n.h[u] = ok ? __ldg(valp + u * kSliceRows) : (V)0;
+    }
+    if (AHEAD) n.d = row_diag<V, M>(a, r);
+}
+
+// The term of row r, lane l, from its columns read ahead.  The own-row loads
+// and the first four gathers leave together; `meanwhile` runs while they are
+// in flight (the next row's loads of the register-pipelined kernel).
+// Arithmetic: H~ x is the diagonal, then the row's entries in stored order;
+// in FP64 with one value, term_row_sum's.
+template <typename V, int L, int SPL, Vals M, bool AHEAD, typename F>
+__device__ __forceinline__ Cv<V, SPL> row_term(const TermArgs &a, uint32_t r, int l,
+                                               const RowAhead<V, M, AHEAD> &cur, F &&meanwhile)
+{
+    typedef typename Val2<V>::type V2;
+    Cv<V, SPL> p, zz;
+    if (a.variant & kVariantStreamHints) {
+        p = ld_cs<V, L, SPL>(a.psi, r, l);
+        if (a.z) zz = ld_cs<V, L, SPL>(a.z, r, l);
+    } else {
+        p = ld_ro<V, L, SPL>(a.psi, r, l);
+        if (a.z) zz = ld<V, L, SPL>(a.z, r, l);
+    }
+    if (!a.z) {
+#pragma unroll
+        for (int j = 0; j < SPL; ++j) { zz.re[j] = 0; zz.im[j] = 0; }
+    }
+    Cv<V, SPL> y;
+    if (sizeof(V) == 4 || M != kOne || !a.zero_diag) {       // x_r is needed
+        y = ld_ro<V, L, SPL>(a.x, r, l);
+    } else {
+#pragma unroll
+        for (int j = 0; j < SPL; ++j) { y.re[j] = 0; y.im[j] = 0; }
+    }
+    Cv<V, SPL> xv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) xv[u] = ld_ro<V, L, SPL>(a.x, cur.c[u], l);
+    const V d = AHEAD ? cur.d : row_diag<V, M>(a, r);
+    meanwhile();
+    // FP32 norm carry: the state scales of the row's sample, or nullptr
+    auto scales = [&]() -> const V * {
+        const V *sc = Coef<V>::scale(a);
+        return sc ? sc + (int64_t)a.chunk_sample[r / kChunkRows] * (L * SPL) + l * SPL : nullptr;
+    };
+    if constexpr (sizeof(V) == 8 && M == kOne) {
+        // FP64 one-value form: neighbours summed in stored order, the
+        // first valid entry starting the sum
+        Cv<V, SPL> sm;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool ok = u < cur.w && cur.c[u] != (int32_t)r;
+#pragma unroll
+            for (int j = 0; j < SPL; ++j) {
+                if (u == 0) {
+                    sm.re[j] = ok ? xv[0].re[j] : 0.0;
+                    sm.im[j] = ok ? xv[0].im[j] : 0.0;
+                } else if (ok) {
+                    sm.re[j] += xv[u].re[j];
+                    sm.im[j] += xv[u].im[j];
+                }
+            }
+        }
+        for (int k = 4; k < cur.w; k += 4) {
+            int w;
+            const int64_t base = row_base(a, r, w);
+            int32_t c[4];
+            bool ok[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                ok[u] = k + u < cur.w;
+                c[u] = ok[u] ? __ldg(a.H.col + base + (k + u) * kSliceRows)
+                             : (int32_t)r;
+                ok[u] = ok[u] && c[u] != (int32_t)r;
+            }
+            Cv<V, SPL> xw[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) xw[u] = ld_ro<V, L, SPL>(a.x, c[u], l);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (ok[u]) {
+#pragma unroll
+                    for (int j = 0; j < SPL; ++j) {
+                        sm.re[j] += xw[u].re[j];
+                        sm.im[j] += xw[u].im[j];
+                    }
+                }
+            }
+        }
+        if (const V *sc = scales()) {
+#pragma unroll
+            for (int j = 0; j < SPL; ++j) {
+                const V sv = sc[j];
+                p.re[j] *= sv;
+                p.im[j] *= sv;
+                if (a.x_is_psi) {
+                    sm.re[j] *= sv;
+                    sm.im[j] *= sv;
+                    y.re[j] *= sv;
+                    y.im[j] *= sv;
+                }
+            }
+        }
+        return combine_sum<SPL>(a, d, y, sm, p, zz);
+    } else {
+#pragma unroll
+        for (int j = 0; j < SPL; ++j) { y.re[j] *= d; y.im[j] *= d; }
+        // four entries a round, the first round's columns and gathers ahead
+        auto round = [&](int k, const int32_t (&c)[4], const Cv<V, SPL> (&xw)[4], auto first) {
+            [[maybe_unused]] int w;
+            [[maybe_unused]] int64_t base = 0;
+            if constexpr (M == kComplex || (M == kReal && !(AHEAD && decltype(first)::value)))
+                base = row_base(a, r, w);
+            [[maybe_unused]] const V *valp = reinterpret_cast<const V *>(a.H.val) + base;
+            [[maybe_unused]] const V2 *valp2 = reinterpret_cast<const V2 *>(a.H.val) + base;
+            V h[4];
+            [[maybe_unused]] V hm[4];
+            bool ok[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                ok[u] = k + u < cur.w;
+                if constexpr (M == kComplex) {
+                    V2 v2;
+                    v2.x = (V)0;
+                    v2.y = (V)0;
+                    if (ok[u]) v2 = __ldg(valp2 + (k + u) * kSliceRows);
+                    h[u] = v2.x;
+                    hm[u] = v2.y;
+                } else if constexpr (M == kOne) {
+                    // one value for all entries; padded slots (col == own row) add nothing
+                    ok[u] = ok[u] && c[u] != (int32_t)r;
+                    h[u] = Coef<V>::hu(a);
+                } else if constexpr (AHEAD && decltype(first)::value) {
+                    h[u] = cur.h[u];
+                } else {
+                    h[u] = ok[u] ? __ldg(valp + (k + u) * kSliceRows) : (V)0;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (ok[u]) {
+#pragma unroll
+                    for (int j = 0; j < SPL; ++j) {
+                        y.re[j] = fma(h[u], xw[u].re[j], y.re[j]);
+                        y.im[j] = fma(h[u], xw[u].im[j], y.im[j]);
+                        if constexpr (M == kComplex) {       // (h + i hm)(x_re + i x_im)
+                            y.re[j] = fma(-hm[u], xw[u].im[j], y.re[j]);
+                            y.im[j] = fma(hm[u], xw[u].re[j], y.im[j]);
+                        }
+                    }
+                }
+            }
+        };
+        round(0, cur.c, xv, std::true_type{});
+        for (int k = 4; k < cur.w; k += 4) {
+            int w;
+            const int64_t base = row_base(a, r, w);
+            int32_t c[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                c[u] = k + u < cur.w ? __ldg(a.H.col + base + (k + u) * kSliceRows)
+                                     : (int32_t)r;
+            Cv<V, SPL> xw[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) xw[u] = ld_ro<V, L, SPL>(a.x, c[u], l);
+            round(k, c, xw, std::false_type{});
+        }
+        if (const V *sc = scales()) {            // psi -> psi * scale (per state)
+#pragma unroll
+            for (int j = 0; j < SPL; ++j) {
+                const V sv = sc[j];
+                p.re[j] *= sv;
+                p.im[j] *= sv;
+                if (a.x_is_psi) { y.re[j] *= sv; y.im[j] *= sv; }
+            }
+        }
+        const V g = Coef<V>::g(a), ch = Coef<V>::hi(a), cl = Coef<V>::lo(a);
+        Cv<V, SPL> o;
+#pragma unroll
+        for (int j = 0; j < SPL; ++j) {
+            // (-i)(y_re + i y_im) = y_im - i y_re
+            V re = fma(g, y.im[j], zz.re[j]);
+            V im = fma(-g, y.re[j], zz.im[j]);
+            if (sizeof(V) == 4) {           // coefficient carried as hi + lo in FP32
+                re = fma(cl, p.re[j], re);
+                im = fma(cl, p.im[j], im);
+            }
+            o.re[j] = fma(ch, p.re[j], re);
+            o.im[j] = fma(ch, p.im[j], im);
+        }
+        return o;
+    }
+}
+
 // Block index in traversal order: with kVariantZigZag the term kernels walk
 // the rows from the end on odd launches, so they start on the rows the
 // previous launch wrote last (still in L2).
@@ -462,28 +678,39 @@ __device__ __forceinline__ int64_t block_in_order(const TermArgs &a)
     return a.reverse ? (int64_t)(gridDim.x - 1 - blockIdx.x) : (int64_t)blockIdx.x;
 }
 
-// FP32: at most 40 registers for 16-byte lanes and 64 for the wide lanes
-// (16 blocks of 64 threads per SM, without spills; the 85-register bound
-// before was 5 % slower per term) -- the kernel is latency-bound, so
-// residency matters; FP64: 64 registers for 16-byte lanes, 85 for the wide
-// lanes (the one-value form's summed path and the general path share the
-// kernel: uncapped, the pair took 94 registers and halved the resident
-// warps).
+// Bound by the column -> gather latency at small sizes, by HBM beyond the L2.
+// The columns are read before dep_wait(), so after it the own-row loads and
+// the gathers leave together; a chain of such launches costs 2.4 us a term on
+// small samples (4.3 us with ordinary launches and the columns read after
+// the own-row loads), 10.1 us against 14.6 us at 4 x 524k FP32 rows.
+// FP32: 48 registers for 16-byte lanes and 64 for the wide lanes (the columns
+// held across the wait spill at 40); FP64: 64 registers for 16-byte lanes,
+// 85 for the wide lanes.
 // Thread t works on row t / (L RS), lane (t / RS) % L, part t % RS.  Rows are
 // a multiple of 1024, so a warp never straddles the last row (the part
 // shuffles see full warps).
-template <typename V, int L, int SPL, bool CX, int RS>
-__global__ void __launch_bounds__(256, sizeof(V) == 4 ? (SPL <= 2 ? 6 : 4) : (SPL == 1 ? 4 : 3)) k_term(TermArgs a)
+template <typename V, int L, int SPL, Vals M, int RS>
+__global__ void __launch_bounds__(256, sizeof(V) == 4 ? (SPL <= 2 ? 5 : 4) : (SPL == 1 ? 4 : 3)) k_term(TermArgs a)
 {
+    dep_launch();
     const int64_t t = block_in_order(a) * blockDim.x + threadIdx.x;
     const int64_t r = t / (L * RS);
     const int l = (int)((t / RS) % L);
-    const int part = (int)(t % RS);
-    if (r >= a.n_rows) return;
-    const V *sc = Coef<V>::scale(a);
-    if (sc) sc += (int64_t)a.chunk_sample[r / kChunkRows] * (L * SPL);
-    Cv<V, SPL> o = term_row<V, L, SPL, CX, RS>(a, r, l, sc, part);
-    if (part == 0) st<V, L, SPL>(a.out, r, l, o);
+    if constexpr (RS == 1) {
+        RowAhead<V, M, false> row;
+        if (r < a.n_rows) row_ahead(a, r, row);
+        dep_wait();
+        if (r >= a.n_rows) return;
+        st<V, L, SPL>(a.out, r, l, row_term<V, L, SPL>(a, r, l, row, [] {}));
+    } else {
+        dep_wait();
+        const int part = (int)(t % RS);
+        if (r >= a.n_rows) return;
+        const V *sc = Coef<V>::scale(a);
+        if (sc) sc += (int64_t)a.chunk_sample[r / kChunkRows] * (L * SPL);
+        Cv<V, SPL> o = term_row<V, L, SPL, RS>(a, r, l, sc, part);
+        if (part == 0) st<V, L, SPL>(a.out, r, l, o);
+    }
 }
 
 // Register-pipelined term (TBPM_VARIANT_PREFETCH; real values): a
@@ -491,218 +718,31 @@ __global__ void __launch_bounds__(256, sizeof(V) == 4 ? (SPL <= 2 ? 6 : 4) : (SP
 // when asked).  A row's first four column indices, their values and its
 // diagonal are loaded one row ahead, so the row's own-row loads and its
 // gathers leave together instead of the gathers waiting on the column
-// loads.  Per row the arithmetic and its order are term_row's (plain
-// kernel; in FP64 with one value, term_row_sum's): the states are
-// bit-identical to it.
-template <typename V>
-struct RowAhead {
-    int64_t base;
-    int w;
-    int32_t c[4];
-    V h[4];
-    V d;
-};
-
-template <typename V, int L, int SPL>
-__device__ __forceinline__ void row_ahead(const TermArgs &a, int64_t r, RowAhead<V> &n)
-{
-    const int64_t q = r / kSliceRows;
-    const int lr = (int)(r % kSliceRows);
-    if (a.fixed_width) {
-        n.w = a.fixed_width;
-        n.base = q * (kSliceRows * (int64_t)n.w);
-    } else {
-        n.base = __ldg(a.H.slice_ptr + q);
-        n.w = (int)((__ldg(a.H.slice_ptr + q + 1) - n.base) / kSliceRows);
-    }
-    const int32_t *colp = a.H.col + n.base + lr;
-    const V *valp = reinterpret_cast<const V *>(a.H.val) + n.base + lr;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const bool ok = u < n.w;
-        n.c[u] = ok ? __ldg(colp + (int64_t)u * kSliceRows) : (int32_t)r;
-        n.h[u] = a.uniform ? Coef<V>::hu(a) : (ok ? __ldg(valp + (int64_t)u * kSliceRows) : (V)0);
-    }
-    n.d = __ldg(reinterpret_cast<const V *>(a.H.diag) + r);
-    if constexpr (sizeof(V) == 8) {              // FP64 one-value form: gamma d
-        if (a.uniform) n.d = a.zero_diag ? 0.0 : gdiag_at(a, r);
-    }
-}
-
-template <typename V, int L, int SPL>
+// loads.  One kernel per kind of values: with one value no value registers
+// are carried, and the 16-byte lanes fit 64 registers.  HBM-bound: 178 us at
+// 4 x 8.3M FP32 rows, 6.7 TB/s (188 us as ordinary launches).
+template <typename V, int L, int SPL, Vals M>
 __global__ void __launch_bounds__(256, sizeof(V) == 4 ? (SPL <= 2 ? 4 : 3) : 2) k_term_pf(TermArgs a)
 {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t rows_per_pass = (int64_t)gridDim.x * blockDim.x / L;
+    dep_launch();
+    // rows are below 2^31, a pass far below: positions fit 32 unsigned bits
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t n_rows = (uint32_t)a.n_rows;
+    const uint32_t rows_per_pass = gridDim.x * blockDim.x / L;
     const int l = (int)(t % L);
-    int64_t i = t / L;                                   // position in traversal order
-    auto row_of = [&](int64_t k) { return a.reverse ? a.n_rows - 1 - k : k; };
-    RowAhead<V> cur;
-    if (i < a.n_rows) row_ahead<V, L, SPL>(a, row_of(i), cur);
-    for (; i < a.n_rows; i += rows_per_pass) {
-        const int64_t r = row_of(i);
-        Cv<V, SPL> p, zz;
-        if (a.variant & kVariantStreamHints) {
-            p = ld_cs<V, L, SPL>(a.psi, r, l);
-            if (a.z) zz = ld_cs<V, L, SPL>(a.z, r, l);
-        } else {
-            p = ld_ro<V, L, SPL>(a.psi, r, l);
-            if (a.z) zz = ld<V, L, SPL>(a.z, r, l);
-        }
-        if (!a.z) {
-#pragma unroll
-            for (int j = 0; j < SPL; ++j) { zz.re[j] = 0; zz.im[j] = 0; }
-        }
-        Cv<V, SPL> y = ld_ro<V, L, SPL>(a.x, r, l);
-        Cv<V, SPL> xv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) xv[u] = ld_ro<V, L, SPL>(a.x, cur.c[u], l);
-        // the next row's indices, values and diagonal, in flight meanwhile
-        RowAhead<V> nxt;
-        const int64_t i2 = i + rows_per_pass;
-        if (i2 < a.n_rows) row_ahead<V, L, SPL>(a, row_of(i2), nxt);
-        if constexpr (sizeof(V) == 8) {
-            if (a.uniform) {
-                // FP64 one-value form (term_row_sum): neighbours summed in
-                // stored order, the first valid entry starting the sum
-                Cv<V, SPL> sm;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const bool ok = u < cur.w && cur.c[u] != (int32_t)r;
-#pragma unroll
-                    for (int j = 0; j < SPL; ++j) {
-                        if (u == 0) {
-                            sm.re[j] = ok ? xv[0].re[j] : 0.0;
-                            sm.im[j] = ok ? xv[0].im[j] : 0.0;
-                        } else if (ok) {
-                            sm.re[j] += xv[u].re[j];
-                            sm.im[j] += xv[u].im[j];
-                        }
-                    }
-                }
-                const int64_t lr0 = r % kSliceRows;
-                for (int k = 4; k < cur.w; k += 4) {
-                    int32_t c[4];
-                    bool okk[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        okk[u] = k + u < cur.w;
-                        c[u] = okk[u] ? __ldg(a.H.col + cur.base + lr0 + (int64_t)(k + u) * kSliceRows)
-                                      : (int32_t)r;
-                        okk[u] = okk[u] && c[u] != (int32_t)r;
-                    }
-                    Cv<V, SPL> xw[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) xw[u] = ld_ro<V, L, SPL>(a.x, c[u], l);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        if (okk[u]) {
-#pragma unroll
-                            for (int j = 0; j < SPL; ++j) {
-                                sm.re[j] += xw[u].re[j];
-                                sm.im[j] += xw[u].im[j];
-                            }
-                        }
-                    }
-                }
-                const V *sc = Coef<V>::scale(a);
-                if (sc) {
-                    sc += (int64_t)a.chunk_sample[r / kChunkRows] * (L * SPL);
-#pragma unroll
-                    for (int j = 0; j < SPL; ++j) {
-                        const V sv = sc[l * SPL + j];
-                        p.re[j] *= sv;
-                        p.im[j] *= sv;
-                        if (a.x_is_psi) {
-                            sm.re[j] *= sv;
-                            sm.im[j] *= sv;
-                            y.re[j] *= sv;
-                            y.im[j] *= sv;
-                        }
-                    }
-                }
-                st<V, L, SPL>(a.out, r, l, combine_sum<SPL>(a, cur.d, y, sm, p, zz));
-                cur = nxt;
-                continue;
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < SPL; ++j) { y.re[j] *= cur.d; y.im[j] *= cur.d; }
-        // the first four entries (as term_row's first round), then the rest
-        bool ok[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            ok[u] = u < cur.w;
-            if (a.uniform) ok[u] = ok[u] && cur.c[u] != (int32_t)r;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (ok[u]) {
-#pragma unroll
-                for (int j = 0; j < SPL; ++j) {
-                    y.re[j] = fma(cur.h[u], xv[u].re[j], y.re[j]);
-                    y.im[j] = fma(cur.h[u], xv[u].im[j], y.im[j]);
-                }
-            }
-        }
-        const int64_t lr = r % kSliceRows;
-        for (int k = 4; k < cur.w; k += 4) {
-            int32_t c[4];
-            V h[4];
-            bool okk[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int ku = k + u;
-                okk[u] = ku < cur.w;
-                c[u] = okk[u] ? __ldg(a.H.col + cur.base + lr + (int64_t)ku * kSliceRows)
-                              : (int32_t)r;
-                if (a.uniform) {
-                    okk[u] = okk[u] && c[u] != (int32_t)r;
-                    h[u] = Coef<V>::hu(a);
-                } else {
-                    h[u] = okk[u] ? __ldg(reinterpret_cast<const V *>(a.H.val) + cur.base + lr +
-                                          (int64_t)ku * kSliceRows)
-                                  : (V)0;
-                }
-            }
-            Cv<V, SPL> xw[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) xw[u] = ld_ro<V, L, SPL>(a.x, c[u], l);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (okk[u]) {
-#pragma unroll
-                    for (int j = 0; j < SPL; ++j) {
-                        y.re[j] = fma(h[u], xw[u].re[j], y.re[j]);
-                        y.im[j] = fma(h[u], xw[u].im[j], y.im[j]);
-                    }
-                }
-            }
-        }
-        const V *sc = Coef<V>::scale(a);
-        if (sc) {
-            sc += (int64_t)a.chunk_sample[r / kChunkRows] * (L * SPL);
-#pragma unroll
-            for (int j = 0; j < SPL; ++j) {
-                const V s = sc[l * SPL + j];
-                p.re[j] *= s;
-                p.im[j] *= s;
-                if (a.x_is_psi) { y.re[j] *= s; y.im[j] *= s; }
-            }
-        }
-        const V g = Coef<V>::g(a), ch = Coef<V>::hi(a), cl = Coef<V>::lo(a);
-        Cv<V, SPL> o;
-#pragma unroll
-        for (int j = 0; j < SPL; ++j) {
-            V re = fma(g, y.im[j], zz.re[j]);
-            V im = fma(-g, y.re[j], zz.im[j]);
-            if (sizeof(V) == 4) {
-                re = fma(cl, p.re[j], re);
-                im = fma(cl, p.im[j], im);
-            }
-            o.re[j] = fma(ch, p.re[j], re);
-            o.im[j] = fma(ch, p.im[j], im);
-        }
+    uint32_t i = t / L;                                  // position in traversal order
+    auto row_of = [&](uint32_t k) { return a.reverse ? n_rows - 1 - k : k; };
+    RowAhead<V, M, true> cur;
+    if (i < n_rows) row_ahead(a, row_of(i), cur);
+    dep_wait();
+    for (; i < n_rows; i += rows_per_pass) {
+        const uint32_t r = row_of(i);
+        RowAhead<V, M, true> nxt;
+        const uint32_t i2 = i + rows_per_pass;
+        const Cv<V, SPL> o = row_term<V, L, SPL>(a, r, l, cur, [&] {
+            // the next row's indices, values and diagonal, in flight meanwhile
+            if (i2 < n_rows) row_ahead(a, row_of(i2), nxt);
+        });
         st<V, L, SPL>(a.out, r, l, o);
         cur = nxt;
     }
@@ -813,21 +853,23 @@ __device__ __forceinline__ void final_reduce(const TermArgs &a, int64_t bid, int
     }
 }
 
-template <typename V, int L, int SPL, bool COMPUTE, bool CX>
+template <typename V, int L, int SPL, bool COMPUTE, Vals M>
 __global__ void __launch_bounds__(kFinalThreads) k_final(TermArgs a)
 {
-    constexpr int B = L * SPL;
+    dep_launch();
     const int64_t bid = block_in_order(a);
     const int64_t t = bid * kFinalThreads + threadIdx.x;
     const int64_t r = t / L;
     const int l = (int)(t % L);
-    const V *sc = Coef<V>::scale(a);
-    if (sc) sc += (int64_t)a.chunk_sample[r / kChunkRows] * B;
     Cv<V, SPL> o;
     if (COMPUTE) {
-        o = term_row<V, L, SPL, CX>(a, r, l, sc);
+        RowAhead<V, M, false> row;
+        row_ahead(a, r, row);
+        dep_wait();
+        o = row_term<V, L, SPL>(a, r, l, row, [] {});
         st<V, L, SPL>(a.out, r, l, o);
     } else {
+        dep_wait();
         o = ld<V, L, SPL>(a.out, r, l);
     }
     const Cv<V, SPL> p0 = ld_ro<V, L, SPL>(a.psi0, r, l);
@@ -851,6 +893,8 @@ __global__ void __launch_bounds__(kFinalThreads) k_final_sums(TermArgs a)
     __shared__ FF redp[P * NV];
     __shared__ double tot[NV];
     __shared__ int last;
+    dep_launch();
+    dep_wait();
     const int64_t bid = block_in_order(a);
     const int lrow = threadIdx.x / L, l = threadIdx.x % L;
     const int64_t r0 = bid * (int64_t)(ROWS * RPT) + lrow;
@@ -1035,6 +1079,10 @@ __global__ void __launch_bounds__(kHaloRows * L, 8 / L) k_term_halo(TermArgs a)
     const int tid = threadIdx.x;
     const int lr = tid / L, l = tid % L;
     const int64_t r = hb * kHaloRows + lr;
+    const int64_t h0 = __ldg(a.halo_ptr + hb);
+    const int H = (int)(__ldg(a.halo_ptr + hb + 1) - h0);
+    dep_launch();
+    dep_wait();
     // own-row streams first: in flight while the halo arrives
     Cv<V, SPL> p = ld_ro<V, L, SPL>(a.psi, r, l), zz;
     if (a.z) {
@@ -1045,8 +1093,6 @@ __global__ void __launch_bounds__(kHaloRows * L, 8 / L) k_term_halo(TermArgs a)
     }
     const V *sc = Coef<V>::scale(a);
     if (sc) sc += (int64_t)a.chunk_sample[r / kChunkRows] * (L * SPL);
-    const int64_t h0 = a.halo_ptr[hb];
-    const int H = (int)(a.halo_ptr[hb + 1] - h0);
     const unsigned char *xg = reinterpret_cast<const unsigned char *>(a.x);
     for (int idx = tid; idx < H * C; idx += NT) {
         const int h = idx / C, c = idx % C;
@@ -1158,8 +1204,7 @@ cudaError_t launch_halo_t(const TermArgs &a, cudaStream_t st)
         configured = smem;
     }
     const unsigned blocks = (unsigned)(a.n_rows / kHaloRows);
-    k_term_halo<V, L, SPL, FINAL><<<blocks, kHaloRows * L, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_term_halo<V, L, SPL, FINAL>, blocks, kHaloRows * L, smem, st, a);
 }
 
 // ---- pipelined staged-gather term (TBPM_VARIANT_HALO | TBPM_VARIANT_PIPE) ----
@@ -1436,6 +1481,7 @@ __global__ void __launch_bounds__(kHaloRows * C) k_term_halo_pipe(TermArgs a, Pi
     };
 
     // prologue: block 0's copies, then the bounds and rows one and two ahead
+    dep_launch();
     int64_t hb = block_at(0);
     int32_t g1[kPipeIdx];
     PipeMeta m1, m2;
@@ -1448,6 +1494,7 @@ __global__ void __launch_bounds__(kHaloRows * C) k_term_halo_pipe(TermArgs a, Pi
         rows_of(m0, g0);
         rows_of(m1, g1);
         row_of(hb, m0, w, off);
+        dep_wait();
         if (hb >= 0) issue(m0, g0, 0);
     }
     for (int64_t i = 0; hb >= 0; ++i) {
@@ -1510,19 +1557,8 @@ __global__ void __launch_bounds__(kHaloRows * C, 2) k_term_staged(TermArgs a, Pi
     const int64_t e0 = __ldg(a.pslice + hb * SPB);
     const int E = (int)(__ldg(a.pslice + (hb + 1) * SPB) - e0);
     const unsigned char *xg = reinterpret_cast<const unsigned char *>(a.x);
-    {
-        int32_t g[kPipeIdx];                         // halo rows lr, lr + 128, ...
-#pragma unroll
-        for (int k = 0; k < kPipeIdx; ++k) {
-            const int h = lr + k * kHaloRows;
-            g[k] = h < H ? __ldg(a.halo_rows + h0 + h) : 0;
-        }
-#pragma unroll
-        for (int k = 0; k < kPipeIdx; ++k) {
-            const int h = lr + k * kHaloRows;
-            if (h < H) cp_async16(sm + (h * C + l) * 16, xg + ((int64_t)g[k] * C + l) * 16);
-        }
-    }
+    dep_launch();
+    // matrix part first: no kernel of the step writes it
     unsigned char *lc = sm + ps.halo_bytes;
     for (int idx = tid; idx < E / 8; idx += NT) cp_async16(lc + idx * 16, a.lcol + e0 + idx * 8);
     if (!a.uniform) {
@@ -1530,6 +1566,20 @@ __global__ void __launch_bounds__(kHaloRows * C, 2) k_term_staged(TermArgs a, Pi
         unsigned char *vs = lc + ps.lcol_bytes;
         for (int idx = tid; idx < E / per; idx += NT)
             cp_async16(vs + idx * 16, reinterpret_cast<const V *>(a.vpack) + e0 + idx * per);
+    }
+    {
+        int32_t g[kPipeIdx];                         // halo rows lr, lr + 128, ...
+#pragma unroll
+        for (int k = 0; k < kPipeIdx; ++k) {
+            const int h = lr + k * kHaloRows;
+            g[k] = h < H ? __ldg(a.halo_rows + h0 + h) : 0;
+        }
+        dep_wait();
+#pragma unroll
+        for (int k = 0; k < kPipeIdx; ++k) {
+            const int h = lr + k * kHaloRows;
+            if (h < H) cp_async16(sm + (h * C + l) * 16, xg + ((int64_t)g[k] * C + l) * 16);
+        }
     }
     cp_async_commit();
     // own-row streams and the row's entry count, in flight while the stage lands
@@ -1576,8 +1626,7 @@ cudaError_t launch_staged_t(const TermArgs &a, cudaStream_t st)
         if (e != cudaSuccess) return e;
         conf = smem;
     }
-    k_term_staged<V, C><<<(unsigned)ps.n_hb, kHaloRows * C, smem, st>>>(a, ps);
-    return cudaGetLastError();
+    return launch_dependent(k_term_staged<V, C>, (unsigned)ps.n_hb, kHaloRows * C, smem, st, a, ps);
 }
 
 cudaError_t dispatch_staged(const TermArgs &a, int fp32, int B, cudaStream_t st)
@@ -1620,8 +1669,7 @@ cudaError_t launch_pipe_t(const TermArgs &a, int num_sms, cudaStream_t st)
         occ_smem[sizeof(V) == 4][C / 4] = smem;
     }
     const int grid = (int)std::min<int64_t>((int64_t)num_sms * occ, ps.n_hb);
-    k_term_halo_pipe<V, C><<<grid, kHaloRows * C, smem, st>>>(a, ps);
-    return cudaGetLastError();
+    return launch_dependent(k_term_halo_pipe<V, C>, grid, kHaloRows * C, smem, st, a, ps);
 }
 
 cudaError_t dispatch_pipe(const TermArgs &a, int fp32, int B, cudaStream_t st)
@@ -1666,6 +1714,8 @@ constexpr int kReduceSplit = 64;
 __global__ void __launch_bounds__(64) k_reduce(ReduceArgs a)
 {
     __shared__ int last;
+    dep_launch();
+    dep_wait();
     const int s = blockIdx.x, j = blockIdx.y;
     const int B3 = a.B * 3;
     const int t = threadIdx.x;
@@ -1816,25 +1866,32 @@ __global__ void k_corr_mean_adjoint(const double2 *gavg, int n_samples, int S, i
     g[i] = make_double2(v.x / S, v.y / S);
 }
 
-template <typename V, int L, int SPL, bool CX, int RS = 1>
+template <typename V, int L, int SPL, Vals M, int RS = 1>
 cudaError_t launch_term_t(const TermArgs &a, int threads, cudaStream_t st)
 {
     const int64_t n_threads = a.n_rows * L * RS;
     const unsigned blocks = (unsigned)((n_threads + threads - 1) / threads);
-    k_term<V, L, SPL, CX, RS><<<blocks, threads, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_term<V, L, SPL, M, RS>, blocks, threads, 0, st, a);
+}
+
+// One row a thread, real values.
+template <typename V, int L, int SPL>
+cudaError_t launch_term_u(const TermArgs &a, int threads, cudaStream_t st)
+{
+    return a.uniform ? launch_term_t<V, L, SPL, kOne>(a, threads, st)
+                     : launch_term_t<V, L, SPL, kReal>(a, threads, st);
 }
 
 // The register-pipelined kernel: a persistent grid of the SMs times the
 // blocks that fit on one, at most one thread per lane-row.
-template <typename V, int L, int SPL>
-cudaError_t launch_term_pf_t(const TermArgs &a, int threads, cudaStream_t st)
+template <typename V, int L, int SPL, Vals M>
+cudaError_t launch_term_pf_m(const TermArgs &a, int threads, cudaStream_t st)
 {
     static int occ[4] = {0, 0, 0, 0};            // resident blocks per SM by threads 64 .. 512
     const int ti = threads <= 64 ? 0 : threads <= 128 ? 1 : threads <= 256 ? 2 : 3;
     if (!occ[ti]) {
         int nb = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_term_pf<V, L, SPL>, threads, 0) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_term_pf<V, L, SPL, M>, threads, 0) !=
             cudaSuccess)
             nb = 1;
         occ[ti] = std::max(1, nb);
@@ -1843,9 +1900,31 @@ cudaError_t launch_term_pf_t(const TermArgs &a, int threads, cudaStream_t st)
     const int64_t want = (n_threads + threads - 1) / threads;
     const unsigned blocks =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)std::max(1, a.num_sms) * occ[ti], want));
-    k_term_pf<V, L, SPL><<<blocks, threads, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_term_pf<V, L, SPL, M>, blocks, threads, 0, st, a);
 }
+
+template <typename V, int L, int SPL>
+cudaError_t launch_term_pf_t(const TermArgs &a, int threads, cudaStream_t st)
+{
+    return a.uniform ? launch_term_pf_m<V, L, SPL, kOne>(a, threads, st)
+                     : launch_term_pf_m<V, L, SPL, kReal>(a, threads, st);
+}
+
+// The widths a TBPM_VARIANT_PREFETCH term runs at, all bit-identical.  FP32
+// interior terms on graphene, us, 16-byte lanes unless said otherwise:
+//   states x rows        one row a thread   persistent   persistent, 32-byte lanes
+//   4 x 131k (4 MB)            4.3              4.7             5.3
+//   4 x 524k (17 MB)          10.1             10.2            13.7
+//   8 x 295k (19 MB)          11.0             10.8            13.4
+//   4 x 2.1M (67 MB)          50               45.9            47.1
+//   4 x 8.3M (266 MB)        204              185             178
+//   16 x 2.1M (266 MB)       191              162             165
+// Up to 2^20 lanes every row of the launch is resident at once or nearly:
+// the persistent loop has nothing to read ahead.  Beyond, reading ahead
+// pays, and once a vector of four states exceeds the L2 (129 MB) one
+// 32-byte lane a row halves the index loads of a kernel that HBM bounds.
+constexpr int64_t kPrefetchMinLanes = (int64_t)1 << 20;
+constexpr int64_t kWideMinBytes = (int64_t)128 << 20;
 
 cudaError_t dispatch_pf(const TermArgs &a, int fp32, int B, int threads, cudaStream_t st)
 {
@@ -1865,13 +1944,18 @@ cudaError_t dispatch_pf(const TermArgs &a, int fp32, int B, int threads, cudaStr
         }
         return cudaErrorInvalidValue;
     }
-    if (a.variant & kVariantWide) {
+    if (a.n_rows * std::max(1, B / 2) <= kPrefetchMinLanes) {
         switch (B) {
-        case 4: return launch_term_pf_t<float, 1, 4>(a, threads, st);
-        case 8: return launch_term_pf_t<float, 2, 4>(a, threads, st);
-        case 16: return launch_term_pf_t<float, 4, 4>(a, threads, st);
+        case 1: return launch_term_u<float, 1, 1>(a, 256, st);
+        case 2: return launch_term_u<float, 1, 2>(a, 256, st);
+        case 4: return launch_term_u<float, 2, 2>(a, 256, st);
+        case 8: return launch_term_u<float, 4, 2>(a, 256, st);
+        case 16: return launch_term_u<float, 8, 2>(a, 256, st);
         }
+        return cudaErrorInvalidValue;
     }
+    if ((a.variant & kVariantWide) && B == 4 && a.n_rows * 32 > kWideMinBytes)
+        return launch_term_pf_t<float, 1, 4>(a, threads, st);
     switch (B) {
     case 1: return launch_term_pf_t<float, 1, 1>(a, threads, st);
     case 2: return launch_term_pf_t<float, 1, 2>(a, threads, st);
@@ -1886,35 +1970,32 @@ cudaError_t dispatch_pf(const TermArgs &a, int fp32, int B, int threads, cudaStr
 template <typename V, int L, int SPL>
 cudaError_t launch_term_split(const TermArgs &a, int threads, cudaStream_t st)
 {
-    if (a.variant & kVariantSplit4) return launch_term_t<V, L, SPL, false, 4>(a, threads, st);
-    return launch_term_t<V, L, SPL, false, 2>(a, threads, st);
+    // (the row split reads TermArgs::uniform at run time)
+    if (a.variant & kVariantSplit4) return launch_term_t<V, L, SPL, kReal, 4>(a, threads, st);
+    return launch_term_t<V, L, SPL, kReal, 2>(a, threads, st);
 }
 
-template <typename V, int L, int SPL, bool CX>
+template <typename V, int L, int SPL, Vals M>
 cudaError_t launch_final_t(const TermArgs &a, int threads, bool compute, cudaStream_t st)
 {
     (void)threads;   // the closing term has its own block size
-    if constexpr (sizeof(V) == 4 && !CX) {
+    if constexpr (sizeof(V) == 4 && M != kComplex) {
         if (!compute) {           // FP32 reduction-only pass: four rows a thread
             constexpr int RPT = 4;
             const unsigned rblocks = (unsigned)(a.n_rows * L / (kFinalThreads * RPT));
-            k_final_sums<L, SPL, RPT><<<rblocks, kFinalThreads, 0, st>>>(a);
-            return cudaGetLastError();
+            return launch_dependent(k_final_sums<L, SPL, RPT>, rblocks, kFinalThreads, 0, st, a);
         }
     }
     const unsigned blocks = (unsigned)(a.n_rows * L / kFinalThreads);
-    if (compute)
-        k_final<V, L, SPL, true, CX><<<blocks, kFinalThreads, 0, st>>>(a);
-    else
-        k_final<V, L, SPL, false, CX><<<blocks, kFinalThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(compute ? k_final<V, L, SPL, true, M> : k_final<V, L, SPL, false, M>,
+                            blocks, kFinalThreads, 0, st, a);
 }
 
-template <bool FINAL, bool CX>
-cudaError_t dispatch_cx(const TermArgs &a, int fp32, int B, int threads, bool compute,
+template <bool FINAL, Vals M>
+cudaError_t dispatch_m(const TermArgs &a, int fp32, int B, int threads, bool compute,
                         cudaStream_t st)
 {
-    if (!FINAL && !CX && (a.variant & (kVariantSplit2 | kVariantSplit4))) {
+    if (!FINAL && M != kComplex && (a.variant & (kVariantSplit2 | kVariantSplit4))) {
         if (a.variant & kVariantWide) {
             if (!fp32) {
                 switch (B) {
@@ -1948,9 +2029,9 @@ cudaError_t dispatch_cx(const TermArgs &a, int fp32, int B, int threads, bool co
         }
     }
 #define TBPM_CASE(V, L, SPL)                                                  \
-    return FINAL ? launch_final_t<V, L, SPL, CX>(a, threads, compute, st)    \
-                 : launch_term_t<V, L, SPL, CX>(a, threads, st)
-    if constexpr (!CX) if (a.variant & kVariantWide) {
+    return FINAL ? launch_final_t<V, L, SPL, M>(a, threads, compute, st)     \
+                 : launch_term_t<V, L, SPL, M>(a, threads, st)
+    if constexpr (M != kComplex) if (a.variant & kVariantWide) {
         // one thread per row and 32-byte lanes: fewer lanes share the index loads
         if (!fp32) {
             switch (B) {
@@ -1990,8 +2071,9 @@ template <bool FINAL>
 cudaError_t dispatch(const TermArgs &a, int fp32, int B, int threads, bool compute,
                      cudaStream_t st)
 {
-    return a.cplx ? dispatch_cx<FINAL, true>(a, fp32, B, threads, compute, st)
-                  : dispatch_cx<FINAL, false>(a, fp32, B, threads, compute, st);
+    if (a.cplx) return dispatch_m<FINAL, kComplex>(a, fp32, B, threads, compute, st);
+    return a.uniform ? dispatch_m<FINAL, kOne>(a, fp32, B, threads, compute, st)
+                     : dispatch_m<FINAL, kReal>(a, fp32, B, threads, compute, st);
 }
 
 }  // namespace
@@ -2095,8 +2177,7 @@ cudaError_t launch_final(const TermArgs &a, int fp32, int B, int threads, cudaSt
 
 cudaError_t launch_reduce(const ReduceArgs &a, cudaStream_t st)
 {
-    k_reduce<<<dim3(a.n_samples, kReduceSplit), 64, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_reduce, dim3(a.n_samples, kReduceSplit), 64, 0, st, a);
 }
 
 cudaError_t kernel_binary_version(int *version)

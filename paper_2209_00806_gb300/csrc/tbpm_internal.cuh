@@ -60,6 +60,43 @@ __device__ __forceinline__ void ff_dot3(float are, float aim, float ore, float o
 }
 #endif
 
+// Dependent launches.  The kernels of a time step form a chain of launches that
+// each need the previous one's vectors; started in the ordinary way, every
+// link pays the drain of one grid and the start of the next.  With
+// launch_dependent a kernel's blocks become resident while the previous
+// kernel's last blocks still run: they read what no kernel of the chain
+// writes (matrix indices, values, diagonal) and stop at dep_wait() until the
+// previous grid has completed and its writes are visible.  Rules of the chain:
+//  - a kernel launched so calls dep_wait() on every path before it reads or
+//    writes anything another kernel of the stream writes or reads;
+//  - vectors are read by plain loads, not through the read-only path (a
+//    read-only load may be moved above the wait);
+//  - data read before dep_wait() was complete on the host's side (stream
+//    synchronised) before the launch.
+// dep_launch() lets the next kernel's blocks start as soon as this grid's
+// blocks are all resident or done.
+#ifdef __CUDACC__
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*k)(P...), dim3 grid, dim3 block, size_t smem,
+                                    cudaStream_t st, const A &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+#endif
+
 // Launch variants of the term kernels (bits of TermArgs::variant).
 constexpr int kVariantZigZag = 1;       // alternate the traversal direction per launch
 constexpr int kVariantStreamHints = 2;  // evict-first loads of the own-row streams

@@ -1,0 +1,54 @@
+"""Launch rules of the register-pipelined variant (TBPM_VARIANT_PREFETCH): the
+states equal the plain kernel's bit for bit on both sides of every rule."""
+import math
+
+import numpy as np
+import pytest
+
+from tbpm_inputs import lattice, rng
+
+pytestmark = pytest.mark.gpu
+Z = math.pi / 2
+PLAIN, PREFETCH = 1, 8257          # ZIGZAG; ZIGZAG | WIDE | PREFETCH
+
+
+def _states(tb, smp, theta, precision, B, variant, steps):
+    import torch
+    from paper_2209_00806_gb300 import _native as N
+    with tb.Propagator() as p:
+        p.launch_config(precision, B, 64, variant)
+        p.build_sample(smp, 9.5)
+        p.set_phase_states(theta)
+        C = p.propagate(Z, steps, precision)
+        out = torch.empty((theta.shape[0], smp.n_orb), dtype=torch.complex128, device="cuda")
+        N.tbpm_get_states(p.ctx, out)
+        return C, out
+
+
+# rows a multiple of 1024: 2^20 lanes of 16 bytes are 2^20 / max(1, B / 2) rows
+@pytest.mark.parametrize("values", ["one", "real"])
+@pytest.mark.parametrize("B", [1, 2, 4, 8, 16])
+@pytest.mark.parametrize("over", [0, 1])
+def test_lane_rule_is_bit_identical(B, over, values):
+    import paper_2209_00806_gb300 as tb
+    rows = (1 << 20) // max(1, B // 2) + 1024 * over
+    smp = lattice.graphene(rows // 1024, 512, pbc=True, seed=3, onsite_w=1.0,
+                           vacancy_frac=0.0 if over else 0.0003,
+                           bond_sigma=0.05 if values == "real" else 0.0)
+    theta = rng.phases(5, B, smp.n_orb)
+    C0, a = _states(tb, smp, theta, tb.TBPM_FP32, B, PLAIN, 2)
+    C1, b = _states(tb, smp, theta, tb.TBPM_FP32, B, PREFETCH, 2)
+    assert (a == b).all()
+    # the sums of float pairs differ in order only: 1e-12 as for the other variants
+    assert np.abs(C0 - C1).max() < 1e-12
+
+
+@pytest.mark.parametrize("sides", [(2048, 1024), (2049, 1024)])   # one vector of 128 MB, and above
+def test_wide_lane_rule_is_bit_identical(sides):
+    import paper_2209_00806_gb300 as tb
+    smp = lattice.graphene(*sides, pbc=True, seed=4, onsite_w=1.0)
+    theta = rng.phases(6, 4, smp.n_orb)
+    C0, a = _states(tb, smp, theta, tb.TBPM_FP32, 4, PLAIN, 2)
+    C1, b = _states(tb, smp, theta, tb.TBPM_FP32, 4, PREFETCH, 2)
+    assert (a == b).all()
+    assert np.abs(C0 - C1).max() < 1e-12
