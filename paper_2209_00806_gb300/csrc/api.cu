@@ -1716,6 +1716,7 @@ extern "C" int tbpm_propagate_adjoint(tbpm_ctx *c, double z, int n_steps, const 
         base.H = Hv;
         base.chunk_sample = c->H.chunk_sample;
         base.n_rows = c->H.n_rows;
+        base.fixed_width = c->H.fixed_width;
         auto term = [&](const void *x, const void *psi, const void *zz, void *out, double cc,
                         double gamma) -> int {
             TermArgs t = base;

@@ -197,9 +197,9 @@ __device__ __forceinline__ double gdiag_at(const TermArgs &a, int64_t r)
     return a.gamma * __ldg(reinterpret_cast<const double *>(a.H.diag) + r);
 }
 
-// the combine above for SPL states; xo is unused when zero_diag
-template <int SPL>
-__device__ __forceinline__ Cv<double, SPL> combine_sum(const TermArgs &a, double gd,
+// the combine above for SPL states; DIAG false: no diagonal term (xo unused)
+template <int SPL, bool DIAG>
+__device__ __forceinline__ Cv<double, SPL> combine_form(const TermArgs &a, double gd,
                                                        const Cv<double, SPL> &xo,
                                                        const Cv<double, SPL> &s,
                                                        const Cv<double, SPL> &p,
@@ -211,7 +211,7 @@ __device__ __forceinline__ Cv<double, SPL> combine_sum(const TermArgs &a, double
     for (int j = 0; j < SPL; ++j) {
         double re = fma(ch, p.re[j], zz.re[j]);
         double im = fma(ch, p.im[j], zz.im[j]);
-        if (!a.zero_diag) {
+        if (DIAG) {
             re = fma(gd, xo.im[j], re);
             im = fma(-gd, xo.re[j], im);
         }
@@ -219,6 +219,18 @@ __device__ __forceinline__ Cv<double, SPL> combine_sum(const TermArgs &a, double
         o.im[j] = fma(-gh, s.re[j], im);
     }
     return o;
+}
+
+// for kernels that serve matrices with and without a diagonal
+template <int SPL>
+__device__ __forceinline__ Cv<double, SPL> combine_sum(const TermArgs &a, double gd,
+                                                       const Cv<double, SPL> &xo,
+                                                       const Cv<double, SPL> &s,
+                                                       const Cv<double, SPL> &p,
+                                                       const Cv<double, SPL> &zz)
+{
+    return a.zero_diag ? combine_form<SPL, false>(a, gd, xo, s, p, zz)
+                       : combine_form<SPL, true>(a, gd, xo, s, p, zz);
 }
 
 template <int L, int SPL, int RS>
@@ -283,11 +295,11 @@ __device__ __forceinline__ Cv<double, SPL> term_row_sum(const TermArgs &a, int64
                     s.re[j] = ok[0] ? xv[0].re[j] : 0.0;
                     s.im[j] = ok[0] ? xv[0].im[j] : 0.0;
                 }
-            } else if (ok[u]) {
+            } else {
 #pragma unroll
                 for (int j = 0; j < SPL; ++j) {
-                    s.re[j] += xv[u].re[j];
-                    s.im[j] += xv[u].im[j];
+                    if (ok[u]) s.re[j] += xv[u].re[j];
+                    if (ok[u]) s.im[j] += xv[u].im[j];
                 }
             }
         }
@@ -386,12 +398,10 @@ __device__ __forceinline__ Cv<V, SPL> term_row(const TermArgs &a, int64_t r, int
         for (int u = 0; u < 4; ++u) xv[u] = ld_ro<V, L, SPL>(a.x, c[u], l);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            if (ok[u]) {
 #pragma unroll
-                for (int j = 0; j < SPL; ++j) {
-                    y.re[j] = fma(h[u], xv[u].re[j], y.re[j]);
-                    y.im[j] = fma(h[u], xv[u].im[j], y.im[j]);
-                }
+            for (int j = 0; j < SPL; ++j) {
+                if (ok[u]) y.re[j] = fma(h[u], xv[u].re[j], y.re[j]);
+                if (ok[u]) y.im[j] = fma(h[u], xv[u].im[j], y.im[j]);
             }
         }
     }
@@ -430,36 +440,35 @@ __device__ __forceinline__ Cv<V, SPL> term_row(const TermArgs &a, int64_t r, int
     return o;
 }
 
-// Matrix values a kernel is compiled for: one real value for all entries
-// (TermArgs::uniform), a real value per entry, a complex one per entry.
-enum Vals { kOne, kReal, kComplex };
-
 // One row's matrix part, read ahead of the vectors: no kernel of the time
 // step writes it, so a dependent launch loads it before dep_wait(), and the
 // register-pipelined kernel loads the next row's before this row's gathers.
 // AHEAD: the values and the diagonal too, else the columns only (the caller's
 // registers then hold the values for a shorter time).
-template <typename V, Vals M, bool AHEAD>
+template <typename V, Vals M, int W, bool AHEAD>
 struct RowAhead {
-    int w;              // entries of the row's slice
-    int32_t c[4];
-    V h[AHEAD && M == kReal ? 4 : 1];
+    int w;                                               // entries of the row's slice
+    int32_t c[W ? W : 4];                                // slots of the first round
+    V h[AHEAD && M == kReal ? (W ? W : 4) : 1];
     V d;
 };
 
 template <typename V, Vals M>
 __device__ __forceinline__ V row_diag(const TermArgs &a, uint32_t r)
 {
-    if constexpr (sizeof(V) == 8 && M == kOne) return a.zero_diag ? 0.0 : gdiag_at(a, r);   // gamma d
+    if constexpr (M == kOneNoDiag) return 0.0;
+    else if constexpr (M == kOneMul) return a.gamma * __ldg(reinterpret_cast<const double *>(a.H.diag) + r);
+    else if constexpr (sizeof(V) == 8 && M == kOne) return xor_sign(__ldg(a.gdiag + r), a.gdiag_sign);
     else return __ldg(reinterpret_cast<const V *>(a.H.diag) + r);
 }
 
 // Offset of row r's first entry and its slice's entries per row.
+template <int W>
 __device__ __forceinline__ int64_t row_base(const TermArgs &a, uint32_t r, int &w)
 {
     const uint32_t q = r / kSliceRows, lr = r % kSliceRows;
-    if (a.fixed_width) {        // no slice-pointer load: one dependent round trip less
-        w = a.fixed_width;
+    if (W || a.fixed_width) {   // no slice-pointer load: one dependent round trip less
+        w = W ? W : a.fixed_width;
         return (int64_t)q * (kSliceRows * w) + lr;
     }
     const int64_t base = __ldg(a.H.slice_ptr + q);
@@ -467,15 +476,15 @@ __device__ __forceinline__ int64_t row_base(const TermArgs &a, uint32_t r, int &
     return base + lr;
 }
 
-template <typename V, Vals M, bool AHEAD>
-__device__ __forceinline__ void row_ahead(const TermArgs &a, uint32_t r, RowAhead<V, M, AHEAD> &n)
+template <typename V, Vals M, int W, bool AHEAD>
+__device__ __forceinline__ void row_ahead(const TermArgs &a, uint32_t r, RowAhead<V, M, W, AHEAD> &n)
 {
-    const int64_t base = row_base(a, r, n.w);
+    const int64_t base = row_base<W>(a, r, n.w);
     const int32_t *colp = a.H.col + base;
     const V *valp = reinterpret_cast<const V *>(a.H.val) + base;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const bool ok = u < n.w;
+    for (int u = 0; u < (W ? W : 4); ++u) {
+        const bool ok = W || u < n.w;
         n.c[u] = ok ? __ldg(colp + u * kSliceRows) : (int32_t)r;
         if constexpr (AHEAD && M == kReal) n.h[u] = ok ? __ldg(valp + u * kSliceRows) : (V)0;
     }
@@ -487,10 +496,11 @@ __device__ __forceinline__ void row_ahead(const TermArgs &a, uint32_t r, RowAhea
 // in flight (the next row's loads of the register-pipelined kernel).
 // Arithmetic: H~ x is the diagonal, then the row's entries in stored order;
 // in FP64 with one value, term_row_sum's.
-template <typename V, int L, int SPL, Vals M, bool AHEAD, typename F>
+template <typename V, int L, int SPL, Vals M, int W, bool AHEAD, typename F>
 __device__ __forceinline__ Cv<V, SPL> row_term(const TermArgs &a, uint32_t r, int l,
-                                               const RowAhead<V, M, AHEAD> &cur, F &&meanwhile)
+                                               const RowAhead<V, M, W, AHEAD> &cur, F &&meanwhile)
 {
+    constexpr int NS = W ? W : 4;
     typedef typename Val2<V>::type V2;
     Cv<V, SPL> p, zz;
     if (a.variant & kVariantStreamHints) {
@@ -505,43 +515,38 @@ __device__ __forceinline__ Cv<V, SPL> row_term(const TermArgs &a, uint32_t r, in
         for (int j = 0; j < SPL; ++j) { zz.re[j] = 0; zz.im[j] = 0; }
     }
     Cv<V, SPL> y;
-    if (sizeof(V) == 4 || M != kOne || !a.zero_diag) {       // x_r is needed
-        y = ld_ro<V, L, SPL>(a.x, r, l);
-    } else {
+    if constexpr (M != kOneNoDiag) y = ld_ro<V, L, SPL>(a.x, r, l);
+    Cv<V, SPL> xv[NS];
 #pragma unroll
-        for (int j = 0; j < SPL; ++j) { y.re[j] = 0; y.im[j] = 0; }
-    }
-    Cv<V, SPL> xv[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) xv[u] = ld_ro<V, L, SPL>(a.x, cur.c[u], l);
+    for (int u = 0; u < NS; ++u) xv[u] = ld_ro<V, L, SPL>(a.x, cur.c[u], l);
     const V d = AHEAD ? cur.d : row_diag<V, M>(a, r);
     meanwhile();
-    // FP32 norm carry: the state scales of the row's sample, or nullptr
-    auto scales = [&]() -> const V * {
+    // norm carry (FP32 only): the state scales of the row's sample, or nullptr
+    [[maybe_unused]] auto scales = [&]() -> const V * {
         const V *sc = Coef<V>::scale(a);
         return sc ? sc + (int64_t)a.chunk_sample[r / kChunkRows] * (L * SPL) + l * SPL : nullptr;
     };
-    if constexpr (sizeof(V) == 8 && M == kOne) {
+    if constexpr (sizeof(V) == 8 && one_value(M)) {
         // FP64 one-value form: neighbours summed in stored order, the
         // first valid entry starting the sum
         Cv<V, SPL> sm;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const bool ok = u < cur.w && cur.c[u] != (int32_t)r;
+        for (int u = 0; u < NS; ++u) {
+            const bool ok = (W || u < cur.w) && cur.c[u] != (int32_t)r;
 #pragma unroll
             for (int j = 0; j < SPL; ++j) {
                 if (u == 0) {
                     sm.re[j] = ok ? xv[0].re[j] : 0.0;
                     sm.im[j] = ok ? xv[0].im[j] : 0.0;
-                } else if (ok) {
-                    sm.re[j] += xv[u].re[j];
-                    sm.im[j] += xv[u].im[j];
+                } else {
+                    if (ok) sm.re[j] += xv[u].re[j];
+                    if (ok) sm.im[j] += xv[u].im[j];
                 }
             }
         }
-        for (int k = 4; k < cur.w; k += 4) {
+        if constexpr (!W) for (int k = 4; k < cur.w; k += 4) {
             int w;
-            const int64_t base = row_base(a, r, w);
+            const int64_t base = row_base<W>(a, r, w);
             int32_t c[4];
             bool ok[4];
 #pragma unroll
@@ -556,47 +561,31 @@ __device__ __forceinline__ Cv<V, SPL> row_term(const TermArgs &a, uint32_t r, in
             for (int u = 0; u < 4; ++u) xw[u] = ld_ro<V, L, SPL>(a.x, c[u], l);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (ok[u]) {
 #pragma unroll
-                    for (int j = 0; j < SPL; ++j) {
-                        sm.re[j] += xw[u].re[j];
-                        sm.im[j] += xw[u].im[j];
-                    }
+                for (int j = 0; j < SPL; ++j) {
+                    if (ok[u]) sm.re[j] += xw[u].re[j];
+                    if (ok[u]) sm.im[j] += xw[u].im[j];
                 }
             }
         }
-        if (const V *sc = scales()) {
-#pragma unroll
-            for (int j = 0; j < SPL; ++j) {
-                const V sv = sc[j];
-                p.re[j] *= sv;
-                p.im[j] *= sv;
-                if (a.x_is_psi) {
-                    sm.re[j] *= sv;
-                    sm.im[j] *= sv;
-                    y.re[j] *= sv;
-                    y.im[j] *= sv;
-                }
-            }
-        }
-        return combine_sum<SPL>(a, d, y, sm, p, zz);
+        return combine_form<SPL, M != kOneNoDiag>(a, d, y, sm, p, zz);
     } else {
 #pragma unroll
         for (int j = 0; j < SPL; ++j) { y.re[j] *= d; y.im[j] *= d; }
         // four entries a round, the first round's columns and gathers ahead
-        auto round = [&](int k, const int32_t (&c)[4], const Cv<V, SPL> (&xw)[4], auto first) {
+        auto round = [&](int k, const int32_t *c, const Cv<V, SPL> *xw, auto first) {
             [[maybe_unused]] int w;
             [[maybe_unused]] int64_t base = 0;
             if constexpr (M == kComplex || (M == kReal && !(AHEAD && decltype(first)::value)))
-                base = row_base(a, r, w);
+                base = row_base<W>(a, r, w);
             [[maybe_unused]] const V *valp = reinterpret_cast<const V *>(a.H.val) + base;
             [[maybe_unused]] const V2 *valp2 = reinterpret_cast<const V2 *>(a.H.val) + base;
-            V h[4];
-            [[maybe_unused]] V hm[4];
-            bool ok[4];
+            V h[NS];
+            [[maybe_unused]] V hm[NS];
+            bool ok[NS];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                ok[u] = k + u < cur.w;
+            for (int u = 0; u < NS; ++u) {
+                ok[u] = W || k + u < cur.w;
                 if constexpr (M == kComplex) {
                     V2 v2;
                     v2.x = (V)0;
@@ -615,24 +604,22 @@ __device__ __forceinline__ Cv<V, SPL> row_term(const TermArgs &a, uint32_t r, in
                 }
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (ok[u]) {
+            for (int u = 0; u < NS; ++u) {
 #pragma unroll
-                    for (int j = 0; j < SPL; ++j) {
-                        y.re[j] = fma(h[u], xw[u].re[j], y.re[j]);
-                        y.im[j] = fma(h[u], xw[u].im[j], y.im[j]);
-                        if constexpr (M == kComplex) {       // (h + i hm)(x_re + i x_im)
-                            y.re[j] = fma(-hm[u], xw[u].im[j], y.re[j]);
-                            y.im[j] = fma(hm[u], xw[u].re[j], y.im[j]);
-                        }
+                for (int j = 0; j < SPL; ++j) {
+                    if (ok[u]) y.re[j] = fma(h[u], xw[u].re[j], y.re[j]);
+                    if (ok[u]) y.im[j] = fma(h[u], xw[u].im[j], y.im[j]);
+                    if constexpr (M == kComplex) {       // (h + i hm)(x_re + i x_im)
+                        if (ok[u]) y.re[j] = fma(-hm[u], xw[u].im[j], y.re[j]);
+                        if (ok[u]) y.im[j] = fma(hm[u], xw[u].re[j], y.im[j]);
                     }
                 }
             }
         };
         round(0, cur.c, xv, std::true_type{});
-        for (int k = 4; k < cur.w; k += 4) {
+        if constexpr (!W) for (int k = 4; k < cur.w; k += 4) {
             int w;
-            const int64_t base = row_base(a, r, w);
+            const int64_t base = row_base<W>(a, r, w);
             int32_t c[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
@@ -643,13 +630,15 @@ __device__ __forceinline__ Cv<V, SPL> row_term(const TermArgs &a, uint32_t r, in
             for (int u = 0; u < 4; ++u) xw[u] = ld_ro<V, L, SPL>(a.x, c[u], l);
             round(k, c, xw, std::false_type{});
         }
-        if (const V *sc = scales()) {            // psi -> psi * scale (per state)
+        if constexpr (sizeof(V) == 4) {
+            if (const V *sc = scales()) {        // psi -> psi * scale (per state)
 #pragma unroll
-            for (int j = 0; j < SPL; ++j) {
-                const V sv = sc[j];
-                p.re[j] *= sv;
-                p.im[j] *= sv;
-                if (a.x_is_psi) { y.re[j] *= sv; y.im[j] *= sv; }
+                for (int j = 0; j < SPL; ++j) {
+                    const V sv = sc[j];
+                    p.re[j] *= sv;
+                    p.im[j] *= sv;
+                    if (a.x_is_psi) { y.re[j] *= sv; y.im[j] *= sv; }
+                }
             }
         }
         const V g = Coef<V>::g(a), ch = Coef<V>::hi(a), cl = Coef<V>::lo(a);
@@ -689,7 +678,7 @@ __device__ __forceinline__ int64_t block_in_order(const TermArgs &a)
 // Thread t works on row t / (L RS), lane (t / RS) % L, part t % RS.  Rows are
 // a multiple of 1024, so a warp never straddles the last row (the part
 // shuffles see full warps).
-template <typename V, int L, int SPL, Vals M, int RS>
+template <typename V, int L, int SPL, Vals M, int W, int RS>
 __global__ void __launch_bounds__(256, sizeof(V) == 4 ? (SPL <= 2 ? 5 : 4) : (SPL == 1 ? 4 : 3)) k_term(TermArgs a)
 {
     dep_launch();
@@ -697,7 +686,7 @@ __global__ void __launch_bounds__(256, sizeof(V) == 4 ? (SPL <= 2 ? 5 : 4) : (SP
     const int64_t r = t / (L * RS);
     const int l = (int)((t / RS) % L);
     if constexpr (RS == 1) {
-        RowAhead<V, M, false> row;
+        RowAhead<V, M, W, false> row;
         if (r < a.n_rows) row_ahead(a, r, row);
         dep_wait();
         if (r >= a.n_rows) return;
@@ -721,7 +710,7 @@ __global__ void __launch_bounds__(256, sizeof(V) == 4 ? (SPL <= 2 ? 5 : 4) : (SP
 // loads.  One kernel per kind of values: with one value no value registers
 // are carried, and the 16-byte lanes fit 64 registers.  HBM-bound: 178 us at
 // 4 x 8.3M FP32 rows, 6.7 TB/s (188 us as ordinary launches).
-template <typename V, int L, int SPL, Vals M>
+template <typename V, int L, int SPL, Vals M, int W>
 __global__ void __launch_bounds__(256, sizeof(V) == 4 ? (SPL <= 2 ? 4 : 3) : 2) k_term_pf(TermArgs a)
 {
     dep_launch();
@@ -732,12 +721,12 @@ __global__ void __launch_bounds__(256, sizeof(V) == 4 ? (SPL <= 2 ? 4 : 3) : 2) 
     const int l = (int)(t % L);
     uint32_t i = t / L;                                  // position in traversal order
     auto row_of = [&](uint32_t k) { return a.reverse ? n_rows - 1 - k : k; };
-    RowAhead<V, M, true> cur;
+    RowAhead<V, M, W, true> cur;
     if (i < n_rows) row_ahead(a, row_of(i), cur);
     dep_wait();
     for (; i < n_rows; i += rows_per_pass) {
         const uint32_t r = row_of(i);
-        RowAhead<V, M, true> nxt;
+        RowAhead<V, M, W, true> nxt;
         const uint32_t i2 = i + rows_per_pass;
         const Cv<V, SPL> o = row_term<V, L, SPL>(a, r, l, cur, [&] {
             // the next row's indices, values and diagonal, in flight meanwhile
@@ -853,7 +842,7 @@ __device__ __forceinline__ void final_reduce(const TermArgs &a, int64_t bid, int
     }
 }
 
-template <typename V, int L, int SPL, bool COMPUTE, Vals M>
+template <typename V, int L, int SPL, bool COMPUTE, Vals M, int W>
 __global__ void __launch_bounds__(kFinalThreads) k_final(TermArgs a)
 {
     dep_launch();
@@ -863,7 +852,7 @@ __global__ void __launch_bounds__(kFinalThreads) k_final(TermArgs a)
     const int l = (int)(t % L);
     Cv<V, SPL> o;
     if (COMPUTE) {
-        RowAhead<V, M, false> row;
+        RowAhead<V, M, W, false> row;
         row_ahead(a, r, row);
         dep_wait();
         o = row_term<V, L, SPL>(a, r, l, row, [] {});
@@ -1038,11 +1027,11 @@ __device__ __forceinline__ Cv<double, SPL> halo_row_sum(const TermArgs &a, const
                     s.re[j] = ok[0] ? xv[0].re[j] : 0.0;
                     s.im[j] = ok[0] ? xv[0].im[j] : 0.0;
                 }
-            } else if (ok[u]) {
+            } else {
 #pragma unroll
                 for (int j = 0; j < SPL; ++j) {
-                    s.re[j] += xv[u].re[j];
-                    s.im[j] += xv[u].im[j];
+                    if (ok[u]) s.re[j] += xv[u].re[j];
+                    if (ok[u]) s.im[j] += xv[u].im[j];
                 }
             }
         }
@@ -1155,12 +1144,10 @@ __global__ void __launch_bounds__(kHaloRows * L, 8 / L) k_term_halo(TermArgs a)
         for (int u = 0; u < 4; ++u) xv[u] = ld_halo<V, L, SPL>(xs, hp[u], l);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            if (ok[u]) {
 #pragma unroll
-                for (int j = 0; j < SPL; ++j) {
-                    y.re[j] = fma(h[u], xv[u].re[j], y.re[j]);
-                    y.im[j] = fma(h[u], xv[u].im[j], y.im[j]);
-                }
+            for (int j = 0; j < SPL; ++j) {
+                if (ok[u]) y.re[j] = fma(h[u], xv[u].re[j], y.re[j]);
+                if (ok[u]) y.im[j] = fma(h[u], xv[u].im[j], y.im[j]);
             }
         }
     }
@@ -1275,9 +1262,9 @@ __device__ __forceinline__ Cv<double, 1> pipe_row_sum(const TermArgs &a, const u
             if (decltype(first)::value && u == 0) {
                 s.re[0] = ok[0] ? xv[0].re[0] : 0.0;
                 s.im[0] = ok[0] ? xv[0].im[0] : 0.0;
-            } else if (ok[u]) {
-                s.re[0] += xv[u].re[0];
-                s.im[0] += xv[u].im[0];
+            } else {
+                if (ok[u]) s.re[0] += xv[u].re[0];
+                if (ok[u]) s.im[0] += xv[u].im[0];
             }
         }
     };
@@ -1363,12 +1350,10 @@ __device__ __forceinline__ Cv<V, 16 / (2 * sizeof(V))> staged_row(
         if (k + 4 < w) load4(k + 4);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            if (ok[u]) {
 #pragma unroll
-                for (int j = 0; j < SPL; ++j) {
-                    y.re[j] = fma(h[u], xv[u].re[j], y.re[j]);
-                    y.im[j] = fma(h[u], xv[u].im[j], y.im[j]);
-                }
+            for (int j = 0; j < SPL; ++j) {
+                if (ok[u]) y.re[j] = fma(h[u], xv[u].re[j], y.re[j]);
+                if (ok[u]) y.im[j] = fma(h[u], xv[u].im[j], y.im[j]);
             }
         }
     }
@@ -1866,32 +1851,50 @@ __global__ void k_corr_mean_adjoint(const double2 *gavg, int n_samples, int S, i
     g[i] = make_double2(v.x / S, v.y / S);
 }
 
-template <typename V, int L, int SPL, Vals M, int RS = 1>
-cudaError_t launch_term_t(const TermArgs &a, int threads, cudaStream_t st)
+template <typename V, int L, int SPL, typename Fm, int RS = 1>
+cudaError_t launch_term_f(const TermArgs &a, int threads, cudaStream_t st)
 {
     const int64_t n_threads = a.n_rows * L * RS;
     const unsigned blocks = (unsigned)((n_threads + threads - 1) / threads);
-    return launch_dependent(k_term<V, L, SPL, M, RS>, blocks, threads, 0, st, a);
+    return launch_dependent(k_term<V, L, SPL, Fm::M, Fm::W, RS>, blocks, threads, 0, st, a);
 }
 
-// One row a thread, real values.
-template <typename V, int L, int SPL>
-cudaError_t launch_term_u(const TermArgs &a, int threads, cudaStream_t st)
+// The forms of one shape: the three-slot kernels for 16-byte lanes.
+template <typename V, int L, int SPL, typename F>
+cudaError_t with_term_form(const TermArgs &a, F &&f)
 {
-    return a.uniform ? launch_term_t<V, L, SPL, kOne>(a, threads, st)
-                     : launch_term_t<V, L, SPL, kReal>(a, threads, st);
+    constexpr bool lane16 = sizeof(V) * 2 * SPL <= 16;
+    return with_form<sizeof(V) == 8, lane16>(a.cplx, a.uniform, a.zero_diag, a.gdiag != nullptr,
+                                             a.fixed_width, f);
+}
+
+// One row a thread.
+template <typename V, int L, int SPL>
+struct TermLaunch {
+    const TermArgs &a;
+    int threads;
+    cudaStream_t st;
+    template <typename Fm> cudaError_t operator()(Fm) const
+    {
+        return launch_term_f<V, L, SPL, Fm>(a, threads, st);
+    }
+};
+template <typename V, int L, int SPL>
+cudaError_t launch_term_t(const TermArgs &a, int threads, cudaStream_t st)
+{
+    return with_term_form<V, L, SPL>(a, TermLaunch<V, L, SPL>{a, threads, st});
 }
 
 // The register-pipelined kernel: a persistent grid of the SMs times the
 // blocks that fit on one, at most one thread per lane-row.
-template <typename V, int L, int SPL, Vals M>
-cudaError_t launch_term_pf_m(const TermArgs &a, int threads, cudaStream_t st)
+template <typename V, int L, int SPL, typename Fm>
+cudaError_t launch_term_pf_f(const TermArgs &a, int threads, cudaStream_t st)
 {
     static int occ[4] = {0, 0, 0, 0};            // resident blocks per SM by threads 64 .. 512
     const int ti = threads <= 64 ? 0 : threads <= 128 ? 1 : threads <= 256 ? 2 : 3;
     if (!occ[ti]) {
         int nb = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_term_pf<V, L, SPL, M>, threads, 0) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_term_pf<V, L, SPL, Fm::M, Fm::W>, threads, 0) !=
             cudaSuccess)
             nb = 1;
         occ[ti] = std::max(1, nb);
@@ -1900,14 +1903,22 @@ cudaError_t launch_term_pf_m(const TermArgs &a, int threads, cudaStream_t st)
     const int64_t want = (n_threads + threads - 1) / threads;
     const unsigned blocks =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)std::max(1, a.num_sms) * occ[ti], want));
-    return launch_dependent(k_term_pf<V, L, SPL, M>, blocks, threads, 0, st, a);
+    return launch_dependent(k_term_pf<V, L, SPL, Fm::M, Fm::W>, blocks, threads, 0, st, a);
 }
 
 template <typename V, int L, int SPL>
 cudaError_t launch_term_pf_t(const TermArgs &a, int threads, cudaStream_t st)
 {
-    return a.uniform ? launch_term_pf_m<V, L, SPL, kOne>(a, threads, st)
-                     : launch_term_pf_m<V, L, SPL, kReal>(a, threads, st);
+    if constexpr (sizeof(V) == 4)
+        if (a.fixed_width == 3)
+            return a.uniform ? launch_term_pf_f<V, L, SPL, Form<kOne, 3>>(a, threads, st)
+                             : launch_term_pf_f<V, L, SPL, Form<kReal, 3>>(a, threads, st);
+    if (!a.uniform) return launch_term_pf_f<V, L, SPL, Form<kReal, 0>>(a, threads, st);
+    if constexpr (sizeof(V) == 8) {
+        if (a.zero_diag) return launch_term_pf_f<V, L, SPL, Form<kOneNoDiag, 0>>(a, threads, st);
+        if (!a.gdiag) return launch_term_pf_f<V, L, SPL, Form<kOneMul, 0>>(a, threads, st);
+    }
+    return launch_term_pf_f<V, L, SPL, Form<kOne, 0>>(a, threads, st);
 }
 
 // The widths a TBPM_VARIANT_PREFETCH term runs at, all bit-identical.  FP32
@@ -1946,11 +1957,11 @@ cudaError_t dispatch_pf(const TermArgs &a, int fp32, int B, int threads, cudaStr
     }
     if (a.n_rows * std::max(1, B / 2) <= kPrefetchMinLanes) {
         switch (B) {
-        case 1: return launch_term_u<float, 1, 1>(a, 256, st);
-        case 2: return launch_term_u<float, 1, 2>(a, 256, st);
-        case 4: return launch_term_u<float, 2, 2>(a, 256, st);
-        case 8: return launch_term_u<float, 4, 2>(a, 256, st);
-        case 16: return launch_term_u<float, 8, 2>(a, 256, st);
+        case 1: return launch_term_t<float, 1, 1>(a, 256, st);
+        case 2: return launch_term_t<float, 1, 2>(a, 256, st);
+        case 4: return launch_term_t<float, 2, 2>(a, 256, st);
+        case 8: return launch_term_t<float, 4, 2>(a, 256, st);
+        case 16: return launch_term_t<float, 8, 2>(a, 256, st);
         }
         return cudaErrorInvalidValue;
     }
@@ -1971,31 +1982,44 @@ template <typename V, int L, int SPL>
 cudaError_t launch_term_split(const TermArgs &a, int threads, cudaStream_t st)
 {
     // (the row split reads TermArgs::uniform at run time)
-    if (a.variant & kVariantSplit4) return launch_term_t<V, L, SPL, kReal, 4>(a, threads, st);
-    return launch_term_t<V, L, SPL, kReal, 2>(a, threads, st);
+    if (a.variant & kVariantSplit4) return launch_term_f<V, L, SPL, Form<kReal, 0>, 4>(a, threads, st);
+    return launch_term_f<V, L, SPL, Form<kReal, 0>, 2>(a, threads, st);
 }
 
-template <typename V, int L, int SPL, Vals M>
+template <typename V, int L, int SPL>
+struct FinalLaunch {
+    const TermArgs &a;
+    unsigned blocks;
+    cudaStream_t st;
+    template <typename Fm> cudaError_t operator()(Fm) const
+    {
+        return launch_dependent(k_final<V, L, SPL, true, Fm::M, Fm::W>, blocks, kFinalThreads, 0, st, a);
+    }
+};
+
+template <typename V, int L, int SPL>
 cudaError_t launch_final_t(const TermArgs &a, int threads, bool compute, cudaStream_t st)
 {
     (void)threads;   // the closing term has its own block size
-    if constexpr (sizeof(V) == 4 && M != kComplex) {
-        if (!compute) {           // FP32 reduction-only pass: four rows a thread
+    if constexpr (sizeof(V) == 4) {
+        if (!compute && !a.cplx) {      // FP32 reduction-only pass: four rows a thread
             constexpr int RPT = 4;
             const unsigned rblocks = (unsigned)(a.n_rows * L / (kFinalThreads * RPT));
             return launch_dependent(k_final_sums<L, SPL, RPT>, rblocks, kFinalThreads, 0, st, a);
         }
     }
     const unsigned blocks = (unsigned)(a.n_rows * L / kFinalThreads);
-    return launch_dependent(compute ? k_final<V, L, SPL, true, M> : k_final<V, L, SPL, false, M>,
-                            blocks, kFinalThreads, 0, st, a);
+    if (!compute)
+        return launch_dependent(k_final<V, L, SPL, false, kReal, 0>, blocks, kFinalThreads, 0,
+                                st, a);
+    return with_term_form<V, L, SPL>(a, FinalLaunch<V, L, SPL>{a, blocks, st});
 }
 
-template <bool FINAL, Vals M>
-cudaError_t dispatch_m(const TermArgs &a, int fp32, int B, int threads, bool compute,
-                        cudaStream_t st)
+template <bool FINAL>
+cudaError_t dispatch(const TermArgs &a, int fp32, int B, int threads, bool compute,
+                     cudaStream_t st)
 {
-    if (!FINAL && M != kComplex && (a.variant & (kVariantSplit2 | kVariantSplit4))) {
+    if (!FINAL && !a.cplx && (a.variant & (kVariantSplit2 | kVariantSplit4))) {
         if (a.variant & kVariantWide) {
             if (!fp32) {
                 switch (B) {
@@ -2029,9 +2053,9 @@ cudaError_t dispatch_m(const TermArgs &a, int fp32, int B, int threads, bool com
         }
     }
 #define TBPM_CASE(V, L, SPL)                                                  \
-    return FINAL ? launch_final_t<V, L, SPL, M>(a, threads, compute, st)     \
-                 : launch_term_t<V, L, SPL, M>(a, threads, st)
-    if constexpr (M != kComplex) if (a.variant & kVariantWide) {
+    return FINAL ? launch_final_t<V, L, SPL>(a, threads, compute, st)        \
+                 : launch_term_t<V, L, SPL>(a, threads, st)
+    if (!a.cplx && (a.variant & kVariantWide)) {
         // one thread per row and 32-byte lanes: fewer lanes share the index loads
         if (!fp32) {
             switch (B) {
@@ -2065,15 +2089,6 @@ cudaError_t dispatch_m(const TermArgs &a, int fp32, int B, int threads, bool com
     }
 #undef TBPM_CASE
     return cudaErrorInvalidValue;
-}
-
-template <bool FINAL>
-cudaError_t dispatch(const TermArgs &a, int fp32, int B, int threads, bool compute,
-                     cudaStream_t st)
-{
-    if (a.cplx) return dispatch_m<FINAL, kComplex>(a, fp32, B, threads, compute, st);
-    return a.uniform ? dispatch_m<FINAL, kOne>(a, fp32, B, threads, compute, st)
-                     : dispatch_m<FINAL, kReal>(a, fp32, B, threads, compute, st);
 }
 
 }  // namespace

@@ -129,6 +129,44 @@ struct SellView {
     const void *diag;          // double or float [n_rows]
 };
 
+// Matrix forms the kernels are compiled for.  A warp's FP64 instruction
+// occupies its share of GB300's FP64 pipe for 64 cycles, and the compiler
+// executes short conditional FP64 code and selects the result, so what a
+// form does not have must not be in its kernel: with the entries in rounds
+// of four under a bound known at run time, and the diagonal under a flag,
+// the FP64 term of pristine graphene executed 14 FP64 operations a state and
+// row for the 8 it needs.
+//   Vals  one real value for all entries (BuildOutput::uniform), in FP64 with
+//         gamma d stored, gamma d multiplied (the first term of a step) or no
+//         diagonal; a real value per entry; a complex one
+//   W     3: every row of every slice has three slots (the graphene family),
+//         0: any widths, read per slice
+enum Vals { kOne, kOneMul, kOneNoDiag, kReal, kComplex };
+constexpr bool one_value(Vals m) { return m == kOne || m == kOneMul || m == kOneNoDiag; }
+template <Vals M_, int W_> struct Form {
+    static constexpr Vals M = M_;
+    static constexpr int W = W_;
+};
+// f(Form) for a matrix.  F64: tell the FP64 one-value forms apart (gd: gamma d
+// is stored); W3: there are three-slot kernels
+template <bool F64, bool W3, typename F>
+inline cudaError_t with_form(int cplx, int uniform, int zero_diag, bool gd, int fixed_width, F &&f)
+{
+    auto widths = [&](auto m) -> cudaError_t {
+        constexpr Vals M = decltype(m)::M;
+        if constexpr (W3)
+            if (fixed_width == 3) return f(Form<M, 3>{});
+        return f(Form<M, 0>{});
+    };
+    if (cplx) return widths(Form<kComplex, 0>{});
+    if (!uniform) return widths(Form<kReal, 0>{});
+    if constexpr (F64) {
+        if (zero_diag) return widths(Form<kOneNoDiag, 0>{});
+        if (!gd) return widths(Form<kOneMul, 0>{});
+    }
+    return widths(Form<kOne, 0>{});
+}
+
 // One Clenshaw term: out = c * psi + gamma * (-i) * H~ x + z, optionally
 // with psi scaled per state (FP32 norm carry).
 struct TermArgs {

@@ -52,3 +52,20 @@ def test_wide_lane_rule_is_bit_identical(sides):
     C1, b = _states(tb, smp, theta, tb.TBPM_FP32, 4, PREFETCH, 2)
     assert (a == b).all()
     assert np.abs(C0 - C1).max() < 1e-12
+
+
+# three-slot rows (fixed slice width 3) against the TMA kernel, which reads the
+# widths at run time: every matrix form, FP32 and FP64
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("B", [1, 2, 8])
+@pytest.mark.parametrize("onsite_w,sigma", [(0.0, 0.0), (1.0, 0.0), (0.0, 0.05), (1.0, 0.05)])
+def test_three_slot_forms_are_bit_identical(precision, B, onsite_w, sigma):
+    import paper_2209_00806_gb300 as tb
+    smp = lattice.graphene(23, 31, pbc=True, seed=8, onsite_w=onsite_w, bond_sigma=sigma,
+                           vacancy_frac=0.01)
+    theta = rng.phases(9, B, smp.n_orb)
+    C0, a = _states(tb, smp, theta, precision, B, 5, 3)       # ZIGZAG | TMA
+    C1, b = _states(tb, smp, theta, precision, B, PLAIN, 3)
+    assert (a == b).all()
+    assert np.abs(C0 - C1).max() < 1e-12
+
