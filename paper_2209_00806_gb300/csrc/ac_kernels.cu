@@ -1,18 +1,20 @@
 // AC-conductivity path (Sec. 2.7 with the Fermi-Dirac operator of Sec. 2.2).
 //
-// Preparation (once per random state, FP64, four lanes per row):
-//   lanes 0, 1 <- psi;  lanes 2, 3 <- J_x psi, J_y psi with
+// Preparation (once per random state, FP64, three lanes per row):
+//   lane 0 <- psi;  lanes 1, 2 <- J_x psi, J_y psi with
 //   (J_a v)_r = -i s sum_c H~_rc d^a_rc v_c   (the hopping current with e / hbar
 //   factored out, units eV nm; d_rc = r_c - r_r is the bond vector of the
 //   stored entry, so periodic bonds carry their own image); then the Fermi
 //   operator by Clenshaw's
-//   recurrence on lanes 1 .. 3, b_k = c_k v + 2 H~ b_{k+1} - b_{k+2},
+//   recurrence on the three, b_k = c_k v + 2 H~ b_{k+1} - b_{k+2},
 //   f v = c_0 v / 2 + H~ b_1 - b_2.
 // Observer (after every time step, in the group's precision): per row and
 // lane quad, g_a = sum_c H~_rc d^a_rc psi_2,c and the four products
 // conj(g_a) psi_1b,r, reduced deterministically per sample.
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "tbpm_internal.cuh"
 
@@ -65,38 +67,19 @@ template <typename VT> __device__ __forceinline__ double diag_of(const void *d, 
     return (double)__ldg(reinterpret_cast<const VT *>(d) + r);
 }
 
-// State element (row r, lane l) of a [row][B] buffer as complex double.
-template <typename V> struct StateLd;
-template <> struct StateLd<double> {
-    __device__ static double2 get(const void *p, int64_t i)
-    {
-        return __ldg(reinterpret_cast<const double2 *>(p) + i);
-    }
-};
-template <> struct StateLd<float> {
-    __device__ static double2 get(const void *p, int64_t i)
-    {
-        const float2 f = __ldg(reinterpret_cast<const float2 *>(p) + i);
-        return make_double2((double)f.x, (double)f.y);
-    }
-};
-
 // ---- preparation ------------------------------------------------------------
 
 __global__ void k_ac_load(const double2 *psi_user, int p, int64_t n_orb,
-                          const int32_t *user_to_row, double2 *v4)
+                          const int32_t *user_to_row, double2 *v3)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n_orb) return;
-    const int64_t r = user_to_row[i];
-    const double2 v = psi_user[(int64_t)p * n_orb + i];
-    v4[r * 4 + 0] = v;
-    v4[r * 4 + 1] = v;
+    v3[(int64_t)user_to_row[i] * kAcLanes] = psi_user[(int64_t)p * n_orb + i];
 }
 
 template <typename VT, bool CX>
-__global__ void k_current4(SellView H, int64_t n_rows, const double *dxe, const double *dye,
-                           double s, double2 *v4)
+__global__ void k_current3(SellView H, int64_t n_rows, const double *dxe, const double *dye,
+                           double s, double2 *v3)
 {
     const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (r >= n_rows) return;
@@ -107,7 +90,7 @@ __global__ void k_current4(SellView H, int64_t n_rows, const double *dxe, const 
     for (int k = 0; k < w; ++k) {
         const int64_t e = base + (int64_t)k * kSliceRows + lr;
         const int32_t c = __ldg(H.col + e);
-        const double2 hv = hmul<CX>(HVal<VT, CX>::get(H.val, e), v4[(int64_t)c * 4]);
+        const double2 hv = hmul<CX>(HVal<VT, CX>::get(H.val, e), v3[(int64_t)c * kAcLanes]);
         const double dx = __ldg(dxe + e), dy = __ldg(dye + e);
         gx.x = fma(dx, hv.x, gx.x);
         gx.y = fma(dx, hv.y, gx.y);
@@ -115,63 +98,122 @@ __global__ void k_current4(SellView H, int64_t n_rows, const double *dxe, const 
         gy.y = fma(dy, hv.y, gy.y);
     }
     // -i s g = s (g.y, -g.x)
-    v4[r * 4 + 2] = make_double2(s * gx.y, -s * gx.x);
-    v4[r * 4 + 3] = make_double2(s * gy.y, -s * gy.x);
+    v3[r * kAcLanes + 1] = make_double2(s * gx.y, -s * gx.x);
+    v3[r * kAcLanes + 2] = make_double2(s * gy.y, -s * gy.x);
 }
 
-// out = c v + gamma (H~ x) + zeta z, one thread per (row, lane) for lanes
-// 1 .. 3 (lane 0 holds psi itself, which needs no Fermi operator); x ==
-// nullptr drops the product, z == nullptr the last term; out may alias z.
-template <typename VT, bool CX>
-__global__ void k_cheb_real4(SellView H, int64_t n_rows, double c, double gamma, double zeta,
-                             const double2 *v, const double2 *x, const double2 *z, double2 *out)
+// out = c v + gamma (H~ x) - z, one thread per (row, lane); x == nullptr drops
+// the product, z == nullptr the last term; out may alias z.  Bound by the
+// FP64 pipe: with one value the neighbours are added first and gamma h and
+// gamma d come as single factors, 2 (E - 1) + 6 operations for E entries (4
+// without a diagonal) instead of 8 + 2E entry by entry -- 8 against 14 on
+// pristine graphene -- and two fewer where c is zero (every other
+// coefficient at mu = 0).  The three lanes are packed (48 bytes a row), so
+// that v, x and z of half a million rows (75 MB) stay in the L2.  524,288
+// rows: 30.2 us a term with v and 23.8 us without, 44.3 us before.
+template <typename VT, Vals M, int W, bool HAS_V>
+__global__ void __launch_bounds__(256) k_ac_cheb(AcChebArgs a)
 {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= n_rows * 3) return;
-    const int64_t r = t / 3;
-    const int l = 1 + (int)(t % 3);
-    double2 y = make_double2(0.0, 0.0);
-    if (x) {
-        const double d = diag_of<VT>(H.diag, r);
-        const double2 xo = x[r * 4 + l];
-        y.x = d * xo.x;
-        y.y = d * xo.y;
-        const int64_t q = r / kSliceRows, lr = r % kSliceRows;
-        const int64_t base = H.slice_ptr[q];
-        const int w = (int)((H.slice_ptr[q + 1] - base) / kSliceRows);
-        for (int k = 0; k < w; ++k) {
-            const int64_t e = base + (int64_t)k * kSliceRows + lr;
-            const int32_t cc = __ldg(H.col + e);
-            const double2 hv = hmul<CX>(HVal<VT, CX>::get(H.val, e), x[(int64_t)cc * 4 + l]);
-            y.x += hv.x;
-            y.y += hv.y;
+    constexpr bool ONE = one_value(M);
+    constexpr int NS = W ? W : 4;                            // slots of the first round
+    dep_launch();
+    // n_rows * 3 is a multiple of 256, and below 2^32: the four buffers would
+    // not fit the device otherwise
+    const uint32_t t = blockIdx.x * 256u + threadIdx.x;
+    const uint32_t r = t / kAcLanes, l = t % kAcLanes;
+    const uint32_t q = r / kSliceRows, lr = r % kSliceRows;
+    int64_t base;
+    int w;
+    if (W || a.fixed_width) {
+        w = W ? W : a.fixed_width;
+        base = (int64_t)q * (kSliceRows * w) + lr;
+    } else {
+        base = __ldg(a.H.slice_ptr + q);
+        w = (int)((__ldg(a.H.slice_ptr + q + 1) - base) / kSliceRows);
+        base += lr;
+    }
+    int32_t c0[NS];
+#pragma unroll
+    for (int u = 0; u < NS; ++u)
+        c0[u] = W || u < w ? __ldg(a.H.col + base + u * kSliceRows) : (int32_t)r;
+    double d = 0.0;
+    if (!ONE) d = diag_of<VT>(a.H.diag, r);
+    else if (M == kOne) d = __ldg(a.gdiag + r);
+    dep_wait();
+    double2 vv = make_double2(0.0, 0.0), zz = vv, xo = vv, y = vv;
+    if (HAS_V) vv = a.v[t];
+    if (a.z) zz = a.z[t];
+    if (!a.x) {             // the first term of the recurrence, b_{K-1} = c_{K-1} v
+        a.out[t] = make_double2(fma(a.c, vv.x, -zz.x), fma(a.c, vv.y, -zz.y));
+        return;
+    }
+    double2 o;
+    if (M != kOneNoDiag) xo = a.x[t];
+    if (!ONE) y = make_double2(d * xo.x, d * xo.y);
+    auto round = [&](int k, const auto &c, auto first) {
+        double2 xv[NS];
+#pragma unroll
+        for (int u = 0; u < NS; ++u) xv[u] = a.x[(int64_t)c[u] * kAcLanes + l];
+#pragma unroll
+        for (int u = 0; u < NS; ++u) {
+            // padded slots (own row) follow a row's entries
+            const bool ok = (W || k + u < w) && (!ONE || c[u] != (int32_t)r);
+            if constexpr (ONE) {
+                if (decltype(first)::value && u == 0) {
+                    y.x = ok ? xv[0].x : 0.0;
+                    y.y = ok ? xv[0].y : 0.0;
+                } else if (ok) {
+                    y.x += xv[u].x;
+                    y.y += xv[u].y;
+                }
+            } else if (ok) {
+                const double2 h = HVal<VT, M == kComplex>::get(a.H.val, base + (int64_t)(k + u) * kSliceRows);
+                y.x = fma(h.x, xv[u].x, y.x);
+                y.y = fma(h.x, xv[u].y, y.y);
+                if (M == kComplex) {
+                    y.x = fma(-h.y, xv[u].y, y.x);
+                    y.y = fma(h.y, xv[u].x, y.y);
+                }
+            }
+        }
+    };
+    round(0, c0, std::true_type{});
+    if (!W) {
+        for (int k = 4; k < w; k += 4) {
+            int32_t c[NS];
+#pragma unroll
+            for (int u = 0; u < NS; ++u)
+                c[u] = k + u < w ? __ldg(a.H.col + base + (int64_t)(k + u) * kSliceRows) : (int32_t)r;
+            round(k, c, std::false_type{});
         }
     }
-    const double2 vv = v[r * 4 + l];
-    double2 o;
-    o.x = fma(c, vv.x, gamma * y.x);
-    o.y = fma(c, vv.y, gamma * y.y);
-    if (z) {
-        const double2 zz = z[r * 4 + l];
-        o.x = fma(zeta, zz.x, o.x);
-        o.y = fma(zeta, zz.y, o.y);
+    // gamma H~ x - z, then + c v
+    const double g = ONE ? a.gh : a.gamma;
+    o.x = fma(g, y.x, -zz.x);
+    o.y = fma(g, y.y, -zz.y);
+    if (M == kOne) {
+        o.x = fma(d, xo.x, o.x);
+        o.y = fma(d, xo.y, o.y);
     }
-    out[r * 4 + l] = o;
+    if (HAS_V) {
+        o.x = fma(a.c, vv.x, o.x);
+        o.y = fma(a.c, vv.y, o.y);
+    }
+    a.out[t] = o;
 }
 
-__global__ void k_ac_store(const double2 *v4, const double2 *f4, int p, int64_t n_orb,
+__global__ void k_ac_store(const double2 *v3, const double2 *f3, int p, int64_t n_orb,
                            const int32_t *user_to_row, double2 *out_user)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n_orb) return;
-    const int64_t r = user_to_row[i];
+    const double2 *v = v3 + (int64_t)user_to_row[i] * kAcLanes;
+    const double2 *f = f3 + (int64_t)user_to_row[i] * kAcLanes;
     double2 *o = out_user + (int64_t)(4 * p) * n_orb + i;
-    o[0] = v4[r * 4 + 0];                       // psi
-    o[n_orb] = f4[r * 4 + 1];                   // f psi
-    const double2 jx = v4[r * 4 + 2], fx = f4[r * 4 + 2];
-    const double2 jy = v4[r * 4 + 3], fy = f4[r * 4 + 3];
-    o[2 * n_orb] = make_double2(jx.x - fx.x, jx.y - fx.y);   // (1 - f) J_x psi
-    o[3 * n_orb] = make_double2(jy.x - fy.x, jy.y - fy.y);   // (1 - f) J_y psi
+    o[0] = v[0];                                // psi
+    o[n_orb] = f[0];                            // f psi
+    o[2 * n_orb] = make_double2(v[1].x - f[1].x, v[1].y - f[1].y);   // (1 - f) J_x psi
+    o[3 * n_orb] = make_double2(v[2].x - f[2].x, v[2].y - f[2].y);   // (1 - f) J_y psi
 }
 
 // Bond vectors onto the stored entries: bond b = (i, j) with d_b = r_j - r_i
@@ -235,10 +277,10 @@ template <typename A> __device__ __forceinline__ C2<A> obs_state(const void *p, 
 {
     C2<A> c;
     if (sizeof(A) == 4) {
-        const float2 f = __ldg(reinterpret_cast<const float2 *>(p) + i);
+        const float2 f = reinterpret_cast<const float2 *>(p)[i];
         c.x = (A)f.x; c.y = (A)f.y;
     } else {
-        const double2 d = __ldg(reinterpret_cast<const double2 *>(p) + i);
+        const double2 d = reinterpret_cast<const double2 *>(p)[i];
         c.x = (A)d.x; c.y = (A)d.y;
     }
     return c;
@@ -253,6 +295,8 @@ template <typename A> __device__ __forceinline__ C2<A> obs_state(const void *p, 
 template <typename A, bool CX>
 __global__ void __launch_bounds__(kAcRows) k_ac_observe(AcArgs a)
 {
+    dep_launch();
+    dep_wait();
     const int64_t r = blockIdx.x * (int64_t)kAcRows + threadIdx.x;   // n_rows % 1024 == 0
     const int quad = blockIdx.y;
     const int B = a.B;
@@ -360,85 +404,101 @@ __global__ void k_vec_to_f32(int64_t n, const double *src, float *dst)
     if (i < n) dst[i] = (float)src[i];
 }
 
-// One CTA of 512 threads per (sample, quad): thread (j, k) sums value k of
-// blocks j, j + 64, ... of the sample; then 8 threads add the 64 partials in
-// order.  Writes i s (sum) at the step index of the sample.
+// Sum of the block partials per (sample, quad): part j = 0 .. 63 adds blocks
+// j, j + 64, ... in order, then the 64 parts are added in order.  The parts are
+// spread over 16 one-warp blocks (four parts of eight values each) and the
+// last block to finish (ticket after a fence) adds them: one block alone
+// waited on its chains of loads, 31 us a step at half a million rows, 13 us so.
+// Writes i s (sum) at the step index of the sample.
 constexpr int kAcSplit = 64;
+constexpr int kAcParts = 4;               // parts per block
 
-__global__ void __launch_bounds__(kAcSplit * 8) k_ac_reduce(AcReduceArgs a)
+__global__ void __launch_bounds__(32) k_ac_reduce(AcReduceArgs a)
 {
+    dep_launch();
+    dep_wait();
     const int smp = blockIdx.x, quad = blockIdx.y;
-    const int k = threadIdx.x & 7, j = threadIdx.x >> 3;
+    const int k = threadIdx.x & 7, j = blockIdx.z * kAcParts + (threadIdx.x >> 3);
     const int per_chunk = kChunkRows / kAcRows;
     const int64_t b0 = a.sample_chunk_off[smp] * per_chunk;
     const int64_t b1 = a.sample_chunk_off[smp + 1] * per_chunk;
     const int nq = a.B / 4;
     double acc = 0.0;
+#pragma unroll 8
     for (int64_t b = b0 + j; b < b1; b += kAcSplit) acc += a.block_partial[(b * nq + quad) * 8 + k];
-    __shared__ double part[kAcSplit][8];
-    part[j][k] = acc;
-    __syncthreads();
+    const int64_t sq = (int64_t)smp * nq + quad;
+    double *mine = a.partial2 + sq * (kAcSplit * 8);
+    mine[j * 8 + k] = acc;
+    __threadfence();
+    __syncwarp();
+    int last = 0;
+    if (threadIdx.x == 0) last = atomicAdd(a.ticket + sq, 1u) == kAcSplit / kAcParts - 1;
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();
+    double t = 0.0;
     if (threadIdx.x < 8) {
-        double t = 0.0;
-        for (int jj = 0; jj < kAcSplit; ++jj) t += part[jj][threadIdx.x];
-        part[0][threadIdx.x] = t;
+#pragma unroll 16
+        for (int jj = 0; jj < kAcSplit; ++jj) t += __ldcg(mine + jj * 8 + threadIdx.x);
     }
-    __syncthreads();
-    if (threadIdx.x < 4) {
-        const int ab = threadIdx.x;
-        const double re = part[0][2 * ab], im = part[0][2 * ab + 1];
+    // value 2 ab is the real part, 2 ab + 1 the imaginary part of ab
+    const double im = __shfl_down_sync(0xffffffffu, t, 1);
+    if (threadIdx.x < 8 && (threadIdx.x & 1) == 0) {
+        const int ab = threadIdx.x / 2;
         const int step = a.step[smp] - 1;
         const int p = a.group_state0 / 4 + quad;
         const int64_t idx = (((int64_t)smp * (a.n_states / 4) + p) * 4 + ab) * (a.n_steps + 1) + step;
-        a.corr_ac[idx] = make_double2(-a.s * im, a.s * re);   // i s (re + i im)
+        a.corr_ac[idx] = make_double2(-a.s * im, a.s * t);   // i s (re + i im)
     }
+    if (threadIdx.x == 0) a.ticket[sq] = 0;                  // ready for the next launch
 }
 
 }  // namespace
 
 cudaError_t launch_ac_load(const double2 *psi_user, int p, int64_t n_orb,
-                           const int32_t *user_to_row, double2 *v4, cudaStream_t st)
+                           const int32_t *user_to_row, double2 *v3, cudaStream_t st)
 {
     const unsigned blocks = (unsigned)((n_orb + 255) / 256);
-    k_ac_load<<<blocks, 256, 0, st>>>(psi_user, p, n_orb, user_to_row, v4);
+    k_ac_load<<<blocks, 256, 0, st>>>(psi_user, p, n_orb, user_to_row, v3);
     return cudaGetLastError();
 }
 
-cudaError_t launch_current4(SellView H, int fp32_vals, int cplx, int64_t n_rows,
-                            const double *dxe, const double *dye, double s, double2 *v4,
+cudaError_t launch_current3(SellView H, int fp32_vals, int cplx, int64_t n_rows,
+                            const double *dxe, const double *dye, double s, double2 *v3,
                             cudaStream_t st)
 {
     const unsigned blocks = (unsigned)((n_rows + 127) / 128);
     if (fp32_vals) {
-        if (cplx) k_current4<float, true><<<blocks, 128, 0, st>>>(H, n_rows, dxe, dye, s, v4);
-        else k_current4<float, false><<<blocks, 128, 0, st>>>(H, n_rows, dxe, dye, s, v4);
+        if (cplx) k_current3<float, true><<<blocks, 128, 0, st>>>(H, n_rows, dxe, dye, s, v3);
+        else k_current3<float, false><<<blocks, 128, 0, st>>>(H, n_rows, dxe, dye, s, v3);
     } else {
-        if (cplx) k_current4<double, true><<<blocks, 128, 0, st>>>(H, n_rows, dxe, dye, s, v4);
-        else k_current4<double, false><<<blocks, 128, 0, st>>>(H, n_rows, dxe, dye, s, v4);
+        if (cplx) k_current3<double, true><<<blocks, 128, 0, st>>>(H, n_rows, dxe, dye, s, v3);
+        else k_current3<double, false><<<blocks, 128, 0, st>>>(H, n_rows, dxe, dye, s, v3);
     }
     return cudaGetLastError();
 }
 
-cudaError_t launch_cheb_real4(SellView H, int fp32_vals, int cplx, int64_t n_rows, double c,
-                              double gamma, double zeta, const double2 *v, const double2 *x,
-                              const double2 *z, double2 *out, cudaStream_t st)
+cudaError_t launch_ac_cheb(const AcChebArgs &a, int fp32_vals, int cplx, int uniform,
+                           cudaStream_t st)
 {
-    const unsigned blocks = (unsigned)((n_rows * 3 + 255) / 256);
-    if (fp32_vals) {
-        if (cplx) k_cheb_real4<float, true><<<blocks, 256, 0, st>>>(H, n_rows, c, gamma, zeta, v, x, z, out);
-        else k_cheb_real4<float, false><<<blocks, 256, 0, st>>>(H, n_rows, c, gamma, zeta, v, x, z, out);
-    } else {
-        if (cplx) k_cheb_real4<double, true><<<blocks, 256, 0, st>>>(H, n_rows, c, gamma, zeta, v, x, z, out);
-        else k_cheb_real4<double, false><<<blocks, 256, 0, st>>>(H, n_rows, c, gamma, zeta, v, x, z, out);
-    }
-    return cudaGetLastError();
+    const unsigned blocks = (unsigned)(a.n_rows * kAcLanes / 256);
+    auto go = [&](auto form, auto vt) -> cudaError_t {
+        typedef decltype(form) Fm;
+        typedef decltype(vt) VT;
+        return launch_dependent(a.c != 0.0 ? k_ac_cheb<VT, Fm::M, Fm::W, true>
+                                           : k_ac_cheb<VT, Fm::M, Fm::W, false>,
+                                blocks, 256, 0, st, a);
+    };
+    if (fp32_vals)      // values rounded to FP32: entry by entry
+        return cplx ? go(Form<kComplex, 0>{}, 0.f) : go(Form<kReal, 0>{}, 0.f);
+    return with_form<true, true>(cplx, uniform, a.zero_diag, true, a.fixed_width,
+                                 [&](auto form) { return go(form, 0.0); });
 }
 
-cudaError_t launch_ac_store(const double2 *v4, const double2 *f4, int p, int64_t n_orb,
+cudaError_t launch_ac_store(const double2 *v3, const double2 *f3, int p, int64_t n_orb,
                             const int32_t *user_to_row, double2 *out_user, cudaStream_t st)
 {
     const unsigned blocks = (unsigned)((n_orb + 255) / 256);
-    k_ac_store<<<blocks, 256, 0, st>>>(v4, f4, p, n_orb, user_to_row, out_user);
+    k_ac_store<<<blocks, 256, 0, st>>>(v3, f3, p, n_orb, user_to_row, out_user);
     return cudaGetLastError();
 }
 
@@ -456,14 +516,11 @@ cudaError_t launch_bond_vectors(int64_t n_hop, const int32_t *bond_rows, const i
 cudaError_t launch_ac_observe(const AcArgs &a, int fp32, int cplx, cudaStream_t st)
 {
     const dim3 grid((unsigned)(a.n_rows / kAcRows), (unsigned)(a.B / 4));
-    if (fp32) {
-        if (cplx) k_ac_observe<float, true><<<grid, kAcRows, 0, st>>>(a);
-        else k_ac_observe<float, false><<<grid, kAcRows, 0, st>>>(a);
-    } else {
-        if (cplx) k_ac_observe<double, true><<<grid, kAcRows, 0, st>>>(a);
-        else k_ac_observe<double, false><<<grid, kAcRows, 0, st>>>(a);
-    }
-    return cudaGetLastError();
+    if (fp32)
+        return launch_dependent(cplx ? k_ac_observe<float, true> : k_ac_observe<float, false>, grid,
+                                kAcRows, 0, st, a);
+    return launch_dependent(cplx ? k_ac_observe<double, true> : k_ac_observe<double, false>, grid,
+                            kAcRows, 0, st, a);
 }
 
 cudaError_t launch_vec_to_f32(int64_t n, const double *src, float *dst, cudaStream_t st)
@@ -475,8 +532,8 @@ cudaError_t launch_vec_to_f32(int64_t n, const double *src, float *dst, cudaStre
 
 cudaError_t launch_ac_reduce(const AcReduceArgs &a, cudaStream_t st)
 {
-    k_ac_reduce<<<dim3((unsigned)a.n_samples, (unsigned)(a.B / 4)), kAcSplit * 8, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_ac_reduce, dim3((unsigned)a.n_samples, (unsigned)(a.B / 4), kAcSplit / kAcParts),
+                            32, 0, st, a);
 }
 
 }  // namespace tbpm

@@ -91,6 +91,8 @@ struct tbpm_ctx {
     bool ac_on = false;
     double2 *d_ac_corr = nullptr;          // [n_samples][n_states / 4][4][n_steps + 1]
     double *d_ac_partial = nullptr;        // [n_rows / kAcRows][4][8]
+    double *d_ac_partial2 = nullptr;       // [n_samples][4][64][8]
+    unsigned int *d_ac_ticket = nullptr;   // [n_samples][4]
     // quasi-eigenstates
     bool qe_on = false;
     int qe_K = 0;
@@ -1124,6 +1126,8 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
             CUDA_OR_FAIL(c, launch_ac_observe(oa, fp32, c->H.cplx, c->st));
             AcReduceArgs ar;
             ar.block_partial = c->d_ac_partial;
+            ar.partial2 = c->d_ac_partial2;
+            ar.ticket = c->d_ac_ticket;
             ar.sample_chunk_off = c->d_sample_chunk_off;
             ar.n_samples = c->n_samples;
             ar.B = g.B;
@@ -2019,19 +2023,19 @@ extern "C" int tbpm_ac_correlation(tbpm_ctx *c, double z, int n_steps, double be
 
     const int S = c->n_states;
     const int64_t n_rows = c->H.n_rows, n_orb = c->n_orb;
-    const size_t v4n = (size_t)n_rows * 4;
-    double2 *v4 = nullptr, *f4 = nullptr, *bb[2] = {nullptr, nullptr}, *D = nullptr;
+    const size_t v3n = (size_t)n_rows * kAcLanes;
+    double2 *v3 = nullptr, *f3 = nullptr, *bb[2] = {nullptr, nullptr}, *D = nullptr;
     auto release = [&]() {
-        cudaFree(v4);
-        cudaFree(f4);
+        cudaFree(v3);
+        cudaFree(f3);
         cudaFree(bb[0]);
         cudaFree(bb[1]);
         cudaFree(D);
     };
-    rc = dalloc(c, &v4, v4n);
-    if (!rc) rc = dalloc(c, &f4, v4n);
-    if (!rc) rc = dalloc(c, &bb[0], v4n);
-    if (!rc) rc = dalloc(c, &bb[1], v4n);
+    rc = dalloc(c, &v3, v3n);
+    if (!rc) rc = dalloc(c, &f3, v3n);
+    if (!rc) rc = dalloc(c, &bb[0], v3n);
+    if (!rc) rc = dalloc(c, &bb[1], v3n);
     if (!rc) rc = dalloc(c, &D, (size_t)4 * S * n_orb);
     if (rc) { release(); return rc; }
 
@@ -2043,16 +2047,46 @@ extern "C" int tbpm_ac_correlation(tbpm_ctx *c, double z, int n_steps, double be
     Hp.val = fp32v ? (const void *)c->H.val32 : (const void *)c->H.val64;
     Hp.diag = fp32v ? (const void *)c->H.diag32 : (const void *)c->H.diag64;
     const int K = (int)cf.size();
+    // coefficients far below the truncation of the series (1e-15 max|c|) are
+    // the rounding of a transform of this length: at mu = 0 every even one
+    // but c_0 (f - 1/2 is odd).  Their terms take no v.
+    double cmax = 0.0;
+    for (double ck : cf) cmax = std::max(cmax, std::fabs(ck));
+    for (double &ck : cf)
+        if (std::fabs(ck) <= 1e-16 * cmax) ck = 0.0;
     auto prep_fail = [&](cudaError_t e) {
         release();
         return fail(c, TBPM_E_CUDA, std::string("AC preparation: ") + cudaGetErrorString(e));
     };
-    cudaError_t e = cudaMemsetAsync(v4, 0, v4n * sizeof(double2), c->st);
+    const bool one = c->H.uniform && !c->H.cplx && !fp32v;
+    if (one && !c->H.zero_diag && !c->H.diag2_64) {
+        std::string msg;
+        rc = build_diag2(c->H, c->st, msg);
+        if (rc) { release(); return fail(c, rc, msg); }
+    }
+    auto cheb = [&](double ck, double gamma, const double2 *x, const double2 *zz, double2 *out) {
+        AcChebArgs ca;
+        memset(&ca, 0, sizeof(ca));
+        ca.H = Hp;
+        ca.fixed_width = c->H.fixed_width;
+        ca.n_rows = n_rows;
+        ca.c = ck;
+        ca.gamma = gamma;
+        ca.v = v3;
+        ca.x = x;
+        ca.z = zz;
+        ca.out = out;
+        ca.zero_diag = c->H.zero_diag;
+        unsigned long long sign = 0;                     // gamma > 0 here
+        if (one) one_value_terms(c->H, gamma, &ca.gh, &ca.gdiag, &sign);
+        return launch_ac_cheb(ca, fp32v, c->H.cplx, one, c->st);
+    };
+    cudaError_t e = cudaMemsetAsync(v3, 0, v3n * sizeof(double2), c->st);
     if (e != cudaSuccess) return prep_fail(e);
     for (int p = 0; p < S; ++p) {
-        e = launch_ac_load(c->d_psi_user, p, n_orb, c->H.user_to_row, v4, c->st);
+        e = launch_ac_load(c->d_psi_user, p, n_orb, c->H.user_to_row, v3, c->st);
         if (e == cudaSuccess)
-            e = launch_current4(Hp, fp32v, c->H.cplx, n_rows, c->d_bond_dx, c->d_bond_dy, c->s, v4,
+            e = launch_current3(Hp, fp32v, c->H.cplx, n_rows, c->d_bond_dx, c->d_bond_dy, c->s, v3,
                                 c->st);
         if (e != cudaSuccess) return prep_fail(e);
         // Clenshaw: b_k = c_k v + 2 H~ b_{k+1} - b_{k+2}, k = K-1 .. 1;
@@ -2060,32 +2094,40 @@ extern "C" int tbpm_ac_correlation(tbpm_ctx *c, double z, int n_steps, double be
         int i1 = -1, i2 = -1;              // buffers of b_{k+1}, b_{k+2}
         for (int k = K - 1; k >= 1 && e == cudaSuccess; --k) {
             const int o = i2 >= 0 ? i2 : (i1 == 0 ? 1 : 0);
-            e = launch_cheb_real4(Hp, fp32v, c->H.cplx, n_rows, cf[k], 2.0, -1.0, v4,
-                                  i1 >= 0 ? bb[i1] : nullptr, i2 >= 0 ? bb[i2] : nullptr, bb[o],
-                                  c->st);
+            e = cheb(cf[k], 2.0, i1 >= 0 ? bb[i1] : nullptr, i2 >= 0 ? bb[i2] : nullptr, bb[o]);
             i2 = i1;
             i1 = o;
         }
         if (e == cudaSuccess)
-            e = launch_cheb_real4(Hp, fp32v, c->H.cplx, n_rows, 0.5 * cf[0], 1.0, -1.0, v4,
-                                  i1 >= 0 ? bb[i1] : nullptr, i2 >= 0 ? bb[i2] : nullptr, f4, c->st);
-        if (e == cudaSuccess) e = launch_ac_store(v4, f4, p, n_orb, c->H.user_to_row, D, c->st);
+            e = cheb(0.5 * cf[0], 1.0, i1 >= 0 ? bb[i1] : nullptr, i2 >= 0 ? bb[i2] : nullptr, f3);
+        if (e == cudaSuccess) e = launch_ac_store(v3, f3, p, n_orb, c->H.user_to_row, D, c->st);
         if (e != cudaSuccess) return prep_fail(e);
     }
     const size_t cnt = (size_t)c->n_samples * S * 4 * (n_steps + 1);
     rc = dalloc(c, &c->d_ac_corr, cnt);
+    const size_t n_sq = (size_t)c->n_samples * 4;          // (sample, quad) pairs of a group
     if (!rc) rc = dalloc(c, &c->d_ac_partial, (size_t)(n_rows / kAcRows) * 4 * 8);
-    if (rc) {
+    if (!rc) rc = dalloc(c, &c->d_ac_partial2, n_sq * 64 * 8);
+    if (!rc) rc = dalloc(c, &c->d_ac_ticket, n_sq);
+    auto free_ac = [&]() {
         cudaFree(c->d_ac_corr);
+        cudaFree(c->d_ac_partial);
+        cudaFree(c->d_ac_partial2);
+        cudaFree(c->d_ac_ticket);
         c->d_ac_corr = nullptr;
+        c->d_ac_partial = c->d_ac_partial2 = nullptr;
+        c->d_ac_ticket = nullptr;
+    };
+    if (rc) {
+        free_ac();
         release();
         return rc;
     }
     e = cudaMemsetAsync(c->d_ac_corr, 0, cnt * sizeof(double2), c->st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_ac_ticket, 0, n_sq * sizeof(unsigned int), c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
     if (e != cudaSuccess) {
-        cudaFree(c->d_ac_corr);
-        c->d_ac_corr = nullptr;
+        free_ac();
         return prep_fail(e);
     }
 
@@ -2118,10 +2160,7 @@ extern "C" int tbpm_ac_correlation(tbpm_ctx *c, double z, int n_steps, double be
     c->d_psi_user = user_psi;
     c->n_states = S;
     c->max_group[precision] = user_group;
-    cudaFree(c->d_ac_corr);
-    cudaFree(c->d_ac_partial);
-    c->d_ac_corr = nullptr;
-    c->d_ac_partial = nullptr;
+    free_ac();
     release();                   // the derived states D included
     if (rc) return fail(c, rc, err);
     c->err.clear();

@@ -258,6 +258,8 @@ struct AcArgs {
 };
 struct AcReduceArgs {
     const double *block_partial;
+    double *partial2;                // [n_samples][B / 4][64][8]
+    unsigned int *ticket;            // [n_samples][B / 4], zero between launches
     const int64_t *sample_chunk_off; // [n_samples + 1] in 1024-row chunks
     int n_samples, B, group_state0, n_states, n_steps;
     const int *step;                 // per sample, already advanced by k_reduce
@@ -284,19 +286,31 @@ cudaError_t launch_qe_finish(const void *acc, int fp32, int K, int S, int64_t n_
 cudaError_t launch_ac_observe(const AcArgs &a, int fp32, int cplx, cudaStream_t st);
 cudaError_t launch_ac_reduce(const AcReduceArgs &a, cudaStream_t st);
 cudaError_t launch_vec_to_f32(int64_t n, const double *src, float *dst, cudaStream_t st);
-// Preparation of the AC states, FP64, four lanes per row ([n_rows][4] complex):
-// lanes 0 and 1 <- psi_p; lanes 2, 3 <- J_x psi_p, J_y psi_p; Fermi Clenshaw
-// terms out = c v + gamma H~ x + zeta z on lanes 1 .. 3; the result goes
-// back to the caller's layout as the four states of p.
+// Preparation of the AC states, FP64, three lanes per row ([n_rows][3]
+// complex): lane 0 <- psi_p; lanes 1, 2 <- J_x psi_p, J_y psi_p; Fermi
+// Clenshaw terms out = c v + gamma H~ x - z on them; the result goes back
+// to the caller's layout as the four states of p.
+constexpr int kAcLanes = 3;
+struct AcChebArgs {
+    SellView H;
+    int fixed_width;
+    int64_t n_rows;
+    double c, gamma;                 // c == 0: no v
+    const double2 *v, *x, *z;        // x, z may be nullptr
+    double2 *out;                    // may alias z
+    // one-value form (FP64 values): gamma H~ x = gh (sum of the neighbours) + gd x_r
+    double gh;
+    const double *gdiag;             // gamma d
+    int zero_diag;
+};
 cudaError_t launch_ac_load(const double2 *psi_user, int p, int64_t n_orb,
-                           const int32_t *user_to_row, double2 *v4, cudaStream_t st);
-cudaError_t launch_current4(SellView H, int fp32_vals, int cplx, int64_t n_rows,
-                            const double *dxe, const double *dye, double s, double2 *v4,
+                           const int32_t *user_to_row, double2 *v3, cudaStream_t st);
+cudaError_t launch_current3(SellView H, int fp32_vals, int cplx, int64_t n_rows,
+                            const double *dxe, const double *dye, double s, double2 *v3,
                             cudaStream_t st);
-cudaError_t launch_cheb_real4(SellView H, int fp32_vals, int cplx, int64_t n_rows, double c,
-                              double gamma, double zeta, const double2 *v, const double2 *x,
-                              const double2 *z, double2 *out, cudaStream_t st);
-cudaError_t launch_ac_store(const double2 *v4, const double2 *f4, int p, int64_t n_orb,
+cudaError_t launch_ac_cheb(const AcChebArgs &a, int fp32_vals, int cplx, int uniform,
+                           cudaStream_t st);
+cudaError_t launch_ac_store(const double2 *v3, const double2 *f3, int p, int64_t n_orb,
                             const int32_t *user_to_row, double2 *out_user, cudaStream_t st);
 cudaError_t launch_bond_vectors(int64_t n_hop, const int32_t *bond_rows, const int64_t *slice_ptr,
                                 const int32_t *col, const double *dx, const double *dy,

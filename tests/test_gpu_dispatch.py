@@ -69,3 +69,24 @@ def test_three_slot_forms_are_bit_identical(precision, B, onsite_w, sigma):
     assert (a == b).all()
     assert np.abs(C0 - C1).max() < 1e-12
 
+
+# the Fermi preparation's one-value forms against the entry-by-entry form of
+# the same matrix (rounding of the FP64 preparation: 1e-10 of the largest
+# value, as against the oracle), uneven samples and several quads a group
+@pytest.mark.parametrize("onsite_w,mu", [(0.0, 0.0), (0.8, 0.0), (0.8, 0.3)])
+def test_fermi_preparation_forms_agree(onsite_w, mu):
+    import paper_2209_00806_gb300 as tb
+    from paper_2209_00806_gb300 import _native as N
+    parts = [lattice.graphene(L, L, pbc=True, seed=L, onsite_w=onsite_w, with_pos=True)
+             for L in (8, 33)]
+    smp, offs = lattice.concat(parts)
+    if not onsite_w:
+        smp.onsite = None
+    out = []
+    for flags in (0, N.TBPM_BUILD_NO_UNIFORM):
+        with tb.Propagator() as p:
+            p.build_sample(smp, 9.5, offs, flags=flags)
+            p.set_bond_vectors(lattice.bond_vectors(smp))
+            p.set_phase_states(rng.phases(11, 3, smp.n_orb))
+            out.append(p.ac_correlation(Z, 6, 20.0, mu, tb.TBPM_FP64))
+    assert np.abs(out[0] - out[1]).max() < 1e-10 * np.abs(out[1]).max()
