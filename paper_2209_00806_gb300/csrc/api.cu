@@ -1678,7 +1678,11 @@ extern "C" int tbpm_propagate_adjoint(tbpm_ctx *c, double z, int n_steps, const 
     const int nseg = (n_steps + K - 1) / K;
     std::vector<void *> ckpt(nseg, nullptr), traj(K, nullptr), stash(M - 1, nullptr);
     double *G = nullptr, *Gd = nullptr, *d_gh = nullptr, *d_go = nullptr;
+    double *val2 = nullptr, *diag2 = nullptr;        // 2 H~ (interior terms)
+    const int64_t nnz = c->H.nnz_pad;
     auto release = [&]() {
+        cudaFree(val2);
+        cudaFree(diag2);
         for (void *p : ckpt) cudaFree(p);
         for (void *p : traj) cudaFree(p);
         for (void *p : stash) cudaFree(p);
@@ -1690,8 +1694,10 @@ extern "C" int tbpm_propagate_adjoint(tbpm_ctx *c, double z, int n_steps, const 
     for (auto &p : ckpt) if (!rc) rc = dalloc(c, (char **)&p, vec);
     for (size_t k = 1; k < traj.size() && !rc; ++k) rc = dalloc(c, (char **)&traj[k], vec);
     for (auto &p : stash) if (!rc) rc = dalloc(c, (char **)&p, vec);
-    if (!rc) rc = dalloc(c, &G, (size_t)std::max<int64_t>(c->H.nnz_pad, 1));
+    if (!rc) rc = dalloc(c, &G, (size_t)std::max<int64_t>(nnz, 1));
     if (!rc) rc = dalloc(c, &Gd, (size_t)c->H.n_rows);
+    if (!rc) rc = dalloc(c, &val2, (size_t)std::max<int64_t>(nnz, 1));
+    if (!rc) rc = dalloc(c, &diag2, (size_t)c->H.n_rows);
     if (!rc && where_out == TBPM_HOST) {
         rc = dalloc(c, &d_gh, (size_t)std::max<int64_t>(c->H.n_hop, 1));
         if (!rc) rc = dalloc(c, &d_go, (size_t)c->n_orb);
@@ -1700,122 +1706,133 @@ extern "C" int tbpm_propagate_adjoint(tbpm_ctx *c, double z, int n_steps, const 
         d_go = grad_onsite;
     }
     if (rc) { release(); return rc; }
-    cudaMemsetAsync(G, 0, std::max<int64_t>(c->H.nnz_pad, 1) * sizeof(double), c->st);
-    cudaMemsetAsync(Gd, 0, c->H.n_rows * sizeof(double), c->st);
+    auto cuda_fail = [&](const char *what, cudaError_t e) {
+        release();
+        return fail(c, e == cudaErrorMemoryAllocation ? TBPM_E_OOM : TBPM_E_CUDA,
+                    std::string(what) + ": " + cudaGetErrorString(e));
+    };
+    {
+        cudaError_t e = cudaMemsetAsync(G, 0, std::max<int64_t>(nnz, 1) * sizeof(double), c->st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(Gd, 0, c->H.n_rows * sizeof(double), c->st);
+        if (e == cudaSuccess) e = launch_double(nnz, c->H.val64, val2, c->st);
+        if (e == cudaSuccess) e = launch_double(c->H.n_rows, c->H.diag64, diag2, c->st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);      // read ahead of dep_wait()
+        if (e != cudaSuccess) return cuda_fail("adjoint setup", e);
+    }
 
-    SellView Hv;
-    Hv.slice_ptr = c->H.slice_ptr;
-    Hv.col = c->H.col;
-    Hv.val = c->H.val64;
-    Hv.diag = c->H.diag64;
-    const int threads = c->threads[TBPM_FP64];
     int64_t launches = 0;
     int fin = 0;
     schedule(a, 0, &fin);
 
     for (auto &g : c->groups) {
         const int B = g.B;
-        TermArgs base;
+        AdjArgs base;
         memset(&base, 0, sizeof(base));
-        base.H = Hv;
+        base.slice_ptr = c->H.slice_ptr;
+        base.col = c->H.col;
+        base.fixed_width = c->H.fixed_width;
         base.chunk_sample = c->H.chunk_sample;
         base.n_rows = c->H.n_rows;
-        base.fixed_width = c->H.fixed_width;
-        auto term = [&](const void *x, const void *psi, const void *zz, void *out, double cc,
-                        double gamma) -> int {
-            TermArgs t = base;
+        base.psi0 = g.psi0;
+        base.n_states = c->n_states;
+        base.state0 = g.s0;
+        base.n_steps = n_steps;
+        base.G = G;
+        base.Gdiag = Gd;
+        // H' for |gamma| = 1 (twice: false) or 2
+        auto with_h = [&](bool twice) {
+            AdjArgs t = base;
+            t.val = twice ? val2 : c->H.val64;
+            t.diag = twice ? diag2 : c->H.diag64;
+            return t;
+        };
+        auto run = [&](const AdjArgs &t, AdjKind kind) -> cudaError_t {
+            ++launches;
+            return launch_adj(t, kind, B, c->st);
+        };
+        // T^_m from T^_{m-1} and T^_{m-2} (m = 1: from T^_0 alone)
+        auto poly = [&](int m, const void *x, const void *zz, void *out) -> cudaError_t {
+            AdjArgs t = with_h(m > 1);
             t.x = x;
-            t.psi = psi;
             t.z = zz;
             t.out = out;
-            t.c_hi = cc;
-            t.gamma = gamma;
-            ++launches;
-            CUDA_OR_FAIL(c, launch_term(t, 0, B, threads, c->st));
-            return TBPM_OK;
+            return run(t, kAdjPoly);
         };
         // one forward Clenshaw step src -> dst (tmp: scratch)
-        auto step_into = [&](void *src, void *dst, void *tmp) -> int {
+        auto step_into = [&](void *src, void *dst, void *tmp) -> cudaError_t {
             void *bufs[3];
             bufs[0] = src;
             bufs[fin] = dst;
             bufs[3 - fin] = tmp;
             int nx = 0;
             for (const Launch &L : schedule(a, 0, &nx)) {
-                int r2 = term(L.x < 0 ? src : bufs[L.x], src, L.z < 0 ? nullptr : bufs[L.z],
-                              bufs[L.out], L.c, L.gamma);
-                if (r2) return r2;
+                AdjArgs t = with_h(L.x >= 0 && !L.final_term);
+                t.x = L.x < 0 ? src : bufs[L.x];
+                t.psi = src;
+                t.z = L.z < 0 ? nullptr : bufs[L.z];
+                t.out = bufs[L.out];
+                t.c = L.c;
+                t.fac = L.gamma;             // of the first term (x is psi)
+                cudaError_t e = run(t, L.x < 0 ? kAdjStepFirst : kAdjStep);
+                if (e != cudaSuccess) return e;
             }
-            return TBPM_OK;
+            return cudaSuccess;
         };
-        CUDA_OR_FAIL(c, launch_set_states(c->d_psi_user, c->n_orb, c->n_states, c->H.user_to_row,
-                                          g.s0, B, 0, g.psi0, c->st));
+        cudaError_t e = launch_set_states(c->d_psi_user, c->n_orb, c->n_states, c->H.user_to_row,
+                                          g.s0, B, 0, g.psi0, c->st);
         const size_t gvec = (size_t)c->H.n_rows * B * sizeof(double2);
-        CUDA_OR_FAIL(c, cudaMemcpyAsync(ckpt[0], g.psi0, gvec, cudaMemcpyDeviceToDevice, c->st));
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(ckpt[0], g.psi0, gvec, cudaMemcpyDeviceToDevice, c->st);
+        if (e != cudaSuccess) return cuda_fail("adjoint states", e);
         // forward pass: checkpoints phi_{jK}
         void *src = ckpt[0];
         for (int n = 0; n + 1 < n_steps; ++n) {
-            void *dst = g.buf[n % 2];
-            if ((rc = step_into(src, dst, g.buf[2]))) { release(); return rc; }
+            void *dst = (n + 1) % K == 0 ? ckpt[(n + 1) / K] : g.buf[n % 2];
+            if ((e = step_into(src, dst, g.buf[2])) != cudaSuccess)
+                return cuda_fail("adjoint forward kernel", e);
             src = dst;
-            if ((n + 1) % K == 0)
-                CUDA_OR_FAIL(c, cudaMemcpyAsync(ckpt[(n + 1) / K], dst, gvec,
-                                                cudaMemcpyDeviceToDevice, c->st));
         }
         // backward pass
         int lc = 0;
-        CUDA_OR_FAIL(c, launch_source_init(c->H.n_rows, B, c->H.chunk_sample, d_gbar, c->n_states,
-                                           g.s0, n_steps, n_steps, g.psi0, g.buf[0], c->st));
+        e = launch_source_init(c->H.n_rows, B, c->H.chunk_sample, d_gbar, c->n_states, g.s0, n_steps,
+                               n_steps, g.psi0, g.buf[0], c->st);
+        if (e != cudaSuccess) return cuda_fail("adjoint source", e);
         for (int seg = nseg - 1; seg >= 0; --seg) {
             const int n0 = seg * K, n1 = std::min(n_steps, n0 + K);
             std::vector<void *> tp(n1 - n0);
             tp[0] = ckpt[seg];
             for (int k = 1; k < n1 - n0; ++k) {
                 tp[k] = traj[k];
-                if ((rc = step_into(tp[k - 1], tp[k], stash[0]))) { release(); return rc; }
+                if ((e = step_into(tp[k - 1], tp[k], stash[0])) != cudaSuccess)
+                    return cuda_fail("adjoint forward kernel", e);
             }
             for (int n = n1 - 1; n >= n0; --n) {
                 void *phi = tp[n - n0];
-                if (M - 2 >= 1 && (rc = term(phi, phi, nullptr, stash[1], 0.0, 1.0))) {
-                    release(); return rc;
+                for (int m = 1; m <= M - 2; ++m) {
+                    e = poly(m, m == 1 ? phi : stash[m - 1],
+                             m == 1 ? nullptr : m == 2 ? phi : stash[m - 2], stash[m]);
+                    if (e != cudaSuccess) return cuda_fail("adjoint polynomial kernel", e);
                 }
-                for (int m = 2; m <= M - 2; ++m)
-                    if ((rc = term(stash[m - 1], stash[m - 1], m == 2 ? phi : stash[m - 2],
-                                   stash[m], 0.0, 2.0))) {
-                        release(); return rc;
-                    }
                 int nx = 0;
                 std::vector<Launch> sch = schedule(a, lc, &nx);
                 for (size_t k = 0; k < sch.size(); ++k) {
                     const Launch &L = sch[k];
                     const int m = M - 2 - (int)k;
-                    AdjArgs aa;
-                    memset(&aa, 0, sizeof(aa));
-                    aa.H = Hv;
-                    aa.x = L.x < 0 ? g.buf[lc] : g.buf[L.x];
-                    aa.psi = g.buf[lc];
-                    aa.z = L.z < 0 ? nullptr : g.buf[L.z];
-                    aa.out = g.buf[L.out];
-                    aa.T_own = m == 0 ? phi : stash[m];
-                    aa.c = L.c;
-                    aa.gamma = -L.gamma;
-                    aa.gfac = L.gamma;
-                    aa.G = G;
-                    aa.Gdiag = Gd;
-                    aa.gbar = m == 0 ? d_gbar : nullptr;
-                    aa.psi0 = g.psi0;
-                    aa.n_states = c->n_states;
-                    aa.state0 = g.s0;
-                    aa.n_steps = n_steps;
-                    aa.step = n;
-                    aa.chunk_sample = c->H.chunk_sample;
-                    aa.n_rows = c->H.n_rows;
-                    ++launches;
-                    cudaError_t e = launch_adj_term(aa, B, threads, c->st);
-                    if (e != cudaSuccess) {
-                        release();
-                        return fail(c, TBPM_E_CUDA, std::string("adjoint kernel: ") + cudaGetErrorString(e));
-                    }
+                    const bool first = L.x < 0;
+                    AdjArgs t = with_h(!first && !L.final_term);
+                    t.sign = 1ull << 63;                 // gamma -> -gamma
+                    t.x = first ? g.buf[lc] : g.buf[L.x];
+                    t.psi = g.buf[lc];
+                    t.z = L.z < 0 ? nullptr : g.buf[L.z];
+                    t.out = g.buf[L.out];
+                    t.T_own = m == 0 ? phi : stash[m];
+                    t.c = L.c;
+                    t.fac = L.gamma;
+                    t.gfac = 0.5 * L.gamma;              // G is half the sum
+                    t.gbar = m == 0 ? d_gbar : nullptr;
+                    t.step = n;
+                    e = run(t, first ? kAdjGradFirst : L.final_term ? kAdjGradLast : kAdjGrad);
+                    if (e != cudaSuccess) return cuda_fail("adjoint kernel", e);
                 }
                 lc = nx;
             }

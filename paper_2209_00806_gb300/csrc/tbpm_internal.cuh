@@ -316,14 +316,25 @@ cudaError_t launch_bond_vectors(int64_t n_hop, const int32_t *bond_rows, const i
                                 const int32_t *col, const double *dx, const double *dy,
                                 int *claim, double *dxe, double *dye, int *err, cudaStream_t st);
 
-// One backward (adjoint) term with gradient accumulation, FP64:
-//   out = c psi + gamma (-i) (H~ x) + z [+ gbar_step psi0],
-//   G_rc += gfac Im(conj(x_c) T_r) for every stored entry, Gdiag_r likewise.
+// One term of the adjoint's forward or backward series, FP64, with the matrix
+// values already scaled by |gamma| (adjoint_kernels.cu).
+enum AdjKind {
+    kAdjPoly,       // z + (-i) H' x: the plain polynomials
+    kAdjStep,       // c psi + z + (-i) H' x: a forward Clenshaw term
+    kAdjStepFirst,  // c psi + fac (-i) H' psi: its first term
+    kAdjGrad,       // c psi + z + i H' x with gradient accumulation
+    kAdjGradFirst,  // c psi + fac i H' psi with it, weight gfac
+    kAdjGradLast    // the closing one: weight gfac, + gbar_step psi0
+};
 struct AdjArgs {
-    SellView H;
+    const int64_t *slice_ptr;
+    const int32_t *col;
+    const double *val, *diag;   // H~ (|gamma| = 1) or 2 H~
+    int fixed_width;
+    unsigned long long sign;    // sign bit applied to H': 0 for -i, 1 << 63 for +i
     const void *x, *psi, *z, *T_own;
     void *out;
-    double c, gamma, gfac;
+    double c, fac, gfac;
     double *G, *Gdiag;
     const double2 *gbar;   // [n_samples][n_states][n_steps + 1] or nullptr
     const void *psi0;
@@ -451,7 +462,8 @@ cudaError_t launch_term_tma(const TermArgs &a, int fp32, int B, int max_width, i
                             int num_sms, cudaStream_t st);
 
 // Adjoint kernels (adjoint_kernels.cu).
-cudaError_t launch_adj_term(const AdjArgs &a, int B, int threads, cudaStream_t st);
+cudaError_t launch_adj(const AdjArgs &a, AdjKind kind, int B, cudaStream_t st);
+cudaError_t launch_double(int64_t n, const double *src, double *dst, cudaStream_t st);
 cudaError_t launch_source_init(int64_t n_rows, int B, const int32_t *chunk_sample,
                                const double2 *gbar, int n_states, int state0, int n_steps,
                                int step, const void *psi0, void *out, cudaStream_t st);

@@ -90,3 +90,28 @@ def test_fermi_preparation_forms_agree(onsite_w, mu):
             p.set_phase_states(rng.phases(11, 3, smp.n_orb))
             out.append(p.ac_correlation(Z, 6, 20.0, mu, tb.TBPM_FP64))
     assert np.abs(out[0] - out[1]).max() < 1e-10 * np.abs(out[1]).max()
+
+
+# gradient kernels per group width and row form against the oracle's reverse
+# mode (1e-11 of the largest, the tolerance of the adjoint tests): widths 1,
+# 2 + 1, 4 and 8, three-slot rows and ragged ones, one step to several segments
+@pytest.mark.parametrize("S", [1, 3, 4, 8])
+@pytest.mark.parametrize("kind", ["graphene", "ragged"])
+@pytest.mark.parametrize("steps,K", [(1, 1), (5, 2)])
+def test_adjoint_forms(S, kind, steps, K):
+    import oracle
+    import paper_2209_00806_gb300 as tb
+    if kind == "graphene":
+        smp = lattice.graphene(9, 7, pbc=True, seed=2, onsite_w=0.5, bond_sigma=0.1)
+    else:
+        smp = lattice.random_graph(130, 400, seed=3, onsite_w=0.5, t_scale=0.7)
+    theta = rng.phases(4, S, smp.n_orb)
+    g = np.random.default_rng(5).normal(size=(1, S, steps + 1, 2)) @ np.array([1, 1j])
+    with tb.Propagator() as p:
+        p.build_sample(smp, 12.0)
+        p.set_phase_states(theta)
+        gh, go = p.adjoint(Z, steps, g, K)
+    rh, ro = oracle.gradient(smp, 12.0, Z, steps, oracle.phase_states(theta), g[0])
+    scale = max(np.abs(rh).max(), np.abs(ro).max())
+    assert np.abs(gh - rh).max() < 1e-11 * scale
+    assert np.abs(go - ro).max() < 1e-11 * scale
