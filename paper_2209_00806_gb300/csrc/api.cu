@@ -2222,8 +2222,7 @@ extern "C" int tbpm_quasi_eigenstates(tbpm_ctx *c, double z, int n_steps, int n_
     if (rc) return rc;
     double2 *d_tab = nullptr, *d_out = nullptr;
     float2 *d_tab_f = nullptr;
-    double *d_norms = nullptr;
-    int64_t *d_off = nullptr;
+    double *d_norms = nullptr, *d_factor = nullptr, *d_part = nullptr;
     auto release = [&]() {
         cudaFree(c->d_qe_acc);
         c->d_qe_acc = nullptr;
@@ -2233,14 +2232,16 @@ extern "C" int tbpm_quasi_eigenstates(tbpm_ctx *c, double z, int n_steps, int n_
         cudaFree(d_tab);
         cudaFree(d_tab_f);
         cudaFree(d_norms);
-        cudaFree(d_off);
+        cudaFree(d_factor);
+        cudaFree(d_part);
         if (where_out == TBPM_HOST) cudaFree(d_out);
     };
     rc = dalloc(c, &c->d_qe_acc, (size_t)K * n_rows * S);
     if (!rc) rc = dalloc(c, &d_tab, tab.size());
     if (!rc) rc = dalloc(c, &d_tab_f, tab_f.size());
     if (!rc) rc = dalloc(c, &d_norms, (size_t)K * S * c->n_samples);
-    if (!rc) rc = dalloc(c, &d_off, (size_t)c->n_samples + 1);
+    if (!rc) rc = dalloc(c, &d_factor, (size_t)K * S * c->n_samples);
+    if (!rc) rc = dalloc(c, &d_part, (size_t)K * (n_rows / kChunkRows) * S);
     if (!rc && where_out == TBPM_HOST) rc = dalloc(c, &d_out, (size_t)K * S * n_orb);
     if (rc) { release(); return rc; }
     if (where_out == TBPM_DEVICE) d_out = reinterpret_cast<double2 *>(out);
@@ -2250,9 +2251,6 @@ extern "C" int tbpm_quasi_eigenstates(tbpm_ctx *c, double z, int n_steps, int n_
                             c->st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d_tab_f, tab_f.data(), tab_f.size() * sizeof(float2),
-                            cudaMemcpyHostToDevice, c->st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_off, c->sample_off.data(), (c->n_samples + 1) * sizeof(int64_t),
                             cudaMemcpyHostToDevice, c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);      // host tables go out of scope
     if (e != cudaSuccess) {
@@ -2278,7 +2276,8 @@ extern "C" int tbpm_quasi_eigenstates(tbpm_ctx *c, double z, int n_steps, int n_
     }
     e = launch_qe_finish(c->d_qe_acc, precision == TBPM_FP32, K, S, n_rows, n_orb, c->n_samples,
                          c->H.user_to_row,
-                         c->H.orb_sample, d_off, d_out, d_norms, c->st);
+                         c->H.orb_sample, c->d_sample_chunk_off, d_part, d_out, d_norms, d_factor,
+                         c->st);
     if (e == cudaSuccess && where_out == TBPM_HOST)
         e = cudaMemcpyAsync(out, d_out, (size_t)K * S * n_orb * sizeof(double2),
                             cudaMemcpyDeviceToHost, c->st);

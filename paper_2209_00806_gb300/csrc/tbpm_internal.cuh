@@ -282,7 +282,8 @@ struct QeArgs {
 cudaError_t launch_qe_acc(const QeArgs &a, int fp32, cudaStream_t st);
 cudaError_t launch_qe_finish(const void *acc, int fp32, int K, int S, int64_t n_rows, int64_t n_orb,
                              int n_samples, const int32_t *user_to_row, const int32_t *orb_sample,
-                             const int64_t *orb_off, double2 *out, double *norms, cudaStream_t st);
+                             const int64_t *chunk_off, double *partial, double2 *out, double *norms,
+                             double *factor, cudaStream_t st);
 cudaError_t launch_ac_observe(const AcArgs &a, int fp32, int cplx, cudaStream_t st);
 cudaError_t launch_ac_reduce(const AcReduceArgs &a, cudaStream_t st);
 cudaError_t launch_vec_to_f32(int64_t n, const double *src, float *dst, cudaStream_t st);

@@ -115,3 +115,24 @@ def test_adjoint_forms(S, kind, steps, K):
     scale = max(np.abs(rh).max(), np.abs(ro).max())
     assert np.abs(gh - rh).max() < 1e-11 * scale
     assert np.abs(go - ro).max() < 1e-11 * scale
+
+
+# quasi-eigenstate accumulation one or two lanes a thread, norms from chunk
+# partials: group splits 1, 2 + 1, 4 + 2, 16 + 1, uneven samples, FP32 against
+# FP64 (2e-5 of the unit norm, the tolerance of the FP32 form)
+@pytest.mark.parametrize("S", [1, 3, 6, 17])
+def test_quasi_lanes_and_norms(S):
+    import paper_2209_00806_gb300 as tb
+    parts = [lattice.graphene(L, L + 2, pbc=True, seed=L, onsite_w=1.0) for L in (5, 30)]
+    smp, offs = lattice.concat(parts)
+    out = []
+    for precision in (tb.TBPM_FP64, tb.TBPM_FP32):
+        with tb.Propagator() as p:
+            p.build_sample(smp, 9.5, offs)
+            p.set_phase_states(rng.phases(12, S, smp.n_orb))
+            out.append(p.quasi_eigenstates(Z, 12, [0.3, -1.1], precision))
+    (a, na), (b, nb) = out
+    for lo, hi in zip(offs, offs[1:]):
+        assert np.abs((np.abs(a[:, :, lo:hi]) ** 2).sum(-1) - 1).max() < 1e-12
+        assert np.linalg.norm(a[:, :, lo:hi] - b[:, :, lo:hi], axis=-1).max() < 2e-5
+    assert np.abs(nb / na - 1).max() < 2e-5
