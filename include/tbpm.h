@@ -364,15 +364,22 @@ int tbpm_dos_adjoint(const double *dl_dd, int n_e, int n_steps, double tau, int 
                                         grid whose threads walk rows with a stride and
                                         load the next row's first four column indices,
                                         values and diagonal before the current row's
-                                        gathers (with TBPM_VARIANT_WIDE: 32-byte lanes);
-                                        ignored otherwise */
+                                        gathers; FP32: one row a thread up to 2^20
+                                        16-byte lanes, 32-byte lanes (with
+                                        TBPM_VARIANT_WIDE) for four states beyond
+                                        128 MB a vector, and the staged gathers
+                                        (HALO | STAGED) for rows of at least 32 values
+                                        on average; ignored otherwise.  All
+                                        bit-identical */
 #define TBPM_VARIANT_STAGED 4096     /* with TBPM_VARIANT_HALO: one block per 128-row
                                         block copying its halo, positions and values
                                         into one shared-memory stage, two blocks per
                                         SM where the stage allows (one block's copies
                                         overlap the other's gathers); same shapes as
                                         TBPM_VARIANT_PIPE, which it takes precedence
-                                        over */
+                                        over.  FP32 values per entry: rows in groups of
+                                        four that share a column list, where the lists
+                                        have at most 3 slots per stored entry */
 int tbpm_set_launch_config(tbpm_ctx *ctx, int precision, int max_group, int threads,
                            int variant);
 

@@ -980,19 +980,42 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     const int threads = c->threads[precision];
     // staged-gather variant: halo lists built on first use; a matrix whose
     // row blocks reference too many other rows keeps the plain kernels
-    bool halo = (c->variant[precision] & kVariantHalo) && !c->H.cplx &&
-                !(c->variant[precision] & (kVariantTma | kVariantFused));
+    int variant = c->variant[precision];
+    // the register-pipelined variant on long rows of real FP32 values: the
+    // staged gathers instead where the lists can be had (twisted bilayer, 68
+    // entries a row, 3.1M rows: 1.84 ms a term through L1, 0.81 ms staged,
+    // less in groups; graphene's three entries hit L1 and lose, 0.27 against
+    // 0.19 ms).  From two steps on the lists' build
+    // (as much as about one step) pays within the call.
+    const bool long_rows = fp32 && (variant & kVariantPrefetch) && !c->H.cplx && !c->H.uniform &&
+                           !(variant & (kVariantHalo | kVariantTma | kVariantFused | kVariantSplit2 |
+                                        kVariantSplit4)) &&
+                           c->H.nnz_true >= kLongRow * c->n_orb && n_steps >= 2;
+    if (long_rows) variant = (variant & ~kVariantPrefetch) | kVariantHalo | kVariantStaged;
+    bool halo = (variant & kVariantHalo) && !c->H.cplx && !(variant & (kVariantTma | kVariantFused));
     if (halo && !c->H.halo_ptr) {
         std::string msg;
         rc = build_halo(c->H, c->st, msg);
-        if (rc == TBPM_E_UNSUPPORTED) halo = false;
+        if (rc == TBPM_E_UNSUPPORTED || (rc == TBPM_E_OOM && long_rows)) halo = false;
         else if (rc) return fail(c, rc, msg);
     }
-    if (halo && (c->variant[precision] & (kVariantPipe | kVariantStaged)) && !c->H.uniform &&
-        !c->H.vpack[fp32]) {
+    // one-stage staged gathers with FP32 values per entry: rows in groups of four
+    if (halo && fp32 && (variant & kVariantStaged) && !c->H.uniform) {
+        std::string msg;
+        rc = build_groups(c->H, c->st, msg);
+        if (rc) return fail(c, rc, msg);
+    }
+    const bool grouped = halo && fp32 && (variant & kVariantStaged) && c->H.gptr;
+    if (halo && (variant & (kVariantPipe | kVariantStaged)) && !c->H.uniform &&
+        !grouped && !c->H.vpack[fp32]) {
         std::string msg;
         rc = build_packed_values(c->H, fp32, c->st, msg);
-        if (rc) return fail(c, rc, msg);
+        if (rc == TBPM_E_OOM && long_rows) halo = false;
+        else if (rc) return fail(c, rc, msg);
+    }
+    if (long_rows && !halo) {                        // no lists: the asked-for kernel
+        cudaGetLastError();
+        variant = c->variant[precision];
     }
     // FP64 one-value form: 2 d for the interior terms' gamma d
     if (!fp32 && c->H.uniform && !c->H.zero_diag && !c->H.diag2_64) {
@@ -1065,6 +1088,12 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
             base.lcol = c->H.lcol;
             base.pslice = c->H.pslice;
             base.vpack = c->H.vpack[fp32];
+            if (grouped) {
+                base.gptr = c->H.gptr;
+                base.gperm = c->H.gperm;
+                base.gpos = c->H.gpos;
+                base.gval = c->H.gval;
+            }
             base.halo_max = c->H.halo_max;
             base.halo_ent_max = c->H.halo_ent_max;
         }
@@ -1146,7 +1175,7 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         FusedArgs fa;
         memset(&fa, 0, sizeof(fa));
         if (fused) {
-            int R = fused_tile_rows(fp32, g.B, (c->variant[precision] >> kVariantFusedTileShift) & 3);
+            int R = fused_tile_rows(fp32, g.B, (variant >> kVariantFusedTileShift) & 3);
             while (R > kChunkRows && c->H.n_rows % R) R /= 4;   // tiles must cover the rows exactly
             const int radius = (int)((c->H.bandwidth + R - 1) / R);
             int maxB = 1;
@@ -1220,7 +1249,7 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         ra.scale_f = g.scale_f;
 
         // cluster-resident stepping: every step of this one FP64 state in one launch
-        const int Kc = (c->variant[precision] & kVariantCluster) && !fp32 && !fused &&
+        const int Kc = (variant & kVariantCluster) && !fp32 && !fused &&
                                c->groups.size() == 1 && g.B == 1 && c->n_samples == 1 &&
                                !c->H.cplx && !c->ac_on && !c->qe_on && c->H.val64 &&
                                c->H.max_width <= kClusterMaxW && n_steps > 0 &&
@@ -1342,7 +1371,7 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
                     ended_interior = true;
                 }
                 TermArgs t = base;
-                t.variant = c->variant[precision];
+                t.variant = variant;
                 // complex values have the plain term kernels only (16-byte lanes)
                 if (c->H.cplx) t.variant &= kVariantZigZag | kVariantStreamHints;
                 if (!halo) t.variant &= ~kVariantHalo;

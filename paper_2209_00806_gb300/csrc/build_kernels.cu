@@ -609,7 +609,167 @@ __global__ void k_pack_values(int64_t n_rows, const int64_t *slice_ptr, const in
             k < w ? val[e0 + (int64_t)k * kSliceRows + lr] : (T)0;
 }
 
+// ---- row groups of the staged-gather kernel for long rows -------------------
+// Four consecutive rows of a halo block share one ascending list of columns
+// (the union of theirs; a column that a row holds twice appears twice), with
+// a 16-bit halo position and four values per list entry, zero where a row has
+// no such entry: one read of a neighbour's states then serves four rows.  The
+// 32 groups of a block are ordered by list length, and each eight of them
+// (an octet, the groups a warp of the term kernel walks together) share a
+// length, a multiple of eight: entry k of the octet's group s is at
+//   values     (gptr[octet] + k) * 32 + s * 4 + row
+//   positions  gptr[octet] * 8 + (k / 4) * 32 + s * 4 + k % 4
+// A row's padded slots (column = own row) end it; the lists are padded with
+// the group's first row and zero values.
+template <typename F>
+__device__ __forceinline__ int merge_group(const int64_t *slice_ptr, const int32_t *col, int64_t r0,
+                                           F &&emit)
+{
+    const int64_t q = r0 / kSliceRows;
+    const int64_t base = slice_ptr[q] + r0 % kSliceRows;
+    const int w = (int)((slice_ptr[q + 1] - slice_ptr[q]) / kSliceRows);
+    int k[kGroupRows] = {};
+    int32_t c[kGroupRows];
+    auto head = [&](int i) {
+        const int32_t v = k[i] < w ? col[base + (int64_t)k[i] * kSliceRows + i] : INT32_MAX;
+        c[i] = v == (int32_t)(r0 + i) ? INT32_MAX : v;
+    };
+#pragma unroll
+    for (int i = 0; i < kGroupRows; ++i) head(i);
+    int n = 0;
+    for (;; ++n) {
+        int32_t m = c[0];
+#pragma unroll
+        for (int i = 1; i < kGroupRows; ++i) m = min(m, c[i]);
+        if (m == INT32_MAX) return n;
+        int take[kGroupRows];
+#pragma unroll
+        for (int i = 0; i < kGroupRows; ++i) take[i] = c[i] == m ? k[i] : -1;
+        emit(n, take);
+#pragma unroll
+        for (int i = 0; i < kGroupRows; ++i)
+            if (take[i] >= 0) {
+                ++k[i];
+                head(i);
+            }
+    }
+}
+
+// One warp per halo block, lane = group: list lengths, the order of the
+// groups (longest first, then by number) and the octets' lengths.
+__global__ void __launch_bounds__(32) k_group_count(const int64_t *slice_ptr, const int32_t *col,
+                                                    uint8_t *perm, int64_t *octet_len)
+{
+    const int64_t hb = blockIdx.x;
+    const int g = threadIdx.x;
+    const int n = merge_group(slice_ptr, col, hb * kHaloRows + g * kGroupRows,
+                              [](int, const int *) {});
+    int rank = 0;
+    for (int o = 0; o < 32; ++o) {
+        const int no = __shfl_sync(0xffffffffu, n, o);
+        rank += no > n || (no == n && o < g);
+    }
+    perm[hb * 32 + rank] = (uint8_t)g;
+    if (rank % 8 == 0) octet_len[hb * 4 + rank / 8] = (n + kGroupStep - 1) / kGroupStep * kGroupStep;
+}
+
+__global__ void __launch_bounds__(32) k_group_fill(const int64_t *slice_ptr, const int32_t *col,
+                                                   const float *val, const int64_t *pslice,
+                                                   const uint16_t *lcol, const uint8_t *perm,
+                                                   const int64_t *gptr, uint16_t *gpos, float4 *gval)
+{
+    const int64_t hb = blockIdx.x;
+    const int slot = threadIdx.x, oct = slot / 8, s8 = slot % 8;
+    const int64_t r0 = hb * kHaloRows + perm[hb * 32 + slot] * kGroupRows;
+    const int64_t q = r0 / kSliceRows, lr = r0 % kSliceRows;
+    const int64_t base = slice_ptr[q] + lr, pbase = pslice[q] + lr * 4;
+    const int64_t k0 = gptr[hb * 4 + oct];
+    const int len = (int)(gptr[hb * 4 + oct + 1] - k0);
+    auto put = [&](int n, int pos, float4 v) {
+        gval[(k0 + n) * 8 + s8] = v;
+        gpos[k0 * 8 + (n / 4) * 32 + s8 * 4 + n % 4] = (uint16_t)pos;
+    };
+    int n = merge_group(slice_ptr, col, r0, [&](int at, const int *take) {
+        float v[kGroupRows];
+        int pos = 0;
+#pragma unroll
+        for (int i = 0; i < kGroupRows; ++i) {
+            v[i] = 0.f;
+            if (take[i] >= 0) {
+                v[i] = val[base + (int64_t)take[i] * kSliceRows + i];
+                pos = lcol[pbase + (take[i] / 4) * (4 * kSliceRows) + i * 4 + take[i] % 4];
+            }
+        }
+        put(at, pos, make_float4(v[0], v[1], v[2], v[3]));
+    });
+    for (; n < len; ++n) put(n, (int)(r0 - hb * kHaloRows), make_float4(0.f, 0.f, 0.f, 0.f));
+}
+
 }  // namespace
+
+int build_groups(BuildOutput &b, cudaStream_t st, std::string &msg)
+{
+    if (b.gptr || b.no_groups) return TBPM_OK;
+    if (!b.halo_ptr || !b.val32 || b.cplx) { msg = "no halo lists or FP32 values"; return TBPM_E_STATE; }
+    const int64_t nb = b.n_rows / kHaloRows, no = nb * 4;
+    int64_t *len = nullptr, *ptr = nullptr;
+    uint8_t *perm = nullptr;
+    uint16_t *pos = nullptr;
+    float4 *val = nullptr;
+    auto drop = [&]() {
+        cudaFree(len);
+        cudaFree(ptr);
+        cudaFree(perm);
+        cudaFree(pos);
+        cudaFree(val);
+    };
+    int64_t total = 0;
+    cudaError_t e = cudaMalloc(&len, (no + 1) * sizeof(int64_t));
+    if (e == cudaSuccess) e = cudaMalloc(&ptr, (no + 1) * sizeof(int64_t));
+    if (e == cudaSuccess) e = cudaMalloc(&perm, nb * 32);
+    if (e == cudaSuccess) {
+        k_group_count<<<(unsigned)nb, 32, 0, st>>>(b.slice_ptr, b.col, perm, len);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) {
+        const int rc = scan_exclusive(len, ptr, no, st, msg);
+        if (rc) { drop(); return rc; }
+        e = cudaMemcpyAsync(&total, ptr + no, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    }
+    // no groups where the zeros would outweigh what the shared reads save
+    if (e == cudaSuccess && total * 32 > kGroupMaxFill * b.nnz_true) {
+        drop();
+        b.no_groups = 1;
+        return TBPM_OK;
+    }
+    if (e == cudaSuccess) e = cudaMalloc(&pos, std::max<int64_t>(total, 1) * 8 * sizeof(uint16_t));
+    if (e == cudaSuccess) e = cudaMalloc(&val, std::max<int64_t>(total, 1) * 8 * sizeof(float4));
+    if (e == cudaSuccess) {
+        k_group_fill<<<(unsigned)nb, 32, 0, st>>>(b.slice_ptr, b.col, b.val32, b.pslice, b.lcol, perm,
+                                                 ptr, pos, val);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaFree(len);
+    len = nullptr;
+    if (e == cudaErrorMemoryAllocation) {        // the packed entries serve instead
+        cudaGetLastError();
+        drop();
+        b.no_groups = 1;
+        return TBPM_OK;
+    }
+    if (e != cudaSuccess) {
+        drop();
+        msg = std::string("row groups: ") + cudaGetErrorString(e);
+        return TBPM_E_CUDA;
+    }
+    b.gptr = ptr;
+    b.gperm = perm;
+    b.gpos = pos;
+    b.gval = val;
+    return TBPM_OK;
+}
 
 int build_halo(BuildOutput &b, cudaStream_t st, std::string &msg)
 {
@@ -760,6 +920,10 @@ void free_build(BuildOutput &b)
     cudaFree(b.pslice);
     cudaFree(b.vpack[0]);
     cudaFree(b.vpack[1]);
+    cudaFree(b.gptr);
+    cudaFree(b.gperm);
+    cudaFree(b.gpos);
+    cudaFree(b.gval);
     b = BuildOutput();
 }
 

@@ -659,13 +659,7 @@ __device__ __forceinline__ Cv<V, SPL> row_term(const TermArgs &a, uint32_t r, in
     }
 }
 
-// Block index in traversal order: with kVariantZigZag the term kernels walk
-// the rows from the end on odd launches, so they start on the rows the
-// previous launch wrote last (still in L2).
-__device__ __forceinline__ int64_t block_in_order(const TermArgs &a)
-{
-    return a.reverse ? (int64_t)(gridDim.x - 1 - blockIdx.x) : (int64_t)blockIdx.x;
-}
+__device__ __forceinline__ int64_t block_in_order(const TermArgs &a) { return block_of(a.reverse); }
 
 // Bound by the column -> gather latency at small sizes, by HBM beyond the L2.
 // The columns are read before dep_wait(), so after it the own-row loads and
@@ -961,15 +955,6 @@ __global__ void __launch_bounds__(kFinalThreads) k_final_sums(TermArgs a)
 // rows sharing a 128-byte bank line spread their chunks over all banks.
 // Real values and 32-byte lanes (two chunks per lane); the arithmetic and
 // its order are term_row's, so the states are bit-identical to it.
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all()
-{
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
-}
 
 // Chunk permutation of halo row h for C chunks per row (C = 2, 4, 8).
 template <int C> __device__ __forceinline__ int halo_swz(int h)
@@ -1203,11 +1188,6 @@ cudaError_t launch_halo_t(const TermArgs &a, cudaStream_t st)
 // gather.  Lanes are 16 bytes (two FP32 or one FP64 state), C lanes per row
 // of x; same arithmetic and order as term_row, so the states are
 // bit-identical to the plain kernel.
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait_group()
-{
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
 
 // Lane l of halo row h in a stage: rows of C 16-byte chunks, chunk l of
 // each row read by the row's thread l (a quarter-warp reads two whole rows,
@@ -1616,6 +1596,7 @@ cudaError_t launch_staged_t(const TermArgs &a, cudaStream_t st)
 
 cudaError_t dispatch_staged(const TermArgs &a, int fp32, int B, cudaStream_t st)
 {
+    if (fp32 && a.gptr) return launch_term_group(a, B, st);
     if (fp32) return B == 4 ? launch_staged_t<float, 2>(a, st) : launch_staged_t<float, 4>(a, st);
     return B == 2 ? launch_staged_t<double, 2>(a, st) : launch_staged_t<double, 4>(a, st);
 }
@@ -2129,7 +2110,7 @@ cudaError_t launch_term(const TermArgs &a, int fp32, int B, int threads, cudaStr
         return dispatch_pf(a, fp32, B, threads, st);
     // the one-stage staged kernel, like the pipelined one, keeps rows unsplit
     if ((a.variant & kVariantHalo) && (a.variant & kVariantStaged) && a.lcol && !a.cplx &&
-        (a.vpack || a.uniform) && !(a.variant & (kVariantSplit2 | kVariantSplit4)) &&
+        (a.vpack || a.uniform || a.gptr) && !(a.variant & (kVariantSplit2 | kVariantSplit4)) &&
         staged_launchable(fp32, B, a.halo_max, a.halo_ent_max, a.uniform))
         return dispatch_staged(a, fp32, B, st);
     // the pipelined kernel does not split rows: with a row split requested,
@@ -2162,7 +2143,7 @@ cudaError_t launch_final(const TermArgs &a, int fp32, int B, int threads, cudaSt
         return dispatch<true>(r, fp32, B, threads, false, st);
     }
     if ((a.variant & kVariantHalo) && (a.variant & kVariantStaged) && a.lcol && !a.cplx &&
-        (a.vpack || a.uniform) && a.H.col &&
+        (a.vpack || a.uniform || a.gptr) && a.H.col &&
         staged_launchable(fp32, B, a.halo_max, a.halo_ent_max, a.uniform)) {
         cudaError_t e = dispatch_staged(a, fp32, B, st);   // then the closing reduction
         if (e != cudaSuccess) return e;

@@ -97,6 +97,31 @@ inline cudaError_t launch_dependent(void (*k)(P...), dim3 grid, dim3 block, size
 }
 #endif
 
+#ifdef __CUDACC__
+// 16-byte asynchronous copies to shared memory and their groups.
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
+{
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all()
+{
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait_group()
+{
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+// Block index in traversal order: with kVariantZigZag the term kernels walk
+// the rows from the end on odd launches, so they start on the rows the
+// previous launch wrote last (still in L2).
+__device__ __forceinline__ int64_t block_of(int reverse)
+{
+    return reverse ? (int64_t)(gridDim.x - 1 - blockIdx.x) : (int64_t)blockIdx.x;
+}
+#endif
+
 // Launch variants of the term kernels (bits of TermArgs::variant).
 constexpr int kVariantZigZag = 1;       // alternate the traversal direction per launch
 constexpr int kVariantStreamHints = 2;  // evict-first loads of the own-row streams
@@ -117,6 +142,13 @@ constexpr int kVariantPrefetch = 8192;  // FP32: persistent term kernel, next ro
 // longest list of the matrix).
 constexpr int kHaloRows = 128;
 constexpr int kHaloMaxExt = 2048;
+constexpr int kLongRow = 32;       // mean entries from which staged gathers are the default
+constexpr int kGroupRows = 4;      // rows sharing a list in the grouped form
+constexpr int kGroupStep = 8;      // list lengths are a multiple of this
+// list slots a stored entry at most: 4 rows x list length over the entries of
+// the rows (1.84 on the twisted bilayer); the shared reads save more than the
+// zeros cost up to about here
+constexpr int kGroupMaxFill = 3;
 constexpr int kHaloSmemMax = 160 * 1024;   // largest shared copy of a halo (bytes)
 constexpr int kPipeSmemMax = 224 * 1024;   // two stages of the pipelined form (bytes)
 
@@ -203,6 +235,10 @@ struct TermArgs {
                                       // pslice[q] + (k/4)*128 + lr*4 + k%4
     const int64_t *pslice;
     const void *vpack;                // packed values (pipelined kernel), or nullptr
+    const int64_t *gptr;              // row groups (kGroupRows rows share a list), or nullptr
+    const uint8_t *gperm;
+    const uint16_t *gpos;
+    const float4 *gval;
     int halo_max;
     int halo_ent_max;     // most stored entries of one halo block (pipelined form)
     int num_sms;          // grid of the persistent pipelined form
@@ -352,6 +388,8 @@ cudaError_t launch_term(const TermArgs &a, int fp32, int B, int threads, cudaStr
 bool halo_launchable(int fp32, int B, bool final_term, int halo_max);
 // The pipelined form serves this shape within the shared-memory budget.
 bool pipe_launchable(int fp32, int B, int halo_max, int ent_max, int uniform);
+// The grouped staged-gather kernel (group_kernels.cu): FP32 groups of 4 or 8.
+cudaError_t launch_term_group(const TermArgs &a, int B, cudaStream_t st);
 // The one-stage staged-gather kernel (kVariantStaged) for that shape.
 bool staged_launchable(int fp32, int B, int halo_max, int ent_max, int uniform);
 cudaError_t launch_final(const TermArgs &a, int fp32, int B, int threads, cudaStream_t st,
@@ -521,10 +559,20 @@ struct BuildOutput {
     int halo_ent_max = 0;            // most packed entries of one block
     int64_t halo_total = 0;          // entries of all lists
     double *diag2_64 = nullptr;      // 2 d (FP64 one-value form; built on first use)
+    // row groups of the staged-gather kernel (build_groups)
+    int64_t *gptr = nullptr;         // [n_rows / kHaloRows * 4 + 1] first list entry of each octet
+    uint8_t *gperm = nullptr;        // [n_rows / kHaloRows][32] group at each slot
+    uint16_t *gpos = nullptr;        // halo positions
+    float4 *gval = nullptr;          // values of the group's four rows
+    int no_groups = 0;               // tried: they do not pay or fit
 };
 
 // 2 d for the FP64 one-value form's interior terms (gamma = +-2), exact.
 int build_diag2(BuildOutput &b, cudaStream_t st, std::string &msg);
+
+// Row groups (FP32, real values) of the staged-gather kernel for long rows,
+// on the halo lists; leaves no_groups set where they do not pay or fit.
+int build_groups(BuildOutput &b, cudaStream_t st, std::string &msg);
 
 // Packed copy of the values of one precision for the pipelined kernel
 // (built on first use).

@@ -136,3 +136,42 @@ def test_quasi_lanes_and_norms(S):
         assert np.abs((np.abs(a[:, :, lo:hi]) ** 2).sum(-1) - 1).max() < 1e-12
         assert np.linalg.norm(a[:, :, lo:hi] - b[:, :, lo:hi], axis=-1).max() < 2e-5
     assert np.abs(nb / na - 1).max() < 2e-5
+
+
+# rows in groups of four (one-stage staged gathers, FP32 values per entry)
+# against the plain kernel: flakes with ragged edges, pairs listed twice, two
+# uneven samples, both group widths the kernel takes, and lists too long for it
+@pytest.mark.parametrize("S", [4, 8, 13])
+@pytest.mark.parametrize("kind", ["flake", "layers", "twice", "batch", "random"])
+def test_grouped_rows_are_bit_identical(S, kind):
+    import torch
+    import paper_2209_00806_gb300 as tb
+    from paper_2209_00806_gb300 import _native as N
+    from tbpm_inputs import tbg
+    offs = None
+    if kind == "random":
+        smp = lattice.random_graph(700, 9000, seed=1, onsite_w=1.0, t_scale=0.2)
+    else:
+        smp = tbg.to_numpy_sample(tbg.twisted_bilayer(7.3, order="layers" if kind == "layers" else
+                                                      "morton"))
+        smp.onsite = rng.uniform_range(5, rng.ONSITE, smp.n_orb, -0.2, 0.2)
+    if kind == "twice":
+        again = np.arange(0, smp.n_hop, 7)
+        for f in ("hop_i", "hop_j"):
+            setattr(smp, f, np.concatenate([getattr(smp, f), getattr(smp, f)[again]]))
+        smp.hop_v = np.concatenate([smp.hop_v, 0.01 * smp.hop_v[again]])
+    if kind == "batch":
+        smp, offs = lattice.concat([smp, tbg.to_numpy_sample(tbg.twisted_bilayer(4.0))])
+    theta = rng.phases(7, S, smp.n_orb)
+    out = []
+    # ZIGZAG | WIDE; ZIGZAG | HALO | STAGED; the default, which takes the staged kernel here
+    for variant in (65, 4609, 8257):
+        with tb.Propagator() as p:
+            p.launch_config(tb.TBPM_FP32, 8, 64, variant)
+            p.build_sample(smp, 13.0, offs)
+            p.set_phase_states(theta)
+            p.propagate(Z, 3, tb.TBPM_FP32)
+            phi = torch.empty((S, smp.n_orb), dtype=torch.complex128, device="cuda")
+            N.tbpm_get_states(p.ctx, phi)
+            out.append(phi)
+    assert (out[0] == out[1]).all() and (out[0] == out[2]).all()
