@@ -57,6 +57,7 @@ struct tbpm_ctx {
     // term-kernel launch variants (FP64, FP32): the fastest on GB300 for
     // graphene-like lattices; tbpm_autotune re-checks for the actual matrix
     int variant[2] = {kVariantZigZag, kVariantZigZag | kVariantWide | kVariantPrefetch};
+    bool cluster_auto = true;    // no FP64 launch shape asked for: small samples step in clusters
     int num_sms = 0;
     double renorm_fp32 = 1e-5, hard_fp32 = 1e-2, hard_fp64 = 1e-6;   // norm policy
     std::vector<Group> groups;
@@ -75,6 +76,7 @@ struct tbpm_ctx {
     int64_t done_len = 0;
     unsigned long long *d_fcounter = nullptr;
     FusedTerm *d_fterms = nullptr;         // [3][kMaxTerms]
+    ClusterState *d_cstates = nullptr;     // [kMaxStates]
     double *d_tile_partial = nullptr;
     int64_t tile_partial_len = 0;
     int *d_step = nullptr;       // [n_samples]
@@ -180,6 +182,8 @@ void free_hamiltonian(tbpm_ctx *c)
     cudaFree(c->d_done);
     cudaFree(c->d_fcounter);
     cudaFree(c->d_fterms);
+    cudaFree(c->d_cstates);
+    c->d_cstates = nullptr;
     cudaFree(c->d_tile_partial);
     c->d_items = nullptr;
     c->d_done = nullptr;
@@ -677,6 +681,7 @@ extern "C" int tbpm_set_launch_config(tbpm_ctx *c, int precision, int max_group,
     c->max_group[precision] = max_group;
     c->threads[precision] = threads;
     c->variant[precision] = variant;
+    if (precision == TBPM_FP64) c->cluster_auto = false;
     return TBPM_OK;
 }
 
@@ -1045,6 +1050,19 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     std::vector<size_t> step_ev;   // index of the first of 5 events per profiled step
     bool cluster_run = false;      // the cluster-resident stepping ran (one launch)
 
+    // cluster-resident stepping: every step of the FP64 states in one launch, a
+    // cluster of Kc blocks per state.  By default up to 512 rows a block: 64 x 64
+    // graphene takes 22 us a step in clusters (25 us with a diagonal, 31 us with
+    // values per entry) against 42-46 us a step and state group in launches;
+    // at 1024 rows a block the two meet (40-57 against 45-50 us).
+    const int Kc = ((variant & kVariantCluster) ||
+                    (c->cluster_auto && c->H.n_rows <= 16 * 512)) && !fp32 && !fused &&
+                           c->n_samples == 1 && !c->H.cplx && !c->ac_on && !c->qe_on &&
+                           c->H.max_width <= kClusterMaxW && n_steps > 0 && M - 1 >= 2 &&
+                           M - 1 <= kClusterMaxTerms
+                       ? cluster_blocks_for(c->H.n_rows, c->H.max_width, c->H.uniform)
+                       : 0;
+
     for (auto &g : c->groups) {
         const size_t bytes = (size_t)c->H.n_rows * g.B * cs;
         if (!resume) {
@@ -1248,81 +1266,7 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         ra.scale = g.scale;
         ra.scale_f = g.scale_f;
 
-        // cluster-resident stepping: every step of this one FP64 state in one launch
-        const int Kc = (variant & kVariantCluster) && !fp32 && !fused &&
-                               c->groups.size() == 1 && g.B == 1 && c->n_samples == 1 &&
-                               !c->H.cplx && !c->ac_on && !c->qe_on && c->H.val64 &&
-                               c->H.max_width <= kClusterMaxW && n_steps > 0 &&
-                               M - 1 >= 2 && M - 1 <= kClusterMaxTerms
-                           ? cluster_blocks_for(c->H.n_rows, c->H.max_width, c->H.uniform)
-                           : 0;
-        if (Kc > 0) {
-            if (!c->d_fterms) {
-                rc = dalloc(c, &c->d_fterms, 3 * (size_t)kMaxTerms);
-                if (rc) return rc;
-            }
-            std::vector<FusedTerm> tabs(3 * (size_t)kMaxTerms);
-            ClusterArgs ca;
-            memset(&ca, 0, sizeof(ca));
-            for (int cur0 = 0; cur0 < 3; ++cur0) {
-                int nx = 0;
-                std::vector<Launch> sch = schedule(a, cur0, &nx);
-                ca.next_cur[cur0] = nx;
-                for (size_t k = 0; k < sch.size(); ++k) {
-                    FusedTerm &ft = tabs[cur0 * kMaxTerms + k];
-                    ft.x = sch[k].x;
-                    ft.z = sch[k].z;
-                    ft.out = sch[k].out;
-                    ft.final_term = sch[k].final_term ? 1 : 0;
-                    split_coeff(sch[k].c, 0, &ft.c_hi, &ft.c_lo);
-                    ft.gamma = tsign * sch[k].gamma;
-                    one_value_table(c->H, ft);
-                }
-            }
-            CUDA_OR_FAIL(c, cudaMemcpyAsync(c->d_fterms, tabs.data(), tabs.size() * sizeof(FusedTerm),
-                                            cudaMemcpyHostToDevice, c->st));
-            ca.col = c->H.col;
-            ca.val = c->H.val64;
-            ca.diag = c->H.diag64;
-            ca.slice_ptr = c->H.slice_ptr;
-            ca.fixed_width = c->H.fixed_width;
-            ca.uniform = c->H.uniform;
-            ca.zero_diag = c->H.zero_diag;
-            ca.h_uniform = c->H.h_uniform;
-            ca.max_w = std::max(1, c->H.max_width);
-            ca.rows_per_cta = (int)(c->H.n_rows / Kc);
-            ca.psi0 = (const double2 *)g.psi0;
-            for (int k = 0; k < 3; ++k) ca.bufs[k] = (double2 *)g.buf[k];
-            ca.cur0 = g.cur;
-            ca.terms = c->d_fterms;
-            ca.J = M - 1;
-            ca.n_steps = n_steps;
-            const int64_t idx0 = (int64_t)g.s0 * (n_steps + 1);
-            ca.corr = c->d_corr + idx0;
-            ca.norms = c->d_norms + idx0;
-            ca.norm_ref = c->d_norm_ref + g.s0;
-            ca.hard_bound = c->hard_fp64;
-            ca.err = c->d_flags;
-            size_t e0 = 0;
-            if (profile) {
-                e0 = ev_used;
-                ev_used += ev_per_step;
-                step_ev.push_back(e0);
-                for (int q = 0; q < 2; ++q) CUDA_OR_FAIL(c, cudaEventRecord(c->events[e0 + q], c->st));
-            }
-            cudaError_t e = launch_cluster_steps(ca, Kc, c->st);
-            if (e != cudaSuccess)
-                return fail(c, TBPM_E_CUDA, std::string("cluster steps: ") + cudaGetErrorString(e));
-            if (profile)
-                for (int q = 2; q < 5; ++q) CUDA_OR_FAIL(c, cudaEventRecord(c->events[e0 + q], c->st));
-            CUDA_OR_FAIL(c, cudaStreamSynchronize(c->st));    // host table goes out of scope
-            int cur = g.cur;
-            for (int n = 0; n < n_steps; ++n) cur = ca.next_cur[cur];
-            g.cur = cur;
-            launches += 1;
-            cluster_run = true;
-            continue;
-        }
+        if (Kc > 0) continue;           // all groups' states step together below
 
         int final_extra = 0;            // launches of the closing term beyond one
         auto run_step = [&](int cur, int *next_cur, bool timed) -> int {
@@ -1444,6 +1388,86 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
             if (c->qe_on) launches += 1; // quasi-eigenstate accumulation
         }
     }
+    if (Kc > 0) {
+        if (!c->d_fterms) {
+            rc = dalloc(c, &c->d_fterms, 3 * (size_t)kMaxTerms);
+            if (rc) return rc;
+        }
+        if (!c->d_cstates) {
+            rc = dalloc(c, &c->d_cstates, (size_t)kMaxStates);
+            if (rc) return rc;
+        }
+        std::vector<FusedTerm> tabs(3 * (size_t)kMaxTerms);
+        ClusterArgs ca;
+        memset(&ca, 0, sizeof(ca));
+        for (int cur0 = 0; cur0 < 3; ++cur0) {
+            int nx = 0;
+            std::vector<Launch> sch = schedule(a, cur0, &nx);
+            ca.next_cur[cur0] = nx;
+            for (size_t k = 0; k < sch.size(); ++k) {
+                FusedTerm &ft = tabs[cur0 * kMaxTerms + k];
+                ft.x = sch[k].x;
+                ft.z = sch[k].z;
+                ft.out = sch[k].out;
+                ft.final_term = sch[k].final_term ? 1 : 0;
+                split_coeff(sch[k].c, 0, &ft.c_hi, &ft.c_lo);
+                ft.gamma = tsign * sch[k].gamma;
+                one_value_table(c->H, ft);
+            }
+        }
+        std::vector<ClusterState> cst;
+        for (auto &g : c->groups)
+            for (int b = 0; b < g.B; ++b) {
+                ClusterState cs1;
+                cs1.psi0 = (const double2 *)g.psi0 + b;
+                for (int k = 0; k < 3; ++k) cs1.bufs[k] = (double2 *)g.buf[k] + b;
+                const int64_t idx0 = (int64_t)(g.s0 + b) * (n_steps + 1);
+                cs1.corr = c->d_corr + idx0;
+                cs1.norms = c->d_norms + idx0;
+                cs1.norm_ref = c->d_norm_ref + g.s0 + b;
+                cs1.B = g.B;
+                cst.push_back(cs1);
+            }
+        CUDA_OR_FAIL(c, cudaMemcpyAsync(c->d_fterms, tabs.data(), tabs.size() * sizeof(FusedTerm),
+                                        cudaMemcpyHostToDevice, c->st));
+        CUDA_OR_FAIL(c, cudaMemcpyAsync(c->d_cstates, cst.data(), cst.size() * sizeof(ClusterState),
+                                        cudaMemcpyHostToDevice, c->st));
+        ca.col = c->H.col;
+        ca.val = c->H.val64;
+        ca.diag = c->H.diag64;
+        ca.slice_ptr = c->H.slice_ptr;
+        ca.fixed_width = c->H.fixed_width;
+        ca.uniform = c->H.uniform;
+        ca.zero_diag = c->H.zero_diag;
+        ca.h_uniform = c->H.h_uniform;
+        ca.max_w = std::max(1, c->H.max_width);
+        ca.rows_per_cta = (int)(c->H.n_rows / Kc);
+        ca.states = c->d_cstates;
+        ca.n_states = (int)cst.size();
+        ca.cur0 = c->groups[0].cur;                  // the groups step alike
+        ca.terms = c->d_fterms;
+        ca.J = M - 1;
+        ca.n_steps = n_steps;
+        ca.hard_bound = c->hard_fp64;
+        ca.err = c->d_flags;
+        size_t e0 = 0;
+        if (profile) {
+            e0 = ev_used;
+            ev_used += ev_per_step;
+            step_ev.push_back(e0);
+            for (int q = 0; q < 2; ++q) CUDA_OR_FAIL(c, cudaEventRecord(c->events[e0 + q], c->st));
+        }
+        cudaError_t e = launch_cluster_steps(ca, Kc, c->st);
+        if (e != cudaSuccess)
+            return fail(c, TBPM_E_CUDA, std::string("cluster steps: ") + cudaGetErrorString(e));
+        if (profile)
+            for (int q = 2; q < 5; ++q) CUDA_OR_FAIL(c, cudaEventRecord(c->events[e0 + q], c->st));
+        CUDA_OR_FAIL(c, cudaStreamSynchronize(c->st));    // host tables go out of scope
+        for (auto &g : c->groups)
+            for (int n = 0; n < n_steps; ++n) g.cur = ca.next_cur[g.cur];
+        launches += 1;
+        cluster_run = true;
+    }
     if (profile) CUDA_OR_FAIL(c, cudaEventRecord(ev_all1, c->st));
 
     // results and checks
@@ -1521,8 +1545,11 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         // fused: the whole step is one launch; report its per-term share;
         // cluster stepping: the whole run is one launch
         S.term_launches = (int64_t)step_ev.size() * (fused ? (M - 1) : n_int);
-        if (cluster_run) S.term_launches = (int64_t)n_steps * (M - 1);
         if (S.term_launches) S.ms_term_avg = t_int / S.term_launches;
+        if (cluster_run) {               // the interior terms, at the average of all M - 1
+            S.term_launches = (int64_t)n_steps * n_int;
+            S.ms_term_avg = t_int / ((double)n_steps * (M - 1));
+        }
         if (!step_ev.empty()) {
             S.ms_final_avg = t_fin / step_ev.size();
             S.ms_reduce_avg = t_red / step_ev.size();
@@ -1942,9 +1969,9 @@ extern "C" int tbpm_autotune(tbpm_ctx *c, int precision, double z, int probe_ste
                 if ((V & kVariantTma) && c->H.n_rows > (1 << 24)) continue;
                 // the register-pipelined kernel takes real values
                 if ((V & kVariantPrefetch) && c->H.cplx) continue;
-                // the cluster stepping takes one FP64 state of a small real sample
+                // the cluster stepping takes the FP64 states of a small real sample
                 if ((V & kVariantCluster) &&
-                    (T != thread_opts[0] || precision != TBPM_FP64 || B != 1 || c->H.cplx ||
+                    (T != thread_opts[0] || precision != TBPM_FP64 || B != widths[0] || c->H.cplx ||
                      c->n_samples != 1 ||
                      !cluster_blocks_for(c->H.n_rows, c->H.max_width, c->H.uniform)))
                     continue;

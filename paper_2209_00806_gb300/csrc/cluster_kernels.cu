@@ -3,7 +3,7 @@
 // A sample of up to 16 x 1024 rows -- the 64 x 64 graphene DOS workload has
 // 8192 -- fits, with psi0, psi and the two Clenshaw buffers, in the shared
 // memory of one thread-block cluster.  All time steps of the propagation then
-// run in one launch: each block holds a contiguous range of rows (one row per
+// run in one launch, one cluster per state: each block holds a contiguous range of rows (one row per
 // thread), gathers x from the owning block's shared memory (distributed
 // shared memory across the cluster), and a cluster barrier separates the
 // Clenshaw terms (Sec. 2.2, Eq. psi_t).  The closing term's sums of
@@ -13,7 +13,7 @@
 // deterministic).  Per row
 // the arithmetic and its order are those of the plain term kernel, so the
 // states equal the per-term launches' bit for bit; the launch cost of
-// 15 kernels per step is gone.  FP64 states, one state, real values, at most
+// 15 kernels per step is gone.  FP64 states, real values, at most
 // kClusterMaxW entries per row, within the shared memory of a block.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -48,14 +48,43 @@ __device__ __forceinline__ double2 ld_cluster(uint32_t addr)
 
 constexpr uint32_t kNoEntry = 0xffffffffu;
 
+// Sums of three values over a warp (lane l: v0, v1, v2 of row l) by a tree that
+// halves the values held as it doubles the lanes summed: six FP64 adds a warp
+// where a butterfly per value takes fifteen, each 64 cycles of the FP64 pipe.
+// Lane 0 returns the sum of v0, lane 16 that of v1, lane 8 that of v2.
+__device__ __forceinline__ double warp_sum3(double v0, double v1, double v2)
+{
+    const int l = threadIdx.x & 31;
+    const bool hi = l & 16, q = l & 8;
+    // lanes 0-15 keep (v0, v2), lanes 16-31 keep (v1, nothing)
+    const double s0 = hi ? v0 : v1, s1 = hi ? v2 : 0.0;          // sent to lane ^ 16
+    double a = (hi ? v1 : v0) + __shfl_xor_sync(0xffffffffu, s0, 16);
+    double b = (hi ? 0.0 : v2) + __shfl_xor_sync(0xffffffffu, s1, 16);
+    // of those, lanes with bit 3 clear keep a, the others b
+    a = (q ? b : a) + __shfl_xor_sync(0xffffffffu, q ? a : b, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
+}
+// the lane of value v in the result
+__device__ __forceinline__ int sum3_lane(int v) { return v == 0 ? 0 : v == 1 ? 16 : 8; }
+
 // MAXW: the widest row the launch allows (its gather addresses stay in
-// registers: 4 for graphene-like lattices, kClusterMaxW otherwise).
-template <int MAXW, int MAXT>
+// registers): 3 when every row has three slots (graphene), else 4 or
+// kClusterMaxW.  M: the matrix form.  What a form lacks is not in its kernel:
+// a conditional FP64 operation costs its 64 cycles of the pipe executed or
+// not, and the FP64 pipes of the cluster's SMs set the time.  64 x 64 graphene
+// executed 14 FP64 instructions a row and term for 8, 15 more a row and
+// step for the sums and 96 in sequence on one warp: 31.4 us a step, 22.0 now
+// (25 with a diagonal, 31 with values per entry).
+template <int MAXW, int MAXT, Vals M>
 __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
 {
+    constexpr bool ONE = one_value(M);
     cg::cluster_group cl = cg::this_cluster();
     const int K = (int)cl.num_blocks();
     const int rank = (int)cl.block_rank();
+    const ClusterState me = a.states[blockIdx.x / K];        // one cluster a state
     const int R = a.rows_per_cta;
     const int t = threadIdx.x;
     const int64_t r = (int64_t)rank * R + t;
@@ -72,8 +101,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
     // this row's entries, as (owning block, local row) pairs
     int w;
     int64_t base;
-    if (a.fixed_width) {
-        w = a.fixed_width;
+    if (MAXW == 3 || a.fixed_width) {
+        w = MAXW == 3 ? 3 : a.fixed_width;
         base = (r / kSliceRows) * (kSliceRows * (int64_t)w) + r % kSliceRows;
     } else {
         const int64_t q = r / kSliceRows;
@@ -82,14 +111,16 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
     }
     for (int k = 0; k < w; ++k) {
         const int32_t c = a.col[base + (int64_t)k * kSliceRows];
-        ent[k * R + t] = c == (int32_t)r && a.uniform ? -1 : ((c / R) << 16) | (c % R);
-        if (!a.uniform) sval[k * R + t] = a.val[base + (int64_t)k * kSliceRows];
+        ent[k * R + t] = c == (int32_t)r && ONE ? -1 : ((c / R) << 16) | (c % R);
+        if (!ONE) sval[k * R + t] = a.val[base + (int64_t)k * kSliceRows];
     }
     const double d = a.diag[r];
     const double d2 = d + d;                 // 2 d, exact: gamma d of the interior terms
-    vec[t] = a.psi0[r];
+    // gamma d of a step's first term (the same in the three tables)
+    const double d_first = M == kOne ? a.terms[0].gamma * d : 0.0;
+    vec[t] = me.psi0[r * me.B];
     for (int b = 0; b < 3; ++b)
-        vec[(1 + b) * R + t] = b == a.cur0 ? a.bufs[b][r] : make_double2(0.0, 0.0);
+        vec[(1 + b) * R + t] = b == a.cur0 ? me.bufs[b][r * me.B] : make_double2(0.0, 0.0);
     cl.sync();
     // gathered entries' shared::cluster addresses in x buffer 0 (a buffer
     // is R rows further on), fixed for the launch; kNoEntry for padding
@@ -98,7 +129,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
 #pragma unroll
     for (int k = 0; k < MAXW; ++k) {
         gsrc[k] = kNoEntry;
-        if (k < w) {
+        if (MAXW == 3 || k < w) {
             const int32_t e = ent[k * R + t];
             if (e >= 0) gsrc[k] = cluster_addr(vec + (e & 0xffff), e >> 16);
         }
@@ -110,8 +141,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
     // until they are all written: the closing term's own barrier completes
     // before the blocks write their parts, the next one after
     int sum_step = 0, sum_waits = 0;
-    // block 0, warp 0: lane k loads block k's parts of step m, the lanes'
-    // values are added in rank order; C_m, the norm and the drift checks
+    // block 0, warp 0: lane k loads block k's parts of step m, added in a fixed
+    // tree; C_m, the norm and the drift checks
     auto cluster_sum = [&](int m) {
         double w0 = 0.0, w1 = 0.0, w2 = 0.0;
         if (t < K) {
@@ -120,16 +151,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
             w1 = pk[1];
             w2 = pk[2];
         }
-        double sm0 = 0.0, sm1 = 0.0, sm2 = 0.0;
-        for (int k = 0; k < K; ++k) {
-            sm0 += __shfl_sync(0xffffffffu, w0, k);
-            sm1 += __shfl_sync(0xffffffffu, w1, k);
-            sm2 += __shfl_sync(0xffffffffu, w2, k);
-        }
+        const double v = warp_sum3(w0, w1, w2);
+        const double sm0 = v, sm1 = __shfl_sync(0xffffffffu, v, sum3_lane(1));
+        const double sm2 = __shfl_sync(0xffffffffu, v, sum3_lane(2));
         if (t == 0) {
-            a.corr[m] = make_double2(sm0, sm1);
-            a.norms[m] = sm2;
-            const double ref = *a.norm_ref;
+            me.corr[m] = make_double2(sm0, sm1);
+            me.norms[m] = sm2;
+            const double ref = *me.norm_ref;
             const double drift = ref > 0.0 ? fabs(sm2 / ref - 1.0) : sm2;
             if (!(sm2 == sm2) || !(sm0 == sm0) || !(sm1 == sm1) || sm2 - sm2 != 0.0)
                 atomicOr(a.err, 2);
@@ -152,14 +180,14 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
             // one-value form: its first product, fma(c, psi, z), needs nothing
             // of this term's x, so it runs before the barrier wait
             double re = 0.0, im = 0.0;
-            if (a.uniform) {
+            if (ONE) {
                 re = fma(tm.c_hi, p.x, zz.x);
                 im = fma(tm.c_hi, p.y, zz.y);
             }
             if (pending) cl.barrier_wait();      // the gathered vector is complete
             pending = false;
             if (sum_waits > 0 && --sum_waits == 0 && rank == 0 && t < 32) cluster_sum(sum_step);
-            if (a.uniform) {
+            if constexpr (ONE) {
                 // the one-value form of the per-term kernels: neighbours summed
                 // in stored order (padding only after a row's entries), then
                 // fma(gh, s, fma(gd, x_r, fma(c, psi, z)))
@@ -167,16 +195,16 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
                 if (gsrc[0] != kNoEntry) sm = ld_cluster(gsrc[0] + xoff_b);
 #pragma unroll
                 for (int k = 1; k < MAXW; ++k) {
-                    if (k < w && gsrc[k] != kNoEntry) {
+                    if ((MAXW == 3 || k < w) && gsrc[k] != kNoEntry) {
                         const double2 x = ld_cluster(gsrc[k] + xoff_b);
                         sm.x += x.x;
                         sm.y += x.y;
                     }
                 }
-                if (!a.zero_diag) {
+                if constexpr (M == kOne) {
                     const double gd = tm.gd_sel == 2 ? xor_sign(d2, tm.gd_sign)
                                     : tm.gd_sel == 1 ? xor_sign(d, tm.gd_sign)
-                                                     : tm.gamma * d;
+                                                     : d_first;
                     const double2 xo = vec[xoff + t];
                     re = fma(gd, xo.y, re);
                     im = fma(-gd, xo.x, im);
@@ -185,17 +213,12 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
                 o.y = fma(-tm.gh, sm.x, im);
             } else {
                 // y = H~ x in the plain kernel's order: diagonal, then the entries
-                // (a zero diagonal contributes only signed zeros: skipped, the
-                // sums stay equal to the plain kernel's)
-                double2 y = make_double2(0.0, 0.0);
-                if (!a.zero_diag) {
-                    y = vec[xoff + t];
-                    y.x *= d;
-                    y.y *= d;
-                }
+                double2 y = vec[xoff + t];
+                y.x *= d;
+                y.y *= d;
 #pragma unroll
                 for (int k = 0; k < MAXW; ++k) {
-                    if (k < w) {
+                    if (MAXW == 3 || k < w) {
                         const double h = sval[k * R + t];
                         const double2 x = ld_cluster(gsrc[k] + xoff_b);
                         y.x = fma(h, x.x, y.x);
@@ -219,18 +242,11 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
                 double v0 = fma(p0.x, o.x, p0.y * o.y);
                 double v1 = fma(p0.x, o.y, -(p0.y * o.x));
                 double v2 = fma(o.x, o.x, o.y * o.y);
-                for (int off = 16; off > 0; off >>= 1) {
-                    v0 += __shfl_xor_sync(0xffffffffu, v0, off);
-                    v1 += __shfl_xor_sync(0xffffffffu, v1, off);
-                    v2 += __shfl_xor_sync(0xffffffffu, v2, off);
-                }
-                if (t % 32 == 0) {
-                    red[t / 32][0] = v0;
-                    red[t / 32][1] = v1;
-                    red[t / 32][2] = v2;
-                }
+                const int lane = t % 32;
+                const double v = warp_sum3(v0, v1, v2);
+                if (lane % 8 == 0 && lane < 24) red[t / 32][lane == 0 ? 0 : lane == 16 ? 1 : 2] = v;
                 __syncthreads();
-                if (t < 32) {               // warp q's sums in order, loaded at once
+                if (t < 32) {               // the warps' sums, in a fixed tree
                     const int nq = (R + 31) / 32;
                     double w0 = 0.0, w1 = 0.0, w2 = 0.0;
                     if (t < nq) {
@@ -238,17 +254,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
                         w1 = red[t][1];
                         w2 = red[t][2];
                     }
-                    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-                    for (int q = 0; q < nq; ++q) {
-                        s0 += __shfl_sync(0xffffffffu, w0, q);
-                        s1 += __shfl_sync(0xffffffffu, w1, q);
-                        s2 += __shfl_sync(0xffffffffu, w2, q);
-                    }
-                    if (t == 0) {
-                        part[n & 1][0] = s0;
-                        part[n & 1][1] = s1;
-                        part[n & 1][2] = s2;
-                    }
+                    const double u = warp_sum3(w0, w1, w2);
+                    if (t % 8 == 0 && t < 24) part[n & 1][t == 0 ? 0 : t == 16 ? 1 : 2] = u;
                 }
                 sum_step = n;
                 sum_waits = 2;
@@ -266,7 +273,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
         cl.sync();
         if (rank == 0 && t < 32) cluster_sum(sum_step);
     }
-    a.bufs[cur][r] = vec[(1 + cur) * R + t];
+    me.bufs[cur][r * me.B] = vec[(1 + cur) * R + t];
     cl.sync();                                           // no block leaves while others read it
 }
 
@@ -280,7 +287,7 @@ int cluster_blocks_for(int64_t n_rows, int max_w, int uniform)
     static int best16 = -1;
     if (best16 < 0) {
         best16 = 0;
-        if (cudaFuncSetAttribute(k_cluster_steps<kClusterMaxW, 1024>,
+        if (cudaFuncSetAttribute(k_cluster_steps<kClusterMaxW, 1024, kReal>,
                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
             cudaLaunchConfig_t cfg = {};
             cudaLaunchAttribute at;
@@ -294,9 +301,9 @@ int cluster_blocks_for(int64_t n_rows, int max_w, int uniform)
             cfg.attrs = &at;
             cfg.numAttrs = 1;
             int n = 0;
-            cudaFuncSetAttribute(k_cluster_steps<kClusterMaxW, 1024>,
+            cudaFuncSetAttribute(k_cluster_steps<kClusterMaxW, 1024, kReal>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-            if (cudaOccupancyMaxActiveClusters(&n, k_cluster_steps<kClusterMaxW, 1024>, &cfg) ==
+            if (cudaOccupancyMaxActiveClusters(&n, k_cluster_steps<kClusterMaxW, 1024, kReal>, &cfg) ==
                     cudaSuccess &&
                 n >= 1)
                 best16 = 1;
@@ -313,14 +320,14 @@ int cluster_blocks_for(int64_t n_rows, int max_w, int uniform)
     return fits(8) ? 8 : 0;
 }
 
-template <int MAXW, int MAXT>
+template <int MAXW, int MAXT, Vals M>
 cudaError_t launch_cluster_t(const ClusterArgs &a, int K, size_t smem, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_cluster_steps<MAXW, MAXT>,
+    cudaError_t e = cudaFuncSetAttribute(k_cluster_steps<MAXW, MAXT, M>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (K > 8) {
-        e = cudaFuncSetAttribute(k_cluster_steps<MAXW, MAXT>,
+        e = cudaFuncSetAttribute(k_cluster_steps<MAXW, MAXT, M>,
                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
     }
@@ -330,13 +337,28 @@ cudaError_t launch_cluster_t(const ClusterArgs &a, int K, size_t smem, cudaStrea
     at.val.clusterDim.x = K;
     at.val.clusterDim.y = 1;
     at.val.clusterDim.z = 1;
-    cfg.gridDim = dim3(K);
+    cfg.gridDim = dim3(K * a.n_states);
     cfg.blockDim = dim3(a.rows_per_cta);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_cluster_steps<MAXW, MAXT>, a);
+    return cudaLaunchKernelEx(&cfg, k_cluster_steps<MAXW, MAXT, M>, a);
+}
+
+template <int MAXW, int MAXT>
+cudaError_t launch_cluster_m(const ClusterArgs &a, int K, size_t smem, cudaStream_t st)
+{
+    if (!a.uniform) return launch_cluster_t<MAXW, MAXT, kReal>(a, K, smem, st);
+    return a.zero_diag ? launch_cluster_t<MAXW, MAXT, kOneNoDiag>(a, K, smem, st)
+                       : launch_cluster_t<MAXW, MAXT, kOne>(a, K, smem, st);
+}
+template <int MAXT>
+cudaError_t launch_cluster_w(const ClusterArgs &a, int K, size_t smem, cudaStream_t st)
+{
+    if (a.fixed_width == 3) return launch_cluster_m<3, MAXT>(a, K, smem, st);
+    return a.max_w <= 4 ? launch_cluster_m<4, MAXT>(a, K, smem, st)
+                        : launch_cluster_m<kClusterMaxW, MAXT>(a, K, smem, st);
 }
 
 cudaError_t launch_cluster_steps(const ClusterArgs &a, int K, cudaStream_t st)
@@ -345,11 +367,7 @@ cudaError_t launch_cluster_steps(const ClusterArgs &a, int K, cudaStream_t st)
     const size_t smem = (size_t)4 * R * sizeof(double2) + (size_t)a.max_w * R * sizeof(int32_t) +
                         (a.uniform ? 0 : (size_t)a.max_w * R * sizeof(double));
     // up to 512 rows per block: 128 registers a thread, else 64
-    if (R <= 512)
-        return a.max_w <= 4 ? launch_cluster_t<4, 512>(a, K, smem, st)
-                            : launch_cluster_t<kClusterMaxW, 512>(a, K, smem, st);
-    return a.max_w <= 4 ? launch_cluster_t<4, 1024>(a, K, smem, st)
-                        : launch_cluster_t<kClusterMaxW, 1024>(a, K, smem, st);
+    return R <= 512 ? launch_cluster_w<512>(a, K, smem, st) : launch_cluster_w<1024>(a, K, smem, st);
 }
 
 }  // namespace tbpm

@@ -463,10 +463,19 @@ struct FusedArgs {
 
 cudaError_t launch_step_fused(const FusedArgs &f, int fp32, int B, int num_sms, cudaStream_t st);
 
-// Cluster-resident time stepping (cluster_kernels.cu): all steps of one FP64
-// state of a sample of up to 16 x 1024 rows in one cluster launch.
+// Cluster-resident time stepping (cluster_kernels.cu): all steps of the FP64
+// states of a sample of up to 16 x 1024 rows in one launch, a cluster a state.
 constexpr int kClusterMaxW = 12;           // entries per row it takes
 constexpr int kClusterMaxTerms = 40;       // Chebyshev terms per step it takes (z <= ~25)
+// One state: row r of its vectors is element r * B of each pointer.
+struct ClusterState {
+    const double2 *psi0;
+    double2 *bufs[3];
+    double2 *corr;              // C_n, n = 0 .. n_steps
+    double *norms;
+    const double *norm_ref;
+    int B;
+};
 struct ClusterArgs {
     const int32_t *col;
     const double *val;
@@ -475,16 +484,13 @@ struct ClusterArgs {
     int fixed_width, uniform, max_w, rows_per_cta;
     int zero_diag;              // every onsite energy is zero
     double h_uniform;
-    const double2 *psi0;
-    double2 *bufs[3];
+    const ClusterState *states;
+    int n_states;
     int cur0;
     const FusedTerm *terms;     // [3][kMaxTerms] schedules by the buffer holding psi
     int J;                      // terms per step
     int next_cur[3];
     int n_steps;
-    double2 *corr;              // C_n, n = 1 .. n_steps (state 0 of sample 0)
-    double *norms;
-    const double *norm_ref;
     double hard_bound;
     int *err;
 };

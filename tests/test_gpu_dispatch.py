@@ -175,3 +175,30 @@ def test_grouped_rows_are_bit_identical(S, kind):
             N.tbpm_get_states(p.ctx, phi)
             out.append(phi)
     assert (out[0] == out[1]).all() and (out[0] == out[2]).all()
+
+
+# cluster stepping of several states at once, and as the default up to 8192
+# rows, against the per-term launches: states bit for bit, C within the
+# rounding of its sums (1e-13, as the one-state test), with a resumed run
+@pytest.mark.parametrize("S", [1, 3, 9])
+@pytest.mark.parametrize("onsite_w,sigma,sides", [(0.0, 0.0, (64, 64)), (1.0, 0.0, (13, 17)),
+                                                  (1.0, 0.05, (40, 51)), (1.0, 0.0, (64, 65))])
+def test_cluster_states_are_bit_identical(S, onsite_w, sigma, sides):
+    import paper_2209_00806_gb300 as tb
+    from paper_2209_00806_gb300 import _native as N
+    smp = lattice.graphene(*sides, pbc=True, seed=6, onsite_w=onsite_w, bond_sigma=sigma)
+    theta = rng.phases(13, S, smp.n_orb)
+    out = []
+    for variant in (1, 2049, None):
+        with tb.Propagator() as p:
+            if variant is not None:
+                p.launch_config(tb.TBPM_FP64, 8, 64, variant)
+            p.build_sample(smp, 9.5)
+            p.set_phase_states(theta)
+            C = p.propagate(Z, 7, tb.TBPM_FP64)
+            D = p.propagate(Z, 4, tb.TBPM_FP64, flags=N.TBPM_PROP_RESUME)
+            out.append((C, D, p.states(), p.norms()))
+    for o in out[1:]:
+        assert np.array_equal(out[0][2], o[2])
+        for a, b in zip((out[0][0], out[0][1], out[0][3]), (o[0], o[1], o[3])):
+            assert np.abs(a - b).max() < 1e-13
