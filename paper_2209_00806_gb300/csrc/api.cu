@@ -30,6 +30,11 @@ struct Group {
 
 }  // namespace
 
+// Results of a call that come back together: up to this many bytes go through
+// a page-locked buffer of the context with one wait; more are copied directly.
+constexpr size_t kResBytes = 64 * 1024;
+constexpr size_t kFlagBytes = 4 * sizeof(int) + sizeof(unsigned long long);
+
 struct tbpm_ctx {
     int device = 0;
     cudaStream_t user = nullptr;
@@ -49,6 +54,9 @@ struct tbpm_ctx {
     // initial states, caller order, complex128 [n_states][n_orb]
     int n_states = 0;
     double2 *d_psi_user = nullptr;
+    size_t psi_count = 0;        // elements it holds
+    cudaEvent_t ev_order = nullptr;        // orders our stream and the user's
+    unsigned char *h_res = nullptr;        // page-locked, kResBytes: small results
 
     // propagation state
     int prec = -1;               // precision of the group buffers
@@ -61,6 +69,7 @@ struct tbpm_ctx {
     int num_sms = 0;
     double renorm_fp32 = 1e-5, hard_fp32 = 1e-2, hard_fp64 = 1e-6;   // norm policy
     std::vector<Group> groups;
+    int group_states = 0;        // states the groups were allocated for
     double *d_partial = nullptr;
     int64_t partial_len = 0;
     double *d_block_partial = nullptr;
@@ -150,6 +159,7 @@ void free_groups(tbpm_ctx *c)
         cudaFree(g.scale_f);
     }
     c->groups.clear();
+    c->group_states = 0;
     c->prec = -1;
     c->have_run = false;
 }
@@ -171,6 +181,7 @@ void free_hamiltonian(tbpm_ctx *c)
     cudaFree(c->d_sample_chunk_off);
     cudaFree(c->d_inv_sqrt_n);
     cudaFree(c->d_psi_user);
+    c->psi_count = 0;
     cudaFree(c->d_partial);
     cudaFree(c->d_block_partial);
     cudaFree(c->d_chunk_count);
@@ -219,22 +230,16 @@ void free_hamiltonian(tbpm_ctx *c)
 int enter(tbpm_ctx *c)
 {
     CUDA_OR_FAIL(c, cudaSetDevice(c->device));
-    cudaEvent_t e;
-    CUDA_OR_FAIL(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    CUDA_OR_FAIL(c, cudaEventRecord(e, c->user));
-    CUDA_OR_FAIL(c, cudaStreamWaitEvent(c->st, e, 0));
-    cudaEventDestroy(e);
+    CUDA_OR_FAIL(c, cudaEventRecord(c->ev_order, c->user));
+    CUDA_OR_FAIL(c, cudaStreamWaitEvent(c->st, c->ev_order, 0));
     return TBPM_OK;
 }
 
 // Make the user's stream wait for our work.
 int leave(tbpm_ctx *c)
 {
-    cudaEvent_t e;
-    CUDA_OR_FAIL(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    CUDA_OR_FAIL(c, cudaEventRecord(e, c->st));
-    CUDA_OR_FAIL(c, cudaStreamWaitEvent(c->user, e, 0));
-    cudaEventDestroy(e);
+    CUDA_OR_FAIL(c, cudaEventRecord(c->ev_order, c->st));
+    CUDA_OR_FAIL(c, cudaStreamWaitEvent(c->user, c->ev_order, 0));
     return TBPM_OK;
 }
 
@@ -379,8 +384,10 @@ extern "C" int tbpm_create(tbpm_ctx **out, int device, void *stream)
     e = cudaSetDevice(device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->st, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_flags, 4 * sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_renorm, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_order, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_flags, kFlagBytes);       // flags, renorm count
+    if (e == cudaSuccess) c->d_renorm = (unsigned long long *)(c->d_flags + 4);
+    if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->h_res, kResBytes, cudaHostAllocDefault);
     if (e != cudaSuccess) {
         std::string m = std::string("context setup: ") + cudaGetErrorString(e);
         tbpm_destroy(c);
@@ -397,7 +404,8 @@ extern "C" void tbpm_destroy(tbpm_ctx *c)
     if (c->st) cudaStreamSynchronize(c->st);
     free_hamiltonian(c);
     cudaFree(c->d_flags);
-    cudaFree(c->d_renorm);
+    cudaFreeHost(c->h_res);
+    if (c->ev_order) cudaEventDestroy(c->ev_order);
     for (auto e : c->events) cudaEventDestroy(e);
     if (c->st) cudaStreamDestroy(c->st);
     delete c;
@@ -600,13 +608,18 @@ static int set_states_common(tbpm_ctx *c, int n_states, const double *src, int w
         return fail(c, TBPM_E_INVALID_ARG, "where must be TBPM_HOST or TBPM_DEVICE");
     int rc = enter(c);
     if (rc) return rc;
-    free_groups(c);
-    cudaFree(c->d_psi_user);
-    c->d_psi_user = nullptr;
+    // new states of the same number keep the buffers of the last ones
+    if (c->group_states != n_states) free_groups(c);
+    c->have_run = false;
     c->n_states = 0;
     const size_t count = (size_t)n_states * c->n_orb;
-    rc = dalloc(c, &c->d_psi_user, count);
-    if (rc) return rc;
+    if (c->psi_count != count) {
+        cudaFree(c->d_psi_user);
+        c->psi_count = 0;
+        rc = dalloc(c, &c->d_psi_user, count);
+        if (rc) return rc;
+        c->psi_count = count;
+    }
     if (phases) {
         const double *d_theta = nullptr;
         bool owned = false;
@@ -701,7 +714,7 @@ extern "C" int tbpm_set_norm_policy(tbpm_ctx *c, double renorm_fp32, double hard
 // widths no wider than the cap (e.g. 3 -> 2 + 1).
 static int ensure_groups(tbpm_ctx *c, int prec)
 {
-    if (c->prec == prec && !c->groups.empty()) return TBPM_OK;
+    if (c->prec == prec && !c->groups.empty() && c->group_states == c->n_states) return TBPM_OK;
     free_groups(c);
     const size_t cs = prec == TBPM_FP64 ? 16 : 8;
     int left = c->n_states, s0 = 0;
@@ -764,6 +777,7 @@ static int ensure_groups(tbpm_ctx *c, int prec)
         cudaMemsetAsync(c->d_sample_ticket, 0, c->n_samples * sizeof(unsigned int), c->st);
     }
     c->prec = prec;
+    c->group_states = c->n_states;
     return TBPM_OK;
 }
 
@@ -964,8 +978,7 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         if (rc) return rc;
         c->corr_steps = n_steps;
     }
-    CUDA_OR_FAIL(c, cudaMemsetAsync(c->d_flags, 0, 4 * sizeof(int), c->st));
-    CUDA_OR_FAIL(c, cudaMemsetAsync(c->d_renorm, 0, sizeof(unsigned long long), c->st));
+    CUDA_OR_FAIL(c, cudaMemsetAsync(c->d_flags, 0, kFlagBytes, c->st));
     {
         const int64_t need = (int64_t)c->n_samples * c->n_states;
         if (need > c->norm_ref_len) {
@@ -1067,14 +1080,15 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         const size_t bytes = (size_t)c->H.n_rows * g.B * cs;
         if (!resume) {
             CUDA_OR_FAIL(c, launch_set_states(c->d_psi_user, c->n_orb, c->n_states,
-                                              c->H.user_to_row, g.s0, g.B, fp32, g.psi0, c->st));
+                                              c->H.user_to_row, g.s0, g.B, fp32, g.psi0, c->st,
+                                              g.scale, g.scale_f, c->n_samples * g.B));
             CUDA_OR_FAIL(c, cudaMemcpyAsync(g.buf[0], g.psi0, bytes, cudaMemcpyDeviceToDevice, c->st));
             g.cur = 0;
             launches += 1;
         }
         for (int k = 0; k < 3; ++k)
             if (g.graph[k]) { cudaGraphExecDestroy(g.graph[k]); g.graph[k] = nullptr; }
-        if (g.scale) {
+        if (g.scale && resume) {        // (a fresh run's scales come with its states)
             std::vector<double> ones((size_t)c->n_samples * g.B, 1.0);
             std::vector<float> ones_f((size_t)c->n_samples * g.B, 1.0f);
             CUDA_OR_FAIL(c, cudaMemcpyAsync(g.scale, ones.data(), ones.size() * sizeof(double),
@@ -1470,21 +1484,31 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     }
     if (profile) CUDA_OR_FAIL(c, cudaEventRecord(ev_all1, c->st));
 
-    // results and checks
+    // results and checks: flags and counts, norms, C
     int h_flags[4];
     unsigned long long h_renorm = 0;
-    CUDA_OR_FAIL(c, cudaMemcpyAsync(h_flags, c->d_flags, sizeof(h_flags), cudaMemcpyDeviceToHost, c->st));
-    CUDA_OR_FAIL(c, cudaMemcpyAsync(&h_renorm, c->d_renorm, sizeof(h_renorm), cudaMemcpyDeviceToHost, c->st));
     const size_t cnt = (size_t)c->n_samples * c->n_states * (n_steps + 1);
     std::vector<double> norms(cnt);
-    CUDA_OR_FAIL(c, cudaMemcpyAsync(norms.data(), c->d_norms, cnt * sizeof(double),
-                                    cudaMemcpyDeviceToHost, c->st));
-    if (corr_out)
+    const size_t norm_b = cnt * sizeof(double);
+    const size_t corr_b = corr_out && where_out == TBPM_HOST ? cnt * sizeof(double2) : 0;
+    const size_t at_norm = 32, at_corr = at_norm + norm_b;
+    const bool small = at_corr + corr_b <= kResBytes;
+    CUDA_OR_FAIL(c, cudaMemcpyAsync(c->h_res, c->d_flags, kFlagBytes, cudaMemcpyDeviceToHost, c->st));
+    CUDA_OR_FAIL(c, cudaMemcpyAsync(small ? (void *)(c->h_res + at_norm) : norms.data(), c->d_norms,
+                                    norm_b, cudaMemcpyDeviceToHost, c->st));
+    if (corr_b)
+        CUDA_OR_FAIL(c, cudaMemcpyAsync(small ? (void *)(c->h_res + at_corr) : corr_out, c->d_corr,
+                                        corr_b, cudaMemcpyDeviceToHost, c->st));
+    else if (corr_out)
         CUDA_OR_FAIL(c, cudaMemcpyAsync(corr_out, c->d_corr, cnt * sizeof(double2),
-                                        where_out == TBPM_HOST ? cudaMemcpyDeviceToHost
-                                                               : cudaMemcpyDeviceToDevice,
-                                        c->st));
+                                        cudaMemcpyDeviceToDevice, c->st));
     CUDA_OR_FAIL(c, cudaStreamSynchronize(c->st));
+    memcpy(h_flags, c->h_res, sizeof(h_flags));
+    memcpy(&h_renorm, c->h_res + sizeof(h_flags), sizeof(h_renorm));
+    if (small) {
+        memcpy(norms.data(), c->h_res + at_norm, norm_b);
+        if (corr_b) memcpy(corr_out, c->h_res + at_corr, corr_b);
+    }
     c->have_run = true;
 
     tbpm_stats &S = c->stats;

@@ -1782,9 +1782,14 @@ __global__ void k_phase_user(const double *theta, int64_t n_orb, int n_states,
 
 template <typename V>
 __global__ void k_set_states(const double2 *src, int64_t n_orb, const int32_t *user_to_row,
-                             int g0, int B, void *psi)
+                             int g0, int B, void *psi, double *scale, float *scale_f, int n_scale)
 {
     const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (scale)                               // FP32 norm carry of a fresh run
+        for (int64_t k = u; k < n_scale; k += (int64_t)gridDim.x * blockDim.x) {
+            scale[k] = 1.0;
+            scale_f[k] = 1.f;
+        }
     if (u >= n_orb) return;
     const int64_t r = user_to_row[u];
     for (int b = 0; b < B; ++b) {
@@ -2212,14 +2217,16 @@ cudaError_t launch_phase_user(const double *theta, int64_t n_orb, int n_states,
 
 cudaError_t launch_set_states(const double2 *psi_user, int64_t n_orb, int n_states,
                               const int32_t *user_to_row, int g0, int B, int fp32, void *psi,
-                              cudaStream_t st)
+                              cudaStream_t st, double *scale, float *scale_f, int n_scale)
 {
     (void)n_states;
     const unsigned blocks = (unsigned)((n_orb + 255) / 256);
     if (fp32)
-        k_set_states<float><<<blocks, 256, 0, st>>>(psi_user, n_orb, user_to_row, g0, B, psi);
+        k_set_states<float><<<blocks, 256, 0, st>>>(psi_user, n_orb, user_to_row, g0, B, psi, scale,
+                                                    scale_f, n_scale);
     else
-        k_set_states<double><<<blocks, 256, 0, st>>>(psi_user, n_orb, user_to_row, g0, B, psi);
+        k_set_states<double><<<blocks, 256, 0, st>>>(psi_user, n_orb, user_to_row, g0, B, psi, scale,
+                                                     scale_f, n_scale);
     return cudaGetLastError();
 }
 

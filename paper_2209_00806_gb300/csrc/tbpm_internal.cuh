@@ -408,7 +408,8 @@ cudaError_t launch_phase_user(const double *theta, int64_t n_orb, int n_states,
                               double2 *psi_user, cudaStream_t st);
 cudaError_t launch_set_states(const double2 *psi_user, int64_t n_orb, int n_states,
                               const int32_t *user_to_row, int group_state0, int B,
-                              int fp32, void *psi, cudaStream_t st);
+                              int fp32, void *psi, cudaStream_t st, double *scale = nullptr,
+                              float *scale_f = nullptr, int n_scale = 0);   // scales set to 1
 cudaError_t launch_get_states(const void *psi, int64_t n_orb, int n_states,
                               const int32_t *user_to_row, int group_state0, int B,
                               int fp32, double2 *out_user, cudaStream_t st);

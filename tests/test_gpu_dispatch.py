@@ -202,3 +202,31 @@ def test_cluster_states_are_bit_identical(S, onsite_w, sigma, sides):
         assert np.array_equal(out[0][2], o[2])
         for a, b in zip((out[0][0], out[0][1], out[0][3]), (o[0], o[1], o[3])):
             assert np.abs(a - b).max() < 1e-13
+
+
+# buffers kept between calls: new states of the same number after a run (one of
+# them not finite), of another number, in both precisions, C over and under
+# the size of the page-locked result buffer (64 KB)
+def test_states_set_again_start_afresh():
+    import paper_2209_00806_gb300 as tb
+    smp = lattice.graphene(12, 9, pbc=True, seed=6, onsite_w=1.0)
+    th = rng.phases(15, 6, smp.n_orb)
+    def fresh(t, steps, precision):
+        with tb.Propagator() as q:
+            q.build_sample(smp, 9.5)
+            q.set_phase_states(t)
+            return q.propagate(Z, steps, precision), q.states(), q.norms()
+    with tb.Propagator() as p:
+        p.build_sample(smp, 9.5)
+        for t, steps, precision in ((th[:3], 5, 1), (th[3:], 5, 1), (th[:3], 5, 0), (th[1:4], 2000, 0),
+                                    (th[:2], 1500, 1), (th, 3, 1)):
+            bad = np.full((t.shape[0], smp.n_orb), np.nan, dtype=np.complex128)
+            p.set_states(bad)
+            with pytest.raises(tb.TbpmError):
+                p.propagate(Z, 3, precision)
+            p.set_phase_states(t)
+            with pytest.raises(tb.TbpmError):       # nothing to resume after new states
+                p.propagate(Z, 3, precision, flags=4)
+            got = (p.propagate(Z, steps, precision), p.states(), p.norms())
+            for a, b in zip(got, fresh(t, steps, precision)):
+                assert np.array_equal(a, b)
