@@ -347,14 +347,17 @@ int tbpm_dos_adjoint(const double *dl_dd, int n_e, int n_steps, double tau, int 
                                         halo lists are built on first use; a matrix
                                         with a block referencing over 2048 other rows
                                         keeps the plain kernel */
-#define TBPM_VARIANT_CLUSTER 2048    /* FP64, one sample of at most 16 x 1024 rows, at
-                                        most 12 entries per row: every time step of
-                                        the states in one launch, a thread-block
-                                        cluster per state, the vectors in the blocks'
-                                        shared memory (distributed shared memory for
-                                        the gathers), a cluster barrier per term;
-                                        otherwise ignored.  Taken by default (until a
-                                        launch shape is set) up to 16 x 512 rows */
+#define TBPM_VARIANT_CLUSTER 2048    /* one sample of at most 16 x 1024 rows (FP32 with
+                                        three slots a row: 16 x 4096), at most 12
+                                        entries per row: every time step of the states
+                                        in one launch, a thread-block cluster per
+                                        state, the vectors in the blocks' shared
+                                        memory (distributed shared memory for the
+                                        gathers), a cluster barrier per term;
+                                        otherwise ignored.  Until a launch shape is
+                                        set it is the default up to 16 x 512 rows
+                                        (FP32: all it takes with up to seven states,
+                                        16 x 1024 rows up to sixteen) */
 #define TBPM_VARIANT_PIPE 1024       /* with TBPM_VARIANT_HALO, interior terms: a
                                         persistent grid (one block per SM) with two
                                         shared-memory stages, the next block's halo,

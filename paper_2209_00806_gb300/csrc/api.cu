@@ -65,7 +65,9 @@ struct tbpm_ctx {
     // term-kernel launch variants (FP64, FP32): the fastest on GB300 for
     // graphene-like lattices; tbpm_autotune re-checks for the actual matrix
     int variant[2] = {kVariantZigZag, kVariantZigZag | kVariantWide | kVariantPrefetch};
-    bool cluster_auto = true;    // no FP64 launch shape asked for: small samples step in clusters
+    // no launch shape asked for (FP64, FP32): small samples step in clusters
+    bool cluster_auto[2] = {true, true};
+    bool cluster_off = false;    // repeating a run whose norm carry must act
     int num_sms = 0;
     double renorm_fp32 = 1e-5, hard_fp32 = 1e-2, hard_fp64 = 1e-6;   // norm policy
     std::vector<Group> groups;
@@ -694,7 +696,7 @@ extern "C" int tbpm_set_launch_config(tbpm_ctx *c, int precision, int max_group,
     c->max_group[precision] = max_group;
     c->threads[precision] = threads;
     c->variant[precision] = variant;
-    if (precision == TBPM_FP64) c->cluster_auto = false;
+    c->cluster_auto[precision] = false;
     return TBPM_OK;
 }
 
@@ -1068,12 +1070,18 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     // graphene takes 22 us a step in clusters (25 us with a diagonal, 31 us with
     // values per entry) against 42-46 us a step and state group in launches;
     // at 1024 rows a block the two meet (40-57 against 45-50 us).
-    const int Kc = ((variant & kVariantCluster) ||
-                    (c->cluster_auto && c->H.n_rows <= 16 * 512)) && !fp32 && !fused &&
+    // FP32, us a step: 64 x 64 10 against 42, 180 x 180 25 against 47-54 (seven
+    // clusters run at once: 16 states 30 against 52 at 64 x 64).
+    const bool auto_cluster = c->cluster_auto[precision] &&
+                       (fp32 ? c->n_states <= 16 &&
+                                   c->H.n_rows <= 16 * (c->n_states <= kClusterStates ? 4096 : 1024)
+                             : c->H.n_rows <= 16 * 512);
+    const int Kc = ((variant & kVariantCluster) || auto_cluster) && !c->cluster_off && !fused &&
                            c->n_samples == 1 && !c->H.cplx && !c->ac_on && !c->qe_on &&
                            c->H.max_width <= kClusterMaxW && n_steps > 0 && M - 1 >= 2 &&
                            M - 1 <= kClusterMaxTerms
-                       ? cluster_blocks_for(c->H.n_rows, c->H.max_width, c->H.uniform)
+                       ? cluster_blocks_for(c->H.n_rows, c->H.max_width, c->H.uniform, fp32,
+                                            c->H.fixed_width)
                        : 0;
 
     for (auto &g : c->groups) {
@@ -1424,17 +1432,30 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
                 ft.z = sch[k].z;
                 ft.out = sch[k].out;
                 ft.final_term = sch[k].final_term ? 1 : 0;
-                split_coeff(sch[k].c, 0, &ft.c_hi, &ft.c_lo);
+                split_coeff(sch[k].c, fp32, &ft.c_hi, &ft.c_lo);
                 ft.gamma = tsign * sch[k].gamma;
+                ft.c_hi_f = (float)ft.c_hi;
+                ft.c_lo_f = (float)ft.c_lo;
+                ft.gamma_f = (float)ft.gamma;
                 one_value_table(c->H, ft);
             }
         }
+        const int cur0 = c->groups[0].cur;           // the groups step alike
+        int cur1 = cur0;
+        for (int n = 0; n < n_steps; ++n) cur1 = ca.next_cur[cur1];
+        // a resumed FP32 run may have to be repeated: its state, kept in a
+        // buffer that the result does not take
+        const int keep = 3 - cur0 - (cur1 == cur0 ? (cur0 + 1) % 3 : cur1);
+        if (fp32 && resume)
+            for (auto &g : c->groups)
+                CUDA_OR_FAIL(c, cudaMemcpyAsync(g.buf[keep], g.buf[cur0], (size_t)c->H.n_rows * g.B * cs,
+                                                cudaMemcpyDeviceToDevice, c->st));
         std::vector<ClusterState> cst;
         for (auto &g : c->groups)
             for (int b = 0; b < g.B; ++b) {
                 ClusterState cs1;
-                cs1.psi0 = (const double2 *)g.psi0 + b;
-                for (int k = 0; k < 3; ++k) cs1.bufs[k] = (double2 *)g.buf[k] + b;
+                cs1.psi0 = (const char *)g.psi0 + b * cs;
+                for (int k = 0; k < 3; ++k) cs1.bufs[k] = (char *)g.buf[k] + b * cs;
                 const int64_t idx0 = (int64_t)(g.s0 + b) * (n_steps + 1);
                 cs1.corr = c->d_corr + idx0;
                 cs1.norms = c->d_norms + idx0;
@@ -1456,13 +1477,17 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         ca.h_uniform = c->H.h_uniform;
         ca.max_w = std::max(1, c->H.max_width);
         ca.rows_per_cta = (int)(c->H.n_rows / Kc);
+        ca.h_uniform_f = (float)c->H.h_uniform;
+        ca.val32 = c->H.val32;
+        ca.diag32 = c->H.diag32;
         ca.states = c->d_cstates;
         ca.n_states = (int)cst.size();
-        ca.cur0 = c->groups[0].cur;                  // the groups step alike
+        ca.cur0 = cur0;
         ca.terms = c->d_fterms;
         ca.J = M - 1;
         ca.n_steps = n_steps;
-        ca.hard_bound = c->hard_fp64;
+        ca.hard_bound = fp32 ? c->hard_fp32 : c->hard_fp64;
+        ca.renorm_bound = c->renorm_fp32;
         ca.err = c->d_flags;
         size_t e0 = 0;
         if (profile) {
@@ -1471,14 +1496,32 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
             step_ev.push_back(e0);
             for (int q = 0; q < 2; ++q) CUDA_OR_FAIL(c, cudaEventRecord(c->events[e0 + q], c->st));
         }
-        cudaError_t e = launch_cluster_steps(ca, Kc, c->st);
+        cudaError_t e = launch_cluster_steps(ca, fp32, Kc, c->st);
         if (e != cudaSuccess)
             return fail(c, TBPM_E_CUDA, std::string("cluster steps: ") + cudaGetErrorString(e));
         if (profile)
             for (int q = 2; q < 5; ++q) CUDA_OR_FAIL(c, cudaEventRecord(c->events[e0 + q], c->st));
-        CUDA_OR_FAIL(c, cudaStreamSynchronize(c->st));    // host tables go out of scope
-        for (auto &g : c->groups)
-            for (int n = 0; n < n_steps; ++n) g.cur = ca.next_cur[g.cur];
+        // (the host tables go out of scope)
+        CUDA_OR_FAIL(c, cudaMemcpyAsync(c->h_res, c->d_flags, kFlagBytes, cudaMemcpyDeviceToHost, c->st));
+        CUDA_OR_FAIL(c, cudaStreamSynchronize(c->st));
+        int hf = 0;
+        memcpy(&hf, c->h_res, sizeof(hf));
+        if (fp32 && (hf & 8)) {
+            // a norm drifted past the renormalisation bound: the per-term kernels,
+            // which rescale the state between steps, from the same start
+            if (resume)
+                for (auto &g : c->groups) {
+                    CUDA_OR_FAIL(c, cudaMemcpyAsync(g.buf[cur0], g.buf[keep],
+                                                    (size_t)c->H.n_rows * g.B * cs,
+                                                    cudaMemcpyDeviceToDevice, c->st));
+                    g.cur = cur0;
+                }
+            c->cluster_off = true;
+            rc = tbpm_propagate(c, z, n_steps, precision, corr_out, where_out, flags);
+            c->cluster_off = false;
+            return rc;
+        }
+        for (auto &g : c->groups) g.cur = cur1;
         launches += 1;
         cluster_run = true;
     }
@@ -1974,6 +2017,7 @@ extern "C" int tbpm_autotune(tbpm_ctx *c, int precision, double z, int probe_ste
                                 kVariantZigZag | kVariantPrefetch,
                                 kVariantZigZag | kVariantWide | kVariantPrefetch,
                                 kVariantZigZag | kVariantCluster};
+    const bool auto0 = c->cluster_auto[precision];
     double best = 1e300;
     int bg = c->max_group[precision], bt = c->threads[precision], bv = c->variant[precision];
     for (int B : widths)
@@ -1997,7 +2041,8 @@ extern "C" int tbpm_autotune(tbpm_ctx *c, int precision, double z, int probe_ste
                 if ((V & kVariantCluster) &&
                     (T != thread_opts[0] || precision != TBPM_FP64 || B != widths[0] || c->H.cplx ||
                      c->n_samples != 1 ||
-                     !cluster_blocks_for(c->H.n_rows, c->H.max_width, c->H.uniform)))
+                     !cluster_blocks_for(c->H.n_rows, c->H.max_width, c->H.uniform, 0,
+                                         c->H.fixed_width)))
                     continue;
                 if ((V & kVariantHalo) && !c->H.halo_ptr) {
                     std::string msg;
@@ -2015,6 +2060,15 @@ extern "C" int tbpm_autotune(tbpm_ctx *c, int precision, double z, int probe_ste
             }
     int rc = tbpm_set_launch_config(c, precision, bg, bt, bv);
     if (rc) return rc;
+    // the default's FP32 cluster stepping stays where it was the default and wins
+    if (auto0 && precision == TBPM_FP32) {
+        c->cluster_auto[precision] = true;
+        rc = tbpm_propagate(c, z, probe_steps, precision, nullptr, TBPM_HOST, TBPM_PROP_PROFILE);
+        if (rc) return rc;
+        const double ms = c->stats.ms_total / probe_steps;
+        c->cluster_auto[precision] = ms < best;
+        best = std::min(best, ms);
+    }
     if (best_group) *best_group = bg;
     if (best_threads) *best_threads = bt;
     if (best_variant) *best_variant = bv;

@@ -118,9 +118,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
     const double d2 = d + d;                 // 2 d, exact: gamma d of the interior terms
     // gamma d of a step's first term (the same in the three tables)
     const double d_first = M == kOne ? a.terms[0].gamma * d : 0.0;
-    vec[t] = me.psi0[r * me.B];
+    vec[t] = reinterpret_cast<const double2 *>(me.psi0)[r * me.B];
     for (int b = 0; b < 3; ++b)
-        vec[(1 + b) * R + t] = b == a.cur0 ? me.bufs[b][r * me.B] : make_double2(0.0, 0.0);
+        vec[(1 + b) * R + t] = b == a.cur0 ? reinterpret_cast<const double2 *>(me.bufs[b])[r * me.B]
+                                           : make_double2(0.0, 0.0);
     cl.sync();
     // gathered entries' shared::cluster addresses in x buffer 0 (a buffer
     // is R rows further on), fixed for the launch; kNoEntry for padding
@@ -273,17 +274,211 @@ __global__ void __launch_bounds__(MAXT, 1) k_cluster_steps(ClusterArgs a)
         cl.sync();
         if (rank == 0 && t < 32) cluster_sum(sum_step);
     }
-    me.bufs[cur][r * me.B] = vec[(1 + cur) * R + t];
+    reinterpret_cast<double2 *>(me.bufs[cur])[r * me.B] = vec[(1 + cur) * R + t];
     cl.sync();                                           // no block leaves while others read it
+}
+
+// ---- FP32 ----------------------------------------------------------------------
+__device__ __forceinline__ float2 ld_cluster_f(uint32_t addr)
+{
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ FF ff_shfl(FF v, int o)
+{
+    return FF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+}
+// warp_sum3 of float pairs
+__device__ __forceinline__ FF warp_sum3(FF v0, FF v1, FF v2)
+{
+    const int l = threadIdx.x & 31;
+    const bool hi = l & 16, q = l & 8;
+    const FF zero = {0.f, 0.f};
+    FF a = ff_add(hi ? v1 : v0, ff_shfl(hi ? v0 : v1, 16));
+    const FF b = ff_add(hi ? zero : v2, ff_shfl(hi ? v2 : zero, 16));
+    a = ff_add(q ? b : a, ff_shfl(q ? a : b, 8));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) a = ff_add(a, ff_shfl(a, o));
+    return a;
+}
+
+// The FP32 form of the stepping: states and arithmetic those of the per-term
+// FP32 kernels (bit-identical), RPT rows a thread (rows t, t + T, ...), the
+// closing sums as float pairs up to the block and FP64 from there.  The
+// per-term kernels rescale a state whose norm has drifted before the next
+// step; here such a drift sets error bit 8 and the caller repeats the run
+// with them.  Bound by the latency of a term (barrier, distributed
+// shared-memory gathers): 64 x 64 graphene, one state, 10 us a step against
+// 42 us of dependent launches; 180 x 180 25 against 47 us.
+template <int MAXW, int RPT, Vals M>
+__global__ void __launch_bounds__(512, 1) k_cluster_steps_f32(ClusterArgs a)
+{
+    cg::cluster_group cl = cg::this_cluster();
+    const int K = (int)cl.num_blocks();
+    const int rank = (int)cl.block_rank();
+    const ClusterState me = a.states[blockIdx.x / K];
+    const int R = a.rows_per_cta, T = blockDim.x, t = threadIdx.x;
+    extern __shared__ __align__(16) unsigned char sm[];
+    float2 *vec = reinterpret_cast<float2 *>(sm);                    // [4][R]
+    float *sval = reinterpret_cast<float *>(vec + 4 * R);            // [W][R] (value per entry)
+    __shared__ double part[2][3];
+    __shared__ FF red[32][3];
+    __shared__ FusedTerm tab[3 * kClusterMaxTerms];
+    for (int i = t; i < 3 * a.J; i += T) tab[i] = a.terms[(i / a.J) * kMaxTerms + i % a.J];
+
+    uint32_t gsrc[RPT][MAXW];
+    float d[RPT];
+    int w[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+        const int row = t + i * T;
+        w[i] = 0;
+        d[i] = 0.f;
+#pragma unroll
+        for (int k = 0; k < MAXW; ++k) gsrc[i][k] = kNoEntry;
+        if (row >= R) continue;
+        const int64_t r = (int64_t)rank * R + row;
+        const int64_t q = r / kSliceRows;
+        int64_t base;
+        if (MAXW == 3) {
+            w[i] = 3;
+            base = q * (3 * kSliceRows) + r % kSliceRows;
+        } else {
+            base = a.slice_ptr[q] + r % kSliceRows;
+            w[i] = (int)((a.slice_ptr[q + 1] - a.slice_ptr[q]) / kSliceRows);
+        }
+        d[i] = a.diag32[r];
+#pragma unroll
+        for (int k = 0; k < MAXW; ++k)
+            if (k < w[i]) {
+                const int32_t c = a.col[base + (int64_t)k * kSliceRows];
+                // one value: padding (own row) adds nothing; else its value is zero
+                if (M != kOne || c != (int32_t)r) gsrc[i][k] = cluster_addr(vec + c % R, c / R);
+                if (M != kOne) sval[k * R + row] = a.val32[base + (int64_t)k * kSliceRows];
+            }
+        vec[row] = reinterpret_cast<const float2 *>(me.psi0)[r * me.B];
+        for (int b = 0; b < 3; ++b)
+            vec[(1 + b) * R + row] = b == a.cur0 ? reinterpret_cast<const float2 *>(me.bufs[b])[r * me.B]
+                                                 : make_float2(0.f, 0.f);
+    }
+    cl.sync();
+
+    int cur = a.cur0;
+    bool pending = false;
+    int sum_step = 0, sum_waits = 0;         // as in the FP64 kernel
+    auto cluster_sum = [&](int m) {
+        double w0 = 0.0, w1 = 0.0, w2 = 0.0;
+        if (t < K) {
+            const double *pk = cl.map_shared_rank(&part[m & 1][0], t);
+            w0 = pk[0];
+            w1 = pk[1];
+            w2 = pk[2];
+        }
+        const double v = warp_sum3(w0, w1, w2);
+        const double sm1 = __shfl_sync(0xffffffffu, v, sum3_lane(1));
+        const double sm2 = __shfl_sync(0xffffffffu, v, sum3_lane(2));
+        if (t == 0) {
+            me.corr[m] = make_double2(v, sm1);
+            me.norms[m] = sm2;
+            const double ref = *me.norm_ref;
+            const double drift = ref > 0.0 ? fabs(sm2 / ref - 1.0) : sm2;
+            if (!(sm2 == sm2) || !(v == v) || !(sm1 == sm1) || sm2 - sm2 != 0.0) atomicOr(a.err, 2);
+            else if (drift > a.hard_bound) atomicOr(a.err, 1);
+            if (drift > a.renorm_bound) atomicOr(a.err, 8);
+        }
+    };
+    for (int n = 1; n <= a.n_steps; ++n) {
+        const FusedTerm *tt = tab + cur * a.J;
+        for (int j = 0; j < a.J; ++j) {
+            const FusedTerm tm = tt[j];
+            const int xoff = (1 + (tm.x < 0 ? cur : tm.x)) * R;
+            const uint32_t xoff_b = (uint32_t)xoff * (uint32_t)sizeof(float2);
+            float2 p[RPT], zz[RPT];          // own rows: written only by this thread
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) {
+                const int row = min(t + i * T, R - 1);
+                p[i] = vec[(1 + cur) * R + row];
+                zz[i] = tm.z >= 0 ? vec[(1 + tm.z) * R + row] : make_float2(0.f, 0.f);
+            }
+            if (pending) cl.barrier_wait();  // the gathered vector is complete
+            pending = false;
+            if (sum_waits > 0 && --sum_waits == 0 && rank == 0 && t < 32) cluster_sum(sum_step);
+            FF v0 = {0.f, 0.f}, v1 = v0, v2 = v0;
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) {
+                const int row = min(t + i * T, R - 1);
+                const bool in = t + i * T < R;
+                float2 x[MAXW];
+#pragma unroll
+                for (int k = 0; k < MAXW; ++k)
+                    if (gsrc[i][k] != kNoEntry) x[k] = ld_cluster_f(gsrc[i][k] + xoff_b);
+                float2 y = vec[xoff + row];
+                y.x *= d[i];
+                y.y *= d[i];
+#pragma unroll
+                for (int k = 0; k < MAXW; ++k)
+                    if (gsrc[i][k] != kNoEntry) {
+                        const float h = M == kOne ? a.h_uniform_f : sval[k * R + row];
+                        y.x = fmaf(h, x[k].x, y.x);
+                        y.y = fmaf(h, x[k].y, y.y);
+                    }
+                float2 o;
+                o.x = fmaf(tm.c_hi_f, p[i].x, fmaf(tm.c_lo_f, p[i].x, fmaf(tm.gamma_f, y.y, zz[i].x)));
+                o.y = fmaf(tm.c_hi_f, p[i].y, fmaf(tm.c_lo_f, p[i].y, fmaf(-tm.gamma_f, y.x, zz[i].y)));
+                if (in) vec[(1 + tm.out) * R + row] = o;
+                if (tm.final_term && in) {
+                    const float2 p0 = vec[row];
+                    FF re, im, nr;
+                    ff_dot3(p0.x, p0.y, o.x, o.y, re, im, nr);
+                    v0 = ff_add(v0, re);
+                    v1 = ff_add(v1, im);
+                    v2 = ff_add(v2, nr);
+                }
+            }
+            cl.barrier_arrive();             // release this term's writes
+            pending = true;
+            if (tm.final_term) {             // the sums, while the other blocks arrive
+                const int lane = t % 32;
+                const FF v = warp_sum3(v0, v1, v2);
+                if (lane % 8 == 0 && lane < 24) red[t / 32][lane == 0 ? 0 : lane == 16 ? 1 : 2] = v;
+                __syncthreads();
+                if (t < 32) {
+                    const FF zero = {0.f, 0.f};
+                    const bool has = t < (T + 31) / 32;
+                    const FF u = warp_sum3(has ? red[t][0] : zero, has ? red[t][1] : zero,
+                                           has ? red[t][2] : zero);
+                    if (t % 8 == 0 && t < 24)
+                        part[n & 1][t == 0 ? 0 : t == 16 ? 1 : 2] = ff_to_double(u);
+                }
+                sum_step = n;
+                sum_waits = 2;
+            }
+        }
+        cur = a.next_cur[cur];
+    }
+    if (pending) {
+        cl.barrier_wait();
+        if (sum_waits > 0) --sum_waits;
+    }
+    if (sum_waits > 0) {
+        cl.sync();
+        if (rank == 0 && t < 32) cluster_sum(sum_step);
+    }
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+        if (t + i * T < R)
+            reinterpret_cast<float2 *>(me.bufs[cur])[((int64_t)rank * R + t + i * T) * me.B] =
+                vec[(1 + cur) * R + t + i * T];
+    cl.sync();                               // no block leaves while others read it
 }
 
 }  // namespace
 
-int cluster_blocks_for(int64_t n_rows, int max_w, int uniform)
+namespace {
+// 16-block clusters (non-portable size) run on this device
+bool cluster16()
 {
-    if (n_rows <= 0 || n_rows > 16 * 1024 || max_w > kClusterMaxW) return 0;
-    // 16 blocks (non-portable size) where the device runs such a cluster:
-    // GB300's FP64 rate per SM makes more SMs pay; else 8
     static int best16 = -1;
     if (best16 < 0) {
         best16 = 0;
@@ -310,25 +505,33 @@ int cluster_blocks_for(int64_t n_rows, int max_w, int uniform)
         }
         cudaGetLastError();
     }
+    return best16 != 0;
+}
+}  // namespace
+
+int cluster_blocks_for(int64_t n_rows, int max_w, int uniform, int fp32, int fixed_width)
+{
+    const int rpt = fp32 && fixed_width == 3 ? 4 : 1;        // rows a thread at most
+    if (n_rows <= 0 || n_rows > 16 * 1024 * rpt || max_w > kClusterMaxW) return 0;
     auto fits = [&](int K) {
-        if (n_rows % K || n_rows / K > 1024) return false;
+        if (n_rows % K || n_rows / K > 1024 * rpt) return false;
         const int64_t R = n_rows / K;
-        const int64_t smem = 4 * R * 16 + (int64_t)std::max(1, max_w) * R * (uniform ? 4 : 12);
+        const int64_t smem = fp32 ? 4 * R * 8 + (int64_t)std::max(1, max_w) * R * (uniform ? 0 : 4)
+                                  : 4 * R * 16 + (int64_t)std::max(1, max_w) * R * (uniform ? 4 : 12);
         return smem <= 200 * 1024;
     };
-    if (best16 && fits(16)) return 16;
+    // GB300's FP64 rate per SM makes more SMs pay; else 8
+    if (cluster16() && fits(16)) return 16;
     return fits(8) ? 8 : 0;
 }
 
-template <int MAXW, int MAXT, Vals M>
-cudaError_t launch_cluster_t(const ClusterArgs &a, int K, size_t smem, cudaStream_t st)
+cudaError_t launch_cluster(void (*k)(ClusterArgs), const ClusterArgs &a, int K, int threads,
+                           size_t smem, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_cluster_steps<MAXW, MAXT, M>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (K > 8) {
-        e = cudaFuncSetAttribute(k_cluster_steps<MAXW, MAXT, M>,
-                                 cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
@@ -338,12 +541,28 @@ cudaError_t launch_cluster_t(const ClusterArgs &a, int K, size_t smem, cudaStrea
     at.val.clusterDim.y = 1;
     at.val.clusterDim.z = 1;
     cfg.gridDim = dim3(K * a.n_states);
-    cfg.blockDim = dim3(a.rows_per_cta);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_cluster_steps<MAXW, MAXT, M>, a);
+    return cudaLaunchKernelEx(&cfg, k, a);
+}
+
+template <int MAXW, int MAXT, Vals M>
+cudaError_t launch_cluster_t(const ClusterArgs &a, int K, size_t smem, cudaStream_t st)
+{
+    return launch_cluster(k_cluster_steps<MAXW, MAXT, M>, a, K, a.rows_per_cta, smem, st);
+}
+
+template <int MAXW, int RPT>
+cudaError_t launch_cluster_f(const ClusterArgs &a, int K, cudaStream_t st)
+{
+    const int R = a.rows_per_cta, threads = ((R + RPT - 1) / RPT + 31) / 32 * 32;
+    const size_t smem = (size_t)4 * R * sizeof(float2) +
+                        (a.uniform ? 0 : (size_t)a.max_w * R * sizeof(float));
+    return a.uniform ? launch_cluster(k_cluster_steps_f32<MAXW, RPT, kOne>, a, K, threads, smem, st)
+                     : launch_cluster(k_cluster_steps_f32<MAXW, RPT, kReal>, a, K, threads, smem, st);
 }
 
 template <int MAXW, int MAXT>
@@ -361,9 +580,19 @@ cudaError_t launch_cluster_w(const ClusterArgs &a, int K, size_t smem, cudaStrea
                         : launch_cluster_m<kClusterMaxW, MAXT>(a, K, smem, st);
 }
 
-cudaError_t launch_cluster_steps(const ClusterArgs &a, int K, cudaStream_t st)
+cudaError_t launch_cluster_steps(const ClusterArgs &a, int fp32, int K, cudaStream_t st)
 {
     const int R = a.rows_per_cta;
+    if (fp32) {
+        // at most 512 threads, 128 registers each, several rows a thread
+        if (a.fixed_width != 3)
+            return R <= 512 ? launch_cluster_f<kClusterMaxW, 1>(a, K, st)
+                            : launch_cluster_f<kClusterMaxW, 2>(a, K, st);
+        return R <= 512    ? launch_cluster_f<3, 1>(a, K, st)
+               : R <= 1024 ? launch_cluster_f<3, 2>(a, K, st)
+               : R <= 2048 ? launch_cluster_f<3, 4>(a, K, st)
+                           : launch_cluster_f<3, 8>(a, K, st);
+    }
     const size_t smem = (size_t)4 * R * sizeof(double2) + (size_t)a.max_w * R * sizeof(int32_t) +
                         (a.uniform ? 0 : (size_t)a.max_w * R * sizeof(double));
     // up to 512 rows per block: 128 registers a thread, else 64

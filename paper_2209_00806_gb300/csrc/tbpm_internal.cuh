@@ -464,14 +464,16 @@ struct FusedArgs {
 
 cudaError_t launch_step_fused(const FusedArgs &f, int fp32, int B, int num_sms, cudaStream_t st);
 
-// Cluster-resident time stepping (cluster_kernels.cu): all steps of the FP64
-// states of a sample of up to 16 x 1024 rows in one launch, a cluster a state.
+// Cluster-resident time stepping (cluster_kernels.cu): all steps of the states
+// of a sample of up to 16 x 1024 rows (FP32 with three slots a row: 16 x 4096)
+// in one launch, a cluster a state.
 constexpr int kClusterMaxW = 12;           // entries per row it takes
+constexpr int kClusterStates = 7;          // 16-block clusters that run at once
 constexpr int kClusterMaxTerms = 40;       // Chebyshev terms per step it takes (z <= ~25)
 // One state: row r of its vectors is element r * B of each pointer.
 struct ClusterState {
-    const double2 *psi0;
-    double2 *bufs[3];
+    const void *psi0;
+    void *bufs[3];
     double2 *corr;              // C_n, n = 0 .. n_steps
     double *norms;
     const double *norm_ref;
@@ -485,6 +487,8 @@ struct ClusterArgs {
     int fixed_width, uniform, max_w, rows_per_cta;
     int zero_diag;              // every onsite energy is zero
     double h_uniform;
+    float h_uniform_f;          // FP32 form: value, values and diagonal
+    const float *val32, *diag32;
     const ClusterState *states;
     int n_states;
     int cur0;
@@ -493,12 +497,13 @@ struct ClusterArgs {
     int next_cur[3];
     int n_steps;
     double hard_bound;
+    double renorm_bound;        // FP32: a drift above it sets error bit 8
     int *err;
 };
 // Blocks of the cluster for n_rows rows (16 where the device runs such a
 // cluster, else 8), or 0 when the sample does not fit.
-int cluster_blocks_for(int64_t n_rows, int max_w, int uniform);
-cudaError_t launch_cluster_steps(const ClusterArgs &a, int K, cudaStream_t st);
+int cluster_blocks_for(int64_t n_rows, int max_w, int uniform, int fp32, int fixed_width);
+cudaError_t launch_cluster_steps(const ClusterArgs &a, int fp32, int K, cudaStream_t st);
 int fused_tile_rows(int fp32, int B, int log4_mult);
 int fused_grid(int fp32, int B, int num_sms);
 

@@ -204,6 +204,56 @@ def test_cluster_states_are_bit_identical(S, onsite_w, sigma, sides):
             assert np.abs(a - b).max() < 1e-13
 
 
+# FP32 cluster stepping against the per-term kernels: one to eight rows a
+# thread and their edges, one value and values per entry, ragged rows; and
+# the repeat by the per-term kernels when the norm carry has to act, from a
+# fresh start and a resumed one
+def _f32(tb, smp, theta, variant, norm=None):
+    from paper_2209_00806_gb300 import _native as N
+    with tb.Propagator() as p:
+        if variant is not None:
+            p.launch_config(tb.TBPM_FP32, 16, 64, variant)
+        p.build_sample(smp, 9.5)
+        p.set_phase_states(theta)
+        C = p.propagate(Z, 6, tb.TBPM_FP32)
+        if norm:
+            N.tbpm_set_norm_policy(p.ctx, norm)
+        D = p.propagate(Z, 5, tb.TBPM_FP32, flags=N.TBPM_PROP_RESUME)
+        st = p.stats()["renormalisations"]
+        if norm:
+            p.set_phase_states(theta)
+            p.propagate(Z, 5, tb.TBPM_FP32)
+            st += p.stats()["renormalisations"]
+        return C, D, p.states(), p.norms(), st
+
+
+@pytest.mark.parametrize("S", [1, 3, 9])
+@pytest.mark.parametrize("kind", [(9, 11), (64, 64), (64, 65), (90, 91), (91, 180), (128, 128),
+                                  (128, 129), (180, 182), "ragged"])
+def test_fp32_cluster_is_bit_identical(S, kind):
+    import paper_2209_00806_gb300 as tb
+    if kind == "ragged":
+        smp = lattice.random_graph(9000, 13000, seed=9, onsite_w=1.0, t_scale=0.8)
+    else:
+        smp = lattice.graphene(*kind, pbc=kind[0] != 90, seed=6, onsite_w=1.0,
+                               bond_sigma=0.05 if kind[0] in (91, 180) else 0.0, vacancy_frac=0.004)
+    theta = rng.phases(14, S, smp.n_orb)
+    out = [_f32(tb, smp, theta, v) for v in (1, 2049, None)]
+    for o in out[1:]:
+        assert np.array_equal(out[0][2], o[2])
+        for a, b in zip(out[0][:2] + out[0][3:4], o[:2] + o[3:4]):
+            assert np.abs(a - b).max() < 1e-12
+
+
+@pytest.mark.parametrize("S", [1, 4])
+def test_fp32_cluster_repeats_for_the_norm_carry(S):
+    import paper_2209_00806_gb300 as tb
+    smp = lattice.graphene(20, 31, pbc=True, seed=6, onsite_w=1.0)
+    theta = rng.phases(15, S, smp.n_orb)
+    # 8257: the default's launch shape set by hand, per-term kernels with the same sums
+    a, b = (_f32(tb, smp, theta, v, norm=1e-12) for v in (8257, None))
+    assert a[4] > 0 and a[4] == b[4]
+    assert np.array_equal(a[2], b[2]) and np.array_equal(a[1], b[1])
 # buffers kept between calls: new states of the same number after a run (one of
 # them not finite), of another number, in both precisions, C over and under
 # the size of the page-locked result buffer (64 KB)
