@@ -297,7 +297,9 @@ int tbpm_dos(const double *corr, int n_steps, double tau, int window, double e_m
  *              `where`): dL/dRe C_n + i dL/dIm C_n of each state's C_n, as
  *              tbpm_propagate defines C_n for the states currently set
  *   K          checkpoint interval (states kept every K steps, recomputed
- *              in between; memory ~ (N/K + K + M) state vectors)
+ *              in between; memory ~ (N/K + K + M) state vectors,
+ *              and K (M - 2) more where they fit 24 GB: the
+ *              polynomials of a segment, kept)
  *   grad_hop   double [n_hop] dL/dt_b, bonds in the order given to
  *              tbpm_build_hamiltonian (host or device, `where_out`)
  *   grad_onsite double [n_orb] dL/deps_i

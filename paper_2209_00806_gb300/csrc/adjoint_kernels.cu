@@ -38,7 +38,9 @@ namespace {
 // four and one thread per state (whose partial gradients had to be added by
 // shuffles).  524,288 rows x 2 states: 68 -> 43 us a gradient term, 36 -> 20 us
 // a plain one.
-template <int L, int SPL, int W, bool HASC, bool FAC, bool GRAD, bool WFAC>
+// ACC (polynomials): the term's share of the next state too, next += ca out
+// (2: the first polynomial, next = c x + ca out); out may then be nullptr.
+template <int L, int SPL, int W, bool HASC, bool FAC, bool GRAD, bool WFAC, int ACC = 0>
 __global__ void __launch_bounds__(128) k_adj(AdjArgs a)
 {
     constexpr int NS = W ? W : 4;
@@ -82,6 +84,10 @@ __global__ void __launch_bounds__(128) k_adj(AdjArgs a)
         if (!FAC && a.z) o[j] = reinterpret_cast<const double2 *>(a.z)[at(r) + j];
     }
     double2 p[SPL];
+    double2 nx[SPL];
+    if (ACC == 1)
+#pragma unroll
+        for (int j = 0; j < SPL; ++j) nx[j] = reinterpret_cast<const double2 *>(a.next)[at(r) + j];
     if (HASC)
 #pragma unroll
         for (int j = 0; j < SPL; ++j) p[j] = reinterpret_cast<const double2 *>(a.psi)[at(r) + j];
@@ -161,6 +167,16 @@ __global__ void __launch_bounds__(128) k_adj(AdjArgs a)
             o[j].y += g.x * p0.y + g.y * p0.x;
         }
     }
+    if (ACC) {
+#pragma unroll
+        for (int j = 0; j < SPL; ++j) {
+            if (ACC == 2) nx[j] = make_double2(a.c * xr[j].x, a.c * xr[j].y);
+            nx[j].x = fma(a.ca, o[j].x, nx[j].x);
+            nx[j].y = fma(a.ca, o[j].y, nx[j].y);
+            reinterpret_cast<double2 *>(a.next)[at(r) + j] = nx[j];
+        }
+        if (!out) return;
+    }
 #pragma unroll
     for (int j = 0; j < SPL; ++j) out[at(r) + j] = o[j];
 }
@@ -228,6 +244,8 @@ cudaError_t launch_adj_w(const AdjArgs &a, AdjKind kind, cudaStream_t st)
     auto go = [&](void (*k)(AdjArgs)) { return launch_dependent(k, blocks, 128, 0, st, a); };
     switch (kind) {
     case kAdjPoly: return go(k_adj<L, SPL, W, false, false, false, false>);
+    case kAdjPolyAcc: return go(k_adj<L, SPL, W, false, false, false, false, 1>);
+    case kAdjPolyFirst: return go(k_adj<L, SPL, W, false, false, false, false, 2>);
     case kAdjStep: return go(k_adj<L, SPL, W, true, false, false, false>);
     case kAdjStepFirst: return go(k_adj<L, SPL, W, true, true, false, false>);
     case kAdjGrad: return go(k_adj<L, SPL, W, true, false, true, false>);

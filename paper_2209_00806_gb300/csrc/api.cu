@@ -1802,10 +1802,12 @@ extern "C" int tbpm_propagate_adjoint(tbpm_ctx *c, double z, int n_steps, const 
     std::vector<void *> ckpt(nseg, nullptr), traj(K, nullptr), stash(M - 1, nullptr);
     double *G = nullptr, *Gd = nullptr, *d_gh = nullptr, *d_go = nullptr;
     double *val2 = nullptr, *diag2 = nullptr;        // 2 H~ (interior terms)
+    char *polys = nullptr;                           // [K][M - 2] polynomials of a segment
     const int64_t nnz = c->H.nnz_pad;
     auto release = [&]() {
         cudaFree(val2);
         cudaFree(diag2);
+        cudaFree(polys);
         for (void *p : ckpt) cudaFree(p);
         for (void *p : traj) cudaFree(p);
         for (void *p : stash) cudaFree(p);
@@ -1816,7 +1818,17 @@ extern "C" int tbpm_propagate_adjoint(tbpm_ctx *c, double z, int n_steps, const 
     };
     for (auto &p : ckpt) if (!rc) rc = dalloc(c, (char **)&p, vec);
     for (size_t k = 1; k < traj.size() && !rc; ++k) rc = dalloc(c, (char **)&traj[k], vec);
-    for (auto &p : stash) if (!rc) rc = dalloc(c, (char **)&p, vec);
+    // the polynomials of a whole segment where they fit: the segment's states
+    // then come out of the same products (a share of the next state per term,
+    // 10 FP64 operations a term and row) instead of a Clenshaw step of their own
+    // (10 more); one allocation, and without it the recomputing form
+    const size_t keep_bytes = (size_t)K * (M - 2) * vec;
+    if (!rc && M > 2 && keep_bytes <= kAdjKeepBytes && cudaMalloc((void **)&polys, keep_bytes) != cudaSuccess) {
+        polys = nullptr;
+        cudaGetLastError();
+    }
+    if (!polys)
+        for (auto &p : stash) if (!rc) rc = dalloc(c, (char **)&p, vec);
     if (!rc) rc = dalloc(c, &G, (size_t)std::max<int64_t>(nnz, 1));
     if (!rc) rc = dalloc(c, &Gd, (size_t)c->H.n_rows);
     if (!rc) rc = dalloc(c, &val2, (size_t)std::max<int64_t>(nnz, 1));
@@ -1873,14 +1885,6 @@ extern "C" int tbpm_propagate_adjoint(tbpm_ctx *c, double z, int n_steps, const 
             ++launches;
             return launch_adj(t, kind, B, c->st);
         };
-        // T^_m from T^_{m-1} and T^_{m-2} (m = 1: from T^_0 alone)
-        auto poly = [&](int m, const void *x, const void *zz, void *out) -> cudaError_t {
-            AdjArgs t = with_h(m > 1);
-            t.x = x;
-            t.z = zz;
-            t.out = out;
-            return run(t, kAdjPoly);
-        };
         // one forward Clenshaw step src -> dst (tmp: scratch)
         auto step_into = [&](void *src, void *dst, void *tmp) -> cudaError_t {
             void *bufs[3];
@@ -1924,17 +1928,39 @@ extern "C" int tbpm_propagate_adjoint(tbpm_ctx *c, double z, int n_steps, const 
             const int n0 = seg * K, n1 = std::min(n_steps, n0 + K);
             std::vector<void *> tp(n1 - n0);
             tp[0] = ckpt[seg];
-            for (int k = 1; k < n1 - n0; ++k) {
-                tp[k] = traj[k];
-                if ((e = step_into(tp[k - 1], tp[k], stash[0])) != cudaSuccess)
-                    return cuda_fail("adjoint forward kernel", e);
+            // T^_m of the segment's step k (m = 1 .. M - 2; T^_0 is its state)
+            auto T = [&](int k, int m) -> void * {
+                if (m == 0) return tp[k];
+                return polys ? (void *)(polys + ((size_t)k * (M - 2) + m - 1) * vec) : stash[m];
+            };
+            for (int k = 0; k < n1 - n0; ++k) {
+                const bool more = k + 1 < n1 - n0;
+                if (more) tp[k + 1] = traj[k + 1];
+                if (!polys) {
+                    if (more && (e = step_into(tp[k], tp[k + 1], stash[0])) != cudaSuccess)
+                        return cuda_fail("adjoint forward kernel", e);
+                    continue;
+                }
+                for (int m = 1; m <= (more ? M - 1 : M - 2); ++m) {
+                    AdjArgs t = with_h(m > 1);
+                    t.x = T(k, m - 1);
+                    t.z = m == 1 ? nullptr : T(k, m - 2);
+                    t.out = m <= M - 2 ? T(k, m) : nullptr;
+                    t.c = a[0];
+                    t.ca = a[m];
+                    t.next = more ? tp[k + 1] : nullptr;
+                    e = run(t, !more ? kAdjPoly : m == 1 ? kAdjPolyFirst : kAdjPolyAcc);
+                    if (e != cudaSuccess) return cuda_fail("adjoint polynomial kernel", e);
+                }
             }
             for (int n = n1 - 1; n >= n0; --n) {
-                void *phi = tp[n - n0];
-                for (int m = 1; m <= M - 2; ++m) {
-                    e = poly(m, m == 1 ? phi : stash[m - 1],
-                             m == 1 ? nullptr : m == 2 ? phi : stash[m - 2], stash[m]);
-                    if (e != cudaSuccess) return cuda_fail("adjoint polynomial kernel", e);
+                for (int m = 1; !polys && m <= M - 2; ++m) {
+                    AdjArgs t = with_h(m > 1);
+                    t.x = T(n - n0, m - 1);
+                    t.z = m == 1 ? nullptr : T(n - n0, m - 2);
+                    t.out = T(n - n0, m);
+                    if ((e = run(t, kAdjPoly)) != cudaSuccess)
+                        return cuda_fail("adjoint polynomial kernel", e);
                 }
                 int nx = 0;
                 std::vector<Launch> sch = schedule(a, lc, &nx);
@@ -1948,7 +1974,7 @@ extern "C" int tbpm_propagate_adjoint(tbpm_ctx *c, double z, int n_steps, const 
                     t.psi = g.buf[lc];
                     t.z = L.z < 0 ? nullptr : g.buf[L.z];
                     t.out = g.buf[L.out];
-                    t.T_own = m == 0 ? phi : stash[m];
+                    t.T_own = T(n - n0, m);
                     t.c = L.c;
                     t.fac = L.gamma;
                     t.gfac = 0.5 * L.gamma;              // G is half the sum

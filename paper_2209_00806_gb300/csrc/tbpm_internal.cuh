@@ -353,10 +353,15 @@ cudaError_t launch_bond_vectors(int64_t n_hop, const int32_t *bond_rows, const i
                                 const int32_t *col, const double *dx, const double *dy,
                                 int *claim, double *dxe, double *dye, int *err, cudaStream_t st);
 
+// A segment's polynomials are kept up to this many bytes (else recomputed
+// per step): 3.8 GB for 512 x 512 graphene, checkpoints of 16 steps, two states.
+constexpr size_t kAdjKeepBytes = (size_t)24 << 30;
 // One term of the adjoint's forward or backward series, FP64, with the matrix
 // values already scaled by |gamma| (adjoint_kernels.cu).
 enum AdjKind {
     kAdjPoly,       // z + (-i) H' x: the plain polynomials
+    kAdjPolyAcc,    // the same, and next += ca out
+    kAdjPolyFirst,  // the first one, and next = c x + ca out
     kAdjStep,       // c psi + z + (-i) H' x: a forward Clenshaw term
     kAdjStepFirst,  // c psi + fac (-i) H' psi: its first term
     kAdjGrad,       // c psi + z + i H' x with gradient accumulation
@@ -372,6 +377,8 @@ struct AdjArgs {
     const void *x, *psi, *z, *T_own;
     void *out;
     double c, fac, gfac;
+    void *next;            // kAdjPolyAcc, kAdjPolyFirst: the next state, its share ca
+    double ca;
     double *G, *Gdiag;
     const double2 *gbar;   // [n_samples][n_states][n_steps + 1] or nullptr
     const void *psi0;

@@ -280,3 +280,18 @@ def test_states_set_again_start_afresh():
             got = (p.propagate(Z, steps, precision), p.states(), p.norms())
             for a, b in zip(got, fresh(t, steps, precision)):
                 assert np.array_equal(a, b)
+
+
+# a segment's polynomials kept (50 steps, 11.7 GB) and recomputed per step (above
+# 24 GB): the same gradients to the rounding of another summation order
+def test_adjoint_segments_kept_and_recomputed():
+    import paper_2209_00806_gb300 as tb
+    smp = lattice.graphene(512, 512, pbc=True, seed=2, onsite_w=0.4, bond_sigma=0.05)
+    theta = rng.phases(4, 2, smp.n_orb)
+    g = np.random.default_rng(5).normal(size=(1, 2, 121, 2)) @ np.array([1, 1j])
+    with tb.Propagator() as p:
+        p.build_sample(smp, 9.5)
+        p.set_phase_states(theta)
+        (ah, ao), (bh, bo) = (p.adjoint(Z, 120, g, K) for K in (50, 120))
+    scale = max(np.abs(ah).max(), np.abs(ao).max())
+    assert np.abs(ah - bh).max() < 1e-11 * scale and np.abs(ao - bo).max() < 1e-11 * scale
