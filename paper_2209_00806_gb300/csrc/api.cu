@@ -56,7 +56,7 @@ struct tbpm_ctx {
     double2 *d_psi_user = nullptr;
     size_t psi_count = 0;        // elements it holds
     cudaEvent_t ev_order = nullptr;        // orders our stream and the user's
-    unsigned char *h_res = nullptr;        // page-locked, kResBytes: small results
+    unsigned char *h_res = nullptr;        // page-locked, kResBytes: small results (first run)
 
     // propagation state
     int prec = -1;               // precision of the group buffers
@@ -389,7 +389,6 @@ extern "C" int tbpm_create(tbpm_ctx **out, int device, void *stream)
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_order, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&c->d_flags, kFlagBytes);       // flags, renorm count
     if (e == cudaSuccess) c->d_renorm = (unsigned long long *)(c->d_flags + 4);
-    if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->h_res, kResBytes, cudaHostAllocDefault);
     if (e != cudaSuccess) {
         std::string m = std::string("context setup: ") + cudaGetErrorString(e);
         tbpm_destroy(c);
@@ -970,6 +969,8 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
 
     int rc = enter(c);
     if (rc) return rc;
+    if (!c->h_res)
+        CUDA_OR_FAIL(c, cudaHostAlloc((void **)&c->h_res, kResBytes, cudaHostAllocDefault));
     rc = ensure_groups(c, precision);
     if (rc) return rc;
     if (c->corr_steps != n_steps) {
@@ -1010,7 +1011,8 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     const bool long_rows = fp32 && (variant & kVariantPrefetch) && !c->H.cplx && !c->H.uniform &&
                            !(variant & (kVariantHalo | kVariantTma | kVariantFused | kVariantSplit2 |
                                         kVariantSplit4)) &&
-                           c->H.nnz_true >= kLongRow * c->n_orb && n_steps >= 2;
+                           c->H.nnz_true >= kLongRow * c->n_orb && n_steps >= 2 &&
+                           (c->H.halo_ptr || fits_beside(10 * (size_t)c->H.nnz_true));
     if (long_rows) variant = (variant & ~kVariantPrefetch) | kVariantHalo | kVariantStaged;
     bool halo = (variant & kVariantHalo) && !c->H.cplx && !(variant & (kVariantTma | kVariantFused));
     if (halo && !c->H.halo_ptr) {
@@ -1818,17 +1820,6 @@ extern "C" int tbpm_propagate_adjoint(tbpm_ctx *c, double z, int n_steps, const 
     };
     for (auto &p : ckpt) if (!rc) rc = dalloc(c, (char **)&p, vec);
     for (size_t k = 1; k < traj.size() && !rc; ++k) rc = dalloc(c, (char **)&traj[k], vec);
-    // the polynomials of a whole segment where they fit: the segment's states
-    // then come out of the same products (a share of the next state per term,
-    // 10 FP64 operations a term and row) instead of a Clenshaw step of their own
-    // (10 more); one allocation, and without it the recomputing form
-    const size_t keep_bytes = (size_t)K * (M - 2) * vec;
-    if (!rc && M > 2 && keep_bytes <= kAdjKeepBytes && cudaMalloc((void **)&polys, keep_bytes) != cudaSuccess) {
-        polys = nullptr;
-        cudaGetLastError();
-    }
-    if (!polys)
-        for (auto &p : stash) if (!rc) rc = dalloc(c, (char **)&p, vec);
     if (!rc) rc = dalloc(c, &G, (size_t)std::max<int64_t>(nnz, 1));
     if (!rc) rc = dalloc(c, &Gd, (size_t)c->H.n_rows);
     if (!rc) rc = dalloc(c, &val2, (size_t)std::max<int64_t>(nnz, 1));
@@ -1840,6 +1831,17 @@ extern "C" int tbpm_propagate_adjoint(tbpm_ctx *c, double z, int n_steps, const 
         d_gh = grad_hop;
         d_go = grad_onsite;
     }
+    // last, the polynomials of a whole segment where they fit: the segment's states
+    // then come out of the same products (a share of the next state per term,
+    // 10 FP64 operations a term and row) instead of a Clenshaw step of their own
+    // (10 more); one allocation, and without it the recomputing form
+    const size_t keep_bytes = (size_t)K * (M - 2) * vec;
+    if (!rc && M > 2 && keep_bytes <= kAdjKeepBytes && cudaMalloc((void **)&polys, keep_bytes) != cudaSuccess) {
+        polys = nullptr;
+        cudaGetLastError();
+    }
+    if (!polys)
+        for (auto &p : stash) if (!rc) rc = dalloc(c, (char **)&p, vec);
     if (rc) { release(); return rc; }
     auto cuda_fail = [&](const char *what, cudaError_t e) {
         release();

@@ -707,6 +707,12 @@ __global__ void __launch_bounds__(32) k_group_fill(const int64_t *slice_ptr, con
 
 }  // namespace
 
+bool fits_beside(size_t bytes)
+{
+    size_t free_b = 0, total_b = 0;
+    return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= free_b / 2;
+}
+
 int build_groups(BuildOutput &b, cudaStream_t st, std::string &msg)
 {
     if (b.gptr || b.no_groups) return TBPM_OK;
@@ -737,8 +743,10 @@ int build_groups(BuildOutput &b, cudaStream_t st, std::string &msg)
         e = cudaMemcpyAsync(&total, ptr + no, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
-    // no groups where the zeros would outweigh what the shared reads save
-    if (e == cudaSuccess && total * 32 > kGroupMaxFill * b.nnz_true) {
+    // no groups where the zeros would outweigh what the shared reads save, or
+    // where they would leave little memory for the caller's next states
+    if (e == cudaSuccess && (total * 32 > kGroupMaxFill * b.nnz_true ||
+                             !fits_beside((size_t)total * 8 * (sizeof(uint16_t) + sizeof(float4))))) {
         drop();
         b.no_groups = 1;
         return TBPM_OK;

@@ -589,6 +589,8 @@ struct BuildOutput {
 // 2 d for the FP64 one-value form's interior terms (gamma = +-2), exact.
 int build_diag2(BuildOutput &b, cudaStream_t st, std::string &msg);
 
+// An optional copy of `bytes` leaves at least as much device memory free.
+bool fits_beside(size_t bytes);
 // Row groups (FP32, real values) of the staged-gather kernel for long rows,
 // on the halo lists; leaves no_groups set where they do not pay or fit.
 int build_groups(BuildOutput &b, cudaStream_t st, std::string &msg);
