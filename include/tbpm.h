@@ -370,13 +370,12 @@ int tbpm_dos_adjoint(const double *dl_dd, int n_e, int n_steps, double tau, int 
                                         grid whose threads walk rows with a stride and
                                         load the next row's first four column indices,
                                         values and diagonal before the current row's
-                                        gathers; FP32: one row a thread up to 2^20
-                                        16-byte lanes, 32-byte lanes (with
-                                        TBPM_VARIANT_WIDE) for four states beyond
-                                        128 MB a vector, and the staged gathers
-                                        (HALO | STAGED) for rows of at least 32 values
-                                        on average; ignored otherwise.  All
-                                        bit-identical */
+                                        gathers; FP32: 16-byte lanes, one row a thread
+                                        up to 2^20 of them, blocks of 128 threads or
+                                        more beyond (TBPM_VARIANT_WIDE: the closing
+                                        pass's lanes), and the staged gathers (HALO |
+                                        STAGED) for rows of at least 32 values on
+                                        average; ignored otherwise.  All bit-identical */
 #define TBPM_VARIANT_STAGED 4096     /* with TBPM_VARIANT_HALO: one block per 128-row
                                         block copying its halo, positions and values
                                         into one shared-memory stage, two blocks per

@@ -702,10 +702,11 @@ __global__ void __launch_bounds__(256, sizeof(V) == 4 ? (SPL <= 2 ? 5 : 4) : (SP
 // diagonal are loaded one row ahead, so the row's own-row loads and its
 // gathers leave together instead of the gathers waiting on the column
 // loads.  One kernel per kind of values: with one value no value registers
-// are carried, and the 16-byte lanes fit 64 registers.  HBM-bound: 178 us at
-// 4 x 8.3M FP32 rows, 6.7 TB/s (188 us as ordinary launches).
+// are carried, and the 16-byte lanes fit 64 registers.  HBM-bound: 171 us at
+// 4 x 8.3M FP32 rows, 7.0 TB/s (188 us as ordinary launches with 32-byte lanes
+// and entries in rounds of four).
 template <typename V, int L, int SPL, Vals M, int W>
-__global__ void __launch_bounds__(256, sizeof(V) == 4 ? (SPL <= 2 ? 4 : 3) : 2) k_term_pf(TermArgs a)
+__global__ void __launch_bounds__(256, sizeof(V) == 4 ? 4 : 2) k_term_pf(TermArgs a)
 {
     dep_launch();
     // rows are below 2^31, a pass far below: positions fit 32 unsigned bits
@@ -1907,21 +1908,22 @@ cudaError_t launch_term_pf_t(const TermArgs &a, int threads, cudaStream_t st)
     return launch_term_pf_f<V, L, SPL, Form<kOne, 0>>(a, threads, st);
 }
 
-// The widths a TBPM_VARIANT_PREFETCH term runs at, all bit-identical.  FP32
-// interior terms on graphene, us, 16-byte lanes unless said otherwise:
-//   states x rows        one row a thread   persistent   persistent, 32-byte lanes
-//   4 x 131k (4 MB)            4.3              4.7             5.3
-//   4 x 524k (17 MB)          10.1             10.2            13.7
-//   8 x 295k (19 MB)          11.0             10.8            13.4
-//   4 x 2.1M (67 MB)          50               45.9            47.1
-//   4 x 8.3M (266 MB)        204              185             178
-//   16 x 2.1M (266 MB)       191              162             165
+// How a TBPM_VARIANT_PREFETCH term runs, all bit-identical.  FP32 interior terms
+// on graphene, us, 16-byte lanes:
+//   states x rows        one row a thread   persistent, blocks of 64   of 128   of 256
+//   4 x 131k (4 MB)            4.3              4.7
+//   4 x 524k (17 MB)          10.1             10.2
+//   8 x 295k (19 MB)          11.0             10.8
+//   4 x 2.1M (67 MB)          50               42.2                     41.7     42.7
+//   4 x 8.3M (266 MB)        204              173.8                    171.0    173.8
+//   16 x 2.1M (266 MB)       191              157.5                    155.9    163.4
 // Up to 2^20 lanes every row of the launch is resident at once or nearly:
-// the persistent loop has nothing to read ahead.  Beyond, reading ahead
-// pays, and once a vector of four states exceeds the L2 (129 MB) one
-// 32-byte lane a row halves the index loads of a kernel that HBM bounds.
+// the persistent loop has nothing to read ahead.  Beyond, reading ahead pays,
+// in blocks of 128 threads unless 256 are asked for.  (One 32-byte lane a row
+// for four states, 172.6 us at 8.3M rows, led while the three-slot rows had a
+// fourth gather.)  The closing pass keeps TBPM_VARIANT_WIDE's lanes: 107 us
+// with a whole row of four states a thread against 119 us.
 constexpr int64_t kPrefetchMinLanes = (int64_t)1 << 20;
-constexpr int64_t kWideMinBytes = (int64_t)128 << 20;
 
 cudaError_t dispatch_pf(const TermArgs &a, int fp32, int B, int threads, cudaStream_t st)
 {
@@ -1951,8 +1953,7 @@ cudaError_t dispatch_pf(const TermArgs &a, int fp32, int B, int threads, cudaStr
         }
         return cudaErrorInvalidValue;
     }
-    if ((a.variant & kVariantWide) && B == 4 && a.n_rows * 32 > kWideMinBytes)
-        return launch_term_pf_t<float, 1, 4>(a, threads, st);
+    threads = std::max(threads, 128);
     switch (B) {
     case 1: return launch_term_pf_t<float, 1, 1>(a, threads, st);
     case 2: return launch_term_pf_t<float, 1, 2>(a, threads, st);
