@@ -1006,20 +1006,36 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     // staged gathers instead where the lists can be had (twisted bilayer, 68
     // entries a row, 3.1M rows: 1.84 ms a term through L1, 0.81 ms staged,
     // less in groups; graphene's three entries hit L1 and lose, 0.27 against
-    // 0.19 ms).  From two steps on the lists' build
-    // (as much as about one step) pays within the call.
+    // 0.19 ms).  The lists are built once the steps run on this matrix pay for
+    // them (built on the first call, two steps of one state went from 10.5 to
+    // 15.3 ms on a 120 nm flake).  ms a step, plain against staged, and the build:
+    //   flake, states   plain  staged  build   meet at (states x steps)
+    //   12 nm, 8         0.27   0.18    1.2     110
+    //   30 nm, 8         0.40   0.26    1.7      97
+    //   30 nm, 4         0.30   0.27    1.7     230
+    //   60 nm, 8         1.75   0.92    3.6      35
+    //   60 nm, 4         0.9    0.71    3.7      78
+    //   120 nm, 8        6.5    3.2    11.8      29
+    //   120 nm, 4        3.7    2.4    11.8      36
+    //   120 nm, 1        2.3    1.65   11.8      18
+    // so from 32 beyond 2^17 rows (between 30 and 60 nm), from 128 below.
+    const int64_t pays = c->H.n_rows >= ((int64_t)1 << 17) ? 32 : 128;
+    if (fp32 && !c->H.halo_ptr) c->H.long_steps += (int64_t)n_steps * c->n_states;
     const bool long_rows = fp32 && (variant & kVariantPrefetch) && !c->H.cplx && !c->H.uniform &&
                            !(variant & (kVariantHalo | kVariantTma | kVariantFused | kVariantSplit2 |
                                         kVariantSplit4)) &&
-                           c->H.nnz_true >= kLongRow * c->n_orb && n_steps >= 2 &&
-                           (c->H.halo_ptr || fits_beside(10 * (size_t)c->H.nnz_true));
+                           c->H.nnz_true >= kLongRow * c->n_orb && !c->H.no_halo &&
+                           (c->H.halo_ptr || (c->H.long_steps >= pays &&
+                                              fits_beside(10 * (size_t)c->H.nnz_true)));
     if (long_rows) variant = (variant & ~kVariantPrefetch) | kVariantHalo | kVariantStaged;
     bool halo = (variant & kVariantHalo) && !c->H.cplx && !(variant & (kVariantTma | kVariantFused));
     if (halo && !c->H.halo_ptr) {
         std::string msg;
         rc = build_halo(c->H, c->st, msg);
-        if (rc == TBPM_E_UNSUPPORTED || (rc == TBPM_E_OOM && long_rows)) halo = false;
-        else if (rc) return fail(c, rc, msg);
+        if (rc == TBPM_E_UNSUPPORTED || (rc == TBPM_E_OOM && long_rows)) {
+            halo = false;
+            c->H.no_halo |= long_rows;      // the default does not try again
+        } else if (rc) return fail(c, rc, msg);
     }
     // one-stage staged gathers with FP32 values per entry: rows in groups of four
     if (halo && fp32 && (variant & kVariantStaged) && !c->H.uniform) {

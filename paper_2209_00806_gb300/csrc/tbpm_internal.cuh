@@ -578,6 +578,8 @@ struct BuildOutput {
     int halo_ent_max = 0;            // most packed entries of one block
     int64_t halo_total = 0;          // entries of all lists
     double *diag2_64 = nullptr;      // 2 d (FP64 one-value form; built on first use)
+    int64_t long_steps = 0;          // FP32 states x steps run without the lists
+    int no_halo = 0;                 // tried by default: no lists for this matrix
     // row groups of the staged-gather kernel (build_groups)
     int64_t *gptr = nullptr;         // [n_rows / kHaloRows * 4 + 1] first list entry of each octet
     uint8_t *gperm = nullptr;        // [n_rows / kHaloRows][32] group at each slot

@@ -164,7 +164,7 @@ def test_grouped_rows_are_bit_identical(S, kind):
         smp, offs = lattice.concat([smp, tbg.to_numpy_sample(tbg.twisted_bilayer(4.0))])
     theta = rng.phases(7, S, smp.n_orb)
     out = []
-    # ZIGZAG | WIDE; ZIGZAG | HALO | STAGED; the default, which takes the staged kernel here
+    # ZIGZAG | WIDE; ZIGZAG | HALO | STAGED; the default
     for variant in (65, 4609, 8257):
         with tb.Propagator() as p:
             p.launch_config(tb.TBPM_FP32, 8, 64, variant)
@@ -175,6 +175,31 @@ def test_grouped_rows_are_bit_identical(S, kind):
             N.tbpm_get_states(p.ctx, phi)
             out.append(phi)
     assert (out[0] == out[1]).all() and (out[0] == out[2]).all()
+
+
+@pytest.mark.parametrize("S,steps", [(1, (100, 27, 1, 2)), (4, (31, 1, 3)), (8, (15, 1, 2)), (3, (42, 2))])
+def test_default_takes_the_lists_between_calls(S, steps):
+    """Long rows: resumed runs on both sides of the step from which the default
+    builds the staged gathers' lists give the plain kernel's states."""
+    import torch
+    import paper_2209_00806_gb300 as tb
+    from paper_2209_00806_gb300 import _native as N
+    from tbpm_inputs import tbg
+    smp = tbg.to_numpy_sample(tbg.twisted_bilayer(6.0, order="morton"))
+    theta = rng.phases(9, S, smp.n_orb)
+    out = []
+    for variant in (65, 8257):
+        with tb.Propagator() as p:
+            p.launch_config(tb.TBPM_FP32, 8, 64, variant)
+            p.build_sample(smp, 13.0)
+            p.set_phase_states(theta)
+            for k, n in enumerate(steps):
+                p.propagate(Z, n, tb.TBPM_FP32, flags=N.TBPM_PROP_RESUME if k else 0)
+                phi = torch.empty((S, smp.n_orb), dtype=torch.complex128, device="cuda")
+                N.tbpm_get_states(p.ctx, phi)
+                out.append(phi)
+    for a, b in zip(out[:len(steps)], out[len(steps):]):
+        assert (a == b).all()
 
 
 # cluster stepping of several states at once, and as the default up to 8192
