@@ -95,7 +95,8 @@ struct tbpm_ctx {
     unsigned long long *d_renorm = nullptr;
     double2 *d_corr = nullptr;
     double *d_norms = nullptr;
-    int corr_steps = -1;         // n_steps of the buffers above
+    int corr_steps = -1;         // n_steps and n_states of the buffers above
+    int corr_states = 0;
     double *d_norm_ref = nullptr;          // [n_samples][n_states] squared norms at t = 0
     int64_t norm_ref_len = 0;
     // AC-conductivity correlation
@@ -973,13 +974,14 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         CUDA_OR_FAIL(c, cudaHostAlloc((void **)&c->h_res, kResBytes, cudaHostAllocDefault));
     rc = ensure_groups(c, precision);
     if (rc) return rc;
-    if (c->corr_steps != n_steps) {
+    if (c->corr_steps != n_steps || c->corr_states != c->n_states) {
         free_outputs(c);
         const size_t cnt = (size_t)c->n_samples * c->n_states * (n_steps + 1);
         rc = dalloc(c, &c->d_corr, cnt);
         if (!rc) rc = dalloc(c, &c->d_norms, cnt);
         if (rc) return rc;
         c->corr_steps = n_steps;
+        c->corr_states = c->n_states;
     }
     CUDA_OR_FAIL(c, cudaMemsetAsync(c->d_flags, 0, kFlagBytes, c->st));
     {

@@ -1,0 +1,80 @@
+"""Host side of the library on a CUDA runtime that has no device (fake_cudart.cpp):
+buffer sizes, shared-memory limits and failing allocations, without a GPU."""
+import os
+import subprocess
+import sys
+import textwrap
+from pathlib import Path
+
+import pytest
+
+ROOT = Path(__file__).resolve().parents[1]
+LIB = ROOT / "paper_2209_00806_gb300" / "_build" / "libtbpm.so"
+HEAD = """
+import ctypes as C, os, sys
+fake = C.CDLL(sys.argv[1], mode=C.RTLD_GLOBAL)
+fake.fake_report.restype = C.c_char_p
+fake.fake_reset.argtypes = [C.c_long]
+fake.fake_live.restype = fake.fake_failed.restype = C.c_long
+lib = C.CDLL(sys.argv[2])
+lib.tbpm_last_error.restype = C.c_char_p
+lib.tbpm_last_error.argtypes = [C.c_void_p]
+lib.tbpm_destroy.argtypes = [C.c_void_p]
+Z = C.c_double(1.5707963267948966)
+FP64, FP32, HOST = 0, 1, 0
+def dbl(n, v=0.0): return (C.c_double * max(n, 1))(*([v] * n))
+def create():
+    h = C.c_void_p()
+    assert lib.tbpm_create(C.byref(h), 0, None) == 0
+    return h
+def build(h, n, onsite=True, flags=0, deg=1):
+    # `deg` bonds an orbital: (u, u + 1), (u, u + 2), ..., all of one value
+    m = n * deg
+    i = (C.c_int64 * m)(*[u for d in range(deg) for u in range(n)])
+    j = (C.c_int64 * m)(*[(u + d + 1) % n for d in range(deg) for u in range(n)])
+    return lib.tbpm_build_hamiltonian(h, C.c_int64(n), dbl(n) if onsite else None, C.c_int64(m), i, j,
+                                      dbl(m, 1.0), C.c_double(10.0), 1, None, HOST, flags)
+def states(h, n, S): return lib.tbpm_set_phase_states(h, S, dbl(n * S), HOST)
+def run(h, S, steps, prec, flags=0):
+    return lib.tbpm_propagate(h, Z, steps, prec, dbl(2 * S * (steps + 1)), HOST, flags)
+def clean(): assert fake.fake_report() == b"", fake.fake_report()
+"""
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    import __graft_entry__
+    bn = __graft_entry__._build_module()
+    bn.build()
+    so = tmp_path_factory.mktemp("fake") / "libfake_cudart.so"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I",
+                    os.path.join(bn.CUDA_HOME, "include"), str(Path(__file__).with_name("fake_cudart.cpp")),
+                    "-o", str(so)], check=True)
+    return so
+
+
+def run_script(fake, body):
+    env = dict(os.environ, LD_PRELOAD=str(fake))
+    r = subprocess.run([sys.executable, "-c", HEAD + textwrap.dedent(body), str(fake), str(LIB)],
+                       capture_output=True, text=True, env=env, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+
+
+# a new number of states with the old number of steps: C and the norms are
+# read back whole, by the per-term kernels and by the cluster stepping
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("config", [None, 1])
+def test_outputs_fit_the_states(fake, prec, config):
+    run_script(fake, f"""
+        h = create()
+        if {config}: assert lib.tbpm_set_launch_config(h, {prec}, 8, 64, {config}) == 0
+        n = 700
+        assert build(h, n) == 0
+        for S in (1, 16, 2, 5):
+            assert states(h, n, S) == 0 and run(h, S, 9, {prec}) == 0, lib.tbpm_last_error(h)
+            avg = dbl(2 * 10)
+            assert lib.tbpm_correlation(h, avg, HOST) == 0
+            clean()
+        lib.tbpm_destroy(h)
+        assert fake.fake_live() == 0
+    """)
