@@ -1168,14 +1168,9 @@ __global__ void __launch_bounds__(kHaloRows * L, 8 / L) k_term_halo(TermArgs a)
 template <typename V, int L, int SPL, bool FINAL>
 cudaError_t launch_halo_t(const TermArgs &a, cudaStream_t st)
 {
-    static int configured = -1;              // dynamic shared bytes already allowed
     const int smem = a.halo_max * (2 * L) * 16;
-    if (smem > configured) {
-        cudaError_t e = cudaFuncSetAttribute(k_term_halo<V, L, SPL, FINAL>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        configured = smem;
-    }
+    const cudaError_t e = allow_shared<k_term_halo<V, L, SPL, FINAL>>(kHaloSmemMax);
+    if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)(a.n_rows / kHaloRows);
     return launch_dependent(k_term_halo<V, L, SPL, FINAL>, blocks, kHaloRows * L, smem, st, a);
 }
@@ -1573,8 +1568,6 @@ __global__ void __launch_bounds__(kHaloRows * C, 2) k_term_staged(TermArgs a, Pi
     st<V, C, SPL>(a.out, r, l, o);
 }
 
-int g_staged_configured[2][2] = {};   // dynamic shared bytes allowed, [fp32][C/4]
-
 template <typename V, int C>
 cudaError_t launch_staged_t(const TermArgs &a, cudaStream_t st)
 {
@@ -1585,13 +1578,8 @@ cudaError_t launch_staged_t(const TermArgs &a, cudaStream_t st)
     ps.stage_bytes = ps.halo_bytes + ps.lcol_bytes + ps.val_bytes;
     ps.n_hb = (int)(a.n_rows / kHaloRows);
     const int smem = ps.stage_bytes;
-    int &conf = g_staged_configured[sizeof(V) == 4][C / 4];
-    if (smem > conf) {
-        cudaError_t e = cudaFuncSetAttribute(k_term_staged<V, C>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        conf = smem;
-    }
+    const cudaError_t e = allow_shared<k_term_staged<V, C>>(kPipeSmemMax);
+    if (e != cudaSuccess) return e;
     return launch_dependent(k_term_staged<V, C>, (unsigned)ps.n_hb, kHaloRows * C, smem, st, a, ps);
 }
 
@@ -1601,8 +1589,6 @@ cudaError_t dispatch_staged(const TermArgs &a, int fp32, int B, cudaStream_t st)
     if (fp32) return B == 4 ? launch_staged_t<float, 2>(a, st) : launch_staged_t<float, 4>(a, st);
     return B == 2 ? launch_staged_t<double, 2>(a, st) : launch_staged_t<double, 4>(a, st);
 }
-
-int g_pipe_configured[2][2] = {};   // dynamic shared bytes allowed, [fp32][C/4]
 
 template <typename V, int C>
 cudaError_t launch_pipe_t(const TermArgs &a, int num_sms, cudaStream_t st)
@@ -1614,26 +1600,19 @@ cudaError_t launch_pipe_t(const TermArgs &a, int num_sms, cudaStream_t st)
     ps.stage_bytes = ps.halo_bytes + ps.lcol_bytes + ps.val_bytes;
     ps.n_hb = (int)(a.n_rows / kHaloRows);
     const int smem = 2 * ps.stage_bytes;
-    int &conf = g_pipe_configured[sizeof(V) == 4][C / 4];
-    if (smem > conf) {
-        cudaError_t e = cudaFuncSetAttribute(k_term_halo_pipe<V, C>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        conf = smem;
-    }
+    const cudaError_t e = allow_shared<k_term_halo_pipe<V, C>>(kPipeSmemMax);
+    if (e != cudaSuccess) return e;
     // as many resident blocks per SM as shared memory and registers allow
     // (one for the twisted bilayer's ~200 KB stages, several for lattices
     // with short rows), the persistent grid a multiple of the SM count
-    static int occ_cache[2][2] = {};
-    static int occ_smem[2][2] = {};
-    int &occ = occ_cache[sizeof(V) == 4][C / 4];
-    if (occ_smem[sizeof(V) == 4][C / 4] != smem) {
+    thread_local int occ = 0, occ_smem = -1;
+    if (occ_smem != smem) {
         int nb = 1;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_term_halo_pipe<V, C>,
                                                           kHaloRows * C, smem) != cudaSuccess)
             nb = 1;
         occ = std::max(1, nb);
-        occ_smem[sizeof(V) == 4][C / 4] = smem;
+        occ_smem = smem;
     }
     const int grid = (int)std::min<int64_t>((int64_t)num_sms * occ, ps.n_hb);
     return launch_dependent(k_term_halo_pipe<V, C>, grid, kHaloRows * C, smem, st, a, ps);
@@ -1877,7 +1856,7 @@ cudaError_t launch_term_t(const TermArgs &a, int threads, cudaStream_t st)
 template <typename V, int L, int SPL, typename Fm>
 cudaError_t launch_term_pf_f(const TermArgs &a, int threads, cudaStream_t st)
 {
-    static int occ[4] = {0, 0, 0, 0};            // resident blocks per SM by threads 64 .. 512
+    static std::atomic<int> occ[4];              // resident blocks per SM by threads 64 .. 512
     const int ti = threads <= 64 ? 0 : threads <= 128 ? 1 : threads <= 256 ? 2 : 3;
     if (!occ[ti]) {
         int nb = 1;

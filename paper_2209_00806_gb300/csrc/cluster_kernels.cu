@@ -476,12 +476,12 @@ __global__ void __launch_bounds__(512, 1) k_cluster_steps_f32(ClusterArgs a)
 }  // namespace
 
 namespace {
+constexpr int kClusterSmem = 200 * 1024;     // dynamic shared memory of a block at most
 // 16-block clusters (non-portable size) run on this device
 bool cluster16()
 {
-    static int best16 = -1;
-    if (best16 < 0) {
-        best16 = 0;
+    static const bool ok = [] {
+        bool best16 = false;
         if (cudaFuncSetAttribute(k_cluster_steps<kClusterMaxW, 1024, kReal>,
                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
             cudaLaunchConfig_t cfg = {};
@@ -496,16 +496,16 @@ bool cluster16()
             cfg.attrs = &at;
             cfg.numAttrs = 1;
             int n = 0;
-            cudaFuncSetAttribute(k_cluster_steps<kClusterMaxW, 1024, kReal>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+            allow_shared<k_cluster_steps<kClusterMaxW, 1024, kReal>>(kClusterSmem);
             if (cudaOccupancyMaxActiveClusters(&n, k_cluster_steps<kClusterMaxW, 1024, kReal>, &cfg) ==
                     cudaSuccess &&
                 n >= 1)
-                best16 = 1;
+                best16 = true;
         }
         cudaGetLastError();
-    }
-    return best16 != 0;
+        return best16;
+    }();
+    return ok;
 }
 }  // namespace
 
@@ -518,17 +518,17 @@ int cluster_blocks_for(int64_t n_rows, int max_w, int uniform, int fp32, int fix
         const int64_t R = n_rows / K;
         const int64_t smem = fp32 ? 4 * R * 8 + (int64_t)std::max(1, max_w) * R * (uniform ? 0 : 4)
                                   : 4 * R * 16 + (int64_t)std::max(1, max_w) * R * (uniform ? 4 : 12);
-        return smem <= 200 * 1024;
+        return smem <= kClusterSmem;
     };
     // GB300's FP64 rate per SM makes more SMs pay; else 8
     if (cluster16() && fits(16)) return 16;
     return fits(8) ? 8 : 0;
 }
 
-cudaError_t launch_cluster(void (*k)(ClusterArgs), const ClusterArgs &a, int K, int threads,
-                           size_t smem, cudaStream_t st)
+template <auto k>
+cudaError_t launch_cluster(const ClusterArgs &a, int K, int threads, size_t smem, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared<k>(kClusterSmem);
     if (e != cudaSuccess) return e;
     if (K > 8) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -552,7 +552,7 @@ cudaError_t launch_cluster(void (*k)(ClusterArgs), const ClusterArgs &a, int K, 
 template <int MAXW, int MAXT, Vals M>
 cudaError_t launch_cluster_t(const ClusterArgs &a, int K, size_t smem, cudaStream_t st)
 {
-    return launch_cluster(k_cluster_steps<MAXW, MAXT, M>, a, K, a.rows_per_cta, smem, st);
+    return launch_cluster<k_cluster_steps<MAXW, MAXT, M>>(a, K, a.rows_per_cta, smem, st);
 }
 
 template <int MAXW, int RPT>
@@ -561,8 +561,8 @@ cudaError_t launch_cluster_f(const ClusterArgs &a, int K, cudaStream_t st)
     const int R = a.rows_per_cta, threads = ((R + RPT - 1) / RPT + 31) / 32 * 32;
     const size_t smem = (size_t)4 * R * sizeof(float2) +
                         (a.uniform ? 0 : (size_t)a.max_w * R * sizeof(float));
-    return a.uniform ? launch_cluster(k_cluster_steps_f32<MAXW, RPT, kOne>, a, K, threads, smem, st)
-                     : launch_cluster(k_cluster_steps_f32<MAXW, RPT, kReal>, a, K, threads, smem, st);
+    return a.uniform ? launch_cluster<k_cluster_steps_f32<MAXW, RPT, kOne>>(a, K, threads, smem, st)
+                     : launch_cluster<k_cluster_steps_f32<MAXW, RPT, kReal>>(a, K, threads, smem, st);
 }
 
 template <int MAXW, int MAXT>

@@ -165,8 +165,7 @@ template <int C>
 cudaError_t launch_group_t(const TermArgs &a, cudaStream_t st)
 {
     const int smem = kGroupRing + a.halo_max * C * 16;
-    cudaError_t e = cudaFuncSetAttribute(k_term_group<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         smem);
+    const cudaError_t e = allow_shared<k_term_group<C>>(kGroupRing + (kHaloRows + kHaloMaxExt) * C * 16);
     if (e != cudaSuccess) return e;
     return launch_dependent(k_term_group<C>, (unsigned)(a.n_rows / kHaloRows), 32 * C, smem, st, a);
 }

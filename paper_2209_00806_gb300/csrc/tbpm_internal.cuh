@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -98,6 +99,21 @@ inline cudaError_t launch_dependent(void (*k)(P...), dim3 grid, dim3 block, size
 #endif
 
 #ifdef __CUDACC__
+// Dynamic shared memory of kernel K.  The limit belongs to the process, not to a
+// context: it is set once a device, to the most that K's launch rule allows.
+// Set to each launch's own size it would refuse the launch of another thread
+// whose sample needs more.
+template <auto K> inline cudaError_t allow_shared(int most)
+{
+    constexpr int kDevices = 64;
+    static std::atomic<bool> done[kDevices];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || (dev < kDevices && done[dev].load())) return e;
+    e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess && dev < kDevices) done[dev].store(true);
+    return e;
+}
 // 16-byte asynchronous copies to shared memory and their groups.
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
 {

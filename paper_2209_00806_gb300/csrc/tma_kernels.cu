@@ -394,10 +394,10 @@ cudaError_t launch_tma_t(const TermArgs &a, int max_width, int *err, int num_sms
         lay = stage_layout(tile_rows, row_bytes, max_width, (int)sizeof(V));
     }
     const size_t smem = 128 + (size_t)kStages * lay.bytes;
-    if (smem > 220 * 1024) return cudaErrorInvalidConfiguration;
+    constexpr int most = 220 * 1024;
+    if (smem > most) return cudaErrorInvalidConfiguration;
     const int threads = tile_rows * L;
-    cudaError_t e = cudaFuncSetAttribute(k_term_tma<V, L, SPL>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared<k_term_tma<V, L, SPL>>(most);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_term_tma<V, L, SPL>, threads, smem);

@@ -78,3 +78,17 @@ def test_outputs_fit_the_states(fake, prec, config):
         lib.tbpm_destroy(h)
         assert fake.fake_live() == 0
     """)
+
+
+# a kernel's shared-memory limit is the process's: a smaller sample in another
+# context does not lower what a larger one's launches need (cluster stepping)
+@pytest.mark.parametrize("prec,sides", [(0, (8000, 5000)), (1, (16000, 9000))])
+def test_shared_memory_limits_are_not_lowered(fake, prec, sides):
+    run_script(fake, f"""
+        a, b = create(), create()
+        for h, n in zip((a, b), {sides}):
+            assert build(h, n) == 0 and states(h, n, 4) == 0
+            assert run(h, 4, 2, {prec}) == 0, lib.tbpm_last_error(h)
+        assert run(a, 4, 2, {prec}) == 0, lib.tbpm_last_error(a)
+        clean()
+    """)
