@@ -67,7 +67,7 @@ struct tbpm_ctx {
     int variant[2] = {kVariantZigZag, kVariantZigZag | kVariantWide | kVariantPrefetch};
     // no launch shape asked for (FP64, FP32): small samples step in clusters
     bool cluster_auto[2] = {true, true};
-    bool cluster_off = false;    // repeating a run whose norm carry must act
+    bool cluster_off = false;    // repeating a run whose norm carry acts at every step
     int num_sms = 0;
     double renorm_fp32 = 1e-5, hard_fp32 = 1e-2, hard_fp64 = 1e-6;   // norm policy
     std::vector<Group> groups;
@@ -1508,6 +1508,7 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         ca.n_steps = n_steps;
         ca.hard_bound = fp32 ? c->hard_fp32 : c->hard_fp64;
         ca.renorm_bound = c->renorm_fp32;
+        ca.renorm_count = c->d_renorm;
         ca.err = c->d_flags;
         size_t e0 = 0;
         if (profile) {
@@ -1527,8 +1528,8 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         int hf = 0;
         memcpy(&hf, c->h_res, sizeof(hf));
         if (fp32 && (hf & 8)) {
-            // a norm drifted past the renormalisation bound: the per-term kernels,
-            // which rescale the state between steps, from the same start
+            // a bound within the rounding of a step, which would rescale and repeat
+            // every one: the launch ended there; the per-term kernels, from the same start
             if (resume)
                 for (auto &g : c->groups) {
                     CUDA_OR_FAIL(c, cudaMemcpyAsync(g.buf[cur0], g.buf[keep],

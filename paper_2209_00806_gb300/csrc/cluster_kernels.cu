@@ -306,9 +306,16 @@ __device__ __forceinline__ FF warp_sum3(FF v0, FF v1, FF v2)
 // The FP32 form of the stepping: states and arithmetic those of the per-term
 // FP32 kernels (bit-identical), RPT rows a thread (rows t, t + T, ...), the
 // closing sums as float pairs up to the block and FP64 from there.  The
-// per-term kernels rescale a state whose norm has drifted before the next
-// step; here such a drift sets error bit 8 and the caller repeats the run
-// with them.  Bound by the latency of a term (barrier, distributed
+// norm carry: a state whose norm has drifted past the bound after step m starts
+// step m + 1 rescaled, as with the per-term kernels.  Step m's sums are known
+// while step m + 1 runs, so it is run once more from its start, which is still
+// in its buffer, with the factor: one step more per rescaling (64 x 64 graphene
+// drifts 8e-9 a step: one in 1,300 at the default bound).  A state that drifts
+// past the bound in the step after a rescaling has a bound within a step's
+// rounding and would run every step twice: the launch ends there with error bit
+// 8, and the caller repeats the run with the per-term kernels.  4,096 steps at
+// the default bound: 9.8 us a step at 64 x 64 and 25 us at 180 x 180 (repeated
+// whole by the per-term kernels: 51 and 70 us).  Bound by the latency of a term (barrier, distributed
 // shared-memory gathers): 64 x 64 graphene, one state, 10 us a step against
 // 42 us of dependent launches; 180 x 180 25 against 47 us.
 template <int MAXW, int RPT, Vals M>
@@ -325,6 +332,14 @@ __global__ void __launch_bounds__(512, 1) k_cluster_steps_f32(ClusterArgs a)
     __shared__ double part[2][3];
     __shared__ FF red[32][3];
     __shared__ FusedTerm tab[3 * kClusterMaxTerms];
+    __shared__ float rescale;        // block 0 -> every block: factor, kStop, or 0
+    __shared__ int start;            // buffer of the last step's starting state
+    __shared__ int scaled;           // (block 0) the last step that called for a factor
+    constexpr float kStop = -1.f;
+    if (t == 0) {
+        rescale = 0.f;
+        scaled = -1;
+    }
     for (int i = t; i < 3 * a.J; i += T) tab[i] = a.terms[(i / a.J) * kMaxTerms + i % a.J];
 
     uint32_t gsrc[RPT][MAXW];
@@ -385,25 +400,54 @@ __global__ void __launch_bounds__(512, 1) k_cluster_steps_f32(ClusterArgs a)
             const double drift = ref > 0.0 ? fabs(sm2 / ref - 1.0) : sm2;
             if (!(sm2 == sm2) || !(v == v) || !(sm1 == sm1) || sm2 - sm2 != 0.0) atomicOr(a.err, 2);
             else if (drift > a.hard_bound) atomicOr(a.err, 1);
-            if (drift > a.renorm_bound) atomicOr(a.err, 8);
+            if (drift > a.renorm_bound && sm2 > 0.0 && ref > 0.0 && sm2 - sm2 == 0.0) {
+                atomicAdd(a.renorm_count, 1ull);
+                if (m < a.n_steps) {
+                    const bool again = m == scaled + 1;
+                    if (again) atomicOr(a.err, 8);
+                    scaled = m;
+                    const float f = again ? kStop : (float)sqrt(ref / sm2);
+                    for (int k = 0; k < K; ++k) *cl.map_shared_rank(&rescale, k) = f;
+                }
+            }
         }
     };
-    for (int n = 1; n <= a.n_steps; ++n) {
+    auto next_vector = [&]() {
+        if (!pending) return;
+        cl.barrier_wait();                   // the gathered vector is complete
+        pending = false;
+        if (sum_waits > 0 && --sum_waits == 0 && rank == 0 && t < 32) cluster_sum(sum_step);
+    };
+    for (int n = 1;; ++n) {
+        next_vector();
+        // step n - 2's factor, written before the barrier just passed: the same
+        // for every thread of the cluster
+        const float f = *(volatile float *)&rescale;
+        if (f > 0.f) {                       // step n - 1 once more, from its rescaled start
+            __syncthreads();
+            if (t == 0) rescale = 0.f;
+            cur = start;
+            sum_waits = 0;                   // not the sums of its first run
+            --n;
+        }
+        const float sc = f > 0.f ? f : 1.f;  // of this step's starting state
+        if (f < 0.f || n > a.n_steps) break;
         const FusedTerm *tt = tab + cur * a.J;
         for (int j = 0; j < a.J; ++j) {
             const FusedTerm tm = tt[j];
             const int xoff = (1 + (tm.x < 0 ? cur : tm.x)) * R;
             const uint32_t xoff_b = (uint32_t)xoff * (uint32_t)sizeof(float2);
+            const float scx = tm.x < 0 ? sc : 1.f;   // (no branch among the rows' gathers)
             float2 p[RPT], zz[RPT];          // own rows: written only by this thread
 #pragma unroll
             for (int i = 0; i < RPT; ++i) {
                 const int row = min(t + i * T, R - 1);
                 p[i] = vec[(1 + cur) * R + row];
+                p[i].x *= sc;
+                p[i].y *= sc;
                 zz[i] = tm.z >= 0 ? vec[(1 + tm.z) * R + row] : make_float2(0.f, 0.f);
             }
-            if (pending) cl.barrier_wait();  // the gathered vector is complete
-            pending = false;
-            if (sum_waits > 0 && --sum_waits == 0 && rank == 0 && t < 32) cluster_sum(sum_step);
+            next_vector();
             FF v0 = {0.f, 0.f}, v1 = v0, v2 = v0;
 #pragma unroll
             for (int i = 0; i < RPT; ++i) {
@@ -423,6 +467,8 @@ __global__ void __launch_bounds__(512, 1) k_cluster_steps_f32(ClusterArgs a)
                         y.x = fmaf(h, x[k].x, y.x);
                         y.y = fmaf(h, x[k].y, y.y);
                     }
+                y.x *= scx;
+                y.y *= scx;
                 float2 o;
                 o.x = fmaf(tm.c_hi_f, p[i].x, fmaf(tm.c_lo_f, p[i].x, fmaf(tm.gamma_f, y.y, zz[i].x)));
                 o.y = fmaf(tm.c_hi_f, p[i].y, fmaf(tm.c_lo_f, p[i].y, fmaf(-tm.gamma_f, y.x, zz[i].y)));
@@ -455,11 +501,12 @@ __global__ void __launch_bounds__(512, 1) k_cluster_steps_f32(ClusterArgs a)
                 sum_waits = 2;
             }
         }
+        if (t == 0) start = cur;
         cur = a.next_cur[cur];
     }
-    if (pending) {
-        cl.barrier_wait();
-        if (sum_waits > 0) --sum_waits;
+    if (rescale < 0.f) {                     // the caller starts again
+        cl.sync();
+        return;
     }
     if (sum_waits > 0) {
         cl.sync();

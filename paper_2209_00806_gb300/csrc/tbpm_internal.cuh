@@ -520,7 +520,8 @@ struct ClusterArgs {
     int next_cur[3];
     int n_steps;
     double hard_bound;
-    double renorm_bound;        // FP32: a drift above it sets error bit 8
+    double renorm_bound;        // FP32: a drift above it rescales the next step's start
+    unsigned long long *renorm_count;
     int *err;
 };
 // Blocks of the cluster for n_rows rows (16 where the device runs such a
