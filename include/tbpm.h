@@ -373,9 +373,11 @@ int tbpm_dos_adjoint(const double *dl_dd, int n_e, int n_steps, double tau, int 
                                         gathers; FP32: 16-byte lanes, one row a thread
                                         up to 2^20 of them, blocks of 128 threads or
                                         more beyond (TBPM_VARIANT_WIDE: the closing
-                                        pass's lanes), and the staged gathers (HALO |
-                                        STAGED) for rows of at least 32 values on
-                                        average; ignored otherwise.  All bit-identical */
+                                        pass's lanes); with at least 32 values a row on
+                                        average, groups of 4 or 8 states take the staged
+                                        gathers (HALO | STAGED) once the steps run pay
+                                        for the lists, groups of 1 or 2 one row a thread;
+                                        ignored otherwise.  All bit-identical */
 #define TBPM_VARIANT_STAGED 4096     /* with TBPM_VARIANT_HALO: one block per 128-row
                                         block copying its halo, positions and values
                                         into one shared-memory stage, two blocks per

@@ -1003,14 +1003,22 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     const int threads = c->threads[precision];
     // staged-gather variant: halo lists built on first use; a matrix whose
     // row blocks reference too many other rows keeps the plain kernels
-    int variant = c->variant[precision];
-    // the register-pipelined variant on long rows of real FP32 values: the
-    // staged gathers instead where the lists can be had (twisted bilayer, 68
-    // entries a row, 3.1M rows: 1.84 ms a term through L1, 0.81 ms staged,
-    // less in groups; graphene's three entries hit L1 and lose, 0.27 against
-    // 0.19 ms).  The lists are built once the steps run on this matrix pay for
-    // them (built on the first call, two steps of one state went from 10.5 to
-    // 15.3 ms on a 120 nm flake).  ms a step, plain against staged, and the build:
+    const int variant = c->variant[precision];
+    // the register-pipelined variant on long rows of real FP32 values, by the
+    // group's width.  Widths 4 and 8 take the staged gathers in row groups where
+    // the lists can be had (twisted bilayer, 68 entries a row, 3.1M rows: 1.84 ms
+    // a term through L1, 0.81 ms staged, less in groups; graphene's three
+    // entries hit L1 and lose, 0.27 against 0.19 ms), widths 1 and 2 one row a
+    // thread, a width of 16 what was asked for.  ms a step (two launches: 2 + 1):
+    //   flake, width   pipelined  one row a thread  k_term_halo
+    //   12 nm, 1, 2    0.19 0.22     0.18 0.21
+    //   120 nm, 1, 2   2.26 2.23     1.64 2.02
+    //   12 nm, 16      0.25          0.25              0.36
+    //   30 nm, 16      0.69          0.77              0.92
+    //   120 nm, 16     12.1          10.9              19.8
+    // The lists are built once the steps that read them pay for them (built on
+    // the first call, two steps of a 120 nm flake take the build's 11.8 ms more).
+    // ms a step, pipelined against staged, and the build:
     //   flake, states   plain  staged  build   meet at (states x steps)
     //   12 nm, 8         0.27   0.18    1.2     110
     //   30 nm, 8         0.40   0.26    1.7      97
@@ -1019,44 +1027,52 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     //   60 nm, 4         0.9    0.71    3.7      78
     //   120 nm, 8        6.5    3.2    11.8      29
     //   120 nm, 4        3.7    2.4    11.8      36
-    //   120 nm, 1        2.3    1.65   11.8      18
     // so from 32 beyond 2^17 rows (between 30 and 60 nm), from 128 below.
-    const int64_t pays = c->H.n_rows >= ((int64_t)1 << 17) ? 32 : 128;
-    if (fp32 && !c->H.halo_ptr) c->H.long_steps += (int64_t)n_steps * c->n_states;
     const bool long_rows = fp32 && (variant & kVariantPrefetch) && !c->H.cplx && !c->H.uniform &&
                            !(variant & (kVariantHalo | kVariantTma | kVariantFused | kVariantSplit2 |
                                         kVariantSplit4)) &&
-                           c->H.nnz_true >= kLongRow * c->n_orb && !c->H.no_halo &&
-                           (c->H.halo_ptr || (c->H.long_steps >= pays &&
-                                              fits_beside(10 * (size_t)c->H.nnz_true)));
-    if (long_rows) variant = (variant & ~kVariantPrefetch) | kVariantHalo | kVariantStaged;
-    bool halo = (variant & kVariantHalo) && !c->H.cplx && !(variant & (kVariantTma | kVariantFused));
+                           c->H.nnz_true >= kLongRow * c->n_orb;
+    int list_states = 0;
+    for (auto &g : c->groups)
+        if (g.B == 4 || g.B == 8) list_states += g.B;
+    const int64_t pays = c->H.n_rows >= ((int64_t)1 << 17) ? 32 : 128;
+    if (long_rows && !c->H.halo_ptr) c->H.long_steps += (int64_t)n_steps * list_states;
+    const bool auto_lists = long_rows && list_states > 0 && !c->H.no_halo &&
+                            (c->H.halo_ptr || (c->H.long_steps >= pays &&
+                                               fits_beside(10 * (size_t)c->H.nnz_true)));
+    const bool staged = auto_lists || (variant & kVariantStaged);
+    bool halo = (auto_lists || (variant & kVariantHalo)) && !c->H.cplx &&
+                !(variant & (kVariantTma | kVariantFused));
     if (halo && !c->H.halo_ptr) {
         std::string msg;
         rc = build_halo(c->H, c->st, msg);
-        if (rc == TBPM_E_UNSUPPORTED || (rc == TBPM_E_OOM && long_rows)) {
+        if (rc == TBPM_E_UNSUPPORTED || (rc == TBPM_E_OOM && auto_lists)) {
             halo = false;
-            c->H.no_halo |= long_rows;      // the default does not try again
+            c->H.no_halo |= auto_lists;     // the default does not try again
         } else if (rc) return fail(c, rc, msg);
     }
     // one-stage staged gathers with FP32 values per entry: rows in groups of four
-    if (halo && fp32 && (variant & kVariantStaged) && !c->H.uniform) {
+    if (halo && fp32 && staged && !c->H.uniform && list_states > 0) {
         std::string msg;
         rc = build_groups(c->H, c->st, msg);
         if (rc) return fail(c, rc, msg);
     }
-    const bool grouped = halo && fp32 && (variant & kVariantStaged) && c->H.gptr;
-    if (halo && (variant & (kVariantPipe | kVariantStaged)) && !c->H.uniform &&
+    const bool grouped = halo && fp32 && staged && c->H.gptr;
+    if (halo && (staged || (variant & kVariantPipe)) && !c->H.uniform &&
         !grouped && !c->H.vpack[fp32]) {
         std::string msg;
         rc = build_packed_values(c->H, fp32, c->st, msg);
-        if (rc == TBPM_E_OOM && long_rows) halo = false;
+        if (rc == TBPM_E_OOM && auto_lists) halo = false;
         else if (rc) return fail(c, rc, msg);
     }
-    if (long_rows && !halo) {                        // no lists: the asked-for kernel
-        cudaGetLastError();
-        variant = c->variant[precision];
-    }
+    if (auto_lists && !halo) cudaGetLastError();     // no lists: the asked-for kernels
+    auto group_variant = [&](int B) {
+        if (!long_rows) return halo ? variant : variant & ~kVariantHalo;
+        if (halo && (B == 4 || B == 8) &&
+            staged_launchable(1, B, c->H.halo_max, c->H.halo_ent_max, 0))
+            return (variant & ~kVariantPrefetch) | kVariantHalo | kVariantStaged;
+        return B <= 2 ? variant & ~kVariantPrefetch : variant;
+    };
     // FP64 one-value form: 2 d for the interior terms' gamma d
     if (!fp32 && c->H.uniform && !c->H.zero_diag && !c->H.diag2_64) {
         std::string msg;
@@ -1357,10 +1373,9 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
                     ended_interior = true;
                 }
                 TermArgs t = base;
-                t.variant = variant;
+                t.variant = group_variant(g.B);
                 // complex values have the plain term kernels only (16-byte lanes)
                 if (c->H.cplx) t.variant &= kVariantZigZag | kVariantStreamHints;
-                if (!halo) t.variant &= ~kVariantHalo;
                 t.reverse = (t.variant & kVariantZigZag) ? (int)(k & 1) : 0;
                 t.x = L.x < 0 ? g.buf[cur] : g.buf[L.x];
                 t.x_is_psi = L.x < 0;
@@ -1603,7 +1618,8 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         const double valb = fp32 ? 4.0 : 8.0;
         bool halo_used = halo;
         for (auto &g : c->groups)
-            halo_used = halo_used && halo_launchable(fp32, g.B, false, c->H.halo_max);
+            halo_used = halo_used && (group_variant(g.B) & kVariantHalo) &&
+                        halo_launchable(fp32, g.B, false, c->H.halo_max);
         const double idxb = halo_used ? 2.0 : 4.0;
         const double entry = idxb + (c->H.uniform ? 0.0 : valb * (c->H.cplx ? 2 : 1));
         S.bytes_term = vb + (double)c->H.nnz_true * entry + (double)c->n_orb * valb;

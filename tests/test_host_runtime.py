@@ -92,3 +92,24 @@ def test_shared_memory_limits_are_not_lowered(fake, prec, sides):
         assert run(a, 4, 2, {prec}) == 0, lib.tbpm_last_error(a)
         clean()
     """)
+
+
+# long rows of FP32 values: the staged gathers' lists (device memory that stays)
+# come only where a group of four or eight states reads them, once the steps
+# pay for them
+@pytest.mark.parametrize("S,lists", [(1, False), (2, False), (3, False), (16, False), (4, True),
+                                     (8, True), (13, True), (20, True)])
+def test_lists_are_built_for_the_widths_that_read_them(fake, S, lists):
+    run_script(fake, f"""
+        h = create()
+        assert build(h, 2000, flags=16, deg=17) == 0        # TBPM_BUILD_NO_UNIFORM, 34 entries a row
+        assert states(h, 2000, {S}) == 0
+        live = []
+        for steps in (3, 130, 130):
+            assert run(h, {S}, steps, FP32) == 0, lib.tbpm_last_error(h)
+            live.append(fake.fake_live())
+        clean()
+        assert (live[1] > live[0]) == {lists} and live[2] == live[1], live
+        lib.tbpm_destroy(h)
+        assert fake.fake_live() == 0
+    """)
