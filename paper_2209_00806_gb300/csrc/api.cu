@@ -1101,17 +1101,17 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     std::vector<size_t> step_ev;   // index of the first of 5 events per profiled step
     bool cluster_run = false;      // the cluster-resident stepping ran (one launch)
 
-    // cluster-resident stepping: every step of the FP64 states in one launch, a
-    // cluster of Kc blocks per state.  By default up to 512 rows a block: 64 x 64
-    // graphene takes 22 us a step in clusters (25 us with a diagonal, 31 us with
-    // values per entry) against 42-46 us a step and state group in launches;
-    // at 1024 rows a block the two meet (40-57 against 45-50 us).
-    // FP32, us a step: 64 x 64 10 against 42, 180 x 180 25 against 47-54 (seven
-    // clusters run at once: 16 states 30 against 52 at 64 x 64).
+    // cluster-resident stepping: every step of the states in one launch, a cluster
+    // of Kc blocks per state.  By default up to 512 rows a block in FP64 and, in
+    // FP32, 4096 (seven states, all clusters at once) or 1024 (sixteen), where it
+    // is estimated to pay (cluster_pays)
+    std::vector<int> widths;
+    for (auto &g : c->groups) widths.push_back(g.B);
     const bool auto_cluster = c->cluster_auto[precision] &&
                        (fp32 ? c->n_states <= 16 &&
                                    c->H.n_rows <= 16 * (c->n_states <= kClusterStates ? 4096 : 1024)
-                             : c->H.n_rows <= 16 * 512);
+                             : c->H.n_rows <= 16 * 512) &&
+                       c->n_samples == 1 && cluster_pays(c->H, fp32, widths);
     const int Kc = ((variant & kVariantCluster) || auto_cluster) && !c->cluster_off && !fused &&
                            c->n_samples == 1 && !c->H.cplx && !c->ac_on && !c->qe_on &&
                            c->H.max_width <= kClusterMaxW && n_steps > 0 && M - 1 >= 2 &&

@@ -271,6 +271,28 @@ __global__ void k_sort_rows(int64_t n_rows, const int64_t *slice_ptr, const int3
     }
 }
 
+// Cluster stepping gives each block a sixteenth of the rows.  A warp's gather of
+// entry k from other blocks costs by the 128-byte lines (eight FP64 rows) that
+// it touches there, not by its lanes; their number over all warps and entries
+// says what a term's traffic between the blocks takes (cluster_pays).
+__global__ void __launch_bounds__(256) k_far_lines(int64_t n_rows, const int64_t *slice_ptr,
+                                                   const int32_t *col, unsigned long long *lines)
+{
+    const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;   // n_rows % 1024 == 0
+    const int64_t q = r / kSliceRows, base = slice_ptr[q] + r % kSliceRows;
+    const int w = (int)((slice_ptr[q + 1] - slice_ptr[q]) / kSliceRows);
+    const int per = (int)(n_rows / 16), own = (int)(r / per), lane = threadIdx.x & 31;
+    unsigned n = 0;
+    for (int k = 0; k < w; ++k) {
+        const int c = col[base + (int64_t)k * kSliceRows];
+        const bool far = c / per != own;
+        const unsigned m = __ballot_sync(0xffffffffu, far);
+        if (far) n += __ffs(__match_any_sync(m, c / 8)) - 1 == lane;
+    }
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0 && n) atomicAdd(lines, (unsigned long long)n);
+}
+
 __global__ void k_bond_rows(int64_t n_hop, const int64_t *hi, const int64_t *hj,
                             const int32_t *user_to_row, int32_t *rows)
 {
@@ -960,16 +982,16 @@ int build_sell(const BuildInput &in, int keep64, int keep32, int detect_uniform,
     int32_t *deg = nullptr, *fill = nullptr;
     int64_t *entries = nullptr;
     int *err = nullptr;           // [0] error bits, [1] max width
-    unsigned long long *gbits = nullptr;   // [0] Gershgorin bits, [1] bandwidth
+    unsigned long long *gbits = nullptr;   // [0] Gershgorin bits, [1] bandwidth, [2] far lines
     CK(cudaMalloc(&deg, n_rows * sizeof(int32_t)));
     CK(cudaMalloc(&fill, n_rows * sizeof(int32_t)));
     CK(cudaMalloc(&entries, (n_slices + 1) * sizeof(int64_t)));
     CK(cudaMalloc(&err, 2 * sizeof(int)));
-    CK(cudaMalloc(&gbits, 2 * sizeof(unsigned long long)));
+    CK(cudaMalloc(&gbits, 3 * sizeof(unsigned long long)));
     CK(cudaMemsetAsync(deg, 0, n_rows * sizeof(int32_t), st));
     CK(cudaMemsetAsync(fill, 0, n_rows * sizeof(int32_t), st));
     CK(cudaMemsetAsync(err, 0, 2 * sizeof(int), st));
-    CK(cudaMemsetAsync(gbits, 0, 2 * sizeof(unsigned long long), st));
+    CK(cudaMemsetAsync(gbits, 0, 3 * sizeof(unsigned long long), st));
 
     if (in.n_hop > 0) {
         k_count<<<blocks_for(in.n_hop, T), T, 0, st>>>(in.n_hop, in.n_orb, in.hop_i, in.hop_j,
@@ -1054,7 +1076,11 @@ int build_sell(const BuildInput &in, int keep64, int keep32, int detect_uniform,
         return cudaGetLastError();
     };
     CK(direct32 ? fill_all(out.val32) : fill_all(out.val64));
-    unsigned long long hg[2] = {0, 0};
+    if (in.n_samples == 1 && n_rows <= kClusterMaxRows && out.max_width <= kClusterMaxW) {
+        k_far_lines<<<blocks_for(n_rows, T), T, 0, st>>>(n_rows, out.slice_ptr, out.col, gbits + 2);
+        CK(cudaGetLastError());
+    }
+    unsigned long long hg[3] = {0, 0, 0};
     CK(cudaMemcpyAsync(hg, gbits, sizeof(hg), cudaMemcpyDeviceToHost, st));
 
     // chunk -> sample table
@@ -1112,6 +1138,7 @@ int build_sell(const BuildInput &in, int keep64, int keep32, int detect_uniform,
     memcpy(&g, &hg[0], sizeof(g));
     out.gershgorin = g;
     out.bandwidth = (int64_t)hg[1];
+    out.far_lines = (int64_t)hg[2];
     if (!keep64) {
         cudaFree(out.val64);
         cudaFree(out.diag64);

@@ -20,7 +20,9 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 #include <string>
+#include <vector>
 
 #include "tbpm_internal.cuh"
 
@@ -570,6 +572,50 @@ int cluster_blocks_for(int64_t n_rows, int max_w, int uniform, int fp32, int fix
     // GB300's FP64 rate per SM makes more SMs pay; else 8
     if (cluster16() && fits(16)) return 16;
     return fits(8) ? 8 : 0;
+}
+
+// Estimated us a step of 15 products, both ways, fitted to sweeps of lattices of 3
+// to 12 entries a row, 1,024 to 65,536 rows, 1 to 16 states, rows in lattice order,
+// with the sublattices apart and in random order (the far lines cost 1.2 to
+// 2 us a thousand and wave of seven clusters):
+//                                      far lines   FP64, cluster / launches   FP32
+//   3 entries, 8,192 rows, 1 state        512          27 /  43              12 / 44
+//     the same, random order           22,419          52 /  45              47 / 45
+//   3 entries, 65,536 rows, 1 state     2,048                                29 / 46
+//     the same, sublattices apart      26,624                                66 / 47
+//     the same, random order          183,884                               287 / 86
+//   8 entries, 4,096 rows, 4 states       896          38 /  82              14 / 50
+//     the same, random order           28,465          83 /  81              68 / 56
+//     the same, 16 states              28,465         240 / 261             222 / 59
+// The slower way is chosen in 20 of the 1,044 points, by 10 % on average (before, every
+// point took the cluster: 35 % over all of them).
+bool cluster_pays(const BuildOutput &H, int fp32, const std::vector<int> &widths)
+{
+    const int w = std::max(1, H.max_width);
+    const double n = (double)H.n_rows, R = n / 16, far = H.far_lines / 1000.0;
+    int S = 0;
+    for (int B : widths) S += B;
+    const int waves = (S + kClusterStates - 1) / kClusterStates;
+    double cluster, launches = 0.0;
+    if (fp32) {
+        // blocks of fewer than 512 rows share an SM
+        const double turns = R < 512 ? std::ceil(S * R / (kClusterStates * 512.0)) : waves;
+        cluster = turns * (10.5 + n / 8192) + waves * (w <= 4 ? 1.5 : 1.95) * far;
+        for (int B : widths) launches += 38 + 1.4 * w + 0.9 * std::min(B * n / 16384, 16.0);
+    } else {
+        // the FP64 pipe: more rows a block or states an SM take longer
+        const double q = std::pow(R / 512, 1.5), each = S / (double)kClusterStates;
+        const double turns = R > 256 ? waves : std::max(1.0, each * (0.2 + R / 270));
+        cluster = turns * (w > 4 ? 24 + 44 * q : 16 + 17 * q) +
+                  std::max(1.0, each) * (w <= 4 ? 1.15 : 1.55) * far;
+        const int rounds = (w + 3) / 4;              // entries in rounds of four
+        for (int B : widths) {
+            const double x = std::max(0.0, B * n / 1000 - 10);
+            launches += H.fixed_width == 3 ? 45 + 0.95 * x
+                                           : 42 + 11 * rounds + (0.75 + 1.15 * rounds) * std::min(x, 23.0);
+        }
+    }
+    return cluster <= launches;
 }
 
 template <auto k>

@@ -524,6 +524,11 @@ struct ClusterArgs {
     unsigned long long *renorm_count;
     int *err;
 };
+struct BuildOutput;
+// Samples whose far lines the builder counts.
+constexpr int64_t kClusterMaxRows = 16 * 4096;
+// The cluster stepping is estimated to take no longer than the per-term launches.
+bool cluster_pays(const BuildOutput &H, int fp32, const std::vector<int> &widths);
 // Blocks of the cluster for n_rows rows (16 where the device runs such a
 // cluster, else 8), or 0 when the sample does not fit.
 int cluster_blocks_for(int64_t n_rows, int max_w, int uniform, int fp32, int fixed_width);
@@ -580,6 +585,8 @@ struct BuildOutput {
     int max_width = 0;
     int fixed_width = 0;             // every slice has this width (0: widths vary)
     int64_t bandwidth = 0;           // max |col - row| over the stored entries
+    int64_t far_lines = 0;           // small single samples: lines a cluster's blocks read of
+                                     // one another a term (k_far_lines)
     int uniform = 0;                 // all off-diagonal values are equal
     int zero_diag = 0;               // no onsite energies were given (H_ii = 0)
     int cplx = 0;                    // values are complex (re, im) per entry

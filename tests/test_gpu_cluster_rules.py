@@ -73,3 +73,40 @@ def test_norm_carry_at_the_end_of_a_run():
         (a, na, ca), (b, nb, cb) = run(PER_TERM, steps), run(None, steps)
         assert ca == cb == (steps >= first)
         assert np.array_equal(a, b) and np.abs(na - nb).max() < 1e-12
+
+
+# which samples step in clusters by default: rows in lattice order do, the same
+# lattice in an order that spreads every neighbour over the blocks does only
+# where it is small; the states are the per-term kernels' either way
+@pytest.mark.parametrize("precision,kind,S,cluster", [
+    (0, (64, 64), 1, True), (0, (64, 64), 8, True), (0, "shuffled 64", 1, False),
+    (0, "shuffled 22", 1, True), (0, "ragged", 1, False), (0, "ragged", 3, True),
+    (1, (64, 64), 16, True), (1, (180, 180), 7, True), (1, "shuffled 180", 1, False),
+    (1, "shuffled 64", 8, False), (1, "shuffled 22", 4, True), (1, "ragged", 16, False)])
+def test_cluster_default_by_row_order(precision, kind, S, cluster):
+    import paper_2209_00806_gb300 as tb
+    if kind == "ragged":
+        smp = lattice.random_graph(8000, 12000, seed=9, onsite_w=1.0, t_scale=0.8)
+    elif isinstance(kind, str):
+        L = int(kind.split()[1])
+        smp = lattice.graphene(L, L, pbc=True, seed=6, onsite_w=1.0)
+        smp = lattice.permute(smp, np.random.default_rng(3).permutation(smp.n_orb))
+    else:
+        smp = lattice.graphene(*kind, pbc=True, seed=6, onsite_w=1.0)
+    theta = rng.phases(4, S, smp.n_orb)
+    out = []
+    for variant in (1, None):
+        with tb.Propagator() as p:
+            if variant is not None:
+                p.launch_config(precision, 8, 64, variant)
+            p.build_sample(smp, 12.0)
+            C = _run_states(p, theta, precision)
+            out.append((C, p.states(), p.stats()["kernel_launches"]))
+    (Ca, a, la), (Cb, b, lb) = out
+    assert np.array_equal(a, b) and np.abs(Ca - Cb).max() < 1e-12
+    assert la > 6 * 15 and (lb < 6 * 15) == cluster
+
+
+def _run_states(p, theta, precision):
+    p.set_phase_states(theta)
+    return p.propagate(Z, 6, precision)
