@@ -406,8 +406,12 @@ int tbpm_set_norm_policy(tbpm_ctx *ctx, double renorm_fp32, double hard_fp32, do
  * block width of the blocked sparse product), threads per block (64, 128, 256)
  * and TBPM_VARIANT_* bits -- and keep the fastest as the context's
  * configuration for `precision`.  The chosen values are written to the
- * non-NULL out pointers.  The slice height is fixed at 32 rows (one warp's
- * rows share a slice).  Leaves no propagation to resume.
+ * non-NULL out pointers; set by hand in another context they run the kernels
+ * that were timed, but for small FP32 samples: where the default's cluster
+ * stepping was the default and is faster, it stays this context's default and
+ * the shape returned is the fastest of the per-term launches.  The slice height
+ * is fixed at 32 rows (one warp's rows share a slice).  Leaves no propagation
+ * to resume.
  * Errors: STATE, INVALID_ARG, OOM, CUDA. */
 int tbpm_autotune(tbpm_ctx *ctx, int precision, double z, int probe_steps, int *best_group,
                   int *best_threads, int *best_variant, double *best_ms_per_step);

@@ -925,6 +925,15 @@ static int ensure_fused(tbpm_ctx *c, int J, int R, int radius, int maxB, int gri
     return TBPM_OK;
 }
 
+// The register-pipelined variant on long rows of real values (FP32): tbpm_propagate
+// chooses the kernel by the group's width.
+static bool takes_long_rows(const tbpm_ctx *c, int variant)
+{
+    return (variant & kVariantPrefetch) && !c->H.cplx && !c->H.uniform &&
+           !(variant & (kVariantHalo | kVariantTma | kVariantFused | kVariantSplit2 | kVariantSplit4)) &&
+           c->H.nnz_true >= kLongRow * c->n_orb;
+}
+
 static int get_events(tbpm_ctx *c, size_t n)
 {
     while (c->events.size() < n) {
@@ -1028,10 +1037,7 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     //   120 nm, 8        6.5    3.2    11.8      29
     //   120 nm, 4        3.7    2.4    11.8      36
     // so from 32 beyond 2^17 rows (between 30 and 60 nm), from 128 below.
-    const bool long_rows = fp32 && (variant & kVariantPrefetch) && !c->H.cplx && !c->H.uniform &&
-                           !(variant & (kVariantHalo | kVariantTma | kVariantFused | kVariantSplit2 |
-                                        kVariantSplit4)) &&
-                           c->H.nnz_true >= kLongRow * c->n_orb;
+    const bool long_rows = fp32 && takes_long_rows(c, variant);
     int list_states = 0;
     for (auto &g : c->groups)
         if (g.B == 4 || g.B == 8) list_states += g.B;
@@ -2086,6 +2092,22 @@ extern "C" int tbpm_autotune(tbpm_ctx *c, int precision, double z, int probe_ste
     for (int B : widths)
         for (int T : thread_opts)
             for (int V : variant_opts) {
+                if (precision == TBPM_FP32 && (V & kVariantPrefetch)) {
+                    // blocks of 128 also stand for 64, and for all where a row a thread
+                    // is launched: one kernel, timed once
+                    if (T == 128 || (T == 256 && c->H.n_rows * std::max(1, B / 2) <= (1 << 20))) continue;
+                    // where the staged gathers take its place (the lists are there by
+                    // now), they are timed and returned under their own name
+                    bool lists = false;
+                    for (int left = c->n_states, b = B; left > 0; left -= b) {
+                        while (b > left) b /= 2;
+                        lists = lists || b == 4 || b == 8;
+                    }
+                    if (lists && c->H.halo_ptr && takes_long_rows(c, V)) {
+                        if (!(V & kVariantWide)) continue;      // a candidate already
+                        V = (V & ~kVariantPrefetch) | kVariantHalo | kVariantStaged;
+                    }
+                }
                 // the staged-gather kernel sets its own block size; it needs real
                 // values and a matrix whose halo lists fit
                 if ((V & kVariantHalo) && (T != thread_opts[0] || c->H.cplx ||
