@@ -124,6 +124,9 @@ int fail(tbpm_ctx *c, int code, const std::string &m)
 {
     if (c) c->err = m;
     g_last_error = m;
+    // a refused allocation stays the thread's last error, which the next call's
+    // launch checks would read as their own
+    if (code == TBPM_E_OOM) cudaGetLastError();
     return code;
 }
 

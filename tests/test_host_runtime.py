@@ -113,3 +113,47 @@ def test_lists_are_built_for_the_widths_that_read_them(fake, S, lists):
         lib.tbpm_destroy(h)
         assert fake.fake_live() == 0
     """)
+
+
+# every allocation of a call fails once: the lists that the default builds on its
+# own are optional (the call succeeds without), any other failure is OOM, leaves
+# the context usable, and nothing of it stays allocated
+@pytest.mark.parametrize("what", ["states", "run", "adjoint"])
+def test_a_failing_allocation(fake, what):
+    run_script(fake, f"""
+        what = {what!r}
+        n, S, OOM = 2000, 4, 3
+        def prepare():
+            h = create()
+            if what == "asked": assert lib.tbpm_set_launch_config(h, FP32, 8, 64, 4609) == 0
+            if what == "build": return h
+            assert build(h, n, flags=16, deg=17) == 0
+            if what == "states": return h
+            assert states(h, n, S) == 0
+            if what == "lists": assert run(h, S, 20, FP32) == 0      # 80 states x steps of the 128
+            return h
+        def call(h):
+            if what == "build": return build(h, n, flags=16, deg=17)
+            if what == "states": return states(h, n, S)
+            if what == "adjoint":
+                g, a, b = dbl(2 * S * 4), dbl(17 * n), dbl(n)
+                return lib.tbpm_propagate_adjoint(h, Z, 3, g, HOST, 2, a, b, HOST)
+            return run(h, S, 20, FP32)
+        k = 0
+        while True:
+            h = prepare()
+            fake.fake_reset(k)
+            rc = call(h)
+            failed = fake.fake_failed()
+            fake.fake_reset(-1)
+            if what == "lists": assert rc == 0, (k, lib.tbpm_last_error(h))
+            else: assert rc == (OOM if failed else 0) or (rc == 0 and what in ("asked", "adjoint")), (k, rc)
+            assert call(h) == 0, (k, lib.tbpm_last_error(h))
+            clean()
+            lib.tbpm_destroy(h)
+            clean()
+            assert fake.fake_live() == 0, (k, fake.fake_live())
+            if not failed: break
+            k += 1
+        assert k >= 2
+    """)
