@@ -496,7 +496,7 @@ extern "C" int tbpm_build_hamiltonian(tbpm_ctx *c, int64_t n_orb, const double *
     // stage inputs on the device
     const double *d_on = nullptr, *d_hv = nullptr;
     const int64_t *d_hi = nullptr, *d_hj = nullptr;
-    bool o1, o2, o3, o4;
+    bool o1 = false, o2 = false, o3 = false, o4 = false;
     rc = stage(c, onsite, n_orb, where, const_cast<double **>(&d_on), &o1);
     if (!rc) rc = stage(c, hop_i, n_hop, where, const_cast<int64_t **>(&d_hi), &o2);
     if (!rc) rc = stage(c, hop_j, n_hop, where, const_cast<int64_t **>(&d_hj), &o3);

@@ -33,6 +33,23 @@ namespace {
         }                                                                     \
     } while (0)
 
+// Device memory of a build step, given back on every way out of it.
+template <typename T> struct Tmp {
+    T *p = nullptr;
+    Tmp() = default;
+    Tmp(const Tmp &) = delete;
+    Tmp &operator=(const Tmp &) = delete;
+    ~Tmp() { cudaFree(p); }
+    T **operator&() { return &p; }
+    operator T *() const { return p; }
+    T *keep()
+    {
+        T *q = p;
+        p = nullptr;
+        return q;
+    }
+};
+
 __device__ __forceinline__ int find_sample(const int64_t *off, int n_samples, int64_t u)
 {
     int lo = 0, hi = n_samples - 1;
@@ -137,7 +154,7 @@ int scan_exclusive(const int64_t *in, int64_t *out, int64_t n, cudaStream_t st,
                    std::string &msg)
 {
     int64_t nb = (n + kScanBlock - 1) / kScanBlock;
-    int64_t *sums = nullptr, *sums_scan = nullptr;
+    Tmp<int64_t> sums, sums_scan;
     CK(cudaMalloc(&sums, (nb + 1) * sizeof(int64_t)));
     CK(cudaMalloc(&sums_scan, (nb + 1) * sizeof(int64_t)));
     k_scan_block<<<(unsigned)nb, kScanBlock, 0, st>>>(in, out, n, sums);
@@ -155,8 +172,6 @@ int scan_exclusive(const int64_t *in, int64_t *out, int64_t n, cudaStream_t st,
         CK(cudaMemcpyAsync(out + n, sums, sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
     }
     CK(cudaStreamSynchronize(st));
-    cudaFree(sums);
-    cudaFree(sums_scan);
     return rc;
 }
 
@@ -807,16 +822,15 @@ int build_halo(BuildOutput &b, cudaStream_t st, std::string &msg)
     if (b.n_rows % kHaloRows) { msg = "rows are not a multiple of the halo block"; return TBPM_E_UNSUPPORTED; }
     const int64_t nb = b.n_rows / kHaloRows;
     const int64_t ns = b.n_slices;
-    int64_t *size = nullptr, *ent = nullptr, *pslice = nullptr;
+    Tmp<int64_t> size, ent, pslice, ptr;
     CK(cudaMalloc(&size, (nb + 1) * sizeof(int64_t)));
     CK(cudaMalloc(&ent, (ns + 1) * sizeof(int64_t)));
     CK(cudaMalloc(&pslice, (ns + 1) * sizeof(int64_t)));
     // packed slice offsets
     k_packed_slice_entries<<<blocks_for(ns, 256), 256, 0, st>>>(ns, b.slice_ptr, ent);
     CK(cudaGetLastError());
-    int rc0 = scan_exclusive(ent, pslice, ns, st, msg);
-    cudaFree(ent);
-    if (rc0) { cudaFree(size); cudaFree(pslice); return rc0; }
+    int rc = scan_exclusive(ent, pslice, ns, st, msg);
+    if (rc) return rc;
     std::vector<int64_t> hp(ns + 1);
     CK(cudaMemcpyAsync(hp.data(), pslice, (ns + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     k_halo_count<<<(unsigned)nb, kHaloThreads, 0, st>>>(b.slice_ptr, b.col, size);
@@ -830,48 +844,32 @@ int build_halo(BuildOutput &b, cudaStream_t st, std::string &msg)
     int64_t mx = 0;
     for (int64_t k = 0; k < nb; ++k) {
         if (hs[k] < 0) {
-            cudaFree(size);
-            cudaFree(pslice);
             msg = "a row block references more than " + std::to_string(kHaloMaxExt) +
                   " other rows: no halo lists for this matrix";
             return TBPM_E_UNSUPPORTED;
         }
         mx = std::max(mx, hs[k]);
     }
-    int64_t *ptr = nullptr;
     CK(cudaMalloc(&ptr, (nb + 1) * sizeof(int64_t)));
-    int rc = scan_exclusive(size, ptr, nb, st, msg);
-    cudaFree(size);
-    if (rc) { cudaFree(ptr); cudaFree(pslice); return rc; }
+    rc = scan_exclusive(size, ptr, nb, st, msg);
+    if (rc) return rc;
     int64_t total = 0;
     CK(cudaMemcpyAsync(&total, ptr + nb, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    int32_t *rows = nullptr;
-    uint16_t *lc = nullptr;
+    Tmp<int32_t> rows;
+    Tmp<uint16_t> lc;
     const int64_t npack = hp[ns];
-    cudaError_t e = cudaMalloc(&rows, total * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMalloc(&lc, (npack > 0 ? npack : 1) * sizeof(uint16_t));
-    if (e != cudaSuccess) {
-        cudaFree(ptr); cudaFree(rows); cudaFree(lc); cudaFree(pslice);
-        msg = std::string("halo lists: ") + cudaGetErrorString(e);
-        return e == cudaErrorMemoryAllocation ? TBPM_E_OOM : TBPM_E_CUDA;
-    }
-    e = cudaFuncSetAttribute(k_halo_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, kColorSmem);
-    if (e == cudaSuccess) {
-        k_halo_fill<<<(unsigned)nb, kHaloThreads, kColorSmem, st>>>(b.slice_ptr, b.col, ptr, pslice,
-                                                                     rows, lc);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) {
-        cudaFree(ptr); cudaFree(rows); cudaFree(lc); cudaFree(pslice);
-        msg = std::string("halo lists: ") + cudaGetErrorString(e);
-        return TBPM_E_CUDA;
-    }
-    b.halo_ptr = ptr;
-    b.halo_rows = rows;
-    b.lcol = lc;
-    b.pslice = pslice;
+    CK(cudaMalloc(&rows, total * sizeof(int32_t)));
+    CK(cudaMalloc(&lc, (npack > 0 ? npack : 1) * sizeof(uint16_t)));
+    CK(cudaFuncSetAttribute(k_halo_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, kColorSmem));
+    k_halo_fill<<<(unsigned)nb, kHaloThreads, kColorSmem, st>>>(b.slice_ptr, b.col, ptr, pslice, rows,
+                                                                 lc);
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(st));
+    b.halo_ptr = ptr.keep();
+    b.halo_rows = rows.keep();
+    b.lcol = lc.keep();
+    b.pslice = pslice.keep();
     b.n_packed = npack;
     b.halo_max = (int)mx;
     b.halo_ent_max = (int)std::min<int64_t>(emx, INT32_MAX);
@@ -979,10 +977,10 @@ int build_sell(const BuildInput &in, int keep64, int keep32, int detect_uniform,
         out.user_to_row, out.orb_sample);
     CK(cudaGetLastError());
 
-    int32_t *deg = nullptr, *fill = nullptr;
-    int64_t *entries = nullptr;
-    int *err = nullptr;           // [0] error bits, [1] max width
-    unsigned long long *gbits = nullptr;   // [0] Gershgorin bits, [1] bandwidth, [2] far lines
+    Tmp<int32_t> deg, fill;
+    Tmp<int64_t> entries;
+    Tmp<int> err;                 // [0] error bits, [1] max width
+    Tmp<unsigned long long> gbits;         // [0] Gershgorin bits, [1] bandwidth, [2] far lines
     CK(cudaMalloc(&deg, n_rows * sizeof(int32_t)));
     CK(cudaMalloc(&fill, n_rows * sizeof(int32_t)));
     CK(cudaMalloc(&entries, (n_slices + 1) * sizeof(int64_t)));
@@ -1002,23 +1000,19 @@ int build_sell(const BuildInput &in, int keep64, int keep32, int detect_uniform,
     int h_err[2] = {0, 0};
     CK(cudaMemcpyAsync(h_err, err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    auto cleanup = [&]() {
-        cudaFree(deg); cudaFree(fill); cudaFree(entries); cudaFree(err); cudaFree(gbits);
-    };
     if (h_err[0]) {
         msg = "invalid bond list:";
         if (h_err[0] & 1) msg += " index out of range;";
         if (h_err[0] & 2) msg += " bond from an orbital to itself;";
         if (h_err[0] & 4) msg += " bond joins two samples;";
         if (h_err[0] & 8) msg += " non-finite hopping;";
-        cleanup();
         return TBPM_E_INVALID_ARG;
     }
     k_slice_width<<<blocks_for(n_slices * 32, T), T, 0, st>>>(n_slices, deg, entries, err + 1);
     CK(cudaGetLastError());
     CK(cudaMalloc(&out.slice_ptr, (n_slices + 1) * sizeof(int64_t)));
     int rc = scan_exclusive(entries, out.slice_ptr, n_slices, st, msg);
-    if (rc) { cleanup(); return rc; }
+    if (rc) return rc;
     CK(cudaMemcpyAsync(&out.nnz_pad, out.slice_ptr + n_slices, sizeof(int64_t),
                        cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(&out.max_width, err + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1035,7 +1029,7 @@ int build_sell(const BuildInput &in, int keep64, int keep32, int detect_uniform,
         out.fixed_width = out.max_width;
         out.nnz_pad = n_slices * kSliceRows * (int64_t)out.max_width;
     }
-    if (out.nnz_pad > (int64_t)1 << 40) { msg = "matrix too large"; cleanup(); return TBPM_E_OOM; }
+    if (out.nnz_pad > (int64_t)1 << 40) { msg = "matrix too large"; return TBPM_E_OOM; }
 
     int64_t nnz_alloc = out.nnz_pad > 0 ? out.nnz_pad : 1;
     CK(cudaMalloc(&out.col, nnz_alloc * sizeof(int32_t)));
@@ -1145,7 +1139,6 @@ int build_sell(const BuildInput &in, int keep64, int keep32, int detect_uniform,
         out.val64 = nullptr;
         out.diag64 = nullptr;
     }
-    cleanup();
     return TBPM_OK;
 }
 
