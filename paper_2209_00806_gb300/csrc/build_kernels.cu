@@ -755,64 +755,45 @@ int build_groups(BuildOutput &b, cudaStream_t st, std::string &msg)
     if (b.gptr || b.no_groups) return TBPM_OK;
     if (!b.halo_ptr || !b.val32 || b.cplx) { msg = "no halo lists or FP32 values"; return TBPM_E_STATE; }
     const int64_t nb = b.n_rows / kHaloRows, no = nb * 4;
-    int64_t *len = nullptr, *ptr = nullptr;
-    uint8_t *perm = nullptr;
-    uint16_t *pos = nullptr;
-    float4 *val = nullptr;
-    auto drop = [&]() {
-        cudaFree(len);
-        cudaFree(ptr);
-        cudaFree(perm);
-        cudaFree(pos);
-        cudaFree(val);
-    };
+    Tmp<int64_t> len, ptr;
+    Tmp<uint8_t> perm;
+    Tmp<uint16_t> pos;
+    Tmp<float4> val;
     int64_t total = 0;
-    cudaError_t e = cudaMalloc(&len, (no + 1) * sizeof(int64_t));
-    if (e == cudaSuccess) e = cudaMalloc(&ptr, (no + 1) * sizeof(int64_t));
-    if (e == cudaSuccess) e = cudaMalloc(&perm, nb * 32);
-    if (e == cudaSuccess) {
+    auto steps = [&]() -> int {
+        CK(cudaMalloc(&len, (no + 1) * sizeof(int64_t)));
+        CK(cudaMalloc(&ptr, (no + 1) * sizeof(int64_t)));
+        CK(cudaMalloc(&perm, nb * 32));
         k_group_count<<<(unsigned)nb, 32, 0, st>>>(b.slice_ptr, b.col, perm, len);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) {
+        CK(cudaGetLastError());
         const int rc = scan_exclusive(len, ptr, no, st, msg);
-        if (rc) { drop(); return rc; }
-        e = cudaMemcpyAsync(&total, ptr + no, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    }
-    // no groups where the zeros would outweigh what the shared reads save, or
-    // where they would leave little memory for the caller's next states
-    if (e == cudaSuccess && (total * 32 > kGroupMaxFill * b.nnz_true ||
-                             !fits_beside((size_t)total * 8 * (sizeof(uint16_t) + sizeof(float4))))) {
-        drop();
-        b.no_groups = 1;
-        return TBPM_OK;
-    }
-    if (e == cudaSuccess) e = cudaMalloc(&pos, std::max<int64_t>(total, 1) * 8 * sizeof(uint16_t));
-    if (e == cudaSuccess) e = cudaMalloc(&val, std::max<int64_t>(total, 1) * 8 * sizeof(float4));
-    if (e == cudaSuccess) {
+        if (rc) return rc;
+        CK(cudaMemcpyAsync(&total, ptr + no, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        // no groups where the zeros would outweigh what the shared reads save, or
+        // where they would leave little memory for the caller's next states
+        b.no_groups = total * 32 > kGroupMaxFill * b.nnz_true ||
+                      !fits_beside((size_t)total * 8 * (sizeof(uint16_t) + sizeof(float4)));
+        if (b.no_groups) return TBPM_OK;
+        CK(cudaMalloc(&pos, std::max<int64_t>(total, 1) * 8 * sizeof(uint16_t)));
+        CK(cudaMalloc(&val, std::max<int64_t>(total, 1) * 8 * sizeof(float4)));
         k_group_fill<<<(unsigned)nb, 32, 0, st>>>(b.slice_ptr, b.col, b.val32, b.pslice, b.lcol, perm,
-                                                 ptr, pos, val);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(len);
-    len = nullptr;
-    if (e == cudaErrorMemoryAllocation) {        // the packed entries serve instead
+                                                  ptr, pos, val);
+        CK(cudaGetLastError());
+        CK(cudaStreamSynchronize(st));
+        return TBPM_OK;
+    };
+    const int rc = steps();
+    if (rc == TBPM_E_OOM) {                      // the packed entries serve instead
         cudaGetLastError();
-        drop();
         b.no_groups = 1;
         return TBPM_OK;
     }
-    if (e != cudaSuccess) {
-        drop();
-        msg = std::string("row groups: ") + cudaGetErrorString(e);
-        return TBPM_E_CUDA;
-    }
-    b.gptr = ptr;
-    b.gperm = perm;
-    b.gpos = pos;
-    b.gval = val;
+    if (rc || b.no_groups) return rc;
+    b.gptr = ptr.keep();
+    b.gperm = perm.keep();
+    b.gpos = pos.keep();
+    b.gval = val.keep();
     return TBPM_OK;
 }
 

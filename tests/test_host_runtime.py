@@ -118,7 +118,7 @@ def test_lists_are_built_for_the_widths_that_read_them(fake, S, lists):
 # every allocation of a call fails once: the lists that the default builds on its
 # own are optional (the call succeeds without), any other failure is OOM, leaves
 # the context usable, and nothing of it stays allocated
-@pytest.mark.parametrize("what", ["asked", "build", "states", "run", "adjoint"])
+@pytest.mark.parametrize("what", ["lists", "asked", "build", "states", "run", "adjoint"])
 def test_a_failing_allocation(fake, what):
     run_script(fake, f"""
         what = {what!r}
