@@ -30,10 +30,13 @@ struct Group {
 
 }  // namespace
 
-// Results of a call that come back together: up to this many bytes go through
-// a page-locked buffer of the context with one wait; more are copied directly.
+// The results of a run are one allocation -- flags and renormalisation count,
+// norms, C -- and come back in one copy, with C up to this many bytes; more of C
+// goes to the caller directly.
 constexpr size_t kResBytes = 64 * 1024;
 constexpr size_t kFlagBytes = 4 * sizeof(int) + sizeof(unsigned long long);
+constexpr size_t kNormsAt = 32;
+static size_t corr_at(size_t cnt) { return (kNormsAt + cnt * sizeof(double) + 15) / 16 * 16; }
 
 struct tbpm_ctx {
     int device = 0;
@@ -56,7 +59,6 @@ struct tbpm_ctx {
     double2 *d_psi_user = nullptr;
     size_t psi_count = 0;        // elements it holds
     cudaEvent_t ev_order = nullptr;        // orders our stream and the user's
-    unsigned char *h_res = nullptr;        // page-locked, kResBytes: small results (first run)
 
     // propagation state
     int prec = -1;               // precision of the group buffers
@@ -91,7 +93,9 @@ struct tbpm_ctx {
     double *d_tile_partial = nullptr;
     int64_t tile_partial_len = 0;
     int *d_step = nullptr;       // [n_samples]
-    int *d_flags = nullptr;      // [0] error bits
+    int *d_flags0 = nullptr;     // without results yet
+    unsigned char *d_out = nullptr;        // the results (see kResBytes)
+    int *d_flags = nullptr;      // [0] error bits; in the results, or d_flags0
     unsigned long long *d_renorm = nullptr;
     double2 *d_corr = nullptr;
     double *d_norms = nullptr;
@@ -172,8 +176,10 @@ void free_groups(tbpm_ctx *c)
 
 void free_outputs(tbpm_ctx *c)
 {
-    cudaFree(c->d_corr);
-    cudaFree(c->d_norms);
+    cudaFree(c->d_out);
+    c->d_out = nullptr;
+    c->d_flags = c->d_flags0;
+    c->d_renorm = nullptr;
     c->d_corr = nullptr;
     c->d_norms = nullptr;
     c->corr_steps = -1;
@@ -391,8 +397,8 @@ extern "C" int tbpm_create(tbpm_ctx **out, int device, void *stream)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->st, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_order, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_flags, kFlagBytes);       // flags, renorm count
-    if (e == cudaSuccess) c->d_renorm = (unsigned long long *)(c->d_flags + 4);
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_flags0, 4 * sizeof(int));
+    if (e == cudaSuccess) c->d_flags = c->d_flags0;
     if (e != cudaSuccess) {
         std::string m = std::string("context setup: ") + cudaGetErrorString(e);
         tbpm_destroy(c);
@@ -408,8 +414,7 @@ extern "C" void tbpm_destroy(tbpm_ctx *c)
     cudaSetDevice(c->device);
     if (c->st) cudaStreamSynchronize(c->st);
     free_hamiltonian(c);
-    cudaFree(c->d_flags);
-    cudaFreeHost(c->h_res);
+    cudaFree(c->d_flags0);
     if (c->ev_order) cudaEventDestroy(c->ev_order);
     for (auto e : c->events) cudaEventDestroy(e);
     if (c->st) cudaStreamDestroy(c->st);
@@ -982,16 +987,17 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
 
     int rc = enter(c);
     if (rc) return rc;
-    if (!c->h_res)
-        CUDA_OR_FAIL(c, cudaHostAlloc((void **)&c->h_res, kResBytes, cudaHostAllocDefault));
     rc = ensure_groups(c, precision);
     if (rc) return rc;
     if (c->corr_steps != n_steps || c->corr_states != c->n_states) {
         free_outputs(c);
         const size_t cnt = (size_t)c->n_samples * c->n_states * (n_steps + 1);
-        rc = dalloc(c, &c->d_corr, cnt);
-        if (!rc) rc = dalloc(c, &c->d_norms, cnt);
+        rc = dalloc(c, &c->d_out, corr_at(cnt) + cnt * sizeof(double2));
         if (rc) return rc;
+        c->d_flags = (int *)c->d_out;
+        c->d_renorm = (unsigned long long *)(c->d_flags + 4);
+        c->d_norms = (double *)(c->d_out + kNormsAt);
+        c->d_corr = (double2 *)(c->d_out + corr_at(cnt));
         c->corr_steps = n_steps;
         c->corr_states = c->n_states;
     }
@@ -1547,10 +1553,9 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         if (profile)
             for (int q = 2; q < 5; ++q) CUDA_OR_FAIL(c, cudaEventRecord(c->events[e0 + q], c->st));
         // (the host tables go out of scope)
-        CUDA_OR_FAIL(c, cudaMemcpyAsync(c->h_res, c->d_flags, kFlagBytes, cudaMemcpyDeviceToHost, c->st));
-        CUDA_OR_FAIL(c, cudaStreamSynchronize(c->st));
         int hf = 0;
-        memcpy(&hf, c->h_res, sizeof(hf));
+        CUDA_OR_FAIL(c, cudaMemcpyAsync(&hf, c->d_flags, sizeof(hf), cudaMemcpyDeviceToHost, c->st));
+        CUDA_OR_FAIL(c, cudaStreamSynchronize(c->st));
         if (fp32 && (hf & 8)) {
             // a bound within the rounding of a step, which would rescale and repeat
             // every one: the launch ended there; the per-term kernels, from the same start
@@ -1576,27 +1581,21 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     int h_flags[4];
     unsigned long long h_renorm = 0;
     const size_t cnt = (size_t)c->n_samples * c->n_states * (n_steps + 1);
-    std::vector<double> norms(cnt);
-    const size_t norm_b = cnt * sizeof(double);
     const size_t corr_b = corr_out && where_out == TBPM_HOST ? cnt * sizeof(double2) : 0;
-    const size_t at_norm = 32, at_corr = at_norm + norm_b;
-    const bool small = at_corr + corr_b <= kResBytes;
-    CUDA_OR_FAIL(c, cudaMemcpyAsync(c->h_res, c->d_flags, kFlagBytes, cudaMemcpyDeviceToHost, c->st));
-    CUDA_OR_FAIL(c, cudaMemcpyAsync(small ? (void *)(c->h_res + at_norm) : norms.data(), c->d_norms,
-                                    norm_b, cudaMemcpyDeviceToHost, c->st));
-    if (corr_b)
-        CUDA_OR_FAIL(c, cudaMemcpyAsync(small ? (void *)(c->h_res + at_corr) : corr_out, c->d_corr,
-                                        corr_b, cudaMemcpyDeviceToHost, c->st));
-    else if (corr_out)
+    const bool small = corr_at(cnt) + corr_b <= kResBytes;
+    const size_t res_b = corr_at(cnt) + (small ? corr_b : 0);
+    std::vector<double> res(res_b / sizeof(double));
+    CUDA_OR_FAIL(c, cudaMemcpyAsync(res.data(), c->d_out, res_b, cudaMemcpyDeviceToHost, c->st));
+    if (corr_b && !small)
+        CUDA_OR_FAIL(c, cudaMemcpyAsync(corr_out, c->d_corr, corr_b, cudaMemcpyDeviceToHost, c->st));
+    else if (corr_out && !corr_b)
         CUDA_OR_FAIL(c, cudaMemcpyAsync(corr_out, c->d_corr, cnt * sizeof(double2),
                                         cudaMemcpyDeviceToDevice, c->st));
     CUDA_OR_FAIL(c, cudaStreamSynchronize(c->st));
-    memcpy(h_flags, c->h_res, sizeof(h_flags));
-    memcpy(&h_renorm, c->h_res + sizeof(h_flags), sizeof(h_renorm));
-    if (small) {
-        memcpy(norms.data(), c->h_res + at_norm, norm_b);
-        if (corr_b) memcpy(corr_out, c->h_res + at_corr, corr_b);
-    }
+    const double *norms = res.data() + kNormsAt / sizeof(double);
+    memcpy(h_flags, res.data(), sizeof(h_flags));
+    memcpy(&h_renorm, res.data() + 2, sizeof(h_renorm));
+    if (small && corr_b) memcpy(corr_out, res.data() + corr_at(cnt) / sizeof(double), corr_b);
     c->have_run = true;
 
     tbpm_stats &S = c->stats;

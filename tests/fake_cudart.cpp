@@ -18,7 +18,7 @@ namespace {
 std::map<char *, size_t> live;
 std::map<const void *, int> limit;
 std::string found;
-long countdown = -1, failed = 0;
+long countdown = -1, failed = 0, pinned = 0;
 cudaError_t last = cudaSuccess;
 
 cudaError_t keep(cudaError_t e)
@@ -59,6 +59,7 @@ void fake_reset(long k) { found.clear(); countdown = k; failed = 0; }
 const char *fake_report() { return found.c_str(); }
 long fake_live() { return (long)live.size(); }
 long fake_failed() { return failed; }
+long fake_pinned() { return pinned; }
 
 cudaError_t cudaMalloc(void **p, size_t n)
 {
@@ -77,7 +78,12 @@ cudaError_t cudaFree(void *p)
     else free(p);
     return cudaSuccess;
 }
-cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { *p = malloc(n); return cudaSuccess; }
+cudaError_t cudaHostAlloc(void **p, size_t n, unsigned)
+{
+    ++pinned;
+    *p = malloc(n);
+    return cudaSuccess;
+}
 cudaError_t cudaFreeHost(void *p) { free(p); return cudaSuccess; }
 cudaError_t cudaMemGetInfo(size_t *f, size_t *t) { *f = *t = (size_t)1 << 38; return cudaSuccess; }
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { return copy(d, s, n); }

@@ -15,7 +15,7 @@ import ctypes as C, os, sys
 fake = C.CDLL(sys.argv[1], mode=C.RTLD_GLOBAL)
 fake.fake_report.restype = C.c_char_p
 fake.fake_reset.argtypes = [C.c_long]
-fake.fake_live.restype = fake.fake_failed.restype = C.c_long
+fake.fake_live.restype = fake.fake_failed.restype = fake.fake_pinned.restype = C.c_long
 lib = C.CDLL(sys.argv[2])
 lib.tbpm_last_error.restype = C.c_char_p
 lib.tbpm_last_error.argtypes = [C.c_void_p]
@@ -156,4 +156,15 @@ def test_a_failing_allocation(fake, what):
             if not failed: break
             k += 1
         assert k >= 2
+    """)
+
+
+# one-shot contexts pay for no page-locked memory (0.2 ms), whatever the size of C
+@pytest.mark.parametrize("steps", [4, 3000])
+def test_a_first_run_locks_no_pages(fake, steps):
+    run_script(fake, f"""
+        h = create()
+        assert build(h, 700) == 0 and states(h, 700, 2) == 0 and run(h, 2, {steps}, FP32) == 0
+        assert fake.fake_pinned() == 0
+        clean()
     """)
