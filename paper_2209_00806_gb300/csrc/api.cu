@@ -1460,6 +1460,10 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
             if (c->qe_on) launches += 1; // quasi-eigenstate accumulation
         }
     }
+    // host tables of the cluster stepping (they live until the results are back)
+    std::vector<FusedTerm> tabs;
+    std::vector<ClusterState> cst;
+    int cur0 = 0, keep = 0;
     if (Kc > 0) {
         if (!c->d_fterms) {
             rc = dalloc(c, &c->d_fterms, 3 * (size_t)kMaxTerms);
@@ -1469,15 +1473,15 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
             rc = dalloc(c, &c->d_cstates, (size_t)kMaxStates);
             if (rc) return rc;
         }
-        std::vector<FusedTerm> tabs(3 * (size_t)kMaxTerms);
+        tabs.resize(3 * (size_t)kMaxTerms);
         ClusterArgs ca;
         memset(&ca, 0, sizeof(ca));
-        for (int cur0 = 0; cur0 < 3; ++cur0) {
+        for (int from = 0; from < 3; ++from) {
             int nx = 0;
-            std::vector<Launch> sch = schedule(a, cur0, &nx);
-            ca.next_cur[cur0] = nx;
+            std::vector<Launch> sch = schedule(a, from, &nx);
+            ca.next_cur[from] = nx;
             for (size_t k = 0; k < sch.size(); ++k) {
-                FusedTerm &ft = tabs[cur0 * kMaxTerms + k];
+                FusedTerm &ft = tabs[from * kMaxTerms + k];
                 ft.x = sch[k].x;
                 ft.z = sch[k].z;
                 ft.out = sch[k].out;
@@ -1490,17 +1494,16 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
                 one_value_table(c->H, ft);
             }
         }
-        const int cur0 = c->groups[0].cur;           // the groups step alike
+        cur0 = c->groups[0].cur;                     // the groups step alike
         int cur1 = cur0;
         for (int n = 0; n < n_steps; ++n) cur1 = ca.next_cur[cur1];
         // a resumed FP32 run may have to be repeated: its state, kept in a
         // buffer that the result does not take
-        const int keep = 3 - cur0 - (cur1 == cur0 ? (cur0 + 1) % 3 : cur1);
+        keep = 3 - cur0 - (cur1 == cur0 ? (cur0 + 1) % 3 : cur1);
         if (fp32 && resume)
             for (auto &g : c->groups)
                 CUDA_OR_FAIL(c, cudaMemcpyAsync(g.buf[keep], g.buf[cur0], (size_t)c->H.n_rows * g.B * cs,
                                                 cudaMemcpyDeviceToDevice, c->st));
-        std::vector<ClusterState> cst;
         for (auto &g : c->groups)
             for (int b = 0; b < g.B; ++b) {
                 ClusterState cs1;
@@ -1552,25 +1555,6 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
             return fail(c, TBPM_E_CUDA, std::string("cluster steps: ") + cudaGetErrorString(e));
         if (profile)
             for (int q = 2; q < 5; ++q) CUDA_OR_FAIL(c, cudaEventRecord(c->events[e0 + q], c->st));
-        // (the host tables go out of scope)
-        int hf = 0;
-        CUDA_OR_FAIL(c, cudaMemcpyAsync(&hf, c->d_flags, sizeof(hf), cudaMemcpyDeviceToHost, c->st));
-        CUDA_OR_FAIL(c, cudaStreamSynchronize(c->st));
-        if (fp32 && (hf & 8)) {
-            // a bound within the rounding of a step, which would rescale and repeat
-            // every one: the launch ended there; the per-term kernels, from the same start
-            if (resume)
-                for (auto &g : c->groups) {
-                    CUDA_OR_FAIL(c, cudaMemcpyAsync(g.buf[cur0], g.buf[keep],
-                                                    (size_t)c->H.n_rows * g.B * cs,
-                                                    cudaMemcpyDeviceToDevice, c->st));
-                    g.cur = cur0;
-                }
-            c->cluster_off = true;
-            rc = tbpm_propagate(c, z, n_steps, precision, corr_out, where_out, flags);
-            c->cluster_off = false;
-            return rc;
-        }
         for (auto &g : c->groups) g.cur = cur1;
         launches += 1;
         cluster_run = true;
@@ -1595,6 +1579,20 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     const double *norms = res.data() + kNormsAt / sizeof(double);
     memcpy(h_flags, res.data(), sizeof(h_flags));
     memcpy(&h_renorm, res.data() + 2, sizeof(h_renorm));
+    if (cluster_run && fp32 && (h_flags[0] & 8)) {
+        // a bound within the rounding of a step, which would rescale and repeat
+        // every one: the launch ended there; the per-term kernels, from the same start
+        for (auto &g : c->groups) {
+            g.cur = cur0;
+            if (resume)
+                CUDA_OR_FAIL(c, cudaMemcpyAsync(g.buf[cur0], g.buf[keep], (size_t)c->H.n_rows * g.B * cs,
+                                                cudaMemcpyDeviceToDevice, c->st));
+        }
+        c->cluster_off = true;
+        rc = tbpm_propagate(c, z, n_steps, precision, corr_out, where_out, flags);
+        c->cluster_off = false;
+        return rc;
+    }
     if (small && corr_b) memcpy(corr_out, res.data() + corr_at(cnt) / sizeof(double), corr_b);
     c->have_run = true;
 

@@ -18,7 +18,7 @@ namespace {
 std::map<char *, size_t> live;
 std::map<const void *, int> limit;
 std::string found;
-long countdown = -1, failed = 0, pinned = 0;
+long countdown = -1, failed = 0, pinned = 0, waits = 0;
 cudaError_t last = cudaSuccess;
 
 cudaError_t keep(cudaError_t e)
@@ -60,6 +60,7 @@ const char *fake_report() { return found.c_str(); }
 long fake_live() { return (long)live.size(); }
 long fake_failed() { return failed; }
 long fake_pinned() { return pinned; }
+long fake_waits() { return waits; }
 
 cudaError_t cudaMalloc(void **p, size_t n)
 {
@@ -141,7 +142,7 @@ cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { *v = 152; retu
 cudaError_t cudaGetSymbolAddress(void **, const void *) { return cudaErrorInvalidValue; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { *s = nullptr; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { ++waits; return cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaErrorNotSupported; }
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *) { return cudaErrorNotSupported; }

@@ -15,7 +15,7 @@ import ctypes as C, os, sys
 fake = C.CDLL(sys.argv[1], mode=C.RTLD_GLOBAL)
 fake.fake_report.restype = C.c_char_p
 fake.fake_reset.argtypes = [C.c_long]
-fake.fake_live.restype = fake.fake_failed.restype = fake.fake_pinned.restype = C.c_long
+fake.fake_live.restype = fake.fake_failed.restype = fake.fake_pinned.restype = fake.fake_waits.restype = C.c_long
 lib = C.CDLL(sys.argv[2])
 lib.tbpm_last_error.restype = C.c_char_p
 lib.tbpm_last_error.argtypes = [C.c_void_p]
@@ -166,5 +166,20 @@ def test_a_first_run_locks_no_pages(fake, steps):
         h = create()
         assert build(h, 700) == 0 and states(h, 700, 2) == 0 and run(h, 2, {steps}, FP32) == 0
         assert fake.fake_pinned() == 0
+        clean()
+    """)
+
+
+# a run waits for the device once, stepped in clusters as term by term
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("config", [None, 1])
+def test_a_run_waits_once(fake, prec, config):
+    run_script(fake, f"""
+        h = create()
+        if {config}: assert lib.tbpm_set_launch_config(h, {prec}, 8, 64, {config}) == 0
+        assert build(h, 700) == 0 and states(h, 700, 3) == 0 and run(h, 3, 5, {prec}) == 0
+        before = fake.fake_waits()
+        assert run(h, 3, 5, {prec}) == 0
+        assert fake.fake_waits() == before + 1
         clean()
     """)
