@@ -107,8 +107,9 @@ typedef struct tbpm_stats {
     double gershgorin;       /* Gershgorin bound of H~ = H / s (dimensionless) */
     double ms_total;         /* device time of the last call (PROFILE) */
     double ms_term_avg;      /* average duration of one interior Chebyshev
-                                term kernel (PROFILE); with the fused step,
-                                its time divided by the M-1 terms */
+                                term kernel (PROFILE); with the fused step or
+                                the cluster stepping, a step's time divided by
+                                the M-1 terms */
     double ms_final_avg;     /* average duration of the closing term kernel */
     double ms_reduce_avg;    /* average duration of the correlation reduction */
     int64_t term_launches;   /* interior term launches that were timed */
@@ -359,7 +360,9 @@ int tbpm_dos_adjoint(const double *dl_dd, int n_e, int n_steps, double tau, int 
                                         otherwise ignored.  Until a launch shape is
                                         set it is the default up to 16 x 512 rows
                                         (FP32: all it takes with up to seven states,
-                                        16 x 1024 rows up to sixteen) */
+                                        16 x 1024 rows up to sixteen) where it is
+                                        estimated to be the faster way: not for rows
+                                        whose neighbours lie scattered over the blocks */
 #define TBPM_VARIANT_PIPE 1024       /* with TBPM_VARIANT_HALO, interior terms: a
                                         persistent grid (one block per SM) with two
                                         shared-memory stages, the next block's halo,

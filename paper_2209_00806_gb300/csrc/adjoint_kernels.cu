@@ -36,8 +36,9 @@ namespace {
 // operations (2 + 2E without c) and 2 + 2E for the gradients: 18 on graphene,
 // against 36 with gamma and the weight multiplied in, entries in rounds of
 // four and one thread per state (whose partial gradients had to be added by
-// shuffles).  524,288 rows x 2 states: 68 -> 43 us a gradient term, 36 -> 20 us
-// a plain one.
+// shuffles).  524,288 rows x 2 states: 36 us a gradient term (68 before; 45 us the
+// first of a step, 52 us the closing one), 19 us a plain one (36 before), 23 us with
+// the next state's share.
 // ACC (polynomials): the term's share of the next state too, next += ca out
 // (2: the first polynomial, next = c x + ca out); out may then be nullptr.
 template <int L, int SPL, int W, bool HASC, bool FAC, bool GRAD, bool WFAC, int ACC = 0>

@@ -1,20 +1,21 @@
 // Cluster-resident time stepping for small samples (TBPM_VARIANT_CLUSTER).
 //
-// A sample of up to 16 x 1024 rows -- the 64 x 64 graphene DOS workload has
-// 8192 -- fits, with psi0, psi and the two Clenshaw buffers, in the shared
-// memory of one thread-block cluster.  All time steps of the propagation then
-// run in one launch, one cluster per state: each block holds a contiguous range of rows (one row per
-// thread), gathers x from the owning block's shared memory (distributed
-// shared memory across the cluster), and a cluster barrier separates the
-// Clenshaw terms (Sec. 2.2, Eq. psi_t).  The closing term's sums of
-// <psi0|phi> and <phi|phi> are formed per block in a fixed tree after the
-// block has arrived at the term's barrier (no later term needs them), and
-// added over the blocks in rank order by block 0 two barriers later (FP64,
-// deterministic).  Per row
-// the arithmetic and its order are those of the plain term kernel, so the
-// states equal the per-term launches' bit for bit; the launch cost of
-// 15 kernels per step is gone.  FP64 states, real values, at most
-// kClusterMaxW entries per row, within the shared memory of a block.
+// A small sample -- the 64 x 64 graphene DOS workload has 8192 rows -- fits, with
+// psi0, psi and the two Clenshaw buffers, in the shared memory of one thread-block
+// cluster of 16 blocks (8 where the device runs no larger one).  All time steps of
+// the propagation then run in one launch, one cluster per state: each block holds a
+// contiguous range of rows, gathers x from the owning block's shared memory
+// (distributed shared memory across the cluster), and a cluster barrier separates
+// the Clenshaw terms (Sec. 2.2, Eq. psi_t).  FP64 takes a row a thread, up to
+// 16 x 1024 rows; FP32 up to eight rows a thread, 16 x 4096 rows with three slots a
+// row and 16 x 1024 otherwise.  Real values, at most kClusterMaxW entries per row.
+// The closing term's sums of <psi0|phi> and <phi|phi> are formed per block in a
+// fixed tree after the block has arrived at the term's barrier (no later term
+// needs them), and added over the blocks in a fixed tree by block 0 two barriers
+// later (FP64 throughout, or float pairs up to the block; deterministic).  Per row
+// the arithmetic and its order are those of the plain term kernel, so the states
+// equal the per-term launches' bit for bit; the launch cost of 15 kernels per step
+// is gone.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -317,9 +318,9 @@ __device__ __forceinline__ FF warp_sum3(FF v0, FF v1, FF v2)
 // rounding and would run every step twice: the launch ends there with error bit
 // 8, and the caller repeats the run with the per-term kernels.  4,096 steps at
 // the default bound: 9.8 us a step at 64 x 64 and 25 us at 180 x 180 (repeated
-// whole by the per-term kernels: 51 and 70 us).  Bound by the latency of a term (barrier, distributed
-// shared-memory gathers): 64 x 64 graphene, one state, 10 us a step against
-// 42 us of dependent launches; 180 x 180 25 against 47 us.
+// whole by the per-term kernels: 51 and 70 us).  Bound by the latency of a term
+// (barrier, distributed shared-memory gathers): 64 x 64 graphene, one state, 10 us
+// a step against 42 us of dependent launches; 180 x 180 25 against 47 us.
 template <int MAXW, int RPT, Vals M>
 __global__ void __launch_bounds__(512, 1) k_cluster_steps_f32(ClusterArgs a)
 {

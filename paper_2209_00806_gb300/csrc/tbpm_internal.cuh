@@ -149,7 +149,7 @@ constexpr int kVariantSplit2 = 128;     // each row's entries over 2 threads
 constexpr int kVariantSplit4 = 256;     // each row's entries over 4 threads
 constexpr int kVariantHalo = 512;       // gathers from a shared-memory copy of the block's halo
 constexpr int kVariantPipe = 1024;      // with kVariantHalo: persistent, two stages in flight
-constexpr int kVariantCluster = 2048;   // small FP64 samples: all steps in one cluster launch
+constexpr int kVariantCluster = 2048;   // small samples: all steps in one launch, a cluster a state
 constexpr int kVariantStaged = 4096;    // with kVariantHalo: one stage, two blocks per SM
 constexpr int kVariantPrefetch = 8192;  // FP32: persistent term kernel, next row's indices loaded ahead
 
