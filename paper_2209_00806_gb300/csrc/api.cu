@@ -1686,7 +1686,7 @@ extern "C" int tbpm_correlation(tbpm_ctx *c, double *out, int where_out)
     if (!c || !out) return fail(c, TBPM_E_INVALID_ARG, "NULL argument");
     if (where_out != TBPM_HOST && where_out != TBPM_DEVICE)
         return fail(c, TBPM_E_INVALID_ARG, "where_out must be TBPM_HOST or TBPM_DEVICE");
-    if (!c->have_run) return fail(c, TBPM_E_STATE, "no propagation yet");
+    if (!c->have_run || !c->d_out) return fail(c, TBPM_E_STATE, "no propagation yet");
     const int n1 = c->corr_steps + 1;
     const size_t cnt = (size_t)c->n_samples * n1;
     int rc = enter(c);
@@ -1778,7 +1778,7 @@ extern "C" int tbpm_get_states(tbpm_ctx *c, double *phi_out, int where_out)
 extern "C" int tbpm_get_norms(tbpm_ctx *c, double *out)
 {
     if (!c || !out) return fail(c, TBPM_E_INVALID_ARG, "NULL argument");
-    if (!c->have_run) return fail(c, TBPM_E_STATE, "no propagation yet");
+    if (!c->have_run || !c->d_out) return fail(c, TBPM_E_STATE, "no propagation yet");
     const size_t cnt = (size_t)c->n_samples * c->n_states * (c->corr_steps + 1);
     CUDA_OR_FAIL(c, cudaMemcpy(out, c->d_norms, cnt * sizeof(double), cudaMemcpyDeviceToHost));
     return TBPM_OK;

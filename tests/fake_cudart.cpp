@@ -2,7 +2,7 @@
 // without a GPU.  Device memory is host memory, kernels do nothing, and every
 // copy, set and launch is checked the way the device would:
 //  - a copy's or set's device range lies inside one live allocation,
-//  - a launch's dynamic shared memory is within its kernel's limit,
+//  - a launch has blocks, and its dynamic shared memory is within its kernel's limit,
 //  - the limit of a kernel is not lowered (it belongs to the process, so
 //    lowering it refuses another thread's launch in between).
 // fake_reset(k) clears the records and makes the k-th allocation from then on
@@ -36,8 +36,9 @@ void check(const char *what, const void *p, size_t n)
         found += std::string(what) + " " + std::to_string(at + n - it->second) +
                  " bytes past an allocation of " + std::to_string(it->second) + "; ";
 }
-cudaError_t launch(const void *f, size_t smem)
+cudaError_t launch(const void *f, dim3 grid, size_t smem)
 {
+    if (!grid.x || !grid.y || !grid.z) return keep(cudaErrorInvalidConfiguration);
     const auto it = limit.find(f);
     const size_t most = it == limit.end() ? 48 * 1024 : it->second;
     if (smem <= most) return cudaSuccess;
@@ -106,16 +107,16 @@ cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute a, int v)
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **)
 {
-    return launch(f, c->dynamicSmemBytes);
+    return launch(f, c->gridDim, c->dynamicSmemBytes);
 }
-cudaError_t cudaLaunchCooperativeKernel(const void *f, dim3, dim3, void **, size_t smem, cudaStream_t)
+cudaError_t cudaLaunchCooperativeKernel(const void *f, dim3 grid, dim3, void **, size_t smem, cudaStream_t)
 {
-    return launch(f, smem);
+    return launch(f, grid, smem);
 }
 cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) { *k = (cudaKernel_t)f; return cudaSuccess; }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **, size_t smem, cudaStream_t)
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void **, size_t smem, cudaStream_t)
 {
-    return launch((const void *)k, smem);
+    return launch((const void *)k, grid, smem);
 }
 cudaError_t cudaFuncGetAttributes(cudaFuncAttributes *a, const void *) { memset(a, 0, sizeof *a); return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned)

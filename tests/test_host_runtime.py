@@ -183,3 +183,21 @@ def test_a_run_waits_once(fake, prec, config):
         assert fake.fake_waits() == before + 1
         clean()
     """)
+
+
+# a run whose result buffers cannot be had leaves no results of the last one to
+# read, but states to go on from
+def test_no_results_after_a_failed_run(fake):
+    run_script(fake, """
+        h = create()
+        assert build(h, 700) == 0 and states(h, 700, 2) == 0 and run(h, 2, 5, FP64) == 0
+        fake.fake_reset(0)
+        assert run(h, 2, 9, FP64) == 3 and fake.fake_failed() == 1
+        fake.fake_reset(-1)
+        avg, norms = dbl(40), dbl(40)
+        assert lib.tbpm_correlation(h, avg, HOST) == 8       # TBPM_E_STATE
+        assert lib.tbpm_get_norms(h, norms) == 8
+        assert run(h, 2, 9, FP64, 4) == 0                    # TBPM_PROP_RESUME
+        assert lib.tbpm_correlation(h, avg, HOST) == 0 and lib.tbpm_get_norms(h, norms) == 0
+        clean()
+    """)
