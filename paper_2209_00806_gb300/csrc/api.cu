@@ -920,7 +920,10 @@ static int ensure_fused(tbpm_ctx *c, int J, int R, int radius, int maxB, int gri
     }
     if (!c->d_fcounter) {
         int rc = dalloc(c, &c->d_fcounter, 1);
-        if (!rc) rc = dalloc(c, &c->d_fterms, 3 * (size_t)kMaxTerms);
+        if (rc) return rc;
+    }
+    if (!c->d_fterms) {             // (the cluster stepping may have it already)
+        int rc = dalloc(c, &c->d_fterms, 3 * (size_t)kMaxTerms);
         if (rc) return rc;
     }
     if (c->tile_partial_len < T * maxB * 3) {

@@ -201,3 +201,15 @@ def test_no_results_after_a_failed_run(fake):
         assert lib.tbpm_correlation(h, avg, HOST) == 0 and lib.tbpm_get_norms(h, norms) == 0
         clean()
     """)
+
+
+# the cluster stepping's tables and the fused step's are the same memory
+def test_fused_after_cluster_keeps_no_memory(fake):
+    run_script(fake, """
+        h = create()
+        assert build(h, 700) == 0 and states(h, 700, 1) == 0
+        assert run(h, 1, 5, FP64) == 0 and run(h, 1, 5, FP64, 8) == 0       # TBPM_PROP_PERSISTENT
+        lib.tbpm_destroy(h)
+        clean()
+        assert fake.fake_live() == 0
+    """)
