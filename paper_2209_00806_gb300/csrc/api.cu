@@ -157,6 +157,19 @@ int dalloc(tbpm_ctx *c, T **p, size_t count)
     return TBPM_OK;
 }
 
+// At least `count` elements in *p, which holds *len: none, and a length of zero,
+// after a failure.
+template <typename T>
+int grow(tbpm_ctx *c, T **p, int64_t *len, int64_t count)
+{
+    if (count <= *len) return TBPM_OK;
+    cudaFree(*p);
+    *len = 0;
+    const int rc = dalloc(c, p, (size_t)count);
+    if (!rc) *len = count;
+    return rc;
+}
+
 void free_groups(tbpm_ctx *c)
 {
     for (auto &g : c->groups) {
@@ -754,38 +767,24 @@ static int ensure_groups(tbpm_ctx *c, int prec)
     }
     int maxB = 1;
     for (auto &g : c->groups) maxB = std::max(maxB, g.B);
-    const int64_t need = c->H.n_rows / kChunkRows * maxB * 3;
-    if (need > c->partial_len) {
-        cudaFree(c->d_partial);
-        c->d_partial = nullptr;
-        int rc = dalloc(c, &c->d_partial, need);
-        if (rc) { free_groups(c); return rc; }
-        c->partial_len = need;
-    }
+    int rc = grow(c, &c->d_partial, &c->partial_len, c->H.n_rows / kChunkRows * maxB * 3);
     // block partials of the closing term: one per block of the launch shape
     int64_t need_b = 0;
     for (auto &g : c->groups) {
         const int L = prec == TBPM_FP64 ? g.B : std::max(1, g.B / 2);
         need_b = std::max<int64_t>(need_b, c->H.n_rows * L / 128 * g.B * 3);   // closing-term blocks of 128
     }
-    if (need_b > c->block_partial_len) {
-        cudaFree(c->d_block_partial);
-        c->d_block_partial = nullptr;
-        int rc = dalloc(c, &c->d_block_partial, need_b);
-        if (rc) { free_groups(c); return rc; }
-        c->block_partial_len = need_b;
+    if (!rc) rc = grow(c, &c->d_block_partial, &c->block_partial_len, need_b);
+    if (!rc && !c->d_chunk_count) {
+        rc = dalloc(c, &c->d_chunk_count, c->H.n_rows / kChunkRows);
+        if (!rc) cudaMemsetAsync(c->d_chunk_count, 0, c->H.n_rows / kChunkRows * sizeof(int), c->st);
     }
-    if (!c->d_chunk_count) {
-        int rc = dalloc(c, &c->d_chunk_count, c->H.n_rows / kChunkRows);
-        if (rc) { free_groups(c); return rc; }
-        cudaMemsetAsync(c->d_chunk_count, 0, c->H.n_rows / kChunkRows * sizeof(int), c->st);
+    if (!rc && !c->d_partial2) rc = dalloc(c, &c->d_partial2, (size_t)c->n_samples * 64 * 16 * 3);
+    if (!rc && !c->d_sample_ticket) {
+        rc = dalloc(c, &c->d_sample_ticket, (size_t)c->n_samples);
+        if (!rc) cudaMemsetAsync(c->d_sample_ticket, 0, c->n_samples * sizeof(unsigned int), c->st);
     }
-    if (!c->d_partial2) {
-        int rc = dalloc(c, &c->d_partial2, (size_t)c->n_samples * 64 * 16 * 3);
-        if (!rc) rc = dalloc(c, &c->d_sample_ticket, (size_t)c->n_samples);
-        if (rc) { free_groups(c); return rc; }
-        cudaMemsetAsync(c->d_sample_ticket, 0, c->n_samples * sizeof(unsigned int), c->st);
-    }
+    if (rc) { free_groups(c); return rc; }
     c->prec = prec;
     c->group_states = c->n_states;
     return TBPM_OK;
@@ -901,7 +900,7 @@ static int ensure_fused(tbpm_ctx *c, int J, int R, int radius, int maxB, int gri
                 if (t >= 0 && t < T) items.push_back((int32_t)(((uint32_t)j << 25) | (uint32_t)t));
             }
         cudaFree(c->d_items);
-        c->d_items = nullptr;
+        c->items_key[0] = -1;
         int rc = dalloc(c, &c->d_items, items.size());
         if (rc) return rc;
         CUDA_OR_FAIL(c, cudaMemcpy(c->d_items, items.data(), items.size() * sizeof(int32_t),
@@ -911,29 +910,17 @@ static int ensure_fused(tbpm_ctx *c, int J, int R, int radius, int maxB, int gri
         c->items_key[1] = R;
         c->items_key[2] = D;
     }
-    if (c->done_len < (int64_t)J * T) {
-        cudaFree(c->d_done);
-        c->d_done = nullptr;
-        int rc = dalloc(c, &c->d_done, (size_t)J * T);
-        if (rc) return rc;
-        c->done_len = (int64_t)J * T;
-    }
+    int rc = grow(c, &c->d_done, &c->done_len, (int64_t)J * T);
+    if (rc) return rc;
     if (!c->d_fcounter) {
-        int rc = dalloc(c, &c->d_fcounter, 1);
+        rc = dalloc(c, &c->d_fcounter, 1);
         if (rc) return rc;
     }
     if (!c->d_fterms) {             // (the cluster stepping may have it already)
-        int rc = dalloc(c, &c->d_fterms, 3 * (size_t)kMaxTerms);
+        rc = dalloc(c, &c->d_fterms, 3 * (size_t)kMaxTerms);
         if (rc) return rc;
     }
-    if (c->tile_partial_len < T * maxB * 3) {
-        cudaFree(c->d_tile_partial);
-        c->d_tile_partial = nullptr;
-        int rc = dalloc(c, &c->d_tile_partial, (size_t)T * maxB * 3);
-        if (rc) return rc;
-        c->tile_partial_len = T * maxB * 3;
-    }
-    return TBPM_OK;
+    return grow(c, &c->d_tile_partial, &c->tile_partial_len, T * maxB * 3);
 }
 
 // The register-pipelined variant on long rows of real values (FP32): tbpm_propagate
@@ -1005,18 +992,11 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
         c->corr_states = c->n_states;
     }
     CUDA_OR_FAIL(c, cudaMemsetAsync(c->d_flags, 0, kFlagBytes, c->st));
-    {
-        const int64_t need = (int64_t)c->n_samples * c->n_states;
-        if (need > c->norm_ref_len) {
-            if (resume) return fail(c, TBPM_E_STATE, "nothing to resume for these states");
-            cudaFree(c->d_norm_ref);
-            c->d_norm_ref = nullptr;
-            c->norm_ref_len = 0;
-            rc = dalloc(c, &c->d_norm_ref, need);
-            if (rc) return rc;
-            c->norm_ref_len = need;
-        }
-    }
+    const int64_t n_ref = (int64_t)c->n_samples * c->n_states;
+    if (resume && n_ref > c->norm_ref_len)
+        return fail(c, TBPM_E_STATE, "nothing to resume for these states");
+    rc = grow(c, &c->d_norm_ref, &c->norm_ref_len, n_ref);
+    if (rc) return rc;
     if (c->ac_on && (!c->d_ac_corr || !c->d_ac_partial || !c->d_bond_dx))
         return fail(c, TBPM_E_STATE, "AC buffers missing");
 

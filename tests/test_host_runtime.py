@@ -213,3 +213,39 @@ def test_fused_after_cluster_keeps_no_memory(fake):
         clean()
         assert fake.fake_live() == 0
     """)
+
+
+# an allocation that fails while a context's buffers grow: a later, smaller run has
+# every buffer that a fresh context has (a null one would be written by a kernel)
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("config", [None, 1, 8])
+def test_buffers_are_whole_after_a_failed_growth(fake, prec, config):
+    run_script(fake, f"""
+        n, small, large = 3000, 1, 8
+        def context():
+            h = create()
+            if {config}: assert lib.tbpm_set_launch_config(h, {prec}, 8, 64, {config}) == 0
+            assert build(h, n) == 0
+            return h
+        def go(h, S, steps): return states(h, n, S) or run(h, S, steps, {prec})
+        h = context()
+        assert go(h, small, 5) == 0
+        whole = fake.fake_live()
+        lib.tbpm_destroy(h)
+        for first in (True, False):             # the growing run is the context's first, or not
+            k = 0
+            while True:
+                h = context()
+                if first: assert go(h, small, 5) == 0
+                fake.fake_reset(k)
+                rc = go(h, large, 5)
+                failed = fake.fake_failed()
+                fake.fake_reset(-1)
+                assert rc == (3 if failed else 0), (k, rc)
+                assert go(h, small, 5) == 0 and fake.fake_live() == whole, (first, k, fake.fake_live(), whole)
+                clean()
+                lib.tbpm_destroy(h)
+                assert fake.fake_live() == 0
+                if not failed: break
+                k += 1
+    """)
