@@ -1118,6 +1118,7 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
                                             c->H.fixed_width)
                        : 0;
 
+    if (!resume) c->have_run = false;       // the states go back to their start
     for (auto &g : c->groups) {
         const size_t bytes = (size_t)c->H.n_rows * g.B * cs;
         if (!resume) {

@@ -249,3 +249,19 @@ def test_buffers_are_whole_after_a_failed_growth(fake, prec, config):
                 if not failed: break
                 k += 1
     """)
+
+
+# a fresh run that fails after it has taken the states back to their start leaves
+# nothing to resume
+def test_a_failed_fresh_run_cannot_be_resumed(fake):
+    run_script(fake, """
+        h = create()
+        assert build(h, 700) == 0 and states(h, 700, 1) == 0
+        assert run(h, 1, 5, FP64, 8) == 0                    # TBPM_PROP_PERSISTENT
+        fake.fake_reset(0)                                   # the cluster stepping's state table
+        assert run(h, 1, 5, FP64) == 3 and fake.fake_failed() == 1
+        fake.fake_reset(-1)
+        assert run(h, 1, 5, FP64, 4) == 8                    # TBPM_PROP_RESUME: TBPM_E_STATE
+        assert run(h, 1, 5, FP64) == 0 and run(h, 1, 5, FP64, 4) == 0
+        clean()
+    """)
