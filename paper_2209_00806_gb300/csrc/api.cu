@@ -1030,27 +1030,40 @@ extern "C" int tbpm_propagate(tbpm_ctx *c, double z, int n_steps, int precision,
     //   120 nm, 4        3.7    2.4    11.8      36
     // so from 32 beyond 2^17 rows (between 30 and 60 nm), from 128 below.
     const bool long_rows = fp32 && takes_long_rows(c, variant);
-    int list_states = 0;
+    int list_states = 0, list_widths = 0;
     for (auto &g : c->groups)
-        if (g.B == 4 || g.B == 8) list_states += g.B;
+        if (g.B == 4 || g.B == 8) {
+            list_widths |= g.B;
+            if (!(g.B & c->H.no_lists)) list_states += g.B;
+        }
     const int64_t pays = c->H.n_rows >= ((int64_t)1 << 17) ? 32 : 128;
     if (long_rows && !c->H.halo_ptr) c->H.long_steps += (int64_t)n_steps * list_states;
-    const bool auto_lists = long_rows && list_states > 0 && !c->H.no_halo &&
+    const bool auto_lists = long_rows && list_states > 0 &&
                             (c->H.halo_ptr || (c->H.long_steps >= pays &&
                                                fits_beside(10 * (size_t)c->H.nnz_true)));
     const bool staged = auto_lists || (variant & kVariantStaged);
     bool halo = (auto_lists || (variant & kVariantHalo)) && !c->H.cplx &&
                 !(variant & (kVariantTma | kVariantFused));
-    if (halo && !c->H.halo_ptr) {
+    const bool had_lists = c->H.halo_ptr != nullptr;
+    if (halo && !had_lists) {
         std::string msg;
         rc = build_halo(c->H, c->st, msg);
         if (rc == TBPM_E_UNSUPPORTED || (rc == TBPM_E_OOM && auto_lists)) {
             halo = false;
-            c->H.no_halo |= auto_lists;     // the default does not try again
+            if (auto_lists) c->H.no_lists = 4 | 8;      // the default does not try again
         } else if (rc) return fail(c, rc, msg);
     }
+    if (halo && auto_lists) {
+        for (int B : {4, 8})
+            if (!staged_launchable(1, B, c->H.halo_max, c->H.halo_ent_max, 0)) c->H.no_lists |= B;
+        if (!(list_widths & ~c->H.no_lists)) {
+            // rows too long for a stage of these widths: new lists are given back
+            if (!had_lists) free_halo(c->H);
+            halo = false;
+        }
+    }
     // one-stage staged gathers with FP32 values per entry: rows in groups of four
-    if (halo && fp32 && staged && !c->H.uniform && list_states > 0) {
+    if (halo && fp32 && staged && !c->H.uniform && list_widths) {
         std::string msg;
         rc = build_groups(c->H, c->st, msg);
         if (rc) return fail(c, rc, msg);

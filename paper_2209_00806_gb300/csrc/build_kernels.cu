@@ -910,6 +910,29 @@ int build_diag2(BuildOutput &b, cudaStream_t st, std::string &msg)
     return TBPM_OK;
 }
 
+void free_halo(BuildOutput &b)
+{
+    cudaFree(b.halo_ptr);
+    cudaFree(b.halo_rows);
+    cudaFree(b.lcol);
+    cudaFree(b.pslice);
+    cudaFree(b.vpack[0]);
+    cudaFree(b.vpack[1]);
+    cudaFree(b.gptr);
+    cudaFree(b.gperm);
+    cudaFree(b.gpos);
+    cudaFree(b.gval);
+    b.halo_ptr = nullptr;
+    b.halo_rows = nullptr;
+    b.lcol = nullptr;
+    b.pslice = nullptr;
+    b.vpack[0] = b.vpack[1] = nullptr;
+    b.gptr = nullptr;
+    b.gperm = nullptr;
+    b.gpos = nullptr;
+    b.gval = nullptr;
+}
+
 void free_build(BuildOutput &b)
 {
     cudaFree(b.diag2_64);
@@ -923,16 +946,7 @@ void free_build(BuildOutput &b)
     cudaFree(b.diag32);
     cudaFree(b.chunk_sample);
     cudaFree(b.bond_rows);
-    cudaFree(b.halo_ptr);
-    cudaFree(b.halo_rows);
-    cudaFree(b.lcol);
-    cudaFree(b.pslice);
-    cudaFree(b.vpack[0]);
-    cudaFree(b.vpack[1]);
-    cudaFree(b.gptr);
-    cudaFree(b.gperm);
-    cudaFree(b.gpos);
-    cudaFree(b.gval);
+    free_halo(b);
     b = BuildOutput();
 }
 

@@ -603,7 +603,7 @@ struct BuildOutput {
     int64_t halo_total = 0;          // entries of all lists
     double *diag2_64 = nullptr;      // 2 d (FP64 one-value form; built on first use)
     int64_t long_steps = 0;          // FP32 states x steps run without the lists
-    int no_halo = 0;                 // tried by default: no lists for this matrix
+    int no_lists = 0;                // tried by default: widths (4 | 8) without staged gathers
     // row groups of the staged-gather kernel (build_groups)
     int64_t *gptr = nullptr;         // [n_rows / kHaloRows * 4 + 1] first list entry of each octet
     uint8_t *gperm = nullptr;        // [n_rows / kHaloRows][32] group at each slot
@@ -635,6 +635,7 @@ constexpr int kLanczosSteps = 64;          // the build's check
 int lanczos_extremes(const BuildOutput &H, int n_iter, cudaStream_t st, double *lo, double *hi,
                      int *steps, std::string &msg);
 
+void free_halo(BuildOutput &b);
 // Halo lists for TBPM_VARIANT_HALO (build_kernels.cu); TBPM_E_UNSUPPORTED
 // when a block references more than kHaloMaxExt other rows.
 int build_halo(BuildOutput &b, cudaStream_t st, std::string &msg);

@@ -37,3 +37,24 @@ def test_default_widths_are_bit_identical(S, kind):
                 out.append(phi)
     for a, b in zip(out[:3], out[3:]):
         assert (a == b).all()
+
+
+# rows too long for a stage of any width (340 entries): the default keeps no lists
+def test_lists_without_a_stage_are_given_back():
+    import numpy as np
+    import torch
+    import paper_2209_00806_gb300 as tb
+    n, w = 20000, 170
+    i = np.repeat(np.arange(n, dtype=np.int64), w)
+    j = (i + np.tile(np.arange(1, w + 1), n)) % n
+    v = np.random.default_rng(1).uniform(-0.05, 0.05, n * w)
+    theta = rng.phases(9, 4, n)
+    with tb.Propagator() as p:
+        p.build(n, None, i, j, v, 20.0)
+        p.set_phase_states(theta)
+        p.propagate(Z, 2, tb.TBPM_FP32)
+        before = torch.cuda.mem_get_info()[0]
+        p.propagate(Z, 40, tb.TBPM_FP32)
+        p.propagate(Z, 40, tb.TBPM_FP32)         # 168 states x steps and 328, of 128
+        # the lists and the values alone would be 41 MB
+        assert before - torch.cuda.mem_get_info()[0] < 8e6
