@@ -422,7 +422,11 @@ __global__ void __launch_bounds__(512, 1) k_cluster_steps_f32(ClusterArgs a)
         if (sum_waits > 0 && --sum_waits == 0 && rank == 0 && t < 32) cluster_sum(sum_step);
     };
     for (int n = 1;; ++n) {
-        next_vector();
+        if (pending) {                       // (the sums come a barrier later)
+            cl.barrier_wait();
+            pending = false;
+            --sum_waits;
+        }
         // step n - 2's factor, written before the barrier just passed: the same
         // for every thread of the cluster
         const float f = *(volatile float *)&rescale;
@@ -440,16 +444,24 @@ __global__ void __launch_bounds__(512, 1) k_cluster_steps_f32(ClusterArgs a)
             const FusedTerm tm = tt[j];
             const int xoff = (1 + (tm.x < 0 ? cur : tm.x)) * R;
             const uint32_t xoff_b = (uint32_t)xoff * (uint32_t)sizeof(float2);
-            const float scx = tm.x < 0 ? sc : 1.f;   // (no branch among the rows' gathers)
+            // the factors without branches among the rows' loads and gathers, which would
+            // cost their overlap.  Eight rows a thread are out of registers: with this
+            // form, 180 x 180, one value and values per entry, 24.6 and 26.2 us a step
+            // (24.3 and 26.2 without a norm carry), with that of fewer rows 25.0 and 26.5
+            const float scx = (RPT < 8 ? tm.x < 0 : j == 0) ? sc : 1.f;
             float2 p[RPT], zz[RPT];          // own rows: written only by this thread
 #pragma unroll
             for (int i = 0; i < RPT; ++i) {
                 const int row = min(t + i * T, R - 1);
                 p[i] = vec[(1 + cur) * R + row];
-                p[i].x *= sc;
-                p[i].y *= sc;
                 zz[i] = tm.z >= 0 ? vec[(1 + tm.z) * R + row] : make_float2(0.f, 0.f);
             }
+            if (RPT < 8 || sc != 1.f)
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) {
+                    p[i].x *= sc;
+                    p[i].y *= sc;
+                }
             next_vector();
             FF v0 = {0.f, 0.f}, v1 = v0, v2 = v0;
 #pragma unroll
